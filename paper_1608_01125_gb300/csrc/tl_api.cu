@@ -183,6 +183,8 @@ TLNarrowConst tl_narrow_const(double dt_fs, double kappa) {
     else sig = sigma_max;
     nk.sbin[i] = round_up(1e12 * kappa * std::min(sig * (1.0 + 1e-5), sigma_max) / TL_PI);
   }
+  nk.suf[TL_SBINS - 1] = nk.sbin[TL_SBINS - 1];
+  for (int i = TL_SBINS - 2; i >= 0; --i) nk.suf[i] = std::max(nk.sbin[i], nk.suf[i + 1]);
   return nk;
 }
 

@@ -135,10 +135,9 @@ constexpr int TL_SBIN_EMAX = 24;
 constexpr int TL_SBINS = 1 + TL_SBIN_OCT * TL_SBIN_EMAX;
 
 __device__ __forceinline__ int tl_sbin(float s) {
-  if (s < 1.0f) return 0;
-  const unsigned b = __float_as_uint(s);
-  const int i = 1 + ((int)(b >> 23) - 127) * TL_SBIN_OCT + (int)((b >> 20) & 7u);
-  return i < TL_SBINS - 1 ? i : TL_SBINS - 1;
+  // below 1 (and below 0) the shifted bits are smaller: bin 0
+  const int i = (__float_as_int(s) >> 20) - 127 * TL_SBIN_OCT + 1;
+  return min(max(i, 0), TL_SBINS - 1);
 }
 
 struct TLNarrowConst {
@@ -152,6 +151,7 @@ struct TLNarrowConst {
   // per bin of s (tl_sbin): an upper bound on r^2 = 1e12 kappa sigma(s) / pi
   // over the bin [um^2] (sigma rises up to its peak near s = 1.97, then falls)
   float sbin[TL_SBINS];
+  float suf[TL_SBINS];  // the largest sbin of the bin or any above it
 };
 
 // Build-time launch helpers (defined in the .cu files).

@@ -102,3 +102,31 @@ __device__ __forceinline__ bool tl_exact_hit(const TLBeam &A, uint32_t i, const 
   return tl_exact_decide(A.px[i], A.py[i], A.pz[i], A.dx[i], A.dy[i], A.dz[i], A.E[i], B.px[j],
                          B.py[j], B.pz[j], B.dx[j], B.dy[j], B.dz[j], B.E[j], ct, dt, kappa);
 }
+
+// true if the decision above is surely false, found without a division, a square root
+// or the logarithm (GB300 does 2 FP64 operations per clock and SM, a division is ~10):
+// below threshold, closest approach outside the window, or farther than r2max, an
+// upper bound of r^2 over s.  |p x v|^2 / v.v is the squared distance; the margins
+// are orders of magnitude above the FP64 rounding of either form.
+__device__ __forceinline__ bool tl_exact_sure_miss(const TLBeam &A, uint32_t i, const TLBeam &B,
+                                                   uint32_t j, double ct, double dt,
+                                                   double r2max) {
+  const double ax = A.dx[i], ay = A.dy[i], az = A.dz[i], bx = B.dx[j], by = B.dy[j], bz = B.dz[j];
+  const double cs = ax * bx + ay * by + az * bz;
+  if (A.E[i] * B.E[j] * (1.0 - cs) < (2.0 * TL_MEC2) * TL_MEC2 * (1.0 - 1e-12) - 1e-14 * A.E[i] * B.E[j])
+    return true;
+  const double vx = TL_C * (ax - bx), vy = TL_C * (ay - by), vz = TL_C * (az - bz);
+  const double vv = vx * vx + vy * vy + vz * vz;
+  const double px = (A.px[i] + ct * ax) - (B.px[j] + ct * bx);
+  const double py = (A.py[i] + ct * ay) - (B.py[j] + ct * by);
+  const double pz = (A.pz[i] + ct * az) - (B.pz[j] + ct * bz);
+  // rounding of the positions themselves, far above it
+  const double sa = fabs(A.px[i]) + fabs(B.px[j]) + fabs(A.py[i]) + fabs(B.py[j]) +
+                    fabs(A.pz[i]) + fabs(B.pz[j]) + 8.0 * fabs(ct);
+  const double pv = px * vx + py * vy + pz * vz;
+  const double ev = 1e-12 * (sa * (fabs(vx) + fabs(vy) + fabs(vz)) + dt * vv) + 1e-200;
+  if (pv > ev || -pv - dt * vv > ev) return true;
+  const double cx = py * vz - pz * vy, cy = pz * vx - px * vz, cz = px * vy - py * vx;
+  const double lim = r2max * (1.0 + 1e-9) + 1e-11 * sa * sa;
+  return cx * cx + cy * cy + cz * cz > vv * lim;
+}

@@ -92,13 +92,37 @@ __device__ __forceinline__ TLNarrowPre tl_narrow32_pre(const float4 pa, const fl
   return r;
 }
 
-// true when the prefix alone makes the pair a sure miss (exactly when
-// tl_narrow32 returns TL_MISS before its error bounds)
-__device__ __forceinline__ bool tl_narrow32_quick_miss(const float4 pa, const float4 da,
-                                                       const float4 pb, const float4 db,
-                                                       const TLNarrowConst &k,
-                                                       const float *sbin) {
-  return tl_narrow32_pre(pa, da, pb, db, k, sbin).early == TL_MISS;
+// The first look at a photon pair: true if it is a sure miss by the threshold or the
+// quick miss above.  It decides most pairs, so it is straight-line code of ~60
+// instructions: one table lookup (k.suf: the largest sbin of the bin or any above it,
+// which covers every s64 >= s - es; suf is its copy in shared memory) and an approximate reciprocal, whose 2u of |tau| raise
+// the last term of dq to |tau||dD| 9.1u <= |q|/14, so dq <= 0.26 |q| and
+// ed2 <= 0.59 d2: 2.5 (1 - 0.59) > 1 still holds.
+__device__ __forceinline__ bool tl_narrow32_sure_miss(const float4 pa, const float4 da,
+                                                      const float4 pb, const float4 db,
+                                                      const TLNarrowConst &k,
+                                                      const float *suf) {
+  const float u = 5.9604644775390625e-8f;  // 2^-24
+  const float cs = fmaf(da.x, db.x, fmaf(da.y, db.y, da.z * db.z));
+  const float eek = (pa.w * pb.w) * k.inv2mc4;
+  const float s = eek * (1.0f - cs);
+  const float es = 2.0f * (9.0f * u * s + 6.0f * u * eek);
+  const bool below = s + es <= 1.0f - 9.5367431640625e-7f;
+  const float dpx = pa.x - pb.x, dpy = pa.y - pb.y, dpz = pa.z - pb.z;
+  const float ddx = da.x - db.x, ddy = da.y - db.y, ddz = da.z - db.z;
+  const float dd = fmaf(ddx, ddx, fmaf(ddy, ddy, ddz * ddz));
+  const float pd = fmaf(dpx, ddx, fmaf(dpy, ddy, dpz * ddz));
+  float rdd;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rdd) : "f"(dd));
+  const float tau = -pd * rdd;
+  const float qx = fmaf(tau, ddx, dpx), qy = fmaf(tau, ddy, dpy), qz = fmaf(tau, ddz, dpz);
+  const float d2 = fmaf(qx, qx, fmaf(qy, qy, qz * qz));
+  const float SA =
+      (fabsf(pa.x) + fabsf(pb.x)) + (fabsf(pa.y) + fabsf(pb.y)) + (fabsf(pa.z) + fabsf(pb.z));
+  const float at = fabsf(tau);
+  const float lim = fmaxf(2.5f * suf[tl_sbin(__fsub_rd(s, es))], at <= 4.0f ? 0x1p-26f : 0x1p-12f);
+  return below ||
+         (dd >= 0x1p-30f && at <= 1024.0f && d2 >= lim && SA * SA <= 0x1p36f * d2);
 }
 
 __device__ __forceinline__ int tl_narrow32(const float4 pa, const float4 da, const float4 pb,

@@ -59,7 +59,11 @@ __global__ void __launch_bounds__(kThreads) k_band_stress(unsigned long long bas
   __shared__ unsigned long long sc[kCats * kFields];
   __shared__ float sbin[TL_SBINS];
   for (int t = threadIdx.x; t < kCats * kFields; t += kThreads) sc[t] = 0ull;
-  for (int t = threadIdx.x; t < TL_SBINS; t += kThreads) sbin[t] = nk.sbin[t];
+  __shared__ float suf[TL_SBINS];
+  for (int t = threadIdx.x; t < TL_SBINS; t += kThreads) {
+    sbin[t] = nk.sbin[t];
+    suf[t] = nk.suf[t];
+  }
   __syncthreads();
   const double two_m2 = (2.0 * TL_MEC2) * TL_MEC2;
   for (int64_t q = q0 + blockIdx.x * (int64_t)kThreads + threadIdx.x; q < q0 + n;
@@ -130,7 +134,10 @@ __global__ void __launch_bounds__(kThreads) k_band_stress(unsigned long long bas
                                   __double2float_rn(dzi), 0.0f);
     const float4 db = make_float4(__double2float_rn(dxj), __double2float_rn(dyj),
                                   __double2float_rn(dzj), 0.0f);
-    const int r32 = tl_narrow32(pa, da, pb, db, nk, sbin);
+    // the first look, then the full test, as the narrow phase decides
+    const int r32 = tl_narrow32_sure_miss(pa, da, pb, db, nk, suf)
+                        ? (int)TL_MISS
+                        : tl_narrow32(pa, da, pb, db, nk, sbin);
     unsigned long long *c = sc + cat * kFields;
     atomicAdd(c + 0, 1ull);
     if (hit) atomicAdd(c + 1, 1ull);
