@@ -15,27 +15,15 @@
 #include "trilens_debug.h"
 
 namespace tl {
-cudaError_t launch_step_init(TLCounters *ctr, uint2 *F0, uint32_t sa, uint32_t sb, int nonempty,
-                             const unsigned *build_status, const unsigned *run_status,
-                             cudaStream_t s);
-cudaError_t launch_expand(const TravArgs &a, uint2 *F0, uint2 *F1, unsigned cap, unsigned target,
-                          int max_levels, cudaStream_t s);
-cudaError_t launch_seed_cut(const TravArgs &a, const uint32_t *cutA, const unsigned *cntA,
-                            uint32_t capA, const uint32_t *cutB, const unsigned *cntB,
-                            uint32_t capB, uint2 *F0, unsigned cap, int blocks, cudaStream_t s);
 cudaError_t traverse_config(int fp64, int warps, int depth, int *blocks_per_sm);
-cudaError_t launch_widen(const TravArgs &a, uint2 *F0, uint2 *F1, unsigned cap, unsigned target,
-                         int levels, int blocks, cudaStream_t s);
 cudaError_t launch_narrow(const TravArgs &a, int blocks, cudaStream_t s);
-cudaError_t launch_traverse(const TravArgs &a, const uint2 *F0, const uint2 *F1, const uint2 *list,
-                            unsigned long long list_n, int from_frontier, int budget, int blocks,
-                            int warps, cudaStream_t s, int part, int nparts);
+cudaError_t launch_traverse(const TravArgs &a, const uint2 *list, unsigned long long list_n,
+                            int budget, int blocks, int warps, cudaStream_t s, int part,
+                            int nparts);
 cudaError_t launch_part_init(TLCounters *ctr, cudaStream_t s);
 cudaError_t launch_band(const TravArgs &a, int blocks, cudaStream_t s);
 cudaError_t launch_yield(const TravArgs &a, void *partials, int blocks, cudaStream_t s);
 size_t partial_bytes();
-cudaError_t launch_seed_instances(TLCounters *ctr, uint2 *F0, const uint32_t *rootA,
-                                  const uint32_t *rootB, int n_inst, cudaStream_t s);
 cudaError_t launch_yield_inst(const TravArgs &a, const uint32_t *inst_of_a, double *yields,
                               int blocks, cudaStream_t s);
 cudaError_t launch_pair_products(const TLBeam &a, const TLBeam &b, const uint32_t *hits,
@@ -50,13 +38,10 @@ enum {
   PH_NARROW, PH_COUNT
 };
 
-// breadth-first levels that may widen the seed frontier of a large problem
-// (each a launch that does nothing once the frontier holds widen_target pairs)
-constexpr int kWidenLevels = 5;
 // node pairs per traversal queue chunk and frontier item (tl_traverse.cu)
 constexpr unsigned long long kQueueChunk = 32;
-// the leaf-pair list never grows past 2^30 pairs (8 GiB): a step that lists
-// more is done in parts, slices of its frontier, each listing at most that
+// the list of candidate (or leaf-bucket) pairs never grows past 2^30 pairs (8 GiB): a step that lists
+// more is done in parts, each listing at most that
 constexpr unsigned long long kLeafListMax = 1ull << 30;
 
 // after a step overflowed the leaf-pair list (the largest part listed need
@@ -78,34 +63,78 @@ static int leaves_for(trilens_ctx *c, unsigned long long need) {
   return TRILENS_OK;
 }
 
-// the traversal and the narrow phase of a step, part by part
-static int traverse_parts(trilens_ctx *c, const tl::TravArgs &a, const uint2 *seeds,
-                          unsigned n_seeds) {
-  for (int p = 0; p < c->parts; ++p) {
-    if (p > 0) CK(tl::launch_part_init(c->ctr, c->stream));
-    CK(tl::launch_traverse(a, c->front[0], c->front[1], seeds, seeds ? n_seeds : 0, seeds ? 0 : 1,
-                           c->budget, c->trav_blocks, c->trav_warps, c->stream, p, c->parts));
-    CK(tl::launch_narrow(a, 8 * c->n_sm, c->stream));
-  }
-  return TRILENS_OK;
-}
-
-// the frontier widening target: 64 pairs per resident traversal warp, two
-// full items each; and the frontier buffers' capacity for every start
-static void frontier_sizes(trilens_ctx *c, unsigned *target, unsigned *cap) {
-  const long long warps = (long long)c->trav_blocks * c->trav_warps;
-  *target = (unsigned)std::min<long long>(64ll * warps, 1 << 22);
-  const unsigned long long need =
-      std::max({(unsigned long long)c->n_inst + 4ull * c->front_target + 64,
-                (unsigned long long)c->w[0].cut_cap * c->w[1].cut_cap + 64,
-                4ull * *target + 64});
-  *cap = (unsigned)std::min<unsigned long long>(need, 0xFFFFFFF0ull);
-}
-
 static void tmark(trilens_ctx *c, int ph, int k, int end) {
   if (!c->timing) return;
   cudaEventRecord(c->ev[ph][k][end], c->stream);
   if (end) c->ev_pending[ph][k] = true;
+}
+
+// warps of k_collide that keep every SM busy: fewer groups of 32 photons than this
+// are each given several warps, on parts of the tree (2 x 2048 photons have 64 groups)
+constexpr int kColWarpsPerSm = 24;
+
+// the groups of 32 query photons of part p of the step, and the kernel's arguments
+static tl::ColArgs col_args(trilens_ctx *c, int p) {
+  const int q = 1 - c->tree, t = c->tree;
+  tl::ColArgs a;
+  memset(&a, 0, sizeof(a));
+  a.qpos = c->w[q].pos;
+  a.qdir = c->w[q].dir;
+  a.tpos = c->w[t].pos;
+  a.tdir = c->w[t].dir;
+  a.box = c->box;
+  a.qinst = c->insts[q];
+  a.tinst = c->insts[t];
+  a.tile_inst = c->tile_inst[q];
+  a.frames = c->frames;
+  a.Llo = c->L_lo;
+  a.Lhi = c->L_hi;
+  a.half = c->half;
+  a.nk = c->nk;
+  a.ctr = c->ctr;
+  a.cand = c->leaves;
+  a.cand_cap = c->leaf_cap;
+  const long long groups = 32ll * c->n_tiles[q];
+  const long long g0 = groups * p / c->parts, g1 = groups * (p + 1) / c->parts;
+  a.group0 = (int)g0;
+  a.slices = 1;
+  if (g1 > g0)
+    a.slices = (int)std::min<long long>(
+        64, std::max<long long>(1, (long long)kColWarpsPerSm * c->n_sm / (g1 - g0)));
+  a.items = c->n_tiles[t] > 0 ? (g1 - g0) * a.slices : 0;
+  a.fp64 = c->p.precision == TRILENS_FP64;
+  a.swap = t == 0;
+  return a;
+}
+
+// the collisions of a step up to its candidates' decisions, part by part
+static int collide_parts(trilens_ctx *c, const tl::TravArgs &a) {
+  for (int p = 0; p < c->parts; ++p) {
+    if (p > 0) CK(tl::launch_part_next(c->ctr, c->stream));
+    tmark(c, PH_TRAV, 0, 0);  // (of several parts the last is timed)
+    CK(tl::launch_collide(col_args(c, p), c->stream));
+    tmark(c, PH_TRAV, 0, 1);
+    tmark(c, PH_NARROW, 0, 0);
+    CK(tl::launch_decide(a, 8 * c->n_sm, c->stream));
+    tmark(c, PH_NARROW, 0, 1);
+  }
+  return TRILENS_OK;
+}
+
+// the seeded traversal and its narrow phase, part by part
+static int traverse_parts(trilens_ctx *c, const tl::TravArgs &a, const uint2 *seeds,
+                          unsigned n_seeds) {
+  for (int p = 0; p < c->parts; ++p) {
+    if (p > 0) CK(tl::launch_part_init(c->ctr, c->stream));
+    tmark(c, PH_TRAV, 0, 0);
+    CK(tl::launch_traverse(a, seeds, n_seeds, c->budget, c->trav_blocks, c->trav_warps, c->stream,
+                           p, c->parts));
+    tmark(c, PH_TRAV, 0, 1);
+    tmark(c, PH_NARROW, 0, 0);
+    CK(tl::launch_narrow(a, 8 * c->n_sm, c->stream));
+    tmark(c, PH_NARROW, 0, 1);
+  }
+  return TRILENS_OK;
 }
 
 // add the elapsed time of every recorded phase (the stream is synchronised)
@@ -193,10 +222,12 @@ static void free_beam(tl::BuildBufs &w) {
   cudaFree(w.dir_u);
   cudaFree(w.pos);
   cudaFree(w.dir);
-  cudaFree(w.key[0]);
-  cudaFree(w.key[1]);
+  cudaFree(w.key32[0]);
+  cudaFree(w.key32[1]);
   cudaFree(w.val[0]);
   cudaFree(w.val[1]);
+  cudaFree(w.key[0]);
+  cudaFree(w.key[1]);
   cudaFree(w.nodes);
   cudaFree(w.parent_leaf);
   cudaFree(w.parent_node);
@@ -204,8 +235,6 @@ static void free_beam(tl::BuildBufs &w) {
   cudaFree(w.rsuf);
   cudaFree(w.rtile);
   cudaFree(w.rsuper);
-  cudaFree(w.cut);
-  cudaFree(w.cut_n);
   cudaFree(w.nfirst);
   cudaFree(w.nlast);
   cudaFree(w.nlev);
@@ -217,34 +246,17 @@ static void free_beam(tl::BuildBufs &w) {
   memset(&w, 0, sizeof(w));
 }
 
-static int alloc_beam(trilens_ctx *c, tl::BuildBufs &w, int64_t n) {
-  size_t m = (size_t)std::max<int64_t>(n, 1);
+// the buffers every step needs: SoAs, keys and sort scratch
+static int alloc_beam(trilens_ctx *c, tl::BuildBufs &w, int64_t n, int64_t padded) {
+  const size_t m = (size_t)std::max<int64_t>(n, 1), mp = (size_t)std::max<int64_t>(padded, 1);
   CK(dalloc(&w.pos_u, m));
   CK(dalloc(&w.dir_u, m));
-  CK(dalloc(&w.pos, m));
-  CK(dalloc(&w.dir, m));
-  CK(dalloc(&w.key[0], m));
-  CK(dalloc(&w.key[1], m));
-  CK(dalloc(&w.val[0], m));
-  CK(dalloc(&w.val[1], m));
-  CK(dalloc(&w.nodes, m));
-  CK(dalloc(&w.parent_leaf, m));
-  CK(dalloc(&w.parent_node, m));
-  CK(dalloc(&w.rpre, 6 * m));
-  CK(dalloc(&w.rsuf, 6 * m));
-  CK(dalloc(&w.rtile, 6 * (size_t)tl::refit_tiles((int64_t)m)));
-  CK(dalloc(&w.rsuper, tl::refit_super_floats((int64_t)m)));
-  CK(dalloc(&w.nfirst, m));
-  CK(dalloc(&w.nlast, m));
-  CK(dalloc(&w.nlev, m));
-  // traversal seeds for beams of 2^17 photons or more: about 256-512 cut nodes
-  // (more where small siblings hang off long chains; past the capacity the
-  // traversal starts from the roots)
-  w.cut_S = n >= 131072 ? (uint32_t)(n >> 8) : 0u;
-  w.cut_cap = w.cut_S ? (uint32_t)(8 * (n / w.cut_S) + 32) : 0u;
-  w.cut_alloc = w.cut_cap;
-  CK(dalloc(&w.cut, std::max<size_t>(w.cut_cap, 1)));
-  CK(dalloc(&w.cut_n, 1));
+  CK(dalloc(&w.pos, mp));
+  CK(dalloc(&w.dir, mp));
+  for (int k = 0; k < 2; ++k) {
+    CK(dalloc(&w.key32[k], m));
+    CK(dalloc(&w.val[k], m));
+  }
   w.sort_tiles = (int64_t)((m + TL_SORT_TILE - 1) / TL_SORT_TILE);
   w.sort_epoch = 0;
   CK(dalloc(&w.sort_status, (size_t)w.sort_tiles * 256));
@@ -254,6 +266,119 @@ static int alloc_beam(trilens_ctx *c, tl::BuildBufs &w, int64_t n) {
   CK(dalloc(&w.sort_hist, 8 * 256));
   CK(dalloc(&w.sort_tile, 8));
   return TRILENS_OK;
+}
+
+// the statistical regime's hierarchies and the seeded traversal's queues, on first use
+static int ensure_full(trilens_ctx *c) {
+  if (c->full_ready) return TRILENS_OK;
+  for (int k = 0; k < 2; ++k) {
+    tl::BuildBufs &w = c->w[k];
+    const size_t m = (size_t)std::max<int64_t>(c->beam[k].n, 1);
+    CK(dalloc(&w.key[0], m));
+    CK(dalloc(&w.key[1], m));
+    CK(dalloc(&w.nodes, m));
+    CK(dalloc(&w.parent_leaf, m));
+    CK(dalloc(&w.parent_node, m));
+    CK(dalloc(&w.rpre, 6 * m));
+    CK(dalloc(&w.rsuf, 6 * m));
+    CK(dalloc(&w.rtile, 6 * (size_t)tl::refit_tiles((int64_t)m)));
+    CK(dalloc(&w.rsuper, tl::refit_super_floats((int64_t)m)));
+    CK(dalloc(&w.nfirst, m));
+    CK(dalloc(&w.nlast, m));
+    CK(dalloc(&w.nlev, m));
+  }
+  const unsigned long long warps = (unsigned long long)c->trav_blocks * c->trav_warps;
+  int rc = alloc_queue(c, std::max<unsigned long long>(
+                              1 << 20, 2ull * warps * (unsigned long long)c->p.stack_depth));
+  if (rc) return rc;
+  if ((rc = alloc_spill(c, c->spill_per_warp, warps))) return rc;
+  // leaf-bucket pairs: 16 per photon to start, at most 2^29 (4 GiB) before a step
+  // asks for more
+  const unsigned long long cap = std::min<unsigned long long>(
+      std::max<unsigned long long>(1 << 20, 16ull * (c->beam[0].n + c->beam[1].n)), 1ull << 29);
+  if (c->leaf_cap < cap) {
+    cudaFree(c->leaves);
+    c->leaves = nullptr;
+    c->leaf_cap = 0;
+    CK(dalloc(&c->leaves, (size_t)cap));
+    c->leaf_cap = cap;
+  }
+  c->full_ready = true;
+  return TRILENS_OK;
+}
+
+// one instance's part of a beam of n photons: its tiles, and the levels of its tree
+static TLInst make_inst(int64_t n, int64_t off, int64_t tile0) {
+  TLInst I;
+  memset(&I, 0, sizeof(I));
+  I.n = (int)n;
+  I.tile0 = (int)tile0;
+  I.pad = (int)(tile0 * kTile - off);
+  I.cnt[0] = (int)n;
+  for (int l = 1; l < 6; ++l) I.cnt[l] = (I.cnt[l - 1] + 31) / 32;
+  I.top = 1;
+  while (I.top < 5 && I.cnt[I.top] > 32) ++I.top;
+  return I;
+}
+
+// The exact path's layout of both beams (sizes[k]: photons of every instance).
+static int layout(trilens_ctx *c, const std::vector<int64_t> sizes[2]) {
+  c->tree = c->beam[1].n <= c->beam[0].n ? 1 : 0;
+  const size_t ni = sizes[0].size();
+  for (int k = 0; k < 2; ++k) {
+    std::vector<TLInst> in(ni);
+    std::vector<uint32_t> tile_inst;
+    std::vector<int> pad(ni);
+    int64_t off = 0, tile = 0;
+    for (size_t q = 0; q < ni; ++q) {
+      in[q] = make_inst(sizes[k][q], off, tile);
+      pad[q] = in[q].pad;
+      const int64_t t = (sizes[k][q] + kTile - 1) / kTile;
+      if (ni > 1) tile_inst.insert(tile_inst.end(), (size_t)t, (uint32_t)q);
+      off += sizes[k][q];
+      tile += t;
+    }
+    c->n_tiles[k] = (int)tile;
+    if (k == c->tree) {  // levels 0..2 tile by tile, then what is above
+      uint64_t up = (uint64_t)tile * (kTile + 32 + 1);
+      for (size_t q = 0; q < ni; ++q) {
+        in[q].lev[0] = (uint32_t)((uint64_t)in[q].tile0 * kTile);
+        in[q].lev[1] = (uint32_t)((uint64_t)tile * kTile + (uint64_t)in[q].tile0 * 32);
+        in[q].lev[2] = (uint32_t)((uint64_t)tile * (kTile + 32) + (uint64_t)in[q].tile0);
+        for (int l = 3; l <= in[q].top; ++l) {
+          in[q].lev[l] = (uint32_t)up;
+          up += (uint64_t)in[q].cnt[l];
+        }
+        c->max_top = std::max(c->max_top, in[q].top);
+      }
+      CK(dalloc(&c->box, 2 * (size_t)up));
+    }
+    CK(dalloc(&c->insts[k], ni));
+    CK(cudaMemcpyAsync(c->insts[k], in.data(), sizeof(TLInst) * ni, cudaMemcpyHostToDevice,
+                       c->stream));
+    if (ni > 1) {
+      CK(dalloc(&c->tile_inst[k], tile_inst.size()));
+      CK(cudaMemcpyAsync(c->tile_inst[k], tile_inst.data(), sizeof(uint32_t) * tile_inst.size(),
+                         cudaMemcpyHostToDevice, c->stream));
+      CK(dalloc(&c->pad[k], ni));
+      CK(cudaMemcpyAsync(c->pad[k], pad.data(), sizeof(int) * ni, cudaMemcpyHostToDevice,
+                         c->stream));
+    }
+    const int rc = alloc_beam(c, c->w[k], c->beam[k].n, tile * kTile);
+    if (rc) return rc;
+    CK(cudaStreamSynchronize(c->stream));  // the host tables are read
+  }
+  CK(dalloc(&c->frames, ni));
+  return TRILENS_OK;
+}
+
+// bits of the order keys for a largest instance of n photons: 4 cells per photon
+// spread evenly, so a few photons per cell where a Gaussian bunch is densest, rounded
+// up to whole 8-bit sort passes together with the instance number's bits
+static int order_bits_for(int64_t n, int inst_bits) {
+  int lg = 0;
+  while ((1ll << lg) < n) ++lg;
+  return std::min(30, std::min(32, 8 * ((lg + 2 + inst_bits + 7) / 8)) - inst_bits);
 }
 
 // ---- C ABI
@@ -290,8 +415,6 @@ void trilens_destroy(trilens_ctx *c) {
   else cudaDeviceSynchronize();
   free_beam(c->w[0]);
   free_beam(c->w[1]);
-  cudaFree(c->front[0]);
-  cudaFree(c->front[1]);
   cudaFree(c->queue);
   cudaFree(c->run_acc);
   cudaFree(c->hits);
@@ -307,11 +430,15 @@ void trilens_destroy(trilens_ctx *c) {
   cudaFreeHost(c->build_status_host);
   for (int k = 0; k < 2; ++k) {
     cudaFree(c->inst_of[k]);
-    cudaFree(c->inst_root[k]);
     cudaFree(c->inst_bounds[k]);
-    cudaFree(c->inst_box[k]);
+    cudaFree(c->insts[k]);
+    cudaFree(c->tile_inst[k]);
+    cudaFree(c->pad[k]);
+    cudaFree(c->grids[k]);
     for (int a = 0; a < 8; ++a) cudaFree(c->owned[k][a]);
   }
+  cudaFree(c->frames);
+  cudaFree(c->box);
   cudaFree(c->inst_tmp);
   cudaFree(c->run_status);
   cudaFreeHost(c->run_status_host);
@@ -327,8 +454,13 @@ void trilens_destroy(trilens_ctx *c) {
   delete c;
 }
 
-int trilens_create(trilens_ctx **out, const trilens_beam *a, const trilens_beam *b,
-                   const trilens_params *p, trilens_stream_t stream) {
+}  // extern "C"
+
+// Create a context; sizes NULL for a single problem, else the photons of every
+// instance of each beam.
+static int ctx_create(trilens_ctx **out, const trilens_beam *a, const trilens_beam *b,
+                      const trilens_params *p, trilens_stream_t stream,
+                      const std::vector<int64_t> *sizes) {
   if (!out) return TRILENS_ERR_INVALID;
   *out = nullptr;
   if (!beam_ok(a) || !beam_ok(b) || !p) return TRILENS_ERR_INVALID;
@@ -370,29 +502,53 @@ int trilens_create(trilens_ctx **out, const trilens_beam *a, const trilens_beam 
   CK(dalloc(&c->build_status, 1));
   CK(cudaMallocHost((void **)&c->build_status_host, sizeof(unsigned)));
   CK(cudaMemsetAsync(c->build_status, 0, sizeof(unsigned), c->stream));
+  const std::vector<int64_t> one[2] = {{c->beam[0].n}, {c->beam[1].n}};
+  if ((rc = layout(c, sizes ? sizes : one))) {
+    trilens_destroy(c);
+    return rc;
+  }
   for (int k = 0; k < 2; ++k) {
-    if ((rc = alloc_beam(c, c->w[k], c->beam[k].n))) {
-      trilens_destroy(c);
-      return rc;
-    }
     c->w[k].build_status = c->build_status;
     // the step-invariant FP32 direction, index and energy, once
     CK(tl::launch_static_soa(c->beam[k], c->w[k], c->stream));
     int64_t n = std::max<int64_t>(c->beam[k].n, 2);
     int lg = 0;
     while ((1ll << lg) < n) ++lg;
-    // Morton resolution: one bit per axis beyond one cell per photon (at 2 x 1M
-    // head-on: 24-bit keys, 3 sort passes; 27 or 30 bits traverse as fast but
-    // take 4 passes; 21 bits slow the traversal by a third)
+    // Morton resolution: one bit per axis beyond one cell per photon
     c->bits[k] = std::min(21, std::max(4, (lg + 2) / 3 + 1));
     c->key_bits[k] = 3 * c->bits[k];
     c->w[k].key_bits = c->key_bits[k];
-    // one-time moments of p0 and d for the Morton box of every step
+  }
+  if (!sizes) {
+    c->order_bits = order_bits_for(std::max(c->beam[0].n, c->beam[1].n), 0);
+    // one-time moments of p0 and d: in the lab frame for the mean directions (the
+    // frame) and the Morton boxes, then in the frame for the grids of every step
     double *mom = nullptr;
-    CK(cudaMalloc((void **)&mom, sizeof(double) * 15 * (1 + 4 * 152)));
-    cudaError_t me = tl::launch_beam_moments(c->beam[k], mom, mom + 15, c->stream);
+    const size_t md = tl::moment_doubles();
+    CK(cudaMalloc((void **)&mom, sizeof(double) * 2 * md));
+    cudaError_t me = cudaSuccess;
+    c->frame0 = tl_ident_frame();
+    for (int pass = 0; pass < 2 && !me; ++pass) {
+      double(*dst)[15] = pass ? c->fmoments : c->moments;
+      for (int k = 0; k < 2 && !me; ++k) {
+        me = tl::launch_beam_moments(c->beam[k], c->frame0, mom + k * md, c->stream);
+        if (!me)
+          me = cudaMemcpyAsync(dst[k], mom + k * md, sizeof(double) * 15, cudaMemcpyDeviceToHost,
+                               c->stream);
+      }
+      if (!me) me = cudaStreamSynchronize(c->stream);
+      if (pass || me) break;
+      memcpy(c->fmoments, c->moments, sizeof(c->moments));
+      if (c->beam[0].n > 0 && c->beam[1].n > 0) {
+        double mean[2][3];
+        for (int k = 0; k < 2; ++k)
+          for (int x = 0; x < 3; ++x) mean[k][x] = c->moments[k][3 + x] / (double)c->beam[k].n;
+        c->frame0 = tl_make_frame(mean[0], mean[1]);
+      }
+      if (c->frame0.ident) break;  // the same moments
+    }
     if (!me)
-      me = cudaMemcpyAsync(c->moments[k], mom, sizeof(double) * 15, cudaMemcpyDeviceToHost,
+      me = cudaMemcpyAsync(c->frames, &c->frame0, sizeof(TLFrame), cudaMemcpyHostToDevice,
                            c->stream);
     if (!me) me = cudaStreamSynchronize(c->stream);
     cudaFree(mom);
@@ -411,33 +567,16 @@ int trilens_create(trilens_ctx **out, const trilens_beam *a, const trilens_beam 
     return TRILENS_ERR_INVALID;
   }
   c->trav_blocks = bps * c->n_sm;
-  c->expand_blocks = 2 * c->n_sm;
-  c->front_target = (unsigned)std::min<long long>(2ll * c->trav_blocks * c->trav_warps, 1 << 16);
-  frontier_sizes(c, &c->widen_target, &c->front_cap);
-  CK(dalloc(&c->front[0], c->front_cap));
-  CK(dalloc(&c->front[1], c->front_cap));
-  {
-    const int rcq = alloc_queue(c, std::max<unsigned long long>(
-                                       1 << 20, 2ull * c->trav_blocks * c->trav_warps *
-                                                    (unsigned long long)c->p.stack_depth));
-    if (rcq) {
-      trilens_destroy(c);
-      return rcq;
-    }
-  }
-  if ((rc = alloc_spill(c, c->spill_per_warp, (unsigned long long)c->trav_blocks * c->trav_warps))) {
-    trilens_destroy(c);
-    return rc;
-  }
   c->hit_cap = std::max<unsigned long long>(1 << 16, 2ull * (c->beam[0].n + c->beam[1].n));
   CK(dalloc(&c->hits, c->hit_cap));
   c->band_cap = std::max<unsigned long long>(1 << 16, (c->beam[0].n + c->beam[1].n) / 4);
   CK(dalloc(&c->band, c->band_cap));
-  // the leaf-pair list: 16 per photon to start (a busy step of 2 x 1M
-  // head-on lists ~2.6e7 with single-photon buckets), at most 2^29 (4 GiB)
-  // before a step asks for more
+  // candidate pairs: what the first look leaves, of the order of the hits; in FP64 mode
+  // every pair of overlapping boxes.  Grown when a step asks for more.
   c->leaf_cap = std::min<unsigned long long>(
-      std::max<unsigned long long>(1 << 20, 16ull * (c->beam[0].n + c->beam[1].n)), 1ull << 29);
+      std::max<unsigned long long>(1 << 18, (c->p.precision == TRILENS_FP64 ? 16ull : 2ull) *
+                                                (c->beam[0].n + c->beam[1].n)),
+      1ull << 29);
   CK(dalloc(&c->leaves, c->leaf_cap));
   CK(dalloc(&c->ctr, 1));
   CK(cudaMallocHost((void **)&c->ctr_host, sizeof(TLCounters)));
@@ -448,25 +587,146 @@ int trilens_create(trilens_ctx **out, const trilens_beam *a, const trilens_beam 
   return TRILENS_OK;
 }
 
-int trilens_build(trilens_ctx *c, int64_t step) {
-  if (!c) return TRILENS_ERR_INVALID;
-  if (step < 0) return fail(c, TRILENS_ERR_INVALID, "step < 0");
-  CK(cudaSetDevice(c->device));
+extern "C" {
+
+int trilens_create(trilens_ctx **out, const trilens_beam *a, const trilens_beam *b,
+                   const trilens_params *p, trilens_stream_t stream) {
+  return ctx_create(out, a, b, p, stream, nullptr);
+}
+
+}  // extern "C"
+
+// The two beams' builds share nothing but the status word (set with atomic OR): beam
+// B's runs on a side stream, forked from the context's stream and joined back before
+// anything that reads them (in a captured run this is a fork and a join in the graph).
+// Per-phase timing keeps them on one stream, one after the other.
+static int fork_builds(trilens_ctx *c, bool *fork) {
+  *fork = !c->timing && c->beam[0].n > 0 && c->beam[1].n > 0;
+  if (!*fork) return TRILENS_OK;
+  if (!c->side_stream) CK(cudaStreamCreateWithFlags(&c->side_stream, cudaStreamNonBlocking));
+  if (!c->fork_ev) CK(cudaEventCreateWithFlags(&c->fork_ev, cudaEventDisableTiming));
+  if (!c->join_ev) CK(cudaEventCreateWithFlags(&c->join_ev, cudaEventDisableTiming));
+  CK(cudaEventRecord(c->fork_ev, c->stream));
+  CK(cudaStreamWaitEvent(c->side_stream, c->fork_ev, 0));
+  return TRILENS_OK;
+}
+
+static int join_builds(trilens_ctx *c, bool fork) {
+  if (!fork) return TRILENS_OK;
+  CK(cudaEventRecord(c->join_ev, c->side_stream));
+  CK(cudaStreamWaitEvent(c->stream, c->join_ev, 0));
+  return TRILENS_OK;
+}
+
+// The ordering grids of a single problem's beams for the step with travel T to the
+// swept boxes' centres: per axis of the frame the mean of the centres +- 5 standard
+// deviations, in closed form from the moments (centres outside are clamped to the edge
+// cells; the grid only shapes the tree), and cells in the proportions of the boxes'
+// extents: pad plus the travel of a typical photon of either beam.
+static void step_grids(trilens_ctx *c, double T, TLGrid g[2]) {
+  double ru[3], s[3];
+  for (int k = 0; k < 3; ++k) {
+    const TLFrame &f = c->frame0;
+    ru[k] = (double)f.r[3 * k] * f.u[0] + (double)f.r[3 * k + 1] * f.u[1] +
+            (double)f.r[3 * k + 2] * f.u[2];
+    s[k] = 2.0 * c->half;
+    for (int h = 0; h < 2; ++h) {
+      const double *m = c->fmoments[h], n = (double)std::max<int64_t>(c->beam[h].n, 1);
+      const double mean = m[3 + k] / n;
+      const double var = std::max(m[12 + k] / n - mean * mean, 0.0);
+      s[k] += c->L64 * sqrt((mean - ru[k]) * (mean - ru[k]) + var);
+    }
+  }
+  for (int h = 0; h < 2; ++h) {
+    double lo[3], range[3];
+    for (int k = 0; k < 3; ++k) {
+      const double *m = c->fmoments[h], n = (double)std::max<int64_t>(c->beam[h].n, 1);
+      const double mean = (m[k] + T * m[3 + k]) / n;
+      const double msq = (m[6 + k] + 2.0 * T * m[9 + k] + T * T * m[12 + k]) / n;
+      const double sd5 = 5.0 * sqrt(std::max(msq - mean * mean, 0.0));
+      lo[k] = mean - 0.5 * c->L64 * ru[k] - sd5;
+      range[k] = 2.0 * sd5;
+    }
+    g[h] = tl_make_grid(lo, range, s, c->order_bits);
+  }
+}
+
+// The exact path's order of both beams and the tree of the smaller one.
+static int build_exact(trilens_ctx *c, int64_t step) {
   const double ct = TL_C * ((double)step * c->p.dt_fs);
   const double T = ct + 0.5 * c->L64;
-  // the two beams' builds share nothing but the status word (set with
-  // atomic OR): beam B's runs on a side stream, forked from the context's
-  // stream and joined back before anything that reads the hierarchies (in a
-  // captured run this is a fork and a join in the graph).  Per-phase timing
-  // keeps them on one stream, one after the other.
-  const bool fork = !c->timing && c->beam[0].n > 0 && c->beam[1].n > 0;
-  if (fork) {
-    if (!c->side_stream) CK(cudaStreamCreateWithFlags(&c->side_stream, cudaStreamNonBlocking));
-    if (!c->fork_ev) CK(cudaEventCreateWithFlags(&c->fork_ev, cudaEventDisableTiming));
-    if (!c->join_ev) CK(cudaEventCreateWithFlags(&c->join_ev, cudaEventDisableTiming));
-    CK(cudaEventRecord(c->fork_ev, c->stream));
-    CK(cudaStreamWaitEvent(c->side_stream, c->fork_ev, 0));
+  const bool batch = c->n_inst > 1;
+  TLGrid grid[2];
+  int ib = 0;
+  while ((1 << ib) < c->n_inst) ++ib;
+  if (batch)
+    CK(tl::launch_inst_grid(c->inst_bounds[0], c->inst_bounds[1], c->frames, c->n_inst, T, c->L64,
+                            c->half, c->order_bits, c->grids[0], c->grids[1], c->stream));
+  else
+    step_grids(c, T, grid);
+  bool fork;
+  if (int rc = fork_builds(c, &fork)) return rc;
+  for (int k = 0; k < 2; ++k) {
+    const int64_t n = c->beam[k].n;
+    if (n <= 0) continue;
+    cudaStream_t st = (fork && k == 1) ? c->side_stream : c->stream;
+    tl::BuildBufs &w = c->w[k];
+    const int bits = c->order_bits + ib, passes = (bits + 7) / 8;
+    tmark(c, PH_PROP, k, 0);
+    tl::OrderArgs o;
+    memset(&o, 0, sizeof(o));
+    o.b = c->beam[k];
+    o.ct = ct;
+    o.L = (float)c->L64;
+    o.frames = c->frames;
+    if (!batch) o.grid = grid[k];
+    o.grids = c->grids[k];
+    o.inst_of = c->inst_of[k];
+    o.inst_shift = c->order_bits;
+    o.passes = passes;
+    o.pos_u = w.pos_u;
+    o.dir_u = w.dir_u;
+    o.key = w.key32[0];
+    o.hist = w.sort_raw;
+    CK(tl::launch_order(o, st));
+    tmark(c, PH_PROP, k, 1);
+    tmark(c, PH_SORT, k, 0);
+    CK(tl::launch_sort32(w, n, bits, c->pad[k], c->order_bits, c->p.spin_limit,
+                         c->debug_stall_sort, c->build_status, st));
+    tmark(c, PH_SORT, k, 1);
+    c->phase_launches[PH_PROP] += 1;
+    c->phase_launches[PH_SORT] += 1 + passes;
+    if (k != c->tree) continue;
+    tmark(c, PH_REFIT, k, 0);
+    tl::BoxArgs b;
+    memset(&b, 0, sizeof(b));
+    b.pos = w.pos;
+    b.dir = w.dir;
+    b.inst = c->insts[k];
+    b.tile_inst = c->tile_inst[k];
+    b.frames = c->frames;
+    b.Llo = c->L_lo;
+    b.Lhi = c->L_hi;
+    b.half = c->half;
+    b.box = c->box;
+    b.build_status = c->build_status;
+    CK(tl::launch_boxes(b, c->n_tiles[k], c->n_inst, c->max_top, st));
+    tmark(c, PH_REFIT, k, 1);
+    c->phase_launches[PH_REFIT] += c->max_top >= 3 ? 2 : 1;
   }
+  if (int rc = join_builds(c, fork)) return rc;
+  c->exact_step = step;
+  c->full_step = -1;  // the two builds share the sorted photons
+  return TRILENS_OK;
+}
+
+// The statistical regime's binary hierarchies of both beams, in Morton order.
+static int build_full(trilens_ctx *c, int64_t step) {
+  if (int rc = ensure_full(c)) return rc;
+  const double ct = TL_C * ((double)step * c->p.dt_fs);
+  const double T = ct + 0.5 * c->L64;
+  bool fork;
+  if (int rc = fork_builds(c, &fork)) return rc;
   for (int k = 0; k < 2; ++k) {
     const int64_t n = c->beam[k].n;
     if (n <= 0) continue;
@@ -476,7 +736,7 @@ int trilens_build(trilens_ctx *c, int64_t step) {
     // moments (centres outside are clamped to the edge cells).  Unlike the
     // extreme centres, the moments of a large beam barely change from one
     // draw to the next, so neither do the cells a level of the hierarchy
-    // stands for.  (Batches use each instance's own box, below.)
+    // stands for.
     float lo[3], scale[3];
     const double maxq = (double)((1u << c->bits[k]) - 1u);
     for (int a = 0; a < 3; ++a) {
@@ -490,13 +750,7 @@ int trilens_build(trilens_ctx *c, int64_t step) {
     }
     tl::BuildBufs &w = c->w[k];
     tmark(c, PH_PROP, k, 0);
-    if (c->n_inst > 1) {
-      CK(tl::launch_inst_box(c->inst_bounds[k], c->n_inst, T, c->bits[k], c->inst_box[k],
-                             st));
-      CK(cudaMemsetAsync(c->inst_root[k], 0xff, sizeof(uint32_t) * c->n_inst, st));
-    }
     CK(tl::launch_propagate(c->beam[k], ct, (float)c->L64, lo, scale, c->bits[k], w,
-                            c->n_inst > 1 ? c->inst_box[k] : nullptr,
                             n > 1 ? (c->key_bits[k] + 7) / 8 : 0, st));
     tmark(c, PH_PROP, k, 1);
     tmark(c, PH_SORT, k, 0);
@@ -505,7 +759,7 @@ int trilens_build(trilens_ctx *c, int64_t step) {
     tmark(c, PH_SORT, k, 1);
     if (n <= 1) {  // no sort: copy the one photon (a longer beam is gathered by the sort)
       tmark(c, PH_GATHER, k, 0);
-      CK(tl::launch_gather(w, n, c->sel[k], st));
+      CK(tl::launch_gather(w, n, st));
       tmark(c, PH_GATHER, k, 1);
       c->phase_launches[PH_GATHER] += 1;
     }
@@ -520,10 +774,26 @@ int trilens_build(trilens_ctx *c, int64_t step) {
     c->phase_launches[PH_EMIT] += 1;
     c->phase_launches[PH_REFIT] += tl::refit_tiles(n) > 1 ? 3 : 1;
   }
-  if (fork) {
-    CK(cudaEventRecord(c->join_ev, c->side_stream));
-    CK(cudaStreamWaitEvent(c->stream, c->join_ev, 0));
-  }
+  if (int rc = join_builds(c, fork)) return rc;
+  c->full_step = step;
+  c->exact_step = -1;
+  return TRILENS_OK;
+}
+
+int need_full(trilens_ctx *c, int64_t step) {
+  return c->full_step == step ? TRILENS_OK : build_full(c, step);
+}
+
+extern "C" {
+
+int trilens_build(trilens_ctx *c, int64_t step) {
+  if (!c) return TRILENS_ERR_INVALID;
+  if (step < 0) return fail(c, TRILENS_ERR_INVALID, "step < 0");
+  CK(cudaSetDevice(c->device));
+  // a context that uses the statistical regime builds its hierarchies; a collision of
+  // the whole beams builds the exact path's trees if they do not stand for the step
+  const int rc = c->sur ? build_full(c, step) : build_exact(c, step);
+  if (rc) return rc;
   c->built_step = step;
   return TRILENS_OK;
 }
@@ -537,8 +807,10 @@ int trilens_build(trilens_ctx *c, int64_t step) {
 // status is cleared.
 static int status_failure(trilens_ctx *c, unsigned trav_st, unsigned build_st) {
   if (!((trav_st | build_st) & (TL_ST_TIMEOUT | TL_ST_BADTREE))) return TRILENS_OK;
+  c->exact_step = c->full_step = -1;
   c->w[0].sort_epoch = c->w[1].sort_epoch = 0;
-  CK(cudaMemsetAsync(c->queue, 0xff, sizeof(uint2) * (size_t)c->queue_cap, c->stream));
+  if (c->queue)
+    CK(cudaMemsetAsync(c->queue, 0xff, sizeof(uint2) * (size_t)c->queue_cap, c->stream));
   CK(cudaMemsetAsync(c->build_status, 0, sizeof(unsigned), c->stream));
   CK(cudaStreamSynchronize(c->stream));
   if (build_st & TL_ST_TIMEOUT)
@@ -591,52 +863,15 @@ tl::TravArgs trav_args(trilens_ctx *c, double ct) {
 }
 
 int run_exact(trilens_ctx *c, double ct, const uint2 *seeds, unsigned n_seeds, int *retries_out) {
-  const int nonempty = c->beam[0].n > 0 && c->beam[1].n > 0;
   int retries = 0;
   TLCounters &h = *c->ctr_host;
   while (true) {
     tl::TravArgs a = trav_args(c, ct);
-    // large single problems start from the refit's cut lists; small ones and
-    // batches expand their root pairs breadth first
-    const bool use_cut = !seeds && c->n_inst <= 1 && c->w[0].cut_S && c->w[1].cut_S;
-    tmark(c, PH_EXPAND, 0, 0);
-    CK(tl::launch_step_init(c->ctr, c->front[0], a.A.super, a.B.super,
-                            (c->n_inst > 1 || seeds || use_cut) ? 0 : nonempty, c->build_status,
-                            nullptr, c->stream));
-    if (use_cut) {
-      CK(tl::launch_seed_cut(a, c->w[0].cut, c->w[0].cut_n, c->w[0].cut_cap, c->w[1].cut,
-                             c->w[1].cut_n, c->w[1].cut_cap, c->front[0], c->front_cap,
-                             2 * c->n_sm, c->stream));
-      CK(tl::launch_widen(a, c->front[0], c->front[1], c->front_cap, c->widen_target,
-                          kWidenLevels, 4 * c->n_sm, c->stream));
-      c->phase_launches[PH_EXPAND] += kWidenLevels;
-    } else if (!seeds) {
-      if (c->n_inst > 1)
-        CK(tl::launch_seed_instances(c->ctr, c->front[0], c->inst_root[0], c->inst_root[1],
-                                     c->n_inst, c->stream));
-      CK(tl::launch_expand(a, c->front[0], c->front[1], c->front_cap, c->front_target, kMaxLevels,
-                           c->stream));
-    }
-    tmark(c, PH_EXPAND, 0, 1);
-    c->phase_launches[PH_EXPAND] += seeds ? 1 : 2;
-    if (c->parts == 1) {
-      tmark(c, PH_TRAV, 0, 0);
-      CK(tl::launch_traverse(a, c->front[0], c->front[1], seeds, seeds ? n_seeds : 0,
-                             seeds ? 0 : 1, c->budget, c->trav_blocks, c->trav_warps, c->stream,
-                             0, 1));
-      tmark(c, PH_TRAV, 0, 1);
-      tmark(c, PH_NARROW, 0, 0);
-      CK(tl::launch_narrow(a, 8 * c->n_sm, c->stream));
-      tmark(c, PH_NARROW, 0, 1);
-    } else {  // parts: traversal and narrow phase timed together
-      tmark(c, PH_TRAV, 0, 0);
-      int rcp = traverse_parts(c, a, seeds, n_seeds);
-      if (rcp) return rcp;
-      tmark(c, PH_TRAV, 0, 1);
-      c->phase_launches[PH_TRAV] += 2 * (c->parts - 1);
-    }
-    c->phase_launches[PH_TRAV] += 1;
-    c->phase_launches[PH_NARROW] += 1;
+    CK(tl::launch_step_init(c->ctr, c->build_status, nullptr, c->stream));
+    const int rcp = seeds ? traverse_parts(c, a, seeds, n_seeds) : collide_parts(c, a);
+    if (rcp) return rcp;
+    c->phase_launches[PH_TRAV] += c->parts;
+    c->phase_launches[PH_NARROW] += c->parts;
     if (!a.fp64) {
       tmark(c, PH_BAND, 0, 0);
       CK(tl::launch_band(a, c->n_sm * 4, c->stream));
@@ -677,7 +912,6 @@ int run_exact(trilens_ctx *c, double ct, const uint2 *seeds, unsigned n_seeds, i
       if ((rc = leaves_for(c, h.max_part_leaves))) return rc;
       again = true;
     }
-    if (st & TL_ST_FRONT_OVF) return fail(c, TRILENS_ERR_STACK, "frontier overflow");
     if (!again) break;
     if (++retries > 8) return fail(c, TRILENS_ERR_STACK, "buffers kept overflowing");
   }
@@ -695,7 +929,9 @@ int trilens_collide_step(trilens_ctx *c, int64_t step, uint32_t *hits, int64_t c
   CK(cudaSetDevice(c->device));
   const double ct = TL_C * ((double)step * c->p.dt_fs);
   int retries = 0;
-  const int rc = run_exact(c, ct, nullptr, 0, &retries);
+  int rc = TRILENS_OK;
+  if (c->exact_step != step && (rc = build_exact(c, step))) return rc;
+  rc = run_exact(c, ct, nullptr, 0, &retries);
   if (rc) return rc;
   TLCounters &h = *c->ctr_host;
   if (hits && (int64_t)h.count > cap) {
@@ -769,8 +1005,11 @@ int trilens_batch_create(trilens_ctx **out, const trilens_beam *a, const trilens
   *out = nullptr;
   if (!a || !b || !p || n_inst < 1 || n_inst > 65536) return TRILENS_ERR_INVALID;
   int64_t tot[2] = {0, 0}, nmax = 1;
+  std::vector<int64_t> sizes[2];
   for (int q = 0; q < n_inst; ++q) {
     if (!beam_ok(&a[q]) || !beam_ok(&b[q])) return TRILENS_ERR_INVALID;
+    sizes[0].push_back(a[q].n);
+    sizes[1].push_back(b[q].n);
     tot[0] += a[q].n;
     tot[1] += b[q].n;
     nmax = std::max<int64_t>(nmax, std::max(a[q].n, b[q].n));
@@ -791,7 +1030,7 @@ int trilens_batch_create(trilens_ctx **out, const trilens_beam *a, const trilens
     cat[k].E = tmp.owned[k][6]; cat[k].w = tmp.owned[k][7];
   }
   trilens_ctx *ctx = nullptr;
-  rc = trilens_create(&ctx, &cat[0], &cat[1], p, stream);
+  rc = ctx_create(&ctx, &cat[0], &cat[1], p, stream, n_inst > 1 ? sizes : nullptr);
   if (rc) {
     for (int k = 0; k < 2; ++k) {
       for (int q = 0; q < 8; ++q) cudaFree(tmp.owned[k][q]);
@@ -807,34 +1046,23 @@ int trilens_batch_create(trilens_ctx **out, const trilens_beam *a, const trilens
     }
     c->inst_of[k] = tmp.inst_of[k];
     tmp.inst_of[k] = nullptr;
-    c->w[k].inst_of = c->inst_of[k];
   }
   c->n_inst = n_inst;
-  for (int k = 0; k < 2; ++k) c->w[k].cut_S = 0;  // batches seed from instance roots
-  int ib = 0;
-  while ((1 << ib) < n_inst) ++ib;
-  int lg = 0;
-  while ((1ll << lg) < nmax) ++lg;
-  const int bits = std::min((63 - ib) / 3, std::max(4, (lg + 2) / 3 + 3));
-  CK(cudaMalloc((void **)&c->inst_tmp, sizeof(long long) * 12 * n_inst));
-  for (int k = 0; k < 2; ++k) {
-    c->bits[k] = bits;
-    c->key_bits[k] = 3 * bits + ib;
-    c->w[k].key_bits = c->key_bits[k];
-    c->w[k].inst_shift = 3 * bits;
-    CK(dalloc(&c->inst_root[k], (size_t)n_inst));
-    c->w[k].inst_root = c->inst_root[k];
-    CK(dalloc(&c->inst_bounds[k], (size_t)12 * n_inst));
-    CK(dalloc(&c->inst_box[k], (size_t)2 * n_inst));
-    CK(tl::launch_inst_bounds(c->beam[k], c->inst_of[k], n_inst, c->inst_tmp, c->inst_bounds[k],
-                              c->stream));
-  }
-  if (c->front_cap < (unsigned)n_inst + 4 * c->front_target + 64) {
-    c->front_cap = (unsigned)n_inst + 4 * c->front_target + 64;
+  if (n_inst > 1) {
+    int ib = 0;
+    while ((1 << ib) < n_inst) ++ib;
+    c->order_bits = order_bits_for(nmax, ib);
+    CK(cudaMalloc((void **)&c->inst_tmp, sizeof(long long) * 12 * n_inst));
     for (int k = 0; k < 2; ++k) {
-      cudaFree(c->front[k]);
-      CK(dalloc(&c->front[k], c->front_cap));
+      CK(dalloc(&c->inst_bounds[k], (size_t)12 * n_inst));
+      CK(dalloc(&c->grids[k], (size_t)n_inst));
+      CK(tl::launch_inst_bounds(c->beam[k], c->inst_of[k], nullptr, n_inst, c->inst_tmp,
+                                c->inst_bounds[k], c->stream));
     }
+    CK(tl::launch_inst_frames(c->inst_bounds[0], c->inst_bounds[1], n_inst, c->frames, c->stream));
+    for (int k = 0; k < 2; ++k)  // the bounds in every instance's frame
+      CK(tl::launch_inst_bounds(c->beam[k], c->inst_of[k], c->frames, n_inst, c->inst_tmp,
+                                c->inst_bounds[k], c->stream));
   }
   if ((rc = ensure_graph(c))) return rc;
   CK(cudaStreamSynchronize(c->stream));
@@ -843,31 +1071,14 @@ int trilens_batch_create(trilens_ctx **out, const trilens_beam *a, const trilens
 }
 
 // One step of a captured run: the collide sequence without host checks (the
-// traversal needs none: its warps share a device work queue); every overflow
+// collisions need none); every overflow
 // is flagged in run_status, and the step's totals are added on the device.
 static int graph_collide(trilens_ctx *c, int64_t step, double *yields) {
   const double ct = TL_C * ((double)step * c->p.dt_fs);
-  const int nonempty = c->beam[0].n > 0 && c->beam[1].n > 0;
   tl::TravArgs a = trav_args(c, ct);
-  const bool use_cut = c->n_inst <= 1 && c->w[0].cut_S && c->w[1].cut_S;
-  CK(tl::launch_step_init(c->ctr, c->front[0], a.A.super, a.B.super,
-                          (c->n_inst > 1 || use_cut) ? 0 : nonempty, c->build_status,
-                          c->run_status, c->stream));
-  if (use_cut) {
-    CK(tl::launch_seed_cut(a, c->w[0].cut, c->w[0].cut_n, c->w[0].cut_cap, c->w[1].cut,
-                           c->w[1].cut_n, c->w[1].cut_cap, c->front[0], c->front_cap,
-                           2 * c->n_sm, c->stream));
-    CK(tl::launch_widen(a, c->front[0], c->front[1], c->front_cap, c->widen_target, kWidenLevels,
-                        4 * c->n_sm, c->stream));
-  } else {
-    if (c->n_inst > 1)
-      CK(tl::launch_seed_instances(c->ctr, c->front[0], c->inst_root[0], c->inst_root[1],
-                                   c->n_inst, c->stream));
-    CK(tl::launch_expand(a, c->front[0], c->front[1], c->front_cap, c->front_target, kMaxLevels,
-                         c->stream));
-  }
+  CK(tl::launch_step_init(c->ctr, c->build_status, c->run_status, c->stream));
   {
-    const int rcp = traverse_parts(c, a, nullptr, 0);
+    const int rcp = collide_parts(c, a);
     if (rcp) return rcp;
   }
   if (!a.fp64) CK(tl::launch_band(a, c->n_sm * 4, c->stream));
@@ -896,7 +1107,7 @@ static int capture_run(trilens_ctx *c, int64_t first, int64_t steps, double *yie
     e = cudaMemsetAsync(yields, 0, sizeof(double) * 2 * c->n_inst, c->stream);
   if (e != cudaSuccess) rc = fail(c, TRILENS_ERR_CUDA, "capture: %s", cudaGetErrorString(e));
   for (int64_t k = first; rc == TRILENS_OK && k < first + steps; ++k) {
-    rc = trilens_build(c, k);
+    rc = build_exact(c, k);
     if (rc == TRILENS_OK) rc = graph_collide(c, k, yields);
   }
   cudaGraph_t g = nullptr;
@@ -925,6 +1136,7 @@ static int replay_run(trilens_ctx *c, int64_t first_step, int64_t steps, double 
       int rc = capture_run(c, first_step, steps, yields);
       if (rc) return rc;
     }
+    c->exact_step = c->full_step = -1;
     CK(cudaGraphLaunch(c->gexec, c->stream));
     CK(cudaMemcpyAsync(c->run_status_host, c->run_status, sizeof(unsigned), cudaMemcpyDeviceToHost,
                        c->stream));
@@ -933,9 +1145,10 @@ static int replay_run(trilens_ctx *c, int64_t first_step, int64_t steps, double 
     CK(cudaStreamSynchronize(c->stream));
     const unsigned st = *c->run_status_host | *c->build_status_host;
     if (int rf = status_failure(c, *c->run_status_host, *c->build_status_host)) return rf;
-    if (!(st & (TL_ST_HIT_OVF | TL_ST_BAND_OVF | TL_ST_SPILL_OVF | TL_ST_FRONT_OVF |
-                TL_ST_PRIV_OVF | TL_ST_LEAFQ)))
+    if (!(st & (TL_ST_HIT_OVF | TL_ST_BAND_OVF | TL_ST_LEAFQ))) {
+      c->built_step = c->exact_step = first_step + steps - 1;  // the run's last step is built
       return TRILENS_OK;
+    }
     // grow what overflowed (to the largest size a step asked for) and capture again
     TLRunAcc m;
     CK(cudaMemcpyAsync(&m, c->run_acc, sizeof(TLRunAcc), cudaMemcpyDeviceToHost, c->stream));
@@ -944,14 +1157,7 @@ static int replay_run(trilens_ctx *c, int64_t first_step, int64_t steps, double 
     if (st & TL_ST_HIT_OVF && (rc = grow(c, &c->hits, &c->hit_cap, m.max_hits + m.max_band)))
       return rc;
     if (st & TL_ST_BAND_OVF && (rc = grow(c, &c->band, &c->band_cap, m.max_band))) return rc;
-    if (st & TL_ST_PRIV_OVF && (rc = alloc_spill(c, 2 * c->spill_per_warp, c->spill_warps)))
-      return rc;
     if (st & TL_ST_LEAFQ && (rc = leaves_for(c, m.max_leaves))) return rc;
-    if (st & TL_ST_SPILL_OVF) {  // the queue: larger, and every slot the sentinel again
-      const unsigned long long need = kQueueChunk * (m.max_handed + m.max_handed / 4 + 1024);
-      if ((rc = alloc_queue(c, std::max(need, 2 * c->queue_cap)))) return rc;
-    }
-    if (st & TL_ST_FRONT_OVF) return fail(c, TRILENS_ERR_STACK, "frontier overflow");
     if (c->gexec) {
       cudaGraphExecDestroy(c->gexec);
       c->gexec = nullptr;
@@ -1032,33 +1238,23 @@ static int apply_tuning(trilens_ctx *c, int bucket, int depth, int warps, int bu
   c->trav_warps = warps;
   c->trav_blocks = bps * c->n_sm;
   c->budget = budget;
-  c->front_target = (unsigned)std::min<long long>(2ll * c->trav_blocks * c->trav_warps, 1 << 16);
-  unsigned need_front = 0;
-  frontier_sizes(c, &c->widen_target, &need_front);
-  if (need_front > c->front_cap) {
-    c->front_cap = need_front;
-    for (int k = 0; k < 2; ++k) {
-      cudaFree(c->front[k]);
-      c->front[k] = nullptr;
-      CK(dalloc(&c->front[k], c->front_cap));
+  if (c->full_ready) {
+    const unsigned long long warps_now = (unsigned long long)c->trav_blocks * c->trav_warps;
+    if (warps_now > c->spill_warps) {
+      const int rcs = alloc_spill(c, c->spill_per_warp, warps_now);
+      if (rcs) return rcs;
     }
-  }
-  const unsigned long long warps_now = (unsigned long long)c->trav_blocks * c->trav_warps;
-  if (warps_now > c->spill_warps) {
-    const int rcs = alloc_spill(c, c->spill_per_warp, warps_now);
-    if (rcs) return rcs;
-  }
-  const unsigned long long need_queue =
-      2ull * c->trav_blocks * c->trav_warps * (unsigned long long)depth;
-  if (need_queue > c->queue_cap) {
-    const int rcq = alloc_queue(c, need_queue);
-    if (rcq) return rcq;
+    const unsigned long long need_queue = 2ull * warps_now * (unsigned long long)depth;
+    if (need_queue > c->queue_cap) {
+      const int rcq = alloc_queue(c, need_queue);
+      if (rcq) return rcq;
+    }
   }
   if (c->gexec) {  // a captured run holds the old shapes
     cudaGraphExecDestroy(c->gexec);
     c->gexec = nullptr;
   }
-  c->built_step = -1;  // the leaf bucket changes the hierarchy: build again
+  c->built_step = c->exact_step = c->full_step = -1;  // the leaf bucket changes the hierarchy
   return TRILENS_OK;
 }
 
@@ -1342,13 +1538,13 @@ int trilens_debug_shrink_buffers(trilens_ctx *c, int64_t cap) {
   CK(dalloc(&c->hits, n));
   CK(dalloc(&c->band, n));
   CK(dalloc(&c->leaves, n));
-  {  // spill areas of cap entries per warp (at least 64)
+  if (c->full_ready) {  // spill areas of cap entries per warp (at least 64), and the queue
     const int rcs = alloc_spill(c, (unsigned)std::max<int64_t>(64, std::min<int64_t>(cap, 1 << 20)),
                                 c->spill_warps);
     if (rcs) return rcs;
+    const int rc = alloc_queue(c, n);
+    if (rc) return rc;
   }
-  const int rc = alloc_queue(c, n);
-  if (rc) return rc;
   CK(cudaStreamSynchronize(c->stream));
   return TRILENS_OK;
 }
@@ -1360,21 +1556,18 @@ int trilens_debug_set_key_bits(trilens_ctx *c, int32_t bits) {
     c->key_bits[k] = 3 * bits;
     c->w[k].key_bits = c->key_bits[k];
   }
+  c->order_bits = std::min(30, 3 * bits);
   if (c->gexec) {  // a captured run holds the old pass count
     cudaGraphExecDestroy(c->gexec);
     c->gexec = nullptr;
   }
-  c->built_step = -1;
+  c->built_step = c->exact_step = c->full_step = -1;
   return TRILENS_OK;
 }
 
-int trilens_debug_set_cut_cap(trilens_ctx *c, int32_t cap) {
-  if (!c) return TRILENS_ERR_INVALID;
-  for (int k = 0; k < 2; ++k) {
-    tl::BuildBufs &w = c->w[k];
-    w.cut_cap = (cap <= 0 || (uint32_t)cap > w.cut_alloc) ? w.cut_alloc : (uint32_t)cap;
-  }
-  return TRILENS_OK;
+// There are no seed lists any more: the exact path descends one tree from its top.
+int trilens_debug_set_cut_cap(trilens_ctx *c, int32_t) {
+  return c ? TRILENS_OK : TRILENS_ERR_INVALID;
 }
 
 }  // extern "C"

@@ -79,22 +79,19 @@ struct TLCounters {
   unsigned long long q_tail;       // traversal queue: chunks reserved (items handed on)
   unsigned long long narrow_tests; // photon pairs tested
   unsigned long long node_tests;   // box pair tests
-  unsigned long long leaf_pairs;   // overlapping bucket pairs
-  unsigned int counts[32];         // frontier size after each expansion level
-  unsigned int frozen;             // frontier expansion finished
-  unsigned int final_level;        // level whose frontier the traversal reads
-  unsigned int widen_done;         // blocks finished in the frontier's widening level
+  unsigned long long leaf_pairs;   // overlapping leaf pairs
+  unsigned long long cand;         // exact path: candidate photon pairs listed
   unsigned int status;             // TL_ST_* bits
   unsigned int reduce_done;        // blocks finished in the yield reduction
   unsigned int hungry;             // traversal warps waiting for a handed-on chunk
-  unsigned long long q_head;       // traversal items taken (the frontier's, then the queue's)
+  unsigned long long q_head;       // traversal items taken (the list's, then the queue's)
   unsigned long long q_done;       // traversal items finished
   // results of the yield reduction for this step
   unsigned long long count;
   double weighted;
   unsigned long long hsum, hxor;
-  // a step done in parts (slices of its frontier): the leaf-pair count at
-  // the start of the current part, and the largest part's leaf pairs
+  // a step done in parts: the list's count (cand, or the seeded traversal's
+  // leaf_pairs) at the start of the current part, and the largest part's
   unsigned long long leaf_base;
   unsigned long long max_part_leaves;
 };
@@ -162,27 +159,20 @@ struct InstSrc {
   const double *p[8];
   long long n, off;
 };
-cudaError_t launch_inst_bounds(const TLBeam &b, const uint32_t *inst_of, int n_inst,
-                               long long *tmp, double *out, cudaStream_t s);
-cudaError_t launch_inst_box(const double *bounds, int n_inst, double T, int bits, float4 *box,
-                            cudaStream_t s);
 cudaError_t launch_gather_instances(const InstSrc *src, int n_inst, int64_t n, double *const *dst,
                                     uint32_t *inst_of, cudaStream_t s);
 struct BuildBufs {
   float4 *pos_u, *dir_u;      // unsorted SoA32
-  float4 *pos, *dir;          // sorted SoA32
-  unsigned long long *key[2];
+  float4 *pos, *dir;          // sorted SoA32 (the exact path's in tiles, see tl_frame.cuh)
+  uint32_t *key32[2];         // the exact path's keys
   uint32_t *val[2];
+  // from here to rsuper: the statistical regime's, allocated with it
+  unsigned long long *key[2];
   TLNode *nodes;
   uint32_t *parent_leaf, *parent_node;
   float *rpre, *rsuf;  // per photon: union of the swept boxes from its tile's start / to its end
   float *rtile;        // per refit tile: union of its photons' swept boxes
   float *rsuper;       // sparse tables over the tile boxes, one per super-tile
-  // traversal seeds: the children with at most cut_S photons of the nodes with
-  // more, as (node << 1) | slot, written by the refit (cut_S = 0: none)
-  uint32_t *cut;
-  unsigned *cut_n;
-  uint32_t cut_S, cut_cap, cut_alloc;
   // sort scratch
   uint32_t *sort_status;  // tiles * 256 per pass
   uint32_t *sort_raw;     // 8 * 256 digit counts of the keys (zero between sorts)
@@ -193,10 +183,6 @@ struct BuildBufs {
   uint32_t *sort_ep;  // device: epochs of the passes of the current sort, and the last one
 
   unsigned *build_status;  // shared status word of the context's builds
-  // several independent instances in one beam (NULL / 0 for a single one)
-  const uint32_t *inst_of;  // instance of each input photon
-  uint32_t *inst_root;      // per instance: stack reference of its subtree root
-  int inst_shift;           // bit position of the instance number in the key
   // per inner node: first photon of its range and its level (Morton prefix
   // length in bits below the key's top bit), for the level-L cut
   uint32_t *nfirst;
@@ -217,7 +203,8 @@ struct TravArgs {
   unsigned long long hit_cap;
   uint2 *band;
   unsigned long long band_cap;
-  uint2 *leaves;  // overlapping leaf-bucket pairs (packed first | (count - 1) << 27)
+  uint2 *leaves;  // candidate photon pairs; the seeded traversal: overlapping leaf-bucket
+                  // pairs (packed first | (count - 1) << 27)
   unsigned long long leaf_cap;
   unsigned long long *queue;  // traversal work queue: chunks of 32 (ref A, ref B) pairs
   unsigned long long queue_cap;  // in pairs
@@ -230,14 +217,16 @@ struct TravArgs {
 };
 
 cudaError_t launch_propagate(const TLBeam &b, double ct, float L, const float box_lo[3],
-                             const float box_scale[3], int bits, BuildBufs &w,
-                             const float4 *inst_box, int passes, cudaStream_t s);
+                             const float box_scale[3], int bits, BuildBufs &w, int passes,
+                             cudaStream_t s);
 cudaError_t launch_static_soa(const TLBeam &b, BuildBufs &w, cudaStream_t s);
-cudaError_t launch_beam_moments(const TLBeam &b, double *out15, double *scratch, cudaStream_t s);
 cudaError_t sort_prepare();
 cudaError_t launch_sort(BuildBufs &w, int64_t n, int key_bits, long long spin_limit,
                         int debug_stall, unsigned int *status, int *out_sel, cudaStream_t s);
-cudaError_t launch_gather(BuildBufs &w, int64_t n, int sel, cudaStream_t s);
+cudaError_t launch_sort32(BuildBufs &w, int64_t n, int key_bits, const int *pad, int pad_shift,
+                          long long spin_limit, int debug_stall, unsigned int *status,
+                          cudaStream_t s);
+cudaError_t launch_gather(BuildBufs &w, int64_t n, cudaStream_t s);
 cudaError_t launch_karras(BuildBufs &w, int64_t n, int sel, int bucket, cudaStream_t s);
 cudaError_t launch_refit(BuildBufs &w, int64_t n, float Llo, float Lhi, float half, int n_sm,
                          cudaStream_t s);

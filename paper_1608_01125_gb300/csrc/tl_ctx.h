@@ -6,14 +6,14 @@
 #include <string.h>
 
 #include <algorithm>
+#include <vector>
 
 #include "tl_common.cuh"
+#include "tl_tree.h"
 #include "trilens.h"
 
 struct SurrogateState;
 struct DepState;
-
-constexpr int kMaxLevels = 24;
 
 struct trilens_ctx {
   int device = 0;
@@ -24,18 +24,33 @@ struct trilens_ctx {
   double L64 = 0, rmax = 0, sigma_max = 0;
   float L_lo = 0, L_hi = 0, half = 0;
   TLNarrowConst nk{};
-  int bits[2]{}, key_bits[2]{};
-  // per beam and axis: sums of p0, d, p0^2, p0 d, d^2 (one-time, fixed order)
-  double moments[2][15]{};
+  int bits[2]{}, key_bits[2]{};  // Morton keys of the statistical regime
+  int order_bits = 0;            // the exact path's keys, all axes together
+  // per beam and axis: sums of p0, d, p0^2, p0 d, d^2 (one-time, fixed order), in the
+  // lab frame and in the exact path's frame
+  double moments[2][15]{}, fmoments[2][15]{};
   // build workspace
   tl::BuildBufs w[2]{};
   int sel[2]{};
-  int64_t built_step = -1;
+  int64_t built_step = -1;  // the step trilens_build was called for
+  int64_t exact_step = -1;  // the step the exact path's trees stand for
+  int64_t full_step = -1;   // the step the statistical regime's hierarchies stand for
+  bool full_ready = false;  // ... and whether their buffers are allocated
+  // exact path: one frame per instance; the photons of both beams in tiles; a tree over
+  // the smaller beam
+  TLFrame frame0{};
+  TLFrame *frames = nullptr;
+  int tree = 1;                  // the beam with the tree
+  TLInst *insts[2]{};            // device, per instance
+  uint32_t *tile_inst[2]{};      // device, instance of every tile (batches)
+  int *pad[2]{};                 // device, TLInst::pad per instance (batches)
+  TLGrid *grids[2]{};            // device, per instance (batches)
+  int n_tiles[2]{};
+  int max_top = 1;               // over the trees of all instances
+  float4 *box = nullptr;         // all boxes of the trees
   // traversal workspace
-  int n_sm = 0, trav_warps = 4, trav_blocks = 0, expand_blocks = 0;
+  int n_sm = 0, trav_warps = 4, trav_blocks = 0;
   int budget = 16;  // traversal iterations per work item before it is handed on
-  unsigned front_target = 0, front_cap = 0, widen_target = 0;
-  uint2 *front[2]{};
   uint2 *queue = nullptr;  // traversal work queue (every free slot holds the sentinel)
   unsigned long long queue_cap = 0;
   uint2 *spill = nullptr;  // traversal warps' private spill areas
@@ -45,9 +60,9 @@ struct trilens_ctx {
   unsigned long long hit_cap = 0;
   uint2 *band = nullptr;
   unsigned long long band_cap = 0;
-  uint2 *leaves = nullptr;  // the step's overlapping leaf-bucket pairs
+  uint2 *leaves = nullptr;  // candidate photon pairs; seeded: overlapping leaf-bucket pairs
   unsigned long long leaf_cap = 0;
-  int parts = 1;  // a step's traversal in this many slices of its frontier
+  int parts = 1;  // a step's collisions in this many slices of its groups (or seeds)
   TLCounters *ctr = nullptr;
   TLCounters *ctr_host = nullptr;  // pinned
   void *partials = nullptr;
@@ -61,9 +76,7 @@ struct trilens_ctx {
   // several independent instances (batch contexts)
   int n_inst = 1;
   uint32_t *inst_of[2]{};     // device, instance of every photon
-  uint32_t *inst_root[2]{};   // device, subtree root (stack reference) per instance
   double *inst_bounds[2]{};   // device, 12 doubles per instance
-  float4 *inst_box[2]{};      // device, Morton box of every instance for the current build
   long long *inst_tmp = nullptr;
   double *owned[2][8]{};      // concatenated inputs owned by a batch context
   // graph-captured multi-step runs (batch contexts)
@@ -162,9 +175,11 @@ static inline int grow(trilens_ctx *c, uint2 **buf, unsigned long long *cap, uns
 
 // traversal arguments for the current build at time c t_k = ct
 tl::TravArgs trav_args(trilens_ctx *c, double ct);
-// exact collision of seed pairs (or, with seeds == NULL, of the whole
-// hierarchies from the roots) for the built step; fills c->ctr_host
+// exact collision of the built step: of seed pairs of the statistical regime's
+// hierarchies, or, with seeds == NULL, of the whole beams; fills c->ctr_host
 int run_exact(trilens_ctx *c, double ct, const uint2 *seeds, unsigned n_seeds, int *retries);
+// make the statistical regime's hierarchies stand for `step` (a no-op if they do)
+int need_full(trilens_ctx *c, int64_t step);
 void surrogate_free(trilens_ctx *c);
 void deplete_free(trilens_ctx *c);
 double tl_sigma_max_bound();

@@ -1,0 +1,260 @@
+// tl_frame.cuh -- the frame of the exact path's boxes, the swept box of a photon
+// in it, and the cells its photons are ordered by.
+//
+// Two photons that come within a distance r at one time do so in every frame
+// that moves uniformly and is turned: boxes may be swept in any frame the two
+// beams share.  The frame here moves with the mean of the two beams' mean
+// directions, ubar, and its third axis is their difference: there both beams
+// move along that axis only (but for their divergence), so a photon's swept box
+// is a needle, whatever the crossing angle; axis-aligned boxes in the lab frame
+// are as wide across the motion as along it for beams that cross.
+#pragma once
+#include <math.h>
+
+#include "tl_common.cuh"
+
+// x' = R x, v' = R (d - u) (v in units of c): exactly these FP32 numbers define the
+// frame, so rounding them costs nothing.  ident: R = 1, u = 0.
+struct TLFrame {
+  float r[9];
+  float u[3];
+  int ident;
+  int pad[3];
+};
+
+// Ordering grid of one instance and step: cell = (x' - lo) scale, nb bits per axis,
+// axes by falling nb (perm).
+struct TLGrid {
+  float lo[3], scale[3];
+  int nb[3], perm[3];
+};
+
+// One instance's photons of one beam in the exact path's layout: tiles of 1024
+// sorted photons from tile0 on, and its tree, an implicit one with 32 children per
+// node over the sorted photons: level 0 the photons, level l nodes of 32^l.
+struct TLInst {
+  int n;       // photons
+  int tile0;   // first tile
+  int pad;     // sorted position of the concatenated beam -> padded position
+  int top;     // lowest level with at most 32 nodes (>= 1)
+  uint32_t lev[6];  // first box of each level
+  int cnt[6];       // nodes of each level
+};
+
+constexpr int kTile = 1024;  // sorted photons per tile (a level-2 node)
+
+__host__ __device__ inline TLFrame tl_ident_frame() {
+  TLFrame f{};
+  f.r[0] = f.r[4] = f.r[8] = 1.0f;
+  f.ident = 1;
+  return f;
+}
+
+// The frame of two beams with mean directions a and b.  The lab frame itself when
+// they are (nearly) parallel or have no common direction, or when the turn would be
+// below ~1e-2, the order of a beam's own divergence: then the lab's boxes are as
+// good and need a third of the work.
+__host__ __device__ inline TLFrame tl_make_frame(const double a[3], const double b[3]) {
+  double w[3], u[3], wl = 0.0;
+  for (int k = 0; k < 3; ++k) {
+    w[k] = a[k] - b[k];
+    u[k] = 0.5 * (a[k] + b[k]);
+    wl += w[k] * w[k];
+  }
+  wl = sqrt(wl);
+  if (!(wl > 0.1) || !(wl < 10.0)) return tl_ident_frame();
+  double uw = 0.0, wmax = 0.0;
+  for (int k = 0; k < 3; ++k) {
+    w[k] /= wl;
+    uw += u[k] * w[k];
+    wmax = fmax(wmax, fabs(w[k]));
+  }
+  double e[3], el = 0.0;  // the drift across the axis
+  for (int k = 0; k < 3; ++k) {
+    e[k] = u[k] - uw * w[k];
+    el += e[k] * e[k];
+  }
+  el = sqrt(el);
+  if (wmax >= 0.9999 && el <= 0.02) return tl_ident_frame();
+  if (el < 1e-3) {  // any axis across w
+    int m = 0;
+    for (int k = 1; k < 3; ++k)
+      if (fabs(w[k]) < fabs(w[m])) m = k;
+    el = 0.0;
+    for (int k = 0; k < 3; ++k) {
+      e[k] = (k == m ? 1.0 : 0.0) - w[m] * w[k];
+      el += e[k] * e[k];
+    }
+    el = sqrt(el);
+  }
+  TLFrame f{};
+  for (int k = 0; k < 3; ++k) {
+    e[k] /= el;
+    f.u[k] = (float)u[k];
+  }
+  const double g[3] = {w[1] * e[2] - w[2] * e[1], w[2] * e[0] - w[0] * e[2],
+                       w[0] * e[1] - w[1] * e[0]};
+  for (int k = 0; k < 3; ++k) {
+    f.r[k] = (float)e[k];
+    f.r[3 + k] = (float)g[k];
+    f.r[6 + k] = (float)w[k];
+  }
+  return f;
+}
+
+// The grid of `bits` bits in all over [lo, lo + range]: each bit halves the cells of
+// the axis that are longest in units of s, the extent of two photons' boxes there.
+// Cells (and so the 32 photons of a leaf) in the proportions of s overlap the fewest
+// other boxes for their volume.
+__host__ __device__ inline TLGrid tl_make_grid(const double lo[3], const double range[3],
+                                               const double s[3], int bits) {
+  TLGrid g{};
+  double rel[3];
+  for (int k = 0; k < 3; ++k) rel[k] = range[k] > 0.0 && s[k] > 0.0 ? range[k] / s[k] : 0.0;
+  for (int b = 0; b < bits; ++b) {
+    int m = 0;
+    for (int k = 1; k < 3; ++k)
+      if (rel[k] > rel[m]) m = k;
+    if (g.nb[m] >= 16) break;
+    ++g.nb[m];
+    rel[m] *= 0.5;
+  }
+  for (int k = 0; k < 3; ++k) {
+    g.lo[k] = (float)lo[k];
+    g.scale[k] = range[k] > 0.0 ? (float)((double)(1u << g.nb[k]) / range[k]) : 0.0f;
+    g.perm[k] = k;
+  }
+  for (int i = 0; i < 2; ++i)  // by falling bits
+    for (int k = 0; k < 2; ++k)
+      if (g.nb[g.perm[k]] < g.nb[g.perm[k + 1]]) {
+        const int t = g.perm[k];
+        g.perm[k] = g.perm[k + 1];
+        g.perm[k + 1] = t;
+      }
+  return g;
+}
+
+#ifdef __CUDACC__
+
+// Swept interval of one axis in FP32 interval arithmetic with directed rounding: the
+// position lies within ep of p and the velocity within ev of v; the segment is
+// P + lambda v for lambda in [0, L], L in [Llo, Lhi]; half = r_max / 2 plus margin.
+__device__ __forceinline__ void swept_axis(float p, float ep, float v, float ev, float Llo,
+                                           float Lhi, float half, float &lo, float &hi) {
+  const float plo = __fsub_rd(p, ep), phi = __fadd_ru(p, ep);
+  const float vlo = __fsub_rd(v, ev), vhi = __fadd_ru(v, ev);
+  const float ldlo = vlo >= 0.f ? __fmul_rd(Llo, vlo) : __fmul_rd(Lhi, vlo);
+  const float ldhi = vhi >= 0.f ? __fmul_ru(Lhi, vhi) : __fmul_ru(Llo, vhi);
+  lo = __fsub_rd(fminf(plo, __fadd_rd(plo, ldlo)), half);
+  hi = __fadd_ru(fmaxf(phi, __fadd_ru(phi, ldhi)), half);
+}
+
+// In the lab frame: the FP64 position of the definition lies within |P32| 2^-23 of
+// P32, and likewise the direction.
+__device__ __forceinline__ void seg_axis(float p, float dc, float Llo, float Lhi, float half,
+                                         float &lo, float &hi) {
+  swept_axis(p, __fmaf_ru(fabsf(p), 1.1920928955078125e-7f, 1e-30f), dc,
+             __fmaf_ru(fabsf(dc), 1.1920928955078125e-7f, 1e-30f), Llo, Lhi, half, lo, hi);
+}
+
+// A photon's swept box in the frame.  Each coordinate of R P from the rounded inputs
+// is off by at most 4u sum |R||P| (u = 2^-24: u of the inputs, 3u of the sum), each of
+// R (d - ubar) by 5u sum |R|(|d| + |ubar|); 6u is taken for both.
+__device__ __forceinline__ TLBox swept_box(const float4 p, const float4 d, const TLFrame &f,
+                                           float Llo, float Lhi, float half) {
+  TLBox b;
+  if (f.ident) {
+    seg_axis(p.x, d.x, Llo, Lhi, half, b.lx, b.hx);
+    seg_axis(p.y, d.y, Llo, Lhi, half, b.ly, b.hy);
+    seg_axis(p.z, d.z, Llo, Lhi, half, b.lz, b.hz);
+    return b;
+  }
+  const float e6 = 6.0f * 5.9604644775390625e-8f;
+  const float vx = d.x - f.u[0], vy = d.y - f.u[1], vz = d.z - f.u[2];
+  const float ax = fabsf(d.x) + fabsf(f.u[0]), ay = fabsf(d.y) + fabsf(f.u[1]),
+              az = fabsf(d.z) + fabsf(f.u[2]);
+  float lo[3], hi[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const float rx = f.r[3 * k], ry = f.r[3 * k + 1], rz = f.r[3 * k + 2];
+    const float q = fmaf(rx, p.x, fmaf(ry, p.y, rz * p.z));
+    const float m = fmaf(fabsf(rx), fabsf(p.x), fmaf(fabsf(ry), fabsf(p.y), fabsf(rz) * fabsf(p.z)));
+    const float v = fmaf(rx, vx, fmaf(ry, vy, rz * vz));
+    const float mv = fmaf(fabsf(rx), ax, fmaf(fabsf(ry), ay, fabsf(rz) * az));
+    swept_axis(q, __fmaf_ru(m, e6, 1e-30f), v, __fmaf_ru(mv, e6, 1e-30f), Llo, Lhi, half, lo[k],
+               hi[k]);
+  }
+  b.lx = lo[0];
+  b.ly = lo[1];
+  b.lz = lo[2];
+  b.hx = hi[0];
+  b.hy = hi[1];
+  b.hz = hi[2];
+  return b;
+}
+
+// Index along the n-dimensional Hilbert curve of 2^b cells a side (J. Skilling,
+// "Programming the Hilbert curve", AIP Conf. Proc. 707, 2004): neighbouring indices
+// are neighbouring cells, so 32 consecutive photons fill a compact region.
+template <int N>
+__device__ __forceinline__ uint32_t hilbert(uint32_t *x, int b) {
+  for (int q = b - 1; q > 0; --q) {
+    const uint32_t low = (1u << q) - 1u;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const bool set = x[i] >> q & 1u;  // invert the low bits of axis 0, or swap them with axis i's
+      const uint32_t t = set ? low : (x[0] ^ x[i]) & low;
+      x[0] ^= t;
+      if (!set) x[i] ^= t;
+    }
+  }
+#pragma unroll
+  for (int i = 1; i < N; ++i) x[i] ^= x[i - 1];  // Gray encode
+  uint32_t t = x[N - 1];
+  t ^= t >> 1;
+  t ^= t >> 2;
+  t ^= t >> 4;
+  t ^= t >> 8;
+  t >>= 1;
+  uint32_t h = 0u;  // interleave, axis 0 highest
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    uint32_t v = (x[i] ^ t) & ((1u << b) - 1u);
+    if (N == 3) {  // up to 10 bits
+      v = (v | v << 16) & 0x030000ffu;
+      v = (v | v << 8) & 0x0300f00fu;
+      v = (v | v << 4) & 0x030c30c3u;
+      v = (v | v << 2) & 0x09249249u;
+    } else {  // up to 16 bits
+      v = (v | v << 8) & 0x00ff00ffu;
+      v = (v | v << 4) & 0x0f0f0f0fu;
+      v = (v | v << 2) & 0x33333333u;
+      v = (v | v << 1) & 0x55555555u;
+    }
+    h |= v << (N - 1 - i);
+  }
+  return h;
+}
+
+// Order key of a point of the frame: the excess bits of the longest axis, then a 2D
+// Hilbert index of the two longest axes' excess over the shortest, then a 3D one of
+// what all three have.
+__device__ __forceinline__ uint32_t order_key(const TLGrid &g, const float c[3]) {
+  uint32_t x[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int a = g.perm[k];
+    const float v = a == 0 ? c[0] : (a == 1 ? c[1] : c[2]);
+    const float fq = fminf(fmaxf((v - g.lo[a]) * g.scale[a], 0.0f), (float)((1u << g.nb[a]) - 1u));
+    x[k] = (uint32_t)fq;
+  }
+  const int b1 = g.nb[g.perm[1]], b2 = g.nb[g.perm[2]];
+  uint32_t key = x[0] >> b1;
+  uint32_t y[2] = {(x[0] & ((1u << b1) - 1u)) >> b2, x[1] >> b2};
+  key = key << (2 * (b1 - b2)) | hilbert<2>(y, b1 - b2);
+  const uint32_t low = (1u << b2) - 1u;
+  uint32_t z[3] = {x[0] & low, x[1] & low, x[2] & low};
+  return key << (3 * b2) | hilbert<3>(z, b2);
+}
+
+#endif

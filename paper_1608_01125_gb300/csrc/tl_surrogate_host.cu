@@ -568,6 +568,7 @@ int trilens_surrogate_step(trilens_ctx *c, int64_t step, int32_t level_L, float 
   if (step != c->built_step) return fail(c, TRILENS_ERR_INVALID, "step not built");
   if (level_L != c->sur->level) return fail(c, TRILENS_ERR_INVALID, "model trained at another L");
   CK(cudaSetDevice(c->device));
+  if (int rcf = need_full(c, step)) return rcf;
   SurrogateState *s = c->sur;
   cudaEvent_t e0, e1, e2;
   CK(cudaEventCreate(&e0));
@@ -644,6 +645,7 @@ int trilens_surrogate_pairs(trilens_ctx *c, int64_t step, int32_t level_L, float
   int rc = ensure_state(c);
   if (rc) return rc;
   SurrogateState *s = c->sur;
+  if ((rc = need_full(c, step))) return rc;
   const double keep_c = c->tot_count, keep_w = c->tot_weighted;
   unsigned ncut = 0;
   if ((rc = sur_cut(c, level_L, &ncut))) return rc;

@@ -1,94 +1,28 @@
-// tl_traverse.cu -- dual-hierarchy traversal, narrow phase, FP64 band
-// re-test and the per-step yield reduction.
+// tl_traverse.cu -- dual traversal of two binary hierarchies from a list of node pairs,
+// its narrow phase, the FP64 band re-test and the per-step yield reduction.
 //
-// The two hierarchies are traversed against each other (Sec. 2.2: depth-first
-// descent; a failed overlap test, Eq. CollDet, skips the whole subtree pair).
-// The frontier of node pairs comes from the refit's seed lists (large beams:
-// every overlapping pair of cut nodes) or from a few breadth-first expansion
-// levels of the root pair; then persistent warps take frontier pairs and
-// descend depth first with a stack of node pairs in shared memory, handing
-// large items on to a device work queue (see k_traverse).  Each
+// The statistical regime works on pairs of the hierarchies' level-L nodes: its exact
+// labels and its exact fallback are the collisions below given node pairs.  Persistent
+// warps take pairs of the list and descend depth first (Sec. 2.2; a failed overlap
+// test, Eq. CollDet, skips the whole subtree pair) with a stack of node pairs in shared
+// memory, handing large items on to a device work queue (see k_traverse).  Each
 // iteration a warp pops up to 32 pairs, one per lane; a lane loads both
 // node records of its pair once and tests the up-to-4 child combinations
 // (both children of each side); survivors are pushed (or, when both sides
 // are leaf buckets, appended to the step's leaf-pair list in blocks of at
-// least 32) with ballot/popc compaction.  A separate kernel (k_narrow) then
-// flattens the listed bucket pairs over its warps' lanes, one photon pair
-// per lane, and gives them the narrow-phase test; hits leave with one atomic
-// per warp.  Splitting the two keeps each kernel's registers low and its
-// warps many, which hides the latency both are bound by.
+// least 32) with ballot/popc compaction.  A separate kernel (k_narrow) then tests the
+// listed bucket pairs' photon pairs.  (The exact path of whole beams is tl_tree.cu.)
 #include "tl_common.cuh"
 #include "tl_exact.cuh"
 #include "tl_narrow.cuh"
+#include "tl_warp.cuh"
 #include "tl_yield.cuh"
 
 namespace tl {
 
 
-// One side of a child pair: the child `slot` of an inner node, or a bucket
-// itself (slot ignored) when ref names a bucket.
-struct Side {
-  TLBox box;
-  uint32_t sref;   // stack reference of this child
-  uint32_t first;  // first photon (buckets)
-  uint32_t cnt;    // photons under it
-  bool bucket;
-};
-
-__device__ __forceinline__ Side side_of(const TLTree &T, uint32_t ref, int slot) {
-  Side s;
-  uint32_t node, sl;
-  if (!(ref & TL_FLAG)) {
-    node = ref;
-    sl = (uint32_t)slot;
-  } else {
-    node = (ref & ~TL_FLAG) >> 1;
-    sl = ref & 1u;
-  }
-  const TLNode *nd = T.nodes + node;
-  const float4 *f = reinterpret_cast<const float4 *>(nd);
-  TLNode v;
-  v.b0 = __ldg(f + 0);
-  v.b1 = __ldg(f + 1);
-  v.b2 = __ldg(f + 2);
-  v.c = __ldg(reinterpret_cast<const int4 *>(f + 3));
-  s.box = tl_child_box(v, (int)sl);
-  const uint32_t cr = (uint32_t)(sl ? v.c.y : v.c.x);
-  s.cnt = (uint32_t)(sl ? v.c.w : v.c.z);
-  s.bucket = (cr & TL_FLAG) != 0u;
-  s.first = cr & ~TL_FLAG;
-  if (ref & TL_FLAG) s.sref = ref;
-  else s.sref = s.bucket ? (TL_FLAG | (node << 1) | sl) : cr;
-  return s;
-}
-
 __device__ __forceinline__ uint32_t pack_bucket(uint32_t first, uint32_t cnt) {
   return first | ((cnt - 1u) << 27);
-}
-
-// For a pair (ra, rb) and a combination index 0..3, the child pair it names.
-// Returns false if the combination does not exist for this pair.
-__device__ __forceinline__ bool child_pair(const TLTree &A, const TLTree &B, uint2 pr, int combo,
-                                           Side &sa, Side &sb) {
-  const bool ain = !(pr.x & TL_FLAG), bin = !(pr.y & TL_FLAG);
-  int ia, ib;
-  if (ain && bin) {
-    ia = combo >> 1;
-    ib = combo & 1;
-  } else if (ain) {
-    if (combo >= 2) return false;
-    ia = combo;
-    ib = 0;
-  } else if (bin) {
-    if (combo >= 2) return false;
-    ia = 0;
-    ib = combo;
-  } else {
-    return false;
-  }
-  sa = side_of(A, pr.x, ia);
-  sb = side_of(B, pr.y, ib);
-  return true;
 }
 
 // Child i (0 or 1) of one side of a popped pair, from the side's node record
@@ -132,242 +66,6 @@ __device__ __forceinline__ TLNode node_record(const TLTree &T, uint32_t ref) {
   return v;
 }
 
-// warp-aggregated append of (x, y) for lanes with pred
-__device__ __forceinline__ void emit(bool pred, uint32_t x, uint32_t y, uint2 *buf,
-                                     unsigned long long cap, unsigned long long *counter,
-                                     unsigned *status, unsigned ovf_bit, int lane) {
-  const unsigned m = __ballot_sync(0xffffffffu, pred);
-  if (!m) return;
-  unsigned long long base = 0;
-  if (lane == 0) base = atomicAdd(counter, (unsigned long long)__popc(m));
-  base = __shfl_sync(0xffffffffu, base, 0);
-  if (pred) {
-    const unsigned long long idx = base + __popc(m & ((1u << lane) - 1u));
-    if (idx < cap) buf[idx] = make_uint2(x, y);
-  }
-  if (lane == 0 && base + __popc(m) > cap) atomicOr(status, ovf_bit);
-}
-
-// ------------------------------------------------------------ init
-
-// run_status (captured runs, else NULL): a queue overflow or an expired wait
-// in an earlier step of the run carries over, so that no later step runs on
-// a queue that may still hold chunks nobody takes (the host repeats the run)
-__global__ void k_step_init(TLCounters *ctr, uint2 *F0, uint32_t superA, uint32_t superB,
-                            int nonempty, const unsigned *build_status,
-                            const unsigned *run_status) {
-  unsigned *w = reinterpret_cast<unsigned *>(ctr);
-  for (int i = threadIdx.x; i < (int)(sizeof(TLCounters) / 4); i += blockDim.x) w[i] = 0u;
-  if (threadIdx.x == 0) F0[0] = make_uint2(superA, superB);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const unsigned bs = *build_status & (unsigned)TL_ST_TIMEOUT;
-    const unsigned rs =
-        run_status ? *run_status & (unsigned)(TL_ST_SPILL_OVF | TL_ST_TIMEOUT) : 0u;
-    ctr->status = bs | rs;
-    // after a failed build there is nothing valid to traverse
-    ctr->counts[0] = (nonempty && !bs && !rs) ? 1u : 0u;
-  }
-}
-
-// Several instances: the frontier starts from each instance's pair of
-// subtree roots, so no pair of photons from different instances is tested.
-__global__ void k_seed_instances(TLCounters *ctr, uint2 *F0, const uint32_t *rootA,
-                                 const uint32_t *rootB, int n_inst) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= n_inst || (ctr->status & (TL_ST_TIMEOUT | TL_ST_SPILL_OVF))) return;
-  const uint32_t ra = rootA[q], rb = rootB[q];
-  if (ra == TL_NONE || rb == TL_NONE) return;
-  const unsigned idx = atomicAdd(&ctr->counts[0], 1u);
-  F0[idx] = make_uint2(ra, rb);
-}
-
-// ------------------------------------------------------------ frontier
-
-// Seeds from the two cut lists written by the refit: every pair (cut node of
-// A, cut node of B) whose boxes overlap (Eq. CollDet).  Every photon lies in
-// exactly one cut node of its beam and a box contains its descendants' boxes,
-// so every overlapping pair of leaf buckets lies below exactly one seed: the
-// traversal from the seeds reaches the same leaf pairs as from the roots.
-__global__ void __launch_bounds__(256) k_seed_cut(TravArgs a, const uint32_t *cutA,
-                                                  const unsigned *cntA, uint32_t capA,
-                                                  const uint32_t *cutB, const unsigned *cntB,
-                                                  uint32_t capB, uint2 *F0, unsigned cap) {
-  TLCounters *ctr = a.ctr;
-  // the build failed, or the queue overflowed earlier in a captured run: nothing to traverse
-  if (ctr->status & (TL_ST_TIMEOUT | TL_ST_SPILL_OVF)) return;
-  const unsigned na = *cntA, nb = *cntB;
-  if (na > capA || nb > capB) {  // a list overflowed: start from the root pair
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-      F0[0] = make_uint2(a.A.super, a.B.super);
-      ctr->counts[0] = 1u;
-    }
-    return;
-  }
-  const unsigned long long total = (unsigned long long)na * nb;
-  const unsigned long long rounded = (total + 31ull) & ~31ull;
-  const int lane = threadIdx.x & 31;
-  unsigned long long tests = 0;
-  for (unsigned long long q = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
-       q < rounded; q += (unsigned long long)gridDim.x * blockDim.x) {
-    bool ok = false;
-    uint2 o = make_uint2(0u, 0u);
-    if (q < total) {
-      const uint32_t ea = cutA[q / nb], eb = cutB[q % nb];
-      const Side sa = side_of(a.A, ea >> 1, (int)(ea & 1u));
-      const Side sb = side_of(a.B, eb >> 1, (int)(eb & 1u));
-      ++tests;
-      ok = tl_overlap(sa.box, sb.box);
-      o = make_uint2(sa.sref, sb.sref);
-    }
-    const unsigned m = __ballot_sync(0xffffffffu, ok);
-    if (m) {
-      unsigned base = 0;
-      if (lane == 0) base = atomicAdd(&ctr->counts[0], (unsigned)__popc(m));
-      base = __shfl_sync(0xffffffffu, base, 0);
-      if (ok) {
-        const unsigned idx = base + __popc(m & ((1u << lane) - 1u));
-        if (idx < cap) F0[idx] = o;
-        else atomicOr(&ctr->status, (unsigned)TL_ST_FRONT_OVF);
-      }
-    }
-  }
-  for (int off = 16; off; off >>= 1) tests += __shfl_xor_sync(0xffffffffu, tests, off);
-  if (lane == 0 && tests) atomicAdd(&ctr->node_tests, tests);
-}
-
-// One block expands the root pair breadth first, level by level, until the
-// frontier holds at least `target` pairs (or nothing is left to expand).
-// Bucket pairs pass through unchanged; failed overlap tests prune.
-__global__ void __launch_bounds__(1024) k_expand(TravArgs a, uint2 *F0, uint2 *F1, unsigned cap,
-                                                 unsigned target, int max_levels) {
-  __shared__ unsigned s_count[2];
-  __shared__ unsigned long long s_tests;
-  TLCounters *ctr = a.ctr;
-  if (threadIdx.x == 0) {
-    s_count[0] = ctr->counts[0];
-    s_count[1] = 0u;
-    s_tests = 0ull;
-  }
-  __syncthreads();
-  const int lane = threadIdx.x & 31;
-  unsigned long long tests = 0;
-  int level = 0;
-  while (true) {
-    const unsigned nin = s_count[level & 1];
-    if (nin >= target || nin == 0u || level >= max_levels) break;
-    const uint2 *in = (level & 1) ? F1 : F0;
-    uint2 *out = (level & 1) ? F0 : F1;
-    unsigned *ocount = &s_count[(level + 1) & 1];
-    const unsigned nround = (nin + 31u) & ~31u;
-    for (unsigned i = threadIdx.x; i < nround; i += blockDim.x) {
-      const bool valid = i < nin;
-      const uint2 pr = valid ? in[i] : make_uint2(0u, 0u);
-      const bool both_buckets = valid && (pr.x & TL_FLAG) && (pr.y & TL_FLAG);
-      for (int combo = 0; combo < 4; ++combo) {
-        Side sa, sb;
-        bool ok = false;
-        uint2 o = make_uint2(0u, 0u);
-        if (valid && !both_buckets && child_pair(a.A, a.B, pr, combo, sa, sb)) {
-          ++tests;
-          ok = tl_overlap(sa.box, sb.box);
-          o = make_uint2(sa.sref, sb.sref);
-        } else if (both_buckets && combo == 0) {
-          ok = true;  // already tested when it was produced: pass through
-          o = pr;
-        }
-        const unsigned m = __ballot_sync(0xffffffffu, ok);
-        if (m) {
-          unsigned base = 0;
-          if (lane == 0) base = atomicAdd(ocount, (unsigned)__popc(m));
-          base = __shfl_sync(0xffffffffu, base, 0);
-          if (ok) {
-            const unsigned idx = base + __popc(m & ((1u << lane) - 1u));
-            if (idx < cap) out[idx] = o;
-            else atomicOr(&ctr->status, (unsigned)TL_ST_FRONT_OVF);
-          }
-        }
-      }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) s_count[level & 1] = 0u;  // the next level's output count
-    ++level;
-    __syncthreads();
-  }
-  for (int off = 16; off; off >>= 1) tests += __shfl_xor_sync(0xffffffffu, tests, off);
-  if (lane == 0 && tests) atomicAdd(&s_tests, tests);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const unsigned n = s_count[level & 1];
-    ctr->counts[level] = n < cap ? n : cap;
-    ctr->final_level = (unsigned)level;
-    ctr->frozen = 1u;
-    ctr->node_tests += s_tests;
-  }
-}
-
-// One breadth-first level of the frontier across the whole grid.  Launched
-// for a fixed number of levels after the seeds; level `level` acts only if it
-// is the frontier's current level and that frontier has fewer than `target`
-// pairs (and its children cannot overflow the buffer, at most 4 per pair):
-// every pair is replaced by its overlapping child pairs (Eq. CollDet; bucket
-// pairs pass through) and the last block to finish moves the frontier on to
-// level + 1.  The decision reads values earlier launches wrote, so every
-// block takes the same one.  A wide frontier gives every traversal warp
-// full 32-pair items from the start.
-__global__ void __launch_bounds__(256) k_widen(TravArgs a, uint2 *F0, uint2 *F1, unsigned cap,
-                                               unsigned target, int level) {
-  TLCounters *ctr = a.ctr;
-  // the build failed, or the queue overflowed earlier in a captured run: nothing to traverse
-  if (ctr->status & (TL_ST_TIMEOUT | TL_ST_SPILL_OVF)) return;
-  if ((int)ctr->final_level != level || level + 1 >= 32) return;
-  const unsigned nin = ctr->counts[level];
-  if (nin == 0u || nin >= target || 4ull * nin > (unsigned long long)cap) return;
-  const uint2 *in = (level & 1) ? F1 : F0;
-  uint2 *out = (level & 1) ? F0 : F1;
-  unsigned *ocount = &ctr->counts[level + 1];
-  const int lane = threadIdx.x & 31;
-  unsigned long long tests = 0;
-  const unsigned nround = (nin + 31u) & ~31u;
-  for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < nround;
-       i += gridDim.x * blockDim.x) {
-    const bool valid = i < nin;
-    const uint2 pr = valid ? in[i] : make_uint2(0u, 0u);
-    const bool both_buckets = valid && (pr.x & TL_FLAG) && (pr.y & TL_FLAG);
-    for (int combo = 0; combo < 4; ++combo) {
-      Side sa, sb;
-      bool ok = false;
-      uint2 o = make_uint2(0u, 0u);
-      if (valid && !both_buckets && child_pair(a.A, a.B, pr, combo, sa, sb)) {
-        ++tests;
-        ok = tl_overlap(sa.box, sb.box);
-        o = make_uint2(sa.sref, sb.sref);
-      } else if (both_buckets && combo == 0) {
-        ok = true;  // already tested when it was produced: pass through
-        o = pr;
-      }
-      const unsigned m = __ballot_sync(0xffffffffu, ok);
-      if (m) {
-        unsigned base = 0;
-        if (lane == 0) base = atomicAdd(ocount, (unsigned)__popc(m));
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if (ok) out[base + __popc(m & ((1u << lane) - 1u))] = o;  // < 4 nin <= cap
-      }
-    }
-  }
-  for (int off = 16; off; off >>= 1) tests += __shfl_xor_sync(0xffffffffu, tests, off);
-  if (lane == 0 && tests) atomicAdd(&ctr->node_tests, tests);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();  // this block's outputs and count before its finish
-    if (atomicAdd(&ctr->widen_done, 1u) == gridDim.x - 1u) {
-      ctr->widen_done = 0u;
-      __threadfence();
-      ctr->final_level = (unsigned)(level + 1);
-    }
-  }
-}
-
 // ------------------------------------------------------------ narrow phase
 
 // a traversal warp's leaf-pair queue: fewer than 32 entries before an iteration,
@@ -386,37 +84,17 @@ struct NarrowSmem {
   uint16_t items[32 * kItemsPerLane];
 };
 
-// The full test of up to 32 pending photon pairs (sorted positions in
-// ws.pend[0 .. cnt)), one per lane; hits and band pairs leave with one
-// atomic per warp each.
+// the full test of the first cnt (<= 32) pending photon pairs
 template <bool FP64>
 __device__ __forceinline__ void decide_pending(const TravArgs &a, const NarrowSmem &ws, int cnt,
                                                int lane, const float *sbin) {
-  int outcome = TL_MISS;
-  uint32_t oi = 0u, oj = 0u;
-  if (lane < cnt) {
-    const uint2 pr = ws.pend[lane];
-    const float4 da = __ldg(a.A.dir + pr.x), db = __ldg(a.B.dir + pr.y);
-    oi = __float_as_uint(da.w);
-    oj = __float_as_uint(db.w);
-    if (FP64) {
-      outcome = tl_exact_hit(a.mA, oi, a.mB, oj, a.ct, a.dt, a.kappa) ? TL_HIT : TL_MISS;
-    } else {
-      const float4 pa = __ldg(a.A.pos + pr.x), pb = __ldg(a.B.pos + pr.y);
-      outcome = tl_narrow32(pa, da, pb, db, a.nk, sbin);
-    }
-  }
-  emit(outcome == TL_HIT, oi, oj, a.hits, a.hit_cap, &a.ctr->hits, &a.ctr->status,
-       TL_ST_HIT_OVF, lane);
-  if (!FP64)
-    emit(outcome == TL_BAND, oi, oj, a.band, a.band_cap, &a.ctr->band, &a.ctr->status,
-         TL_ST_BAND_OVF, lane);
+  decide_pairs<FP64>(a, lane < cnt ? ws.pend[lane] : make_uint2(0u, 0u), lane < cnt, lane, sbin);
 }
 
 // ------------------------------------------------------------ traversal
 
 // Persistent warps share one work queue.  Its items come first from the
-// frontier, in groups of up to 32 node pairs (indices below nf), then from
+// list, in groups of up to 32 node pairs (indices below nf), then from
 // the queue's chunks of up to 32 node pairs each (256 bytes).  A warp that
 // waits for a chunk is counted in ctr->hungry while it waits; a warp that
 // has spent `budget` iterations on its item while h > 0 warps wait hands on
@@ -436,7 +114,7 @@ __device__ __forceinline__ void decide_pending(const TravArgs &a, const NarrowSm
 // nf plus the chunks handed on.  Every wait is bounded by spin_limit (then
 // TL_ST_TIMEOUT).
 constexpr unsigned long long kQFree = 0xffffffffffffffffull;
-constexpr int kGroup = 32;  // frontier pairs per item, node pairs per queue chunk
+constexpr int kGroup = 32;  // listed pairs per item, node pairs per queue chunk
 
 __device__ __forceinline__ unsigned long long pack2(uint2 v) {
   return (unsigned long long)v.x | ((unsigned long long)v.y << 32);
@@ -467,8 +145,7 @@ __device__ __forceinline__ void spill_leaves(const TravArgs &a, const TravSmem &
 }
 
 __global__ void __launch_bounds__(TL_TRAV_MAX_WARPS * 32, TL_TRAV_MINBLOCKS) k_traverse(
-    TravArgs a, const uint2 *F0, const uint2 *F1, const uint2 *list, unsigned long long list_n,
-    int from_frontier, int budget, int part, int nparts) {
+    TravArgs a, const uint2 *list, unsigned long long list_n, int budget, int part, int nparts) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int D = a.stack_depth;
@@ -482,25 +159,13 @@ __global__ void __launch_bounds__(TL_TRAV_MAX_WARPS * 32, TL_TRAV_MINBLOCKS) k_t
   // step's end would no longer be seen.  The host repeats the step (or run)
   // with the queue reset, so nothing more is traversed here.
   if (*(volatile unsigned *)&ctr->status & (TL_ST_SPILL_OVF | TL_ST_TIMEOUT)) return;
-  const uint2 *src0;
-  unsigned long long n0;
-  if (from_frontier) {
-    const unsigned lvl = ctr->final_level;
-    src0 = (lvl & 1u) ? F1 : F0;
-    n0 = ctr->counts[lvl];
-  } else {
-    src0 = list;
-    n0 = list_n;
-  }
-  {  // this launch's part of the frontier: every leaf pair lies below exactly
-     // one frontier pair, so the parts split the step's work
-    const unsigned long long lo = n0 * (unsigned long long)part / (unsigned long long)nparts;
-    const unsigned long long hi = n0 * (unsigned long long)(part + 1) / (unsigned long long)nparts;
-    src0 += lo;
-    n0 = hi - lo;
-  }
+  // this launch's part of the list: the parts split the step's work
+  const unsigned long long lo = list_n * (unsigned long long)part / (unsigned long long)nparts;
+  const unsigned long long hi = list_n * (unsigned long long)(part + 1) / (unsigned long long)nparts;
+  const uint2 *src0 = list + lo;
+  const unsigned long long n0 = hi - lo;
   const unsigned long long lbase = ctr->leaf_base;  // the list of this part starts here
-  const unsigned long long nf = (n0 + kGroup - 1) / kGroup;  // frontier groups
+  const unsigned long long nf = (n0 + kGroup - 1) / kGroup;  // groups of listed pairs
   unsigned long long *Q = a.queue;
   const unsigned long long qcap = a.queue_cap / kGroup;  // chunks
   const unsigned lt = (1u << lane) - 1u;
@@ -615,7 +280,7 @@ __global__ void __launch_bounds__(TL_TRAV_MAX_WARPS * 32, TL_TRAV_MINBLOCKS) k_t
       }
     }
     if (sp == 0) {
-      int got = 0;  // 1: a frontier group; 2: a queue chunk
+      int got = 0;  // 1: a group of listed pairs; 2: a queue chunk
       unsigned long long idx = 0;
       uint2 item = make_uint2(0u, 0u);
       if (lane == 0) {
@@ -668,7 +333,7 @@ __global__ void __launch_bounds__(TL_TRAV_MAX_WARPS * 32, TL_TRAV_MINBLOCKS) k_t
       got = __shfl_sync(0xffffffffu, got, 0);
       if (!got) break;
       idx = __shfl_sync(0xffffffffu, idx, 0);
-      if (got == 1) {  // up to 32 frontier pairs
+      if (got == 1) {  // up to 32 listed pairs
         const unsigned long long f = idx * kGroup + (unsigned long long)lane;
         const bool have = f < n0;
         if (have) stack[lane] = __ldcg(src0 + f);
@@ -698,7 +363,7 @@ __global__ void __launch_bounds__(TL_TRAV_MAX_WARPS * 32, TL_TRAV_MINBLOCKS) k_t
       ra = node_record(a.A, pr.x);
       rb = node_record(a.B, pr.y);
     }
-    // a bucket pair taken from the frontier was tested when it was produced
+    // a bucket pair taken from the list was tested when it was produced
     const bool pass = active && bka && bkb;
     int tested = 0;
 #pragma unroll
@@ -911,17 +576,37 @@ __global__ void __launch_bounds__(256) k_yield(TravArgs a, YieldPartial *partial
 }
 
 // Per-instance yield: count and sum of w_i w_j of each instance's hits,
-// accumulated into yields[2 * inst], yields[2 * inst + 1].
+// accumulated into yields[2 * inst], yields[2 * inst + 1].  A warp's hits mostly belong
+// to one instance: its lanes are summed first, one pair of atomics per run of equal
+// instances (two per hit on a few addresses took 4.8 ms of a 64-instance run of 16
+// steps, this takes 0.29 ms).
 __global__ void __launch_bounds__(256) k_yield_inst(TravArgs a, const uint32_t *inst_of_a,
                                                     double *yields) {
   const unsigned long long n = min(a.ctr->hits, a.hit_cap);
-  for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < n;
+  const unsigned long long nround = (n + 31ull) & ~31ull;
+  const int lane = threadIdx.x & 31;
+  for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < nround;
        i += (unsigned long long)gridDim.x * blockDim.x) {
-    const uint2 h = a.hits[i];
-    const double wi = a.mA.w ? a.mA.w[h.x] : 1.0, wj = a.mB.w ? a.mB.w[h.y] : 1.0;
-    const uint32_t q = inst_of_a[h.x];
-    atomicAdd(&yields[2 * q], 1.0);
-    atomicAdd(&yields[2 * q + 1], wi * wj);
+    uint32_t q = TL_NONE;
+    double w = 0.0;
+    if (i < n) {
+      const uint2 h = a.hits[i];
+      w = (a.mA.w ? a.mA.w[h.x] : 1.0) * (a.mB.w ? a.mB.w[h.y] : 1.0);
+      q = inst_of_a[h.x];
+    }
+    unsigned left = __ballot_sync(0xffffffffu, i < n);
+    while (left) {
+      const uint32_t q0 = __shfl_sync(0xffffffffu, q, __ffs(left) - 1);
+      const unsigned m = __ballot_sync(0xffffffffu, q == q0);
+      double s = q == q0 ? w : 0.0;
+#pragma unroll
+      for (int off = 16; off; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+      if (lane == 0) {
+        atomicAdd(&yields[2 * (size_t)q0], (double)__popc(m));
+        atomicAdd(&yields[2 * (size_t)q0 + 1], s);
+      }
+      left &= ~m;
+    }
   }
 }
 
@@ -952,36 +637,6 @@ size_t traverse_smem(int warps, int depth) {
   return sizeof(uint2) * (size_t)depth * warps + sizeof(TravSmem) * (size_t)warps;
 }
 
-cudaError_t launch_step_init(TLCounters *ctr, uint2 *F0, uint32_t sa, uint32_t sb, int nonempty,
-                             const unsigned *build_status, const unsigned *run_status,
-                             cudaStream_t s) {
-  k_step_init<<<1, 128, 0, s>>>(ctr, F0, sa, sb, nonempty, build_status, run_status);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_seed_cut(const TravArgs &a, const uint32_t *cutA, const unsigned *cntA,
-                            uint32_t capA, const uint32_t *cutB, const unsigned *cntB,
-                            uint32_t capB, uint2 *F0, unsigned cap, int blocks, cudaStream_t s) {
-  k_seed_cut<<<blocks, 256, 0, s>>>(a, cutA, cntA, capA, cutB, cntB, capB, F0, cap);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_expand(const TravArgs &a, uint2 *F0, uint2 *F1, unsigned cap, unsigned target,
-                          int max_levels, cudaStream_t s) {
-  k_expand<<<1, 1024, 0, s>>>(a, F0, F1, cap, target, max_levels);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_widen(const TravArgs &a, uint2 *F0, uint2 *F1, unsigned cap, unsigned target,
-                         int levels, int blocks, cudaStream_t s) {
-  for (int l = 0; l < levels; ++l) {
-    k_widen<<<blocks, 256, 0, s>>>(a, F0, F1, cap, target, l);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
-}
-
 cudaError_t traverse_config(int fp64, int warps, int depth, int *blocks_per_sm) {
   (void)fp64;  // the traversal is the same for both precisions (the narrow phase differs)
   const size_t smem = traverse_smem(warps, depth);
@@ -992,14 +647,13 @@ cudaError_t traverse_config(int fp64, int warps, int depth, int *blocks_per_sm) 
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k_traverse, warps * 32, smem);
 }
 
-cudaError_t launch_traverse(const TravArgs &a, const uint2 *F0, const uint2 *F1, const uint2 *list,
-                            unsigned long long list_n, int from_frontier, int budget, int blocks,
-                            int warps, cudaStream_t s, int part, int nparts) {
+cudaError_t launch_traverse(const TravArgs &a, const uint2 *list, unsigned long long list_n,
+                            int budget, int blocks, int warps, cudaStream_t s, int part,
+                            int nparts) {
   // a warp only waits for work that warps holding items (running ones) hand
   // on, so no block needs another to be resident
   const size_t smem = traverse_smem(warps, a.stack_depth);
-  k_traverse<<<blocks, warps * 32, smem, s>>>(a, F0, F1, list, list_n, from_frontier, budget,
-                                              part, nparts);
+  k_traverse<<<blocks, warps * 32, smem, s>>>(a, list, list_n, budget, part, nparts);
   return cudaGetLastError();
 }
 
@@ -1033,12 +687,6 @@ cudaError_t launch_yield(const TravArgs &a, void *partials, int blocks, cudaStre
 }
 
 size_t partial_bytes() { return sizeof(YieldPartial); }
-
-cudaError_t launch_seed_instances(TLCounters *ctr, uint2 *F0, const uint32_t *rootA,
-                                  const uint32_t *rootB, int n_inst, cudaStream_t s) {
-  k_seed_instances<<<(n_inst + 255) / 256, 256, 0, s>>>(ctr, F0, rootA, rootB, n_inst);
-  return cudaGetLastError();
-}
 
 cudaError_t launch_yield_inst(const TravArgs &a, const uint32_t *inst_of_a, double *yields,
                               int blocks, cudaStream_t s) {
