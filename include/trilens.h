@@ -2,12 +2,12 @@
  * trilens.h -- C ABI of the GB300 (sm_103a) Breit-Wheeler collision library.
  *
  * Two beams of photons (macro-photons) move on straight lines.  Each time
- * step the library builds, for each beam, a bounding-volume hierarchy over
- * the boxes swept by its photons during the step (Sec. 2.1: a BV grows by the
- * distance its particles travel in one step, so collisions are found before
- * they happen), traverses the two hierarchies against each other with the
- * axis-aligned overlap test (Eq. CollDet; depth-first descent, Sec. 2.2), and
- * tests the surviving photon pairs.  A pair (i in A, j in B) collides in step
+ * step the library orders both beams along a space-filling curve and builds a
+ * bounding-volume hierarchy over the boxes swept by the smaller beam's photons
+ * during the step (Sec. 2.1: a BV grows by the distance its particles travel in
+ * one step, so collisions are found before they happen), descends it with groups
+ * of the other beam's photons by the axis-aligned overlap test (Eq. CollDet;
+ * depth first, Sec. 2.2), and tests the surviving photon pairs.  A pair (i in A, j in B) collides in step
  * k when
  *     s = E_i E_j (1 - cos Phi) / (2 m_e^2 c^4) > 1           (Eq. eq.Cond)
  *     t* = time of the pair's closest approach, 0 <= t* - t_k < dt
@@ -76,6 +76,8 @@ typedef struct {
   double dt_fs;        /* time step [fs], > 0 */
   double kappa;        /* cross-section amplification, > 0 (r^2 = kappa sigma / pi) */
   int32_t precision;   /* enum trilens_precision */
+  /* the statistical regime's hierarchies and its seeded traversal (the exact path
+   * has no knobs): */
   int32_t leaf_bucket; /* photons per hierarchy leaf, 1..32 (0: 4) */
   int32_t stack_depth; /* traversal stack entries per warp, 64..4096 (0: 512) */
   int32_t block_shape; /* traversal warps per block, 1..8 (0: 4) */
@@ -89,9 +91,12 @@ typedef struct {
   double weighted;      /* sum over H_k of w_i w_j (FP64) */
   uint64_t hsum;        /* sum of splitmix64((i << 32) | j) mod 2^64 over H_k */
   uint64_t hxor;        /* xor of the same (order-free checksum pair) */
-  int64_t narrow_tests; /* photon pairs given the narrow-phase test */
+  int64_t narrow_tests; /* photon pairs given the narrow-phase test: those of two
+                           overlapping leaves that neither photon's box against the
+                           other leaf's has decided (first the pair's swept boxes are
+                           tested, then the closest approach) */
   int64_t node_tests;   /* box-pair overlap tests during traversal */
-  int64_t leaf_pairs;   /* overlapping leaf pairs */
+  int64_t leaf_pairs;   /* overlapping leaves (32 photons each) */
   int64_t band;         /* pairs re-tested in FP64 (FP32_BAND mode) */
   int64_t retries;      /* internal buffer regrowths in this step */
 } trilens_step_stats;
@@ -103,14 +108,16 @@ typedef struct {
 int trilens_create(trilens_ctx **out, const trilens_beam *a, const trilens_beam *b,
                    const trilens_params *p, trilens_stream_t stream);
 
-/* Build both hierarchies for step `step` (t_k = step * dt): propagate
- * positions in closed form p0 + c t_k d (FP64), form the FP32 swept boxes
- * (Sec. 2.1), Morton-sort them and emit the hierarchy (Sec. 2.1, 2.2).
+/* Prepare step `step` (t_k = step * dt): propagate positions in closed form
+ * p0 + c t_k d (FP64), sort both beams along a Hilbert curve, form the FP32 swept
+ * boxes (Sec. 2.1) and the smaller beam's hierarchy (Sec. 2.1, 2.2); in a context
+ * that uses the statistical regime, the two binary hierarchies in Morton order that
+ * it works on (a collision of the whole beams then builds what it needs itself).
  * Asynchronous.  INVALID if step < 0. */
 int trilens_build(trilens_ctx *c, int64_t step);
 
-/* Collide the hierarchies built for `step` (trilens_build must have been
- * called with the same step).  Adds the step's counters to the cumulative
+/* Collide the beams at `step` (trilens_build must have been called with the
+ * same step).  Adds the step's counters to the cumulative
  * yield.  If hits != NULL (device, 2*cap uint32: (i_A, j_B) pairs, order
  * unspecified), the step's pairs are written to it; if more than cap exist
  * the call writes nothing, adds nothing to the yield, returns CAPACITY and
@@ -135,9 +142,7 @@ int trilens_yield(trilens_ctx *c, int32_t mode, int32_t level_L, double *count,
 /* Run time steps first_step .. first_step+steps-1 of a single (non-batch)
  * context -- trilens_build + trilens_collide_step for each, in step order --
  * as one captured CUDA graph on the context's stream, with no host round
- * trip between steps (each step's traversal is one launch whose warps share
- * a device work queue, so no step needs the host).  The graph is captured on the
- * first call and replayed while (first_step, steps) stay the same.  Adds the
+ * trip between steps.  The graph is captured on the first call and replayed while (first_step, steps) stay the same.  Adds the
  * run's yield to the cumulative yield; out (host, may be NULL) receives the
  * run's totals: step = steps, count, weighted, the checksums (hsum summed,
  * hxor xored over the steps) and the work counters.  Hit lists are not

@@ -24,34 +24,30 @@ extern "C" {
  * normal operation.  INVALID for a NULL context. */
 int trilens_debug_stall_sort(trilens_ctx *c, int on);
 
-/* Do the traversal and narrow phase of every following step in `parts`
- * slices of its frontier (1..4096), as the library does by itself when a
- * step's leaf-pair list would exceed its largest size (2^30 pairs).  The hit
- * set never depends on it.  INVALID for a NULL context or parts outside
- * 1..4096. */
+/* Do the collisions of every following step in `parts` slices of the query
+ * beam's photons (a seeded traversal: of its seeds; 1..4096), as the library does
+ * by itself when a step's candidate list would exceed its largest size (2^30
+ * pairs).  The hit set never depends on it.  INVALID for a NULL context or parts
+ * outside 1..4096. */
 int trilens_debug_set_parts(trilens_ctx *c, int32_t parts);
 
 /* Replace the context's spin limit (iterations of every bounded device wait,
  * >= 1).  INVALID for a NULL context or limit < 1. */
 int trilens_debug_set_spin_limit(trilens_ctx *c, int64_t limit);
 
-/* Morton resolution of a single context's keys: bits per axis (4..21; the
- * default is a few bits beyond one cell per photon).  The hit set never
- * depends on it (the hierarchy only prunes); tests use it to check that, and
- * to time the sort (ceil(3 bits / 8) digit passes) against tree quality.
- * The next collisions need a fresh build.  INVALID for a NULL or batch
- * context or bits outside 4..21. */
+/* Resolution of a single context's keys: bits per axis of the statistical regime's
+ * Morton keys (4..21), and three times as many (at most 30) for the exact path's
+ * Hilbert keys.  The hit set never depends on it (the hierarchy only prunes); tests
+ * use it to check that, and to time the sort against tree quality.  The next
+ * collisions need a fresh build.  INVALID for a NULL or batch context or bits
+ * outside 4..21. */
 int trilens_debug_set_key_bits(trilens_ctx *c, int32_t bits);
 
-/* Capacity of the traversal-seed lists the refit writes (children with at
- * most n/64 photons of nodes with more; normally a few hundred).  cap
- * below the list's length makes the next collisions start from the root pair
- * instead -- the path taken when a list overflows -- so tests can check that
- * both starts give the same hits.  cap <= 0 restores the allocated capacity.
+/* Kept for its callers and without effect: the traversal has no seed lists any more.
  * INVALID for a NULL context. */
 int trilens_debug_set_cut_cap(trilens_ctx *c, int32_t cap);
 
-/* Replace the internal hit, band, leaf-pair and hand-on buffers with buffers of cap
+/* Replace the internal hit, band, candidate and hand-on buffers with buffers of cap
  * pairs each (>= 1), so that the next collisions overflow them and exercise
  * the regrow-and-repeat path.  Synchronises the stream.  INVALID for a NULL
  * context or cap < 1. */
@@ -67,10 +63,10 @@ int trilens_debug_eval64(const double *x, double *out, int64_t n, int32_t which,
 
 /* Per-phase device time.  on != 0 records CUDA events around every kernel
  * phase on the context's stream (cheap, but adds event records).  The
- * phases, in order: 0 propagate+Morton, 1 radix sort, 2 gather, 3 hierarchy
- * emit, 4 refit, 5 frontier (seeds, expansion, widening), 6 dual traversal
- * (listing the overlapping leaf-bucket pairs), 7 FP64 band re-test, 8 yield
- * reduction, 9 FP32 narrow phase of the listed leaf pairs. */
+ * phases, in order: 0 propagate and key, 1 radix sort, 2 gather, 3 emit of the
+ * statistical regime's hierarchies, 4 boxes (their refit), 5 unused, 6 collisions
+ * (descent and first look; seeded: the dual traversal), 7 FP64 band re-test, 8 yield
+ * reduction, 9 narrow phase of what the descent leaves (seeded: of the leaf pairs). */
 int trilens_debug_timing(trilens_ctx *c, int on);
 
 /* Copy the accumulated milliseconds of the 10 phases into out[0..9], the

@@ -269,7 +269,7 @@ static int alloc_beam(trilens_ctx *c, tl::BuildBufs &w, int64_t n, int64_t padde
 }
 
 // the statistical regime's hierarchies and the seeded traversal's queues, on first use
-static int ensure_full(trilens_ctx *c) {
+int ensure_full(trilens_ctx *c) {
   if (c->full_ready) return TRILENS_OK;
   for (int k = 0; k < 2; ++k) {
     tl::BuildBufs &w = c->w[k];

@@ -180,6 +180,7 @@ tl::TravArgs trav_args(trilens_ctx *c, double ct);
 int run_exact(trilens_ctx *c, double ct, const uint2 *seeds, unsigned n_seeds, int *retries);
 // make the statistical regime's hierarchies stand for `step` (a no-op if they do)
 int need_full(trilens_ctx *c, int64_t step);
+int ensure_full(trilens_ctx *c);  // its buffers
 void surrogate_free(trilens_ctx *c);
 void deplete_free(trilens_ctx *c);
 double tl_sigma_max_bound();

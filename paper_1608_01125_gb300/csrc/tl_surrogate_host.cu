@@ -145,6 +145,7 @@ static int cut_buffers(trilens_ctx *c, unsigned cap) {
 
 static int ensure_state(trilens_ctx *c) {
   if (c->sur) return TRILENS_OK;
+  if (int rc = ensure_full(c)) return rc;
   c->sur = new SurrogateState();
   SurrogateState *s = c->sur;
   CK(tl::mlp_prepare());
