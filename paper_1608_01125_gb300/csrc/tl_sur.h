@@ -1,7 +1,5 @@
 // tl_sur.h -- declarations shared by the surrogate translation units.
 #pragma once
-#include <cuda_bf16.h>
-
 #include "tl_common.cuh"
 
 namespace tl {
@@ -31,18 +29,6 @@ struct CutArgs {
   unsigned *cut_count;
   unsigned cut_cap;
   unsigned *status;
-};
-
-// device workspace of the network
-struct MLPWork {
-  __nv_bfloat16 *W1, *W2, *W3, *W4;
-  __nv_bfloat16 *Z[3], *dZ[3];
-  float *dout;
-  float *wpart;  // per-block partial weight gradients (rows / 512 slices of all parameters)
-  float *grad;
-  float *loss;
-  int *err;
-  int64_t cap;  // rows the training buffers hold
 };
 
 cudaError_t launch_prefix_moments(const TLBeam &B, const float4 *pos, const float4 *dir, int64_t n,
@@ -75,14 +61,12 @@ cudaError_t launch_sur_misc(int op, const void *a, const void *b, void *c, int64
                             cudaStream_t s);
 
 cudaError_t mlp_prepare();
-cudaError_t mlp_work_alloc(MLPWork &w, int64_t rows);
-void mlp_work_free(MLPWork &w);
-cudaError_t mlp_pack(const float *prm, MLPWork &w, cudaStream_t s);
-cudaError_t mlp_forward(const float *prm, const float *norm, const MLPWork &w, const float *x,
-                        int64_t M, float *out, int blocks, long long spin, cudaStream_t s);
-cudaError_t mlp_grad(const float *prm, const float *norm, const MLPWork &w, const float *x,
-                     const float *y, int64_t M, int blocks, long long spin, cudaStream_t s,
-                     int kind, const float *st, float st_scale);
+size_t mlp_grad_floats(int64_t M, int sms);  // workspace of mlp_grad
+cudaError_t mlp_forward(const float *prm, const float *norm, const float *x, int64_t M, float *out,
+                        int sms, int *err, long long spin, cudaStream_t s);
+cudaError_t mlp_grad(const float *prm, const float *norm, const float *x, const float *y, int64_t M,
+                     int sms, float *part, float *grad, float *loss, int *err, long long spin,
+                     cudaStream_t s, int kind, const float *st, float st_scale);
 cudaError_t mlp_adamw(float *prm, const float *grad, float *m, float *v, float lr, float wd,
                       int step, cudaStream_t s);
 

@@ -21,7 +21,8 @@ static inline double tau_edge(int g) { return std::ldexp(1.0, -10) * std::pow(2.
 struct SurrogateState {
   // model
   float *prm = nullptr, *mom1 = nullptr, *mom2 = nullptr, *norm = nullptr;
-  tl::MLPWork work{};
+  float *part = nullptr, *grad = nullptr, *loss = nullptr;  // training workspace
+  int *err = nullptr;  // device: a tensor-core wait ran out
   bool trained = false;
   int level = -1;
   double calib = 1.0, st_calib = 1.0, st_only_calib = 1.0;
@@ -66,7 +67,10 @@ static void sfree(SurrogateState *s) {
   cudaFree(s->mom1);
   cudaFree(s->mom2);
   cudaFree(s->norm);
-  tl::mlp_work_free(s->work);
+  cudaFree(s->part);
+  cudaFree(s->grad);
+  cudaFree(s->loss);
+  cudaFree(s->err);
   for (int k = 0; k < 2; ++k) {
     cudaFree(s->pre[k]);
     cudaFree(s->bsum[k]);
@@ -153,7 +157,11 @@ static int ensure_state(trilens_ctx *c) {
   CK(dalloc(&s->mom1, TRILENS_MLP_PARAMS));
   CK(dalloc(&s->mom2, TRILENS_MLP_PARAMS));
   CK(dalloc(&s->norm, 48));
-  CK(tl::mlp_work_alloc(s->work, kBatch));
+  CK(dalloc(&s->part, tl::mlp_grad_floats(kBatch, c->n_sm)));
+  CK(dalloc(&s->grad, TRILENS_MLP_PARAMS));
+  CK(dalloc(&s->loss, 1));
+  CK(dalloc(&s->err, 1));
+  CK(cudaMemsetAsync(s->err, 0, sizeof(int), c->stream));
   for (int k = 0; k < 2; ++k) {
     const int64_t n = std::max<int64_t>(c->beam[k].n, 1);
     CK(dalloc(&s->pre[k], (size_t)6 * (n + 1)));
@@ -466,17 +474,17 @@ int trilens_surrogate_fit(trilens_ctx *c, int32_t epochs, uint64_t seed) {
       const int64_t r0 = b * kBatch, m = std::min<int64_t>(kBatch, Ntr - r0);
       const double t = (double)s->adam_step / (double)std::max<int64_t>(total_steps - 1, 1);
       const float lr = (float)(lr1 + 0.5 * (lr0 - lr1) * (1.0 + cos(3.14159265358979323846 * t)));
-      if (tl::mlp_pack(s->prm, s->work, c->stream) ||
-          tl::mlp_grad(s->prm, s->norm, s->work, dx + 24 * r0, dy + r0, m, c->n_sm,
-                       c->p.spin_limit, c->stream, 1, dst + r0, (float)s->st_calib) ||
-          tl::mlp_adamw(s->prm, s->work.grad, s->mom1, s->mom2, lr, 1e-4f, ++s->adam_step,
+      if (tl::mlp_grad(s->prm, s->norm, dx + 24 * r0, dy + r0, m, c->n_sm, s->part, s->grad,
+                       s->loss, s->err, c->p.spin_limit, c->stream, 1, dst + r0,
+                       (float)s->st_calib) ||
+          tl::mlp_adamw(s->prm, s->grad, s->mom1, s->mom2, lr, 1e-4f, ++s->adam_step,
                         c->stream)) {
         rc = fail(c, TRILENS_ERR_CUDA, "training step failed");
         break;
       }
       if (b == nb - 1 || (b & 63) == 63) {
         float l = 0;
-        cudaMemcpyAsync(&l, s->work.loss, sizeof(float), cudaMemcpyDeviceToHost, c->stream);
+        cudaMemcpyAsync(&l, s->loss, sizeof(float), cudaMemcpyDeviceToHost, c->stream);
         cudaStreamSynchronize(c->stream);
         lsum = l / (double)m;
       }
@@ -485,7 +493,7 @@ int trilens_surrogate_fit(trilens_ctx *c, int32_t epochs, uint64_t seed) {
   }
   int herr = 0;
   if (!rc) {
-    CK(cudaMemcpy(&herr, s->work.err, sizeof(int), cudaMemcpyDeviceToHost));
+    CK(cudaMemcpy(&herr, s->err, sizeof(int), cudaMemcpyDeviceToHost));
     if (herr) rc = fail(c, TRILENS_ERR_TIMEOUT, "a tensor-core wait ran out during training");
   }
   // calibration of the summed estimates on the samples (for the network,
@@ -495,12 +503,11 @@ int trilens_surrogate_fit(trilens_ctx *c, int32_t epochs, uint64_t seed) {
   std::vector<double> bl(kTauBins + 1, 0.0), be(kTauBins + 1, 0.0);  // per spread bin
   std::vector<float> hout;
   std::vector<double> hpred, hlb;
-  if (!rc && tl::mlp_pack(s->prm, s->work, c->stream)) rc = fail(c, TRILENS_ERR_CUDA, "pack");
   for (int64_t r0 = c0; !rc && r0 < N; r0 += s->cut_cap) {
     const int64_t m = std::min<int64_t>(s->cut_cap, N - r0);
     const unsigned mm = (unsigned)m;
     double a = 0, b = 0, d = 0;
-    if (tl::mlp_forward(s->prm, s->norm, s->work, dx + 24 * r0, m, s->out, c->n_sm,
+    if (tl::mlp_forward(s->prm, s->norm, dx + 24 * r0, m, s->out, c->n_sm, s->err,
                         c->p.spin_limit, c->stream) ||
         cudaMemcpyAsync(s->cut_count, &mm, sizeof(unsigned), cudaMemcpyHostToDevice, c->stream) ||
         cudaMemsetAsync(s->fb_count, 0, sizeof(unsigned), c->stream) ||
@@ -580,8 +587,7 @@ int trilens_surrogate_step(trilens_ctx *c, int64_t step, int32_t level_L, float 
   int rc = sur_cut(c, level_L, &ncut);
   if (rc) return rc;
   CK(cudaEventRecord(e1, c->stream));
-  CK(tl::mlp_pack(s->prm, s->work, c->stream));
-  CK(tl::mlp_forward(s->prm, s->norm, s->work, s->feat, ncut, s->out, c->n_sm, c->p.spin_limit,
+  CK(tl::mlp_forward(s->prm, s->norm, s->feat, ncut, s->out, c->n_sm, s->err, c->p.spin_limit,
                      c->stream));
   CK(cudaMemsetAsync(s->fb_count, 0, sizeof(unsigned), c->stream));
   CK(tl::launch_estimate(s->out, s->st, (float)s->st_calib, s->cut, s->cut_count, s->cut_cap, tau,
@@ -662,9 +668,8 @@ int trilens_surrogate_pairs(trilens_ctx *c, int64_t step, int32_t level_L, float
   uint8_t *flag = nullptr;
   if (want_net) {
     CK(dalloc(&flag, ncut));
-    CK(tl::mlp_pack(s->prm, s->work, c->stream));
-    CK(tl::mlp_forward(s->prm, s->norm, s->work, s->feat, ncut, s->out, c->n_sm,
-                       c->p.spin_limit, c->stream));
+    CK(tl::mlp_forward(s->prm, s->norm, s->feat, ncut, s->out, c->n_sm, s->err, c->p.spin_limit,
+                       c->stream));
     CK(cudaMemsetAsync(s->fb_count, 0, sizeof(unsigned), c->stream));
     CK(tl::launch_estimate(s->out, s->st, (float)s->st_calib, s->cut, s->cut_count, s->cut_cap,
                            tau, s->pred, s->fb, s->fb_count, s->cut_cap, 4 * c->n_sm, c->stream,
