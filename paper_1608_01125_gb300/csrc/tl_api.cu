@@ -78,13 +78,13 @@ static tl::ColArgs col_args(trilens_ctx *c, int p) {
   const int q = 1 - c->tree, t = c->tree;
   tl::ColArgs a;
   memset(&a, 0, sizeof(a));
-  a.qpos = c->w[q].pos;
-  a.qdir = c->w[q].dir;
-  a.tpos = c->w[t].pos;
-  a.tdir = c->w[t].dir;
+  a.q = c->w[q].rec;
+  a.t = c->w[t].rec;
   a.box = c->box;
   a.qinst = c->insts[q];
   a.tinst = c->insts[t];
+  a.qstart = c->w[q].start;
+  a.tstart = c->w[t].start;
   a.tile_inst = c->tile_inst[q];
   a.frames = c->frames;
   a.Llo = c->L_lo;
@@ -218,12 +218,14 @@ TLNarrowConst tl_narrow_const(double dt_fs, double kappa) {
 }
 
 static void free_beam(tl::BuildBufs &w) {
+  cudaFree(w.stat);
   cudaFree(w.pos_u);
   cudaFree(w.dir_u);
-  cudaFree(w.pos);
-  cudaFree(w.dir);
-  cudaFree(w.key32[0]);
-  cudaFree(w.key32[1]);
+  cudaFree(w.rec);
+  cudaFree(w.cell);
+  cudaFree(w.count);
+  cudaFree(w.start);
+  cudaFree(w.scan_st);
   cudaFree(w.val[0]);
   cudaFree(w.val[1]);
   cudaFree(w.key[0]);
@@ -246,36 +248,70 @@ static void free_beam(tl::BuildBufs &w) {
   memset(&w, 0, sizeof(w));
 }
 
-// the buffers every step needs: SoAs, keys and sort scratch
-static int alloc_beam(trilens_ctx *c, tl::BuildBufs &w, int64_t n, int64_t padded) {
+// the buffers every step needs: SoAs and the counting sort's cells
+static int alloc_beam(trilens_ctx *c, tl::BuildBufs &w, int64_t n, int64_t padded, int64_t cells) {
   const size_t m = (size_t)std::max<int64_t>(n, 1), mp = (size_t)std::max<int64_t>(padded, 1);
-  CK(dalloc(&w.pos_u, m));
-  CK(dalloc(&w.dir_u, m));
-  CK(dalloc(&w.pos, mp));
-  CK(dalloc(&w.dir, mp));
-  for (int k = 0; k < 2; ++k) {
-    CK(dalloc(&w.key32[k], m));
-    CK(dalloc(&w.val[k], m));
+  CK(dalloc(&w.stat, 2 * m));
+  CK(dalloc(&w.rec, 2 * mp));
+  w.pos = w.rec;  // the statistical regime's two arrays
+  w.dir = w.rec + mp;
+  CK(dalloc(&w.cell, m));
+  w.cells = cells;
+  CK(dalloc(&w.count, (size_t)cells));
+  CK(cudaMemsetAsync(w.count, 0, sizeof(uint32_t) * (size_t)cells, c->stream));
+  CK(dalloc(&w.start, (size_t)cells + 1));
+  CK(dalloc(&w.scan_st, (size_t)tl::scan_tiles(cells) + 1));
+  return TRILENS_OK;
+}
+
+// moments of both beams in a frame, and their extremes (ext NULL: not wanted)
+static int beam_moments(trilens_ctx *c, const TLFrame &f, double mom[2][15], double ext[2][14]) {
+  const size_t md = tl::moment_doubles();
+  double *dev = nullptr, h[2][29];
+  CK(cudaMalloc((void **)&dev, sizeof(double) * 2 * md));
+  cudaError_t e = cudaSuccess;
+  for (int k = 0; k < 2 && !e; ++k) {
+    e = tl::launch_beam_moments(c->beam[k], f, dev + k * md, c->stream);
+    if (!e)
+      e = cudaMemcpyAsync(h[k], dev + k * md, sizeof(h[k]), cudaMemcpyDeviceToHost, c->stream);
   }
-  w.sort_tiles = (int64_t)((m + TL_SORT_TILE - 1) / TL_SORT_TILE);
-  w.sort_epoch = 0;
-  CK(dalloc(&w.sort_status, (size_t)w.sort_tiles * 256));
-  CK(dalloc(&w.sort_ep, 9));
-  CK(dalloc(&w.sort_raw, 8 * 256));
-  CK(cudaMemsetAsync(w.sort_raw, 0, sizeof(uint32_t) * 8 * 256, c->stream));
-  CK(dalloc(&w.sort_hist, 8 * 256));
-  CK(dalloc(&w.sort_tile, 8));
+  if (!e) e = cudaStreamSynchronize(c->stream);
+  cudaFree(dev);
+  CK(e);
+  for (int k = 0; k < 2; ++k) {
+    memcpy(mom[k], h[k], sizeof(double) * 15);
+    if (ext) memcpy(ext[k], h[k] + 15, sizeof(double) * 14);
+  }
   return TRILENS_OK;
 }
 
 // the statistical regime's hierarchies and the seeded traversal's queues, on first use
 int ensure_full(trilens_ctx *c) {
   if (c->full_ready) return TRILENS_OK;
+  if (c->frame0.ident) {
+    memcpy(c->moments, c->fmoments, sizeof(c->moments));
+  } else {
+    const int rcm = beam_moments(c, tl_ident_frame(), c->moments, nullptr);
+    if (rcm) return rcm;
+  }
   for (int k = 0; k < 2; ++k) {
     tl::BuildBufs &w = c->w[k];
     const size_t m = (size_t)std::max<int64_t>(c->beam[k].n, 1);
-    CK(dalloc(&w.key[0], m));
-    CK(dalloc(&w.key[1], m));
+    CK(dalloc(&w.pos_u, m));
+    CK(dalloc(&w.dir_u, m));
+    CK(tl::launch_static_soa(c->beam[k], w, c->stream));
+    for (int q = 0; q < 2; ++q) {
+      CK(dalloc(&w.key[q], m));
+      CK(dalloc(&w.val[q], m));
+    }
+    w.sort_tiles = (int64_t)((m + TL_SORT_TILE - 1) / TL_SORT_TILE);
+    w.sort_epoch = 0;
+    CK(dalloc(&w.sort_status, (size_t)w.sort_tiles * 256));
+    CK(dalloc(&w.sort_ep, 9));
+    CK(dalloc(&w.sort_raw, 8 * 256));
+    CK(cudaMemsetAsync(w.sort_raw, 0, sizeof(uint32_t) * 8 * 256, c->stream));
+    CK(dalloc(&w.sort_hist, 8 * 256));
+    CK(dalloc(&w.sort_tile, 8));
     CK(dalloc(&w.nodes, m));
     CK(dalloc(&w.parent_leaf, m));
     CK(dalloc(&w.parent_node, m));
@@ -307,18 +343,13 @@ int ensure_full(trilens_ctx *c) {
   return TRILENS_OK;
 }
 
-// one instance's part of a beam of n photons: its tiles, and the levels of its tree
-static TLInst make_inst(int64_t n, int64_t off, int64_t tile0) {
-  TLInst I;
-  memset(&I, 0, sizeof(I));
-  I.n = (int)n;
-  I.tile0 = (int)tile0;
-  I.pad = (int)(tile0 * kTile - off);
-  I.cnt[0] = (int)n;
-  for (int l = 1; l < 6; ++l) I.cnt[l] = (I.cnt[l - 1] + 31) / 32;
-  I.top = 1;
-  while (I.top < 5 && I.cnt[I.top] > 32) ++I.top;
-  return I;
+// bits of the cells that order n photons: 2 to 4 cells per photon spread evenly, so up
+// to a leaf's worth of photons per cell where a Gaussian bunch is densest (ten times the
+// cells per photon cost more to scan than the finer order saves)
+static int order_bits_for(int64_t n) {
+  int lg = 0;
+  while ((1ll << lg) < n) ++lg;
+  return std::max(4, lg + 1);
 }
 
 // The exact path's layout of both beams (sizes[k]: photons of every instance).
@@ -328,14 +359,17 @@ static int layout(trilens_ctx *c, const std::vector<int64_t> sizes[2]) {
   for (int k = 0; k < 2; ++k) {
     std::vector<TLInst> in(ni);
     std::vector<uint32_t> tile_inst;
-    std::vector<int> pad(ni);
-    int64_t off = 0, tile = 0;
+    int64_t tile = 0, cells = 0;
     for (size_t q = 0; q < ni; ++q) {
-      in[q] = make_inst(sizes[k][q], off, tile);
-      pad[q] = in[q].pad;
+      TLInst &I = in[q];
+      memset(&I, 0, sizeof(I));
+      I.n = (int)sizes[k][q];
+      I.tile0 = (int)tile;
+      I.bits = order_bits_for(sizes[k][q]);
+      I.cell0 = (uint32_t)cells;
+      cells += 1ll << in[q].bits;
       const int64_t t = (sizes[k][q] + kTile - 1) / kTile;
       if (ni > 1) tile_inst.insert(tile_inst.end(), (size_t)t, (uint32_t)q);
-      off += sizes[k][q];
       tile += t;
     }
     c->n_tiles[k] = (int)tile;
@@ -345,11 +379,12 @@ static int layout(trilens_ctx *c, const std::vector<int64_t> sizes[2]) {
         in[q].lev[0] = (uint32_t)((uint64_t)in[q].tile0 * kTile);
         in[q].lev[1] = (uint32_t)((uint64_t)tile * kTile + (uint64_t)in[q].tile0 * 32);
         in[q].lev[2] = (uint32_t)((uint64_t)tile * (kTile + 32) + (uint64_t)in[q].tile0);
-        for (int l = 3; l <= in[q].top; ++l) {
+        const int top = tl_top_level(in[q].n);
+        for (int l = 3; l <= top; ++l) {
           in[q].lev[l] = (uint32_t)up;
-          up += (uint64_t)in[q].cnt[l];
+          up += (uint64_t)tl_level_count(in[q].n, l);
         }
-        c->max_top = std::max(c->max_top, in[q].top);
+        c->max_top = std::max(c->max_top, top);
       }
       CK(dalloc(&c->box, 2 * (size_t)up));
     }
@@ -360,25 +395,13 @@ static int layout(trilens_ctx *c, const std::vector<int64_t> sizes[2]) {
       CK(dalloc(&c->tile_inst[k], tile_inst.size()));
       CK(cudaMemcpyAsync(c->tile_inst[k], tile_inst.data(), sizeof(uint32_t) * tile_inst.size(),
                          cudaMemcpyHostToDevice, c->stream));
-      CK(dalloc(&c->pad[k], ni));
-      CK(cudaMemcpyAsync(c->pad[k], pad.data(), sizeof(int) * ni, cudaMemcpyHostToDevice,
-                         c->stream));
     }
-    const int rc = alloc_beam(c, c->w[k], c->beam[k].n, tile * kTile);
+    const int rc = alloc_beam(c, c->w[k], c->beam[k].n, tile * kTile, cells);
     if (rc) return rc;
-    CK(cudaStreamSynchronize(c->stream));  // the host tables are read
+    // (copies from pageable memory have read the host tables when they return)
   }
   CK(dalloc(&c->frames, ni));
   return TRILENS_OK;
-}
-
-// bits of the order keys for a largest instance of n photons: 4 cells per photon
-// spread evenly, so a few photons per cell where a Gaussian bunch is densest, rounded
-// up to whole 8-bit sort passes together with the instance number's bits
-static int order_bits_for(int64_t n, int inst_bits) {
-  int lg = 0;
-  while ((1ll << lg) < n) ++lg;
-  return std::min(30, std::min(32, 8 * ((lg + 2 + inst_bits + 7) / 8)) - inst_bits);
 }
 
 // ---- C ABI
@@ -433,7 +456,6 @@ void trilens_destroy(trilens_ctx *c) {
     cudaFree(c->inst_bounds[k]);
     cudaFree(c->insts[k]);
     cudaFree(c->tile_inst[k]);
-    cudaFree(c->pad[k]);
     cudaFree(c->grids[k]);
     for (int a = 0; a < 8; ++a) cudaFree(c->owned[k][a]);
   }
@@ -509,8 +531,7 @@ static int ctx_create(trilens_ctx **out, const trilens_beam *a, const trilens_be
   }
   for (int k = 0; k < 2; ++k) {
     c->w[k].build_status = c->build_status;
-    // the step-invariant FP32 direction, index and energy, once
-    CK(tl::launch_static_soa(c->beam[k], c->w[k], c->stream));
+    CK(tl::launch_static(c->beam[k], c->w[k].stat, c->stream));
     int64_t n = std::max<int64_t>(c->beam[k].n, 2);
     int lg = 0;
     while ((1ll << lg) < n) ++lg;
@@ -520,39 +541,35 @@ static int ctx_create(trilens_ctx **out, const trilens_beam *a, const trilens_be
     c->w[k].key_bits = c->key_bits[k];
   }
   if (!sizes) {
-    c->order_bits = order_bits_for(std::max(c->beam[0].n, c->beam[1].n), 0);
-    // one-time moments of p0 and d: in the lab frame for the mean directions (the
-    // frame) and the Morton boxes, then in the frame for the grids of every step
-    double *mom = nullptr;
-    const size_t md = tl::moment_doubles();
-    CK(cudaMalloc((void **)&mom, sizeof(double) * 2 * md));
-    cudaError_t me = cudaSuccess;
+    for (int k = 0; k < 2; ++k) c->order_bits[k] = order_bits_for(c->beam[k].n);
+    // one-time: the beams' mean directions (the frame), then their moments and extremes in
+    // the frame, for the grids and boxes of every step
     c->frame0 = tl_ident_frame();
-    for (int pass = 0; pass < 2 && !me; ++pass) {
-      double(*dst)[15] = pass ? c->fmoments : c->moments;
-      for (int k = 0; k < 2 && !me; ++k) {
-        me = tl::launch_beam_moments(c->beam[k], c->frame0, mom + k * md, c->stream);
-        if (!me)
-          me = cudaMemcpyAsync(dst[k], mom + k * md, sizeof(double) * 15, cudaMemcpyDeviceToHost,
-                               c->stream);
-      }
+    if (c->beam[0].n > 0 && c->beam[1].n > 0) {
+      const int nd = tl::mean_doubles();
+      std::vector<double> h(2 * (size_t)nd);
+      double *part = nullptr;
+      CK(cudaMalloc((void **)&part, sizeof(double) * h.size()));
+      cudaError_t me = cudaSuccess;
+      for (int k = 0; k < 2 && !me; ++k)
+        me = tl::launch_mean_dir(c->beam[k], part + k * nd, c->stream);
+      if (!me)
+        me = cudaMemcpyAsync(h.data(), part, sizeof(double) * h.size(), cudaMemcpyDeviceToHost,
+                             c->stream);
       if (!me) me = cudaStreamSynchronize(c->stream);
-      if (pass || me) break;
-      memcpy(c->fmoments, c->moments, sizeof(c->moments));
-      if (c->beam[0].n > 0 && c->beam[1].n > 0) {
-        double mean[2][3];
-        for (int k = 0; k < 2; ++k)
-          for (int x = 0; x < 3; ++x) mean[k][x] = c->moments[k][3 + x] / (double)c->beam[k].n;
-        c->frame0 = tl_make_frame(mean[0], mean[1]);
-      }
-      if (c->frame0.ident) break;  // the same moments
+      cudaFree(part);
+      CK(me);
+      double mean[2][3] = {};
+      for (int k = 0; k < 2; ++k)
+        for (int q = 0; q < nd; ++q)
+          mean[k][q % 3] += h[(size_t)k * nd + q] / (double)tl::mean_count(c->beam[k].n);
+      c->frame0 = tl_make_frame(mean[0], mean[1]);
     }
-    if (!me)
-      me = cudaMemcpyAsync(c->frames, &c->frame0, sizeof(TLFrame), cudaMemcpyHostToDevice,
-                           c->stream);
-    if (!me) me = cudaStreamSynchronize(c->stream);
-    cudaFree(mom);
-    CK(me);
+    CK(cudaMemcpyAsync(c->frames, &c->frame0, sizeof(TLFrame), cudaMemcpyHostToDevice, c->stream));
+    if ((rc = beam_moments(c, c->frame0, c->fmoments, c->ext))) {
+      trilens_destroy(c);
+      return rc;
+    }
   }
   CK(tl::sort_prepare());
   CK(tl::refit_prepare());
@@ -647,7 +664,8 @@ static void step_grids(trilens_ctx *c, double T, TLGrid g[2]) {
       lo[k] = mean - 0.5 * c->L64 * ru[k] - sd5;
       range[k] = 2.0 * sd5;
     }
-    g[h] = tl_make_grid(lo, range, s, c->order_bits);
+    g[h] = tl_make_grid(lo, range, s, c->order_bits[h]);
+    tl_beam_box(c->ext[1 - h], c->ext[1 - h][12], c->ext[1 - h][13], c->frame0, T - 0.5 * c->L64, c->L64, c->half, g[h].clo, g[h].chi);
   }
 }
 
@@ -657,52 +675,71 @@ static int build_exact(trilens_ctx *c, int64_t step) {
   const double T = ct + 0.5 * c->L64;
   const bool batch = c->n_inst > 1;
   TLGrid grid[2];
-  int ib = 0;
-  while ((1 << ib) < c->n_inst) ++ib;
   if (batch)
-    CK(tl::launch_inst_grid(c->inst_bounds[0], c->inst_bounds[1], c->frames, c->n_inst, T, c->L64,
-                            c->half, c->order_bits, c->grids[0], c->grids[1], c->stream));
+    CK(tl::launch_inst_grid(c->inst_bounds[0], c->inst_bounds[1], c->frames, c->insts[0],
+                            c->insts[1], c->n_inst, T, c->L64, c->half, c->grids[0], c->grids[1],
+                            c->stream));
   else
     step_grids(c, T, grid);
+  c->exact_step = step;
+  c->full_step = -1;  // the two builds share the sorted photons
+  // The root of the descent, tested on the host: where the boxes of all swept boxes of
+  // the two beams do not meet (Eq. CollDet), no photon of one meets one of the other,
+  // and the step has nothing to order or to test.
+  c->apart = c->beam[0].n <= 0 || c->beam[1].n <= 0;
+  for (int k = 0; k < 3 && !batch; ++k)
+    c->apart = c->apart || grid[0].clo[k] > grid[1].chi[k] || grid[1].clo[k] > grid[0].chi[k];
+  if (c->apart) return TRILENS_OK;
   bool fork;
   if (int rc = fork_builds(c, &fork)) return rc;
   for (int k = 0; k < 2; ++k) {
-    const int64_t n = c->beam[k].n;
-    if (n <= 0) continue;
     cudaStream_t st = (fork && k == 1) ? c->side_stream : c->stream;
     tl::BuildBufs &w = c->w[k];
-    const int bits = c->order_bits + ib, passes = (bits + 7) / 8;
     tmark(c, PH_PROP, k, 0);
     tl::OrderArgs o;
     memset(&o, 0, sizeof(o));
-    o.b = c->beam[k];
-    o.ct = ct;
+    o.n = c->beam[k].n;
+    o.stat = w.stat;
+    o.ct = (float)ct;
     o.L = (float)c->L64;
+    o.half = c->half;
     o.frames = c->frames;
     if (!batch) o.grid = grid[k];
     o.grids = c->grids[k];
     o.inst_of = c->inst_of[k];
-    o.inst_shift = c->order_bits;
-    o.passes = passes;
-    o.pos_u = w.pos_u;
-    o.dir_u = w.dir_u;
-    o.key = w.key32[0];
-    o.hist = w.sort_raw;
+    o.inst = c->insts[k];
+    o.cell = w.cell;
+    o.count = w.count;
+    o.scan_st = w.scan_st;
+    o.scan_tiles = (int)tl::scan_tiles(w.cells);
+    if (c->n_inst <= 1) o.inst_of = nullptr;
     CK(tl::launch_order(o, st));
     tmark(c, PH_PROP, k, 1);
     tmark(c, PH_SORT, k, 0);
-    CK(tl::launch_sort32(w, n, bits, c->pad[k], c->order_bits, c->p.spin_limit,
-                         c->debug_stall_sort, c->build_status, st));
+    CK(tl::launch_cell_scan(w.count, w.start, w.cells, w.scan_st, c->p.spin_limit,
+                            c->debug_stall_sort, c->build_status, st));
+    tl::PlaceArgs pl;
+    memset(&pl, 0, sizeof(pl));
+    pl.b = c->beam[k];
+    pl.ct = ct;
+    pl.n_pad = (int64_t)c->n_tiles[k] * kTile;
+    pl.stat = w.stat;
+    pl.cell = w.cell;
+    pl.start = w.start;
+    pl.inst_of = o.inst_of;
+    pl.inst = c->insts[k];
+    pl.rec = w.rec;
+    CK(tl::launch_place(pl, st));
     tmark(c, PH_SORT, k, 1);
     c->phase_launches[PH_PROP] += 1;
-    c->phase_launches[PH_SORT] += 1 + passes;
+    c->phase_launches[PH_SORT] += 2;
     if (k != c->tree) continue;
     tmark(c, PH_REFIT, k, 0);
     tl::BoxArgs b;
     memset(&b, 0, sizeof(b));
-    b.pos = w.pos;
-    b.dir = w.dir;
+    b.rec = w.rec;
     b.inst = c->insts[k];
+    b.start = w.start;
     b.tile_inst = c->tile_inst[k];
     b.frames = c->frames;
     b.Llo = c->L_lo;
@@ -714,10 +751,7 @@ static int build_exact(trilens_ctx *c, int64_t step) {
     tmark(c, PH_REFIT, k, 1);
     c->phase_launches[PH_REFIT] += c->max_top >= 3 ? 2 : 1;
   }
-  if (int rc = join_builds(c, fork)) return rc;
-  c->exact_step = step;
-  c->full_step = -1;  // the two builds share the sorted photons
-  return TRILENS_OK;
+  return join_builds(c, fork);
 }
 
 // The statistical regime's binary hierarchies of both beams, in Morton order.
@@ -831,8 +865,10 @@ tl::TravArgs trav_args(trilens_ctx *c, double ct) {
   memset(&a, 0, sizeof(a));
   for (int k = 0; k < 2; ++k) {
     TLTree &t = k ? a.B : a.A;
-    t.pos = c->w[k].pos;
-    t.dir = c->w[k].dir;
+    const bool full = c->full_step >= 0;  // the buffers hold the statistical regime's order
+    t.pos = full ? c->w[k].pos : c->w[k].rec;
+    t.dir = full ? c->w[k].dir : c->w[k].rec + 1;
+    t.stride = full ? 1u : 2u;
     t.nodes = c->w[k].nodes;
     t.n = c->beam[k].n;
     t.super = (uint32_t)(t.n > 1 ? t.n - 1 : 0);
@@ -868,7 +904,8 @@ int run_exact(trilens_ctx *c, double ct, const uint2 *seeds, unsigned n_seeds, i
   while (true) {
     tl::TravArgs a = trav_args(c, ct);
     CK(tl::launch_step_init(c->ctr, c->build_status, nullptr, c->stream));
-    const int rcp = seeds ? traverse_parts(c, a, seeds, n_seeds) : collide_parts(c, a);
+    const int rcp = seeds ? traverse_parts(c, a, seeds, n_seeds)
+                          : (c->apart ? TRILENS_OK : collide_parts(c, a));
     if (rcp) return rcp;
     c->phase_launches[PH_TRAV] += c->parts;
     c->phase_launches[PH_NARROW] += c->parts;
@@ -1004,7 +1041,7 @@ int trilens_batch_create(trilens_ctx **out, const trilens_beam *a, const trilens
   if (!out) return TRILENS_ERR_INVALID;
   *out = nullptr;
   if (!a || !b || !p || n_inst < 1 || n_inst > 65536) return TRILENS_ERR_INVALID;
-  int64_t tot[2] = {0, 0}, nmax = 1;
+  int64_t tot[2] = {0, 0};
   std::vector<int64_t> sizes[2];
   for (int q = 0; q < n_inst; ++q) {
     if (!beam_ok(&a[q]) || !beam_ok(&b[q])) return TRILENS_ERR_INVALID;
@@ -1012,7 +1049,6 @@ int trilens_batch_create(trilens_ctx **out, const trilens_beam *a, const trilens
     sizes[1].push_back(b[q].n);
     tot[0] += a[q].n;
     tot[1] += b[q].n;
-    nmax = std::max<int64_t>(nmax, std::max(a[q].n, b[q].n));
   }
   if (tot[0] >= (1ll << 27) || tot[1] >= (1ll << 27)) return TRILENS_ERR_INVALID;
   // a throwaway context holds the owned inputs while they are gathered
@@ -1049,9 +1085,6 @@ int trilens_batch_create(trilens_ctx **out, const trilens_beam *a, const trilens
   }
   c->n_inst = n_inst;
   if (n_inst > 1) {
-    int ib = 0;
-    while ((1 << ib) < n_inst) ++ib;
-    c->order_bits = order_bits_for(nmax, ib);
     CK(cudaMalloc((void **)&c->inst_tmp, sizeof(long long) * 12 * n_inst));
     for (int k = 0; k < 2; ++k) {
       CK(dalloc(&c->inst_bounds[k], (size_t)12 * n_inst));
@@ -1108,7 +1141,7 @@ static int capture_run(trilens_ctx *c, int64_t first, int64_t steps, double *yie
   if (e != cudaSuccess) rc = fail(c, TRILENS_ERR_CUDA, "capture: %s", cudaGetErrorString(e));
   for (int64_t k = first; rc == TRILENS_OK && k < first + steps; ++k) {
     rc = build_exact(c, k);
-    if (rc == TRILENS_OK) rc = graph_collide(c, k, yields);
+    if (rc == TRILENS_OK && !c->apart) rc = graph_collide(c, k, yields);
   }
   cudaGraph_t g = nullptr;
   e = cudaStreamEndCapture(c->cap_stream, &g);
@@ -1146,7 +1179,7 @@ static int replay_run(trilens_ctx *c, int64_t first_step, int64_t steps, double 
     const unsigned st = *c->run_status_host | *c->build_status_host;
     if (int rf = status_failure(c, *c->run_status_host, *c->build_status_host)) return rf;
     if (!(st & (TL_ST_HIT_OVF | TL_ST_BAND_OVF | TL_ST_LEAFQ))) {
-      c->built_step = c->exact_step = first_step + steps - 1;  // the run's last step is built
+      c->built_step = first_step + steps - 1;  // (collided again, it is ordered again)
       return TRILENS_OK;
     }
     // grow what overflowed (to the largest size a step asked for) and capture again
@@ -1556,7 +1589,8 @@ int trilens_debug_set_key_bits(trilens_ctx *c, int32_t bits) {
     c->key_bits[k] = 3 * bits;
     c->w[k].key_bits = c->key_bits[k];
   }
-  c->order_bits = std::min(30, 3 * bits);
+  for (int k = 0; k < 2; ++k)  // at most what the cells are allocated for
+    c->order_bits[k] = std::min(order_bits_for(c->beam[k].n), 3 * bits);
   if (c->gexec) {  // a captured run holds the old pass count
     cudaGraphExecDestroy(c->gexec);
     c->gexec = nullptr;

@@ -117,6 +117,7 @@ struct TLBeam {
 struct TLTree {
   const float4 *pos;    // sorted: x y z E (FP32)
   const float4 *dir;    // sorted: dx dy dz, w = input index (int bits)
+  uint32_t stride;      // float4s from one photon to the next in pos and dir
   const TLNode *nodes;  // n - 1 inner nodes, then the super root at index n - 1
   uint32_t super;       // index of the super root (max(n - 1, 0))
   int64_t n;
@@ -162,12 +163,21 @@ struct InstSrc {
 cudaError_t launch_gather_instances(const InstSrc *src, int n_inst, int64_t n, double *const *dst,
                                     uint32_t *inst_of, cudaStream_t s);
 struct BuildBufs {
+  float4 *stat;               // the step-invariant FP32 records (two float4 per photon)
+  // sorted photons: the exact path's in tiles (tl_frame.cuh), position and direction of a
+  // photon side by side (one 32-byte sector); the statistical regime's as two arrays in
+  // the same buffer
+  float4 *rec;
+  float4 *pos, *dir;
+  // exact path: cell and rank in it of every photon; photons per cell (zero between
+  // steps), their running sum, and the scan's tile words and tile counter
+  uint2 *cell;
+  uint32_t *count, *start, *scan_st;
+  int64_t cells;
+  // from here to sort_ep: the statistical regime's, allocated with it
   float4 *pos_u, *dir_u;      // unsorted SoA32
-  float4 *pos, *dir;          // sorted SoA32 (the exact path's in tiles, see tl_frame.cuh)
-  uint32_t *key32[2];         // the exact path's keys
-  uint32_t *val[2];
-  // from here to rsuper: the statistical regime's, allocated with it
   unsigned long long *key[2];
+  uint32_t *val[2];
   TLNode *nodes;
   uint32_t *parent_leaf, *parent_node;
   float *rpre, *rsuf;  // per photon: union of the swept boxes from its tile's start / to its end
@@ -223,9 +233,6 @@ cudaError_t launch_static_soa(const TLBeam &b, BuildBufs &w, cudaStream_t s);
 cudaError_t sort_prepare();
 cudaError_t launch_sort(BuildBufs &w, int64_t n, int key_bits, long long spin_limit,
                         int debug_stall, unsigned int *status, int *out_sel, cudaStream_t s);
-cudaError_t launch_sort32(BuildBufs &w, int64_t n, int key_bits, const int *pad, int pad_shift,
-                          long long spin_limit, int debug_stall, unsigned int *status,
-                          cudaStream_t s);
 cudaError_t launch_gather(BuildBufs &w, int64_t n, cudaStream_t s);
 cudaError_t launch_karras(BuildBufs &w, int64_t n, int sel, int bucket, cudaStream_t s);
 cudaError_t launch_refit(BuildBufs &w, int64_t n, float Llo, float Lhi, float half, int n_sm,

@@ -25,10 +25,10 @@ struct trilens_ctx {
   float L_lo = 0, L_hi = 0, half = 0;
   TLNarrowConst nk{};
   int bits[2]{}, key_bits[2]{};  // Morton keys of the statistical regime
-  int order_bits = 0;            // the exact path's keys, all axes together
+  int order_bits[2]{};           // the exact path's cells, all axes together (not batches)
   // per beam and axis: sums of p0, d, p0^2, p0 d, d^2 (one-time, fixed order), in the
-  // lab frame and in the exact path's frame
-  double moments[2][15]{}, fmoments[2][15]{};
+  // exact path's frame and (for the statistical regime) in the lab frame
+  double fmoments[2][15]{}, moments[2][15]{};
   // build workspace
   tl::BuildBufs w[2]{};
   int sel[2]{};
@@ -43,10 +43,11 @@ struct trilens_ctx {
   int tree = 1;                  // the beam with the tree
   TLInst *insts[2]{};            // device, per instance
   uint32_t *tile_inst[2]{};      // device, instance of every tile (batches)
-  int *pad[2]{};                 // device, TLInst::pad per instance (batches)
   TLGrid *grids[2]{};            // device, per instance (batches)
   int n_tiles[2]{};
   int max_top = 1;               // over the trees of all instances
+  double ext[2][14]{};           // extremes of R p0 and R d (tl_beam_box; not batches)
+  bool apart = false;            // the beams' boxes do not meet at exact_step
   float4 *box = nullptr;         // all boxes of the trees
   // traversal workspace
   int n_sm = 0, trav_warps = 4, trav_blocks = 0;

@@ -23,23 +23,37 @@ struct TLFrame {
 };
 
 // Ordering grid of one instance and step: cell = (x' - lo) scale, nb bits per axis,
-// axes by falling nb (perm).
+// axes by falling nb (perm); and the box that holds every swept box of the other beam's
+// photons: a photon whose own misses it can meet none of them.
 struct TLGrid {
   float lo[3], scale[3];
   int nb[3], perm[3];
+  float clo[3], chi[3];
 };
 
 // One instance's photons of one beam in the exact path's layout: tiles of 1024
 // sorted photons from tile0 on, and its tree, an implicit one with 32 children per
-// node over the sorted photons: level 0 the photons, level l nodes of 32^l.
+// node over the sorted photons: level 0 the photons, level l nodes of 32^l.  Only the
+// photons that can meet the other beam in a step are sorted; how many, the running sum
+// of the cells tells (tl_live).
 struct TLInst {
-  int n;       // photons
-  int tile0;   // first tile
-  int pad;     // sorted position of the concatenated beam -> padded position
-  int top;     // lowest level with at most 32 nodes (>= 1)
+  int n;            // photons
+  int tile0;        // first tile
+  int bits;         // its photons are ordered by 2^bits cells,
+  uint32_t cell0;   // from this one on
   uint32_t lev[6];  // first box of each level
-  int cnt[6];       // nodes of each level
 };
+
+// nodes of level l over n photons
+__host__ __device__ inline int tl_level_count(int n, int l) {
+  return (int)(((long long)n + (1ll << (5 * l)) - 1) >> (5 * l));
+}
+// the lowest level (>= 1) with at most 32 nodes
+__host__ __device__ inline int tl_top_level(int n) {
+  int l = 1;
+  while (l < 5 && tl_level_count(n, l) > 32) ++l;
+  return l;
+}
 
 constexpr int kTile = 1024;  // sorted photons per tile (a level-2 node)
 
@@ -134,7 +148,29 @@ __host__ __device__ inline TLGrid tl_make_grid(const double lo[3], const double 
   return g;
 }
 
+// The box of every swept box of a beam at the step: from the extremes pmin, dmin,
+// pmax, dmax of R p0 and R d (e[0..11]), ct = c t_k >= 0, the travel L and the pad half.
+// p1, d1: the largest |p0|_1 and |d|_1 where the extremes were found in FP32 (each is off
+// by less than 2^-22 of them), else 0.
+__host__ __device__ inline void tl_beam_box(const double *e, double p1, double d1,
+                                            const TLFrame &f, double ct, double L, double half,
+                                            float clo[3], float chi[3]) {
+  for (int k = 0; k < 3; ++k) {
+    const double ru = (double)f.r[3 * k] * f.u[0] + (double)f.r[3 * k + 1] * f.u[1] +
+                      (double)f.r[3 * k + 2] * f.u[2];
+    const double lo = e[k] + ct * e[3 + k], hi = e[6 + k] + ct * e[9 + k];
+    const double m = half + 1e-6 * (1.0 + fabs(lo) + fabs(hi) + ct + L + p1 + (ct + L) * d1);
+    clo[k] = (float)(lo + fmin(0.0, L * (e[3 + k] - ru)) - m);
+    chi[k] = (float)(hi + fmax(0.0, L * (e[9 + k] - ru)) + m);
+  }
+}
+
 #ifdef __CUDACC__
+
+// photons of an instance that are sorted this step
+__device__ __forceinline__ int tl_live(const TLInst &I, const uint32_t *start) {
+  return (int)(__ldg(start + I.cell0 + (1u << I.bits)) - __ldg(start + I.cell0));
+}
 
 // Swept interval of one axis in FP32 interval arithmetic with directed rounding: the
 // position lies within ep of p and the velocity within ev of v; the segment is

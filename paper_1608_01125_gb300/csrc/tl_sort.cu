@@ -1,4 +1,5 @@
-// tl_sort.cu -- stable LSD radix sort of (32- or 64-bit key, 32-bit index) pairs.
+// tl_sort.cu -- stable LSD radix sort of (64-bit key, 32-bit index) pairs, for the
+// statistical regime's Morton order (the exact path counts its cells: tl_tree.cu).
 //
 // 8-bit digits.  The key kernel counts every digit of every pass while it
 // writes the keys; one scan turns the counts into digit offsets; then one
@@ -68,9 +69,8 @@ __global__ void k_sort_scan(uint32_t *raw, uint32_t *hist, uint32_t *tile_ctr, u
   }
 }
 
-template <class K>
 struct SortSmem {
-  K keys[kSortTile];
+  unsigned long long keys[kSortTile];
   uint32_t vals[kSortTile];
   uint32_t wcnt[8][kRadix];  // per-warp digit counts, then per-warp offsets
   uint32_t dexcl[kRadix];    // tile-local exclusive digit offsets
@@ -79,19 +79,16 @@ struct SortSmem {
   uint32_t tile;
 };
 
-// vin NULL: the first pass, whose values are the positions themselves.  kout NULL: the
-// last pass of a sort whose keys nobody reads.  pad (with pad_shift): photons of
-// instance key >> pad_shift move on by pad[instance] (batches).
-template <class K>
+// vin NULL: the first pass, whose values are the positions themselves.
 __global__ void __launch_bounds__(256, 4) k_sort_pass(
-    const K *__restrict__ kin, const uint32_t *__restrict__ vin, K *__restrict__ kout,
-    uint32_t *__restrict__ vout, int64_t n, int shift,
+    const unsigned long long *__restrict__ kin, const uint32_t *__restrict__ vin,
+    unsigned long long *__restrict__ kout, uint32_t *__restrict__ vout, int64_t n, int shift,
     const uint32_t *__restrict__ digit_base, uint32_t *status, uint32_t *tile_ctr,
     const uint32_t *epoch_p, long long spin_limit, int debug_stall, unsigned int *st_flags,
     const float4 *__restrict__ pos_u, const float4 *__restrict__ dir_u, float4 *__restrict__ pos,
-    float4 *__restrict__ dir, const int *__restrict__ pad, int pad_shift) {
+    float4 *__restrict__ dir) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  SortSmem<K> &sm = *reinterpret_cast<SortSmem<K> *>(smem_raw);
+  SortSmem &sm = *reinterpret_cast<SortSmem *>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid == 0) sm.tile = atomicAdd(tile_ctr, 1u);
   for (int i = tid; i < 8 * kRadix; i += kSortThreads) (&sm.wcnt[0][0])[i] = 0;
@@ -100,7 +97,7 @@ __global__ void __launch_bounds__(256, 4) k_sort_pass(
   const int64_t base = (int64_t)tile * kSortTile;
   const unsigned lt = (1u << lane) - 1u;
 
-  K k[kSortItems];
+  unsigned long long k[kSortItems];
   uint32_t v[kSortItems];
   uint32_t rank[kSortItems];
   uint32_t dig[kSortItems];
@@ -108,7 +105,7 @@ __global__ void __launch_bounds__(256, 4) k_sort_pass(
   for (int it = 0; it < kSortItems; ++it) {
     const int64_t idx = base + warp * (32 * kSortItems) + it * 32 + lane;
     const bool valid = idx < n;
-    k[it] = valid ? kin[idx] : (K)0;
+    k[it] = valid ? kin[idx] : 0ull;
     v[it] = valid ? (vin ? vin[idx] : (uint32_t)idx) : 0u;
     dig[it] = valid ? (uint32_t)((k[it] >> shift) & 255u) : 256u;
   }
@@ -198,15 +195,15 @@ __global__ void __launch_bounds__(256, 4) k_sort_pass(
   const int64_t rem = n - base;
   const int tcount = rem < kSortTile ? (int)rem : kSortTile;
   for (int j = tid; j < tcount; j += kSortThreads) {
-    const K kk = sm.keys[j];
+    const unsigned long long kk = sm.keys[j];
     const uint32_t d = (uint32_t)((kk >> shift) & 255u);
     const uint32_t g = sm.gbase[d] + (uint32_t)j - sm.dexcl[d];
     if ((int64_t)g < n) {  // always true unless a wait expired (then the result is discarded)
-      if (kout) kout[g] = kk;
-      if (pos) {  // last pass: gather the photon itself into the sorted order
-        const uint32_t src = sm.vals[j], to = g + (pad ? (uint32_t)pad[kk >> pad_shift] : 0u);
-        pos[to] = pos_u[src];
-        dir[to] = dir_u[src];
+      kout[g] = kk;
+      if (pos) {  // last pass: gather the photon itself into Morton order
+        const uint32_t src = sm.vals[j];
+        pos[g] = pos_u[src];
+        dir[g] = dir_u[src];
       } else {
         vout[g] = sm.vals[j];
       }
@@ -216,65 +213,41 @@ __global__ void __launch_bounds__(256, 4) k_sort_pass(
 
 // Kernel attributes of the sort (before any launch or stream capture).
 cudaError_t sort_prepare() {
-  cudaError_t e = cudaFuncSetAttribute(k_sort_pass<uint32_t>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)sizeof(SortSmem<uint32_t>));
-  if (e) return e;
-  return cudaFuncSetAttribute(k_sort_pass<unsigned long long>,
-                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)sizeof(SortSmem<unsigned long long>));
+  return cudaFuncSetAttribute(k_sort_pass, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)sizeof(SortSmem));
 }
 
-// Sort key[0] by the low key_bits bits and gather the SoA into w.pos / w.dir in the
-// sorted order (the last pass does it).  The key kernel has counted every pass's
-// digits into w.sort_raw (which the scan clears again, as it does the tile counters;
-// both are zero when allocated).  n <= 1: nothing is sorted or gathered.  keys: the
-// sorted keys are wanted; *out_sel receives the buffer that holds them.
-template <class K>
-static cudaError_t sort_keys(BuildBufs &w, K *const key[2], int64_t n, int key_bits, bool keys,
-                             const int *pad, int pad_shift, long long spin_limit, int debug_stall,
-                             unsigned int *status, int *out_sel, cudaStream_t s) {
+// Sort w.key[0] by the low key_bits bits and gather the SoA into w.pos / w.dir in the
+// sorted order (the last pass does it).  *out_sel receives the buffer index holding the
+// sorted keys.  The key kernel has counted every pass's digits into w.sort_raw (which
+// the scan clears again, as it does the tile counters; both are zero when allocated).
+// n <= 1: nothing is sorted or gathered.
+cudaError_t launch_sort(BuildBufs &w, int64_t n, int key_bits, long long spin_limit,
+                        int debug_stall, unsigned int *status, int *out_sel, cudaStream_t s) {
+  *out_sel = 0;
+  if (n <= 1) return cudaSuccess;
   const int passes = (key_bits + 7) / 8;
   const int64_t tiles = (n + kSortTile - 1) / kSortTile;
   cudaError_t e;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if ((e = cudaStreamIsCapturing(s, &cap))) return e;
-  const bool capturing = cap != cudaStreamCaptureStatusNone;
   if (w.sort_epoch == 0) {  // fresh buffers, or a wait expired: clear the words once
     if ((e = cudaMemsetAsync(w.sort_status, 0, sizeof(uint32_t) * kRadix * tiles, s))) return e;
     if ((e = cudaMemsetAsync(w.sort_ep, 0, sizeof(uint32_t) * 9, s))) return e;
-    if (!capturing) w.sort_epoch = 1;
+    w.sort_epoch = 1;
   }
   k_sort_scan<<<1, kRadix, 0, s>>>(w.sort_raw, w.sort_hist, w.sort_tile, w.sort_ep, passes);
   int sel = 0;
   for (int p = 0; p < passes; ++p) {
     const bool last = p == passes - 1;
-    k_sort_pass<K><<<(unsigned)tiles, kSortThreads, sizeof(SortSmem<K>), s>>>(
-        key[sel], p ? w.val[sel] : nullptr, last && !keys ? nullptr : key[sel ^ 1],
-        w.val[sel ^ 1], n, 8 * p, w.sort_hist + p * kRadix, w.sort_status, w.sort_tile + p,
-        w.sort_ep + p, spin_limit, debug_stall && p == 0, status, last ? w.pos_u : nullptr,
-        last ? w.dir_u : nullptr, last ? w.pos : nullptr, last ? w.dir : nullptr, pad, pad_shift);
+    k_sort_pass<<<(unsigned)tiles, kSortThreads, sizeof(SortSmem), s>>>(
+        w.key[sel], p ? w.val[sel] : nullptr, w.key[sel ^ 1], w.val[sel ^ 1], n, 8 * p,
+        w.sort_hist + p * kRadix, w.sort_status, w.sort_tile + p, w.sort_ep + p, spin_limit,
+        debug_stall && p == 0, status, last ? w.pos_u : nullptr, last ? w.dir_u : nullptr,
+        last ? w.pos : nullptr, last ? w.dir : nullptr);
     if ((e = cudaGetLastError())) return e;
     sel ^= 1;
   }
-  if (out_sel) *out_sel = sel;
+  *out_sel = sel;
   return cudaSuccess;
-}
-
-cudaError_t launch_sort(BuildBufs &w, int64_t n, int key_bits, long long spin_limit,
-                        int debug_stall, unsigned int *status, int *out_sel, cudaStream_t s) {
-  *out_sel = 0;
-  if (n <= 1) return cudaSuccess;
-  return sort_keys<unsigned long long>(w, w.key, n, key_bits, true, nullptr, 0, spin_limit,
-                                       debug_stall, status, out_sel, s);
-}
-
-cudaError_t launch_sort32(BuildBufs &w, int64_t n, int key_bits, const int *pad, int pad_shift,
-                          long long spin_limit, int debug_stall, unsigned int *status,
-                          cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  return sort_keys<uint32_t>(w, w.key32, n, key_bits, false, pad, pad_shift, spin_limit,
-                             debug_stall, status, nullptr, s);
 }
 
 }  // namespace tl

@@ -1,6 +1,7 @@
 // tl_tree.cu -- the exact path: order, trees and collisions of a step.
 //
-// Both beams are propagated and sorted along a Hilbert curve (k_order, tl_sort.cu).
+// Both beams are propagated and ordered by the cells of a Hilbert curve (k_order,
+// k_cell_scan, k_place: one counting sort).
 // The smaller beam (the tree's) gets a packed tree over its sorted photons with 32
 // children per node (as in Kamel and Faloutsos, "Hilbert R-tree", VLDB 1994: leaves
 // are runs of the curve, so there are no links to build): k_boxes writes every
@@ -19,11 +20,46 @@ namespace tl {
 
 // ---------------------------------------------------------------- frames and grids
 
+// Sums of d over up to kSample photons of a beam, evenly spaced (3 FP64 values per block,
+// added by the host): the beam's mean direction, for the choice of the frame.
+constexpr int kSampleBlocks = 64, kSample = 65536;
+
+__global__ void __launch_bounds__(256) k_mean_dir(TLBeam b, double *part) {
+  __shared__ double sm[8][3];
+  const int64_t n = b.n < kSample ? b.n : kSample;
+  double m[3] = {0.0, 0.0, 0.0};
+  for (int64_t t = blockIdx.x * 256 + threadIdx.x; t < n; t += kSampleBlocks * 256) {
+    const int64_t i = t * b.n / n;
+    m[0] += b.dx[i];
+    m[1] += b.dy[i];
+    m[2] += b.dz[i];
+  }
+  for (int q = 0; q < 3; ++q)
+    for (int off = 16; off; off >>= 1) m[q] += __shfl_xor_sync(0xffffffffu, m[q], off);
+  if ((threadIdx.x & 31) == 0)
+    for (int q = 0; q < 3; ++q) sm[threadIdx.x >> 5][q] = m[q];
+  __syncthreads();
+  if (threadIdx.x < 3) {
+    double t = 0.0;
+    for (int w = 0; w < 8; ++w) t += sm[w][threadIdx.x];
+    part[blockIdx.x * 3 + threadIdx.x] = t;
+  }
+}
+
+int mean_doubles() { return 3 * kSampleBlocks; }
+int64_t mean_count(int64_t n) { return n < kSample ? n : kSample; }
+
+cudaError_t launch_mean_dir(const TLBeam &b, double *part, cudaStream_t s) {
+  k_mean_dir<<<kSampleBlocks, 256, 0, s>>>(b, part);
+  return cudaGetLastError();
+}
+
 // Per-axis sums of p', d', p'^2, p' d', d'^2 with p' = R p0, d' = R d (15 FP64 values),
-// in a fixed order (per-block sums, then one block over the blocks).  With the
-// frame the means and variances of the swept boxes' centres follow in closed form for
-// every step.
-constexpr int kMomentBlocks = 4 * 152;
+// in a fixed order (per-block sums, then one block over the blocks), from which the means
+// and variances of the swept boxes' centres follow in closed form for every step; and the
+// extremes of p' and d' and the largest |p0|_1 and |d|_1 (FP32; tl_beam_box takes their
+// rounding into account), 14 more values.
+constexpr int kMomentBlocks = 4 * 152, kMom = 29;
 
 __device__ __forceinline__ void turn(const TLFrame &f, double v[3]) {
   if (f.ident) return;
@@ -32,51 +68,73 @@ __device__ __forceinline__ void turn(const TLFrame &f, double v[3]) {
     v[k] = (double)f.r[3 * k] * x + (double)f.r[3 * k + 1] * y + (double)f.r[3 * k + 2] * z;
 }
 
+// value q of two partial results joined: sums, then 6 minima, 6 maxima, 2 maxima
+__device__ __forceinline__ double mom_join(int q, double a, double b) {
+  return q < 15 ? a + b : (q < 21 ? fmin(a, b) : fmax(a, b));
+}
+
 __global__ void __launch_bounds__(256) k_beam_moments(TLBeam b, TLFrame f, double *part) {
   double m[15];
+  float e[14];
+  const float inf = __int_as_float(0x7f800000);
   for (int q = 0; q < 15; ++q) m[q] = 0.0;
+  for (int q = 0; q < 14; ++q) e[q] = q < 6 ? inf : -inf;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < b.n;
        i += (int64_t)gridDim.x * blockDim.x) {
     double p[3] = {b.px[i], b.py[i], b.pz[i]}, d[3] = {b.dx[i], b.dy[i], b.dz[i]};
+    e[12] = fmaxf(e[12], fabsf((float)p[0]) + fabsf((float)p[1]) + fabsf((float)p[2]));
+    e[13] = fmaxf(e[13], fabsf((float)d[0]) + fabsf((float)d[1]) + fabsf((float)d[2]));
     turn(f, p);
     turn(f, d);
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
       m[a] += p[a];
       m[3 + a] += d[a];
       m[6 + a] += p[a] * p[a];
       m[9 + a] += p[a] * d[a];
       m[12 + a] += d[a] * d[a];
+      const float pf = (float)p[a], df = (float)d[a];
+      e[a] = fminf(e[a], pf);  // (a photon at NaN meets nothing)
+      e[3 + a] = fminf(e[3 + a], df);
+      e[6 + a] = fmaxf(e[6 + a], pf);
+      e[9 + a] = fmaxf(e[9 + a], df);
     }
   }
-  __shared__ double sm[8][15];
-  for (int q = 0; q < 15; ++q)
-    for (int off = 16; off; off >>= 1) m[q] += __shfl_xor_sync(0xffffffffu, m[q], off);
+  __shared__ double sm[8][kMom];
+  double v[kMom];
+#pragma unroll
+  for (int q = 0; q < kMom; ++q) {
+    v[q] = q < 15 ? m[q] : (double)e[q - 15];
+    for (int off = 16; off; off >>= 1)
+      v[q] = mom_join(q, v[q], __shfl_xor_sync(0xffffffffu, v[q], off));
+  }
   if ((threadIdx.x & 31) == 0)
-    for (int q = 0; q < 15; ++q) sm[threadIdx.x >> 5][q] = m[q];
+#pragma unroll
+    for (int q = 0; q < kMom; ++q) sm[threadIdx.x >> 5][q] = v[q];
   __syncthreads();
-  if (threadIdx.x < 15) {
-    double t = 0.0;
-    for (int w8 = 0; w8 < 8; ++w8) t += sm[w8][threadIdx.x];
-    part[blockIdx.x * 15 + threadIdx.x] = t;
+  if (threadIdx.x < kMom) {
+    double t = sm[0][threadIdx.x];
+    for (int w8 = 1; w8 < 8; ++w8) t = mom_join(threadIdx.x, t, sm[w8][threadIdx.x]);
+    part[blockIdx.x * kMom + threadIdx.x] = t;
   }
 }
 
 __global__ void k_beam_moments_final(const double *part, int nparts, double *out) {
-  if (threadIdx.x < 15) {
-    double t = 0.0;
-    for (int k = 0; k < nparts; ++k) t += part[k * 15 + threadIdx.x];
+  if (threadIdx.x < kMom) {
+    double t = part[threadIdx.x];
+    for (int k = 1; k < nparts; ++k) t = mom_join(threadIdx.x, t, part[k * kMom + threadIdx.x]);
     out[threadIdx.x] = t;
   }
 }
 
-size_t moment_doubles() { return 15 * (1 + kMomentBlocks); }
+size_t moment_doubles() { return kMom * (1 + kMomentBlocks); }
 
-// out: device, moment_doubles() doubles, the 15 moments first
+// out: device, moment_doubles() doubles, the 29 values first
 cudaError_t launch_beam_moments(const TLBeam &b, const TLFrame &f, double *out, cudaStream_t s) {
   const int64_t nb = (b.n + 255) / 256;
   const int blocks = (int)(nb < 1 ? 1 : (nb < kMomentBlocks ? nb : kMomentBlocks));
-  k_beam_moments<<<blocks, 256, 0, s>>>(b, f, out + 15);
-  k_beam_moments_final<<<1, 32, 0, s>>>(out + 15, blocks, out);
+  k_beam_moments<<<blocks, 256, 0, s>>>(b, f, out + kMom);
+  k_beam_moments_final<<<1, 32, 0, s>>>(out + kMom, blocks, out);
   return cudaGetLastError();
 }
 
@@ -179,8 +237,9 @@ cudaError_t launch_inst_frames(const double *ba, const double *bb, int n_inst, T
 // Ordering grids of both beams of a batch's instances for the step with travel
 // T = c t_k + L / 2 to the swept boxes' centres: the range of the centres, and cells in
 // the proportions of the boxes' extents (pad + travel of a typical photon).
-__global__ void k_inst_grid(const double *ba, const double *bb, const TLFrame *frames, int n_inst,
-                            double T, double L, double half, int bits, TLGrid *ga, TLGrid *gb) {
+__global__ void k_inst_grid(const double *ba, const double *bb, const TLFrame *frames,
+                            const TLInst *ia, const TLInst *ib, int n_inst, double T, double L,
+                            double half, TLGrid *ga, TLGrid *gb) {
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= n_inst) return;
   const TLFrame f = frames[q];
@@ -202,14 +261,17 @@ __global__ void k_inst_grid(const double *ba, const double *bb, const TLFrame *f
       lo[k] = bd[h][k] + T * bd[h][3 + k] - 0.5 * L * ru[k];
       range[k] = bd[h][6 + k] + T * bd[h][9 + k] - 0.5 * L * ru[k] - lo[k];
     }
-    (h ? gb : ga)[q] = tl_make_grid(lo, range, s, bits);
+    TLGrid g = tl_make_grid(lo, range, s, (h ? ib : ia)[q].bits);
+    tl_beam_box(bd[1 - h], 0.0, 0.0, f, T - 0.5 * L, L, half, g.clo, g.chi);
+    (h ? gb : ga)[q] = g;
   }
 }
 
-cudaError_t launch_inst_grid(const double *ba, const double *bb, const TLFrame *frames, int n_inst,
-                             double T, double L, double half, int bits, TLGrid *ga, TLGrid *gb,
-                             cudaStream_t s) {
-  k_inst_grid<<<(n_inst + 127) / 128, 128, 0, s>>>(ba, bb, frames, n_inst, T, L, half, bits, ga, gb);
+cudaError_t launch_inst_grid(const double *ba, const double *bb, const TLFrame *frames,
+                             const TLInst *ia, const TLInst *ib, int n_inst, double T, double L,
+                             double half, TLGrid *ga, TLGrid *gb, cudaStream_t s) {
+  k_inst_grid<<<(n_inst + 127) / 128, 128, 0, s>>>(ba, bb, frames, ia, ib, n_inst, T, L, half, ga,
+                                                   gb);
   return cudaGetLastError();
 }
 
@@ -240,59 +302,233 @@ cudaError_t launch_gather_instances(const InstSrc *src, int n_inst, int64_t n, d
 
 // ---------------------------------------------------------------- order
 
-// Propagate p = p0 + c t_k d in FP64 (closed form), round to the FP32 SoA, and key
-// every photon by its swept box's centre in the frame, with several instances below
-// the instance's number.  Also counts the 8-bit digits of every sort pass in shared
-// memory, flushed once per block.  Bound by GB300's FP64 pipe (six operations and
-// three conversions per photon at 2 per clock and SM), beside which the key's integer
-// work is free.  A fixed grid of at most kPropBlocks blocks, grid-stride.
-constexpr int kPropBlocks = 4 * 152;
+// The step-invariant FP32 record of every photon, once per context: p0 and energy,
+// direction and index.
+__global__ void __launch_bounds__(256) k_static(TLBeam b, float4 *stat) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < b.n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    stat[2 * i] = make_float4(__double2float_rn(b.px[i]), __double2float_rn(b.py[i]),
+                              __double2float_rn(b.pz[i]), __double2float_rn(b.E[i]));
+    stat[2 * i + 1] = make_float4(__double2float_rn(b.dx[i]), __double2float_rn(b.dy[i]),
+                                  __double2float_rn(b.dz[i]), __int_as_float((int)i));
+  }
+}
+
+cudaError_t launch_static(const TLBeam &b, float4 *stat, cudaStream_t s) {
+  if (b.n <= 0) return cudaSuccess;
+  const int64_t nb = (b.n + 255) / 256;
+  k_static<<<(unsigned)(nb < 8 * 152 ? nb : 8 * 152), 256, 0, s>>>(b, stat);
+  return cudaGetLastError();
+}
+
+// Every photon's cell, from its swept box's centre in the frame (FP32), counted there:
+// the count it finds is its rank in the cell.  With the cells' running sum that is its
+// place, so a beam is ordered by one counting sort with 2 to 4 cells per photon (three
+// or four radix passes took 29 us each for 1M photons; the scan takes 13 us, the move
+// 30).
+// The order inside a cell is that of the atomics and changes from run to run; it shapes
+// the tree and nothing else.  A photon whose swept box misses the box of the whole other
+// beam is left out of the step here: its 32 bytes are all that is read of it.  The test
+// takes 2^-20 of the sums of the lengths involved for the rounding of the FP32 record
+// and arithmetic (16u; 8u bound it).  Bound by memory: 32 bytes in, 8 out, one atomic
+// per photon; a warp whose photons share one cell adds once, so that a beam on one point
+// does not queue at one word.
+constexpr int kOrderBlocks = 8 * 152;
 
 __global__ void __launch_bounds__(256) k_order(OrderArgs a) {
-  __shared__ uint32_t sh[4][256];
-  for (int t = threadIdx.x; t < 4 * 256; t += 256) (&sh[0][0])[t] = 0u;
-  __syncthreads();
-  const float halfL = 0.5f * a.L;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.b.n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const double dx = a.b.dx[i], dy = a.b.dy[i], dz = a.b.dz[i];
-    const float3 p = make_float3(__double2float_rn(__dadd_rn(a.b.px[i], __dmul_rn(a.ct, dx))),
-                                 __double2float_rn(__dadd_rn(a.b.py[i], __dmul_rn(a.ct, dy))),
-                                 __double2float_rn(__dadd_rn(a.b.pz[i], __dmul_rn(a.ct, dz))));
-    const float4 d = a.dir_u[i];  // the FP32 direction, written once (k_static_soa)
-    float *pu = reinterpret_cast<float *>(a.pos_u + i);  // x, y, z; w holds the energy
-    *reinterpret_cast<float2 *>(pu) = make_float2(p.x, p.y);
-    pu[2] = p.z;
-    const uint32_t q = a.inst_of ? a.inst_of[i] : 0u;
-    const TLFrame &f = a.frames[q];
-    float c[3];
-    if (f.ident) {
-      c[0] = fmaf(halfL, d.x, p.x);
-      c[1] = fmaf(halfL, d.y, p.y);
-      c[2] = fmaf(halfL, d.z, p.z);
-    } else {
-      const float mx = fmaf(halfL, d.x - f.u[0], p.x), my = fmaf(halfL, d.y - f.u[1], p.y),
-                  mz = fmaf(halfL, d.z - f.u[2], p.z);
+  const int64_t gtid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  for (int64_t t = gtid; t < a.scan_tiles + 1; t += (int64_t)gridDim.x * blockDim.x)
+    a.scan_st[t] = 0u;
+  const int lane = threadIdx.x & 31;
+  const int64_t nround = (a.n + 31) & ~(int64_t)31;
+  for (int64_t i = gtid; i < nround; i += (int64_t)gridDim.x * blockDim.x) {
+    uint32_t cell = TL_NONE;
+    if (i < a.n) {
+      const float4 p0 = a.stat[2 * i], d = a.stat[2 * i + 1];
+      const uint32_t q = a.inst_of ? a.inst_of[i] : 0u;
+      const TLFrame &f = a.frames[q];
+      const TLGrid &g = a.inst_of ? a.grids[q] : a.grid;
+      const float px = fmaf(a.ct, d.x, p0.x), py = fmaf(a.ct, d.y, p0.y),
+                  pz = fmaf(a.ct, d.z, p0.z);
+      const float d1 = fabsf(d.x) + fabsf(d.y) + fabsf(d.z);
+      const float e = a.half + 0x1p-20f * (fabsf(p0.x) + fabsf(p0.y) + fabsf(p0.z) +
+                                           fmaf(a.ct, d1, a.L * (d1 + 3.0f)));
+      float x[3] = {px, py, pz}, v[3] = {d.x, d.y, d.z};
+      if (!f.ident) {
+        const float vx = d.x - f.u[0], vy = d.y - f.u[1], vz = d.z - f.u[2];
 #pragma unroll
-      for (int k = 0; k < 3; ++k)
-        c[k] = fmaf(f.r[3 * k], mx, fmaf(f.r[3 * k + 1], my, f.r[3 * k + 2] * mz));
+        for (int k = 0; k < 3; ++k) {
+          x[k] = fmaf(f.r[3 * k], px, fmaf(f.r[3 * k + 1], py, f.r[3 * k + 2] * pz));
+          v[k] = fmaf(f.r[3 * k], vx, fmaf(f.r[3 * k + 1], vy, f.r[3 * k + 2] * vz));
+        }
+      }
+      bool apart = false;
+      float c[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const float t = a.L * v[k];
+        apart = apart || x[k] + fminf(t, 0.0f) - e > g.chi[k] || x[k] + fmaxf(t, 0.0f) + e < g.clo[k];
+        c[k] = fmaf(0.5f, t, x[k]);
+      }
+      if (!apart) cell = (a.inst_of ? a.inst[q].cell0 : 0u) + order_key(g, c);
     }
-    const uint32_t key =
-        a.inst_of ? (q << a.inst_shift | order_key(a.grids[q], c)) : order_key(a.grid, c);
-    a.key[i] = key;
-    for (int r = 0; r < a.passes; ++r) atomicAdd(&sh[r][(key >> (8 * r)) & 255u], 1u);
-  }
-  __syncthreads();
-  for (int t = threadIdx.x; t < a.passes * 256; t += 256) {
-    const uint32_t v = (&sh[0][0])[t];
-    if (v) atomicAdd(&a.hist[t], v);
+    const uint32_t c0 = __shfl_sync(0xffffffffu, cell, 0);
+    uint32_t r = 0u;
+    if (__all_sync(0xffffffffu, cell == c0)) {
+      if (c0 != TL_NONE) {
+        if (lane == 0) r = atomicAdd(a.count + c0, 32u);
+        r = __shfl_sync(0xffffffffu, r, 0) + lane;
+      }
+    } else if (cell != TL_NONE) {
+      r = atomicAdd(a.count + cell, 1u);
+    }
+    if (i < a.n) a.cell[i] = make_uint2(cell, r);
   }
 }
 
 cudaError_t launch_order(const OrderArgs &a, cudaStream_t s) {
+  if (a.n <= 0) return cudaSuccess;
+  const int64_t nb = (a.n + 255) / 256;
+  k_order<<<(int)(nb < kOrderBlocks ? nb : kOrderBlocks), 256, 0, s>>>(a);
+  return cudaGetLastError();
+}
+
+// Exclusive running sum of the cells' counts, tile by tile of kScanTile cells, with the
+// counts cleared for the next step.  A tile's sum is published at once; warp 0 looks back
+// over the preceding tiles' words 32 at a time (Merrill and Garland 2016, "Single-pass
+// parallel prefix scan with decoupled look-back").  Tiles are numbered in the order blocks
+// start, so a tile only waits on running ones; every wait is bounded by spin (then
+// TL_ST_TIMEOUT is recorded and the sums are not used).  Words: 2 flag bits and a 27-bit
+// sum (beams hold fewer than 2^27 photons), cleared by k_order.
+constexpr int kScanThreads = 1024, kScanCells = 16, kScanTile = kScanThreads * kScanCells;
+constexpr uint32_t kScanSum = 1u << 30, kScanPre = 2u << 30, kScanVal = (1u << 28) - 1u;
+
+__global__ void __launch_bounds__(kScanThreads) k_cell_scan(uint32_t *count, uint32_t *start,
+                                                            int64_t cells, uint32_t *st,
+                                                            long long spin, int debug_stall,
+                                                            unsigned *status) {
+  __shared__ uint32_t ws[32], tile_s, before_s;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  if (t == 0) tile_s = atomicAdd(st, 1u);
+  __syncthreads();
+  const uint32_t tile = tile_s;
+  const int64_t c0 = (int64_t)tile * kScanTile + (int64_t)t * kScanCells;
+  uint4 v[kScanCells / 4];
+  uint32_t sum = 0u;
+#pragma unroll
+  for (int q = 0; q < kScanCells / 4; ++q) {  // (cells is a multiple of 16)
+    uint4 *p = reinterpret_cast<uint4 *>(count + c0) + q;
+    v[q] = c0 < cells ? *p : make_uint4(0u, 0u, 0u, 0u);
+    if (c0 < cells) *p = make_uint4(0u, 0u, 0u, 0u);
+    sum += v[q].x + v[q].y + v[q].z + v[q].w;
+  }
+  uint32_t inc = sum;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const uint32_t u = __shfl_up_sync(0xffffffffu, inc, off);
+    if (lane >= off) inc += u;
+  }
+  if (lane == 31) ws[warp] = inc;
+  __syncthreads();
+  if (warp == 0) {
+    uint32_t w = ws[lane];
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const uint32_t u = __shfl_up_sync(0xffffffffu, w, off);
+      if (lane >= off) w += u;
+    }
+    ws[lane] = w;  // inclusive sums of the warps
+    const uint32_t total = __shfl_sync(0xffffffffu, w, 31);
+    uint32_t *my = st + 1 + tile;
+    uint32_t before = 0u;
+    if (tile == 0) {
+      if (lane == 0 && !debug_stall) atomicExch(my, kScanPre | total);
+    } else {
+      if (lane == 0) atomicExch(my, kScanSum | total);
+      long long j = (long long)tile - 1, spins = 0;
+      while (j >= 0) {  // lane l looks at tile j - l
+        uint32_t w1 = kScanPre;
+        if (j - lane >= 0) w1 = *(volatile uint32_t *)(st + 1 + j - lane);
+        const unsigned none = __ballot_sync(0xffffffffu, (w1 >> 30) == 0u);
+        const unsigned pre = __ballot_sync(0xffffffffu, (w1 >> 30) == 2u);
+        // the words up to the first prefix, or up to the first one not published
+        int use = none ? __ffs(none) - 1 : 32;
+        const bool done = pre && __ffs(pre) - 1 < use;
+        if (done) use = __ffs(pre);
+        uint32_t x = lane < use ? w1 & kScanVal : 0u;
+#pragma unroll
+        for (int off = 16; off; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+        before += x;
+        if (done) break;
+        j -= use;
+        if (use == 0) {
+          if (++spins > spin) {
+            if (lane == 0) atomicOr(status, (unsigned)TL_ST_TIMEOUT);
+            break;
+          }
+          __nanosleep(32);
+        }
+      }
+      if (lane == 0) atomicExch(my, kScanPre | ((before + total) & kScanVal));
+    }
+    if (lane == 0) before_s = before;
+  }
+  __syncthreads();
+  uint32_t run = before_s + (warp ? ws[warp - 1] : 0u) + inc - sum;
+  if (c0 >= cells) return;
+  if (c0 + kScanCells == cells) start[cells] = run + sum;  // the photons in all
+#pragma unroll
+  for (int q = 0; q < kScanCells / 4; ++q) {
+    uint4 o;
+    o.x = run;
+    o.y = o.x + v[q].x;
+    o.z = o.y + v[q].y;
+    o.w = o.z + v[q].z;
+    run = o.w + v[q].w;
+    reinterpret_cast<uint4 *>(start + c0)[q] = o;
+  }
+}
+
+int64_t scan_tiles(int64_t cells) { return (cells + kScanTile - 1) / kScanTile; }
+
+cudaError_t launch_cell_scan(uint32_t *count, uint32_t *start, int64_t cells, uint32_t *st,
+                             long long spin, int debug_stall, unsigned *status, cudaStream_t s) {
+  k_cell_scan<<<(unsigned)scan_tiles(cells), kScanThreads, 0, s>>>(count, start, cells, st, spin,
+                                                                   debug_stall, status);
+  return cudaGetLastError();
+}
+
+// Every photon that stays in the step to its place, at its position of the step:
+// p = p0 + c t_k d in FP64 (closed form), rounded to FP32.  Coalesced reads (88 bytes),
+// one full 32-byte sector written per photon; beside that it keeps GB300's FP64 pipe
+// busy (six operations and three conversions per photon at 2 per clock and SM).
+__global__ void __launch_bounds__(256) k_place(PlaceArgs a) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.b.n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const uint2 c = a.cell[i];
+    if (c.x == TL_NONE) continue;
+    int64_t to = (int64_t)__ldg(a.start + c.x) + c.y;
+    const float4 s0 = a.stat[2 * i], d = a.stat[2 * i + 1];
+    const double dx = a.b.dx[i], dy = a.b.dy[i], dz = a.b.dz[i];
+    const float4 p =
+        make_float4(__double2float_rn(__dadd_rn(a.b.px[i], __dmul_rn(a.ct, dx))),
+                    __double2float_rn(__dadd_rn(a.b.py[i], __dmul_rn(a.ct, dy))),
+                    __double2float_rn(__dadd_rn(a.b.pz[i], __dmul_rn(a.ct, dz))), s0.w);
+    if (a.inst_of) {
+      const TLInst &I = a.inst[a.inst_of[i]];
+      to += (int64_t)I.tile0 * kTile - (int64_t)__ldg(a.start + I.cell0);
+    }
+    if ((uint64_t)to < (uint64_t)a.n_pad) {  // always, unless the scan's wait expired
+      a.rec[2 * to] = p;
+      a.rec[2 * to + 1] = d;
+    }
+  }
+}
+
+cudaError_t launch_place(const PlaceArgs &a, cudaStream_t s) {
   if (a.b.n <= 0) return cudaSuccess;
   const int64_t nb = (a.b.n + 255) / 256;
-  k_order<<<(int)(nb < kPropBlocks ? nb : kPropBlocks), 256, 0, s>>>(a);
+  k_place<<<(int)(nb < 8 * 152 ? nb : 8 * 152), 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -347,17 +583,19 @@ __global__ void __launch_bounds__(kTile) k_boxes(BoxArgs a) {
   const int tile = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const uint32_t q = a.tile_inst ? a.tile_inst[tile] : 0u;
   const TLInst &I = a.inst[q];
+  const int n = tl_live(I, a.start);
   const int k = tile - I.tile0, r = k * kTile + t;
+  if (k * kTile >= n) return;
   TLBox b = empty_box();
-  if (r < I.n) {
+  if (r < n) {
     const int64_t p = (int64_t)tile * kTile + t;
-    b = swept_box(a.pos[p], a.dir[p], a.frames[q], a.Llo, a.Lhi, a.half);
+    b = swept_box(a.rec[2 * p], a.rec[2 * p + 1], a.frames[q], a.Llo, a.Lhi, a.half);
     put_box(a.box + 2 * ((size_t)I.lev[0] + r), b);
   }
   b = warp_union(b);
   if (lane == 0) {
     wb[warp] = b;
-    if (r < I.n) put_box(a.box + 2 * ((size_t)I.lev[1] + k * 32 + warp), b);
+    if (r < n) put_box(a.box + 2 * ((size_t)I.lev[1] + k * 32 + warp), b);
   }
   __syncthreads();
   if (warp == 0) {
@@ -367,13 +605,16 @@ __global__ void __launch_bounds__(kTile) k_boxes(BoxArgs a) {
 }
 
 // Levels 3 and up of one instance's tree per block, a warp per node.
-__global__ void __launch_bounds__(1024) k_upper(const TLInst *inst, float4 *box) {
+__global__ void __launch_bounds__(1024) k_upper(const TLInst *inst, const uint32_t *start,
+                                                float4 *box) {
   const TLInst &I = inst[blockIdx.x];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int l = 3; l <= I.top; ++l) {
-    for (int j = warp; j < I.cnt[l]; j += 32) {
+  const int n = tl_live(I, start), top = tl_top_level(n);
+  for (int l = 3; l <= top; ++l) {
+    const int cnt = tl_level_count(n, l), below = tl_level_count(n, l - 1);
+    for (int j = warp; j < cnt; j += 32) {
       const int c = 32 * j + lane;
-      TLBox b = c < I.cnt[l - 1] ? get_box(box + 2 * ((size_t)I.lev[l - 1] + c)) : empty_box();
+      TLBox b = c < below ? get_box(box + 2 * ((size_t)I.lev[l - 1] + c)) : empty_box();
       b = warp_union(b);
       if (lane == 0) put_box(box + 2 * ((size_t)I.lev[l] + j), b);
     }
@@ -384,7 +625,7 @@ __global__ void __launch_bounds__(1024) k_upper(const TLInst *inst, float4 *box)
 cudaError_t launch_boxes(const BoxArgs &a, int tiles, int n_inst, int max_top, cudaStream_t s) {
   if (tiles <= 0) return cudaSuccess;
   k_boxes<<<tiles, kTile, 0, s>>>(a);
-  if (max_top >= 3) k_upper<<<n_inst, 1024, 0, s>>>(a.inst, a.box);
+  if (max_top >= 3) k_upper<<<n_inst, 1024, 0, s>>>(a.inst, a.start, a.box);
   return cudaGetLastError();
 }
 
@@ -393,17 +634,19 @@ cudaError_t launch_boxes(const BoxArgs &a, int tiles, int n_inst, int max_top, c
 constexpr int kColWarps = 4;
 constexpr uint32_t kIdxMask = (1u << 27) - 1u;  // beams hold fewer than 2^27 photons
 
+constexpr int kPend = 256;
+
 struct ColSmem {
   float4 qpos[32], qdir[32];  // the warp's photons
-  float4 qbox[64];            // their boxes
-  float4 cbox[64];            // boxes of the visited node's children
-  uint32_t pend[64];          // (lane << 27 | photon of the tree): boxes overlap
+  float4 cbox[64];            // boxes tested by every lane
+  uint32_t pend[kPend];       // (lane << 27 | photon of the tree): boxes overlap
   uint32_t cand[64];          // undecided by the first look
   uint32_t mask[6], base[6];  // per level: children still to descend into
+  uint8_t id[32];             // lane of each tested box
 };
 
-// Photon pairs whose boxes overlap: the first look, 32 at a time; what it leaves goes
-// to the step's candidate list.
+// Photon pairs whose boxes overlap: the first look, 32 at a time, from the end of the
+// pending list; what it leaves goes to the step's candidate list.
 template <bool FP64>
 struct Pairs {
   const ColArgs &a;
@@ -413,7 +656,8 @@ struct Pairs {
   int lane, np, nc;
   unsigned long long lbase;
 
-  __device__ __forceinline__ void write(int cnt) {  // the first cnt candidates
+  __device__ __forceinline__ void write(int cnt) {  // the last cnt (<= 32) candidates
+    nc -= cnt;
     unsigned long long at = 0;
     if (lane == 0) {
       at = atomicAdd(&a.ctr->cand, (unsigned long long)cnt) - lbase;
@@ -421,46 +665,68 @@ struct Pairs {
     }
     at = __shfl_sync(0xffffffffu, at, 0);
     if (lane < cnt && at + lane < a.cand_cap) {
-      const uint32_t e = ws.cand[lane], q = qpos0 + (e >> 27), t = tpos0 + (e & kIdxMask);
+      const uint32_t e = ws.cand[nc + lane], q = qpos0 + (e >> 27), t = tpos0 + (e & kIdxMask);
       a.cand[at + lane] = a.swap ? make_uint2(t, q) : make_uint2(q, t);
     }
+    __syncwarp();
   }
-  __device__ __forceinline__ void look(int cnt) {  // the first cnt (<= 32) pending pairs
+  __device__ __forceinline__ void look(int cnt) {  // the last cnt (<= 32) pending pairs
+    np -= cnt;
     bool open = false;
     uint32_t e = 0u;
     if (lane < cnt) {
-      e = ws.pend[lane];
+      e = ws.pend[np + lane];
       open = true;
       if (!FP64) {
-        const uint32_t t = tpos0 + (e & kIdxMask), q = e >> 27;
-        const float4 pb = __ldg(a.tpos + t), db = __ldg(a.tdir + t);
+        const size_t t = 2 * (size_t)(tpos0 + (e & kIdxMask));
+        const uint32_t q = e >> 27;
+        const float4 pb = __ldg(a.t + t), db = __ldg(a.t + t + 1);
         open = !tl_narrow32_sure_miss(ws.qpos[q], ws.qdir[q], pb, db, a.nk, suf);
       }
     }
     const unsigned m = __ballot_sync(0xffffffffu, open);
-    if (!m) return;
     if (open) ws.cand[nc + __popc(m & ((1u << lane) - 1u))] = e;
     nc += __popc(m);
     __syncwarp();
-    if (nc < 32) return;
-    write(32);
-    nc -= 32;
-    const uint32_t v = lane < nc ? ws.cand[32 + lane] : 0u;
-    __syncwarp();
-    if (lane < nc) ws.cand[lane] = v;
-    __syncwarp();
+    if (nc >= 32) write(32);
   }
-  __device__ __forceinline__ void add(bool ok, unsigned m, uint32_t e) {  // m = ballot(ok) != 0
-    if (ok) ws.pend[np + __popc(m & ((1u << lane) - 1u))] = e;
-    np += __popc(m);
-    __syncwarp();
-    if (np < 32) return;
-    look(32);
-    np -= 32;
-    const uint32_t v = lane < np ? ws.pend[32 + lane] : 0u;
-    __syncwarp();
-    if (lane < np) ws.pend[lane] = v;
-    __syncwarp();
+  // every lane's pairs: bit r of bits stands for box r of the cnt last tested, this lane
+  // for its photon (by_tree) or for photon j0 + lane of the tree
+  __device__ __forceinline__ void add(uint32_t bits, bool by_tree, uint32_t j0) {
+    int inc = __popc(bits);
+    const int own = inc;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, inc, off);
+      if (lane >= off) inc += t;
+    }
+    const int total = __shfl_sync(0xffffffffu, inc, 31);
+    if (total == 0) return;
+    // what does not fit the list at once (dense leaves) goes in rounds of one per lane
+    if (np + total <= kPend) {
+      int at = np + inc - own;
+      while (bits) {
+        const uint32_t k = ws.id[__ffs(bits) - 1];
+        bits &= bits - 1u;
+        ws.pend[at++] = by_tree ? (uint32_t)lane << 27 | (j0 + k) : k << 27 | (j0 + lane);
+      }
+      np += total;
+      __syncwarp();
+      while (np >= 32) look(32);
+      return;
+    }
+    unsigned m;
+    while ((m = __ballot_sync(0xffffffffu, bits != 0u)) != 0u) {
+      if (bits) {
+        const uint32_t k = ws.id[__ffs(bits) - 1];
+        bits &= bits - 1u;
+        ws.pend[np + __popc(m & ((1u << lane) - 1u))] =
+            by_tree ? (uint32_t)lane << 27 | (j0 + k) : k << 27 | (j0 + lane);
+      }
+      np += __popc(m);
+      __syncwarp();
+      while (np >= 32) look(32);
+    }
   }
   __device__ __forceinline__ void finish() {
     if (np) look(np);
@@ -468,22 +734,41 @@ struct Pairs {
   }
 };
 
+// The boxes src of the lanes in sel against box cmp of every lane: bit r of the result,
+// the r-th of them overlaps.  The boxes pass through shared memory, compacted, and come
+// back by broadcast: ~10 instructions for 32 box pairs.
+__device__ __forceinline__ uint32_t test_boxes(ColSmem &ws, const TLBox &src, unsigned sel,
+                                               const TLBox &cmp, int lane) {
+  __syncwarp();
+  if (sel >> lane & 1u) {
+    const int r = __popc(sel & ((1u << lane) - 1u));
+    put_box(ws.cbox + 2 * r, src);
+    ws.id[r] = (uint8_t)lane;
+  }
+  __syncwarp();
+  const int cnt = __popc(sel);
+  uint32_t bits = 0u;
+#pragma unroll 4
+  for (int r = 0; r < cnt; ++r)
+    if (tl_overlap(get_box(ws.cbox + 2 * r), cmp)) bits |= 1u << r;
+  return bits;
+}
+
 // One warp: 32 consecutive photons of the query beam, one per lane, against the tree.
 // A node's 32 children are tested by 32 lanes at once against the union of the warp's
-// boxes; each that overlaps it is then tested by every lane against its own box, and
-// the node is descended into if any lane overlaps.  At the photons, the two sides'
-// survivors are tested against each other along the shorter list: survivors of the
-// tree one by one against all lanes, or the lanes one by one against all 32.  What
-// bounds it is issue: one coalesced load serves 32 tests and boxes come from shared
-// memory by broadcast, so a box test costs ~12 warp instructions for 32 pairs (the
-// dual descent of two binary trees took 25 warp instructions per popped node pair and
-// lane-private 64-byte records).  Few groups (small beams): the tree is cut into
+// boxes; those that overlap it are tested by every lane against its own box, and
+// the node's child is descended into if any lane overlaps it.  At the photons, the two
+// sides' survivors are tested against each other along the shorter list: survivors of the
+// tree against all lanes, or the lanes against all 32.  What bounds it is issue: one
+// coalesced load serves 32 tests, and box tests cost ~10 warp instructions for 32 pairs
+// (the dual descent of two binary trees took 25 warp instructions per popped node pair
+// and lane-private 64-byte records).  Few groups (small beams): the tree is cut into
 // `slices` contiguous parts of its sorted photons, one warp each per group.
 // Measured (with the first look, which was k_narrow's): 2 x 4M statistical step 15.0 ms
-// for the dual descent and its narrow phase, 6.4 ms now; 2 x 16M at 90 degrees 7.3 ms,
-// 1.1 ms now (there the turned frame is most of it).
+// for the dual descent and its narrow phase, 6.1 ms now; 2 x 16M at 90 degrees
+// 7.3 ms, 1.1 ms now (there the turned frame is most of it).
 template <bool FP64>
-__global__ void __launch_bounds__(32 * kColWarps) k_collide(ColArgs a) {
+__global__ void __launch_bounds__(32 * kColWarps, 8) k_collide(ColArgs a) {
   __shared__ ColSmem wsm[kColWarps];
   __shared__ float suf[TL_SBINS];
   if (a.ctr->status & (TL_ST_TIMEOUT | TL_ST_SPILL_OVF)) return;  // the build failed
@@ -498,49 +783,46 @@ __global__ void __launch_bounds__(32 * kColWarps) k_collide(ColArgs a) {
   const int tile = g >> 5;
   const uint32_t inst = a.tile_inst ? a.tile_inst[tile] : 0u;
   const TLInst &Q = a.qinst[inst], &T = a.tinst[inst];
-  const int r0 = (g - Q.tile0 * 32) * 32;
-  if (r0 >= Q.n || T.n == 0) return;
-  const int c0 = (int)((long long)T.cnt[1] * slice / a.slices);
-  const int c1 = (int)((long long)T.cnt[1] * (slice + 1) / a.slices);
+  const int r0 = (g - Q.tile0 * 32) * 32, qn = tl_live(Q, a.qstart);
+  if (r0 >= qn) return;
+  const int tn = tl_live(T, a.tstart), leaves_n = tl_level_count(tn, 1);
+  const int c0 = (int)((long long)leaves_n * slice / a.slices);
+  const int c1 = (int)((long long)leaves_n * (slice + 1) / a.slices);
   if (c0 == c1) return;
   ColSmem &ws = wsm[warp];
   Pairs<FP64> out{a, ws, suf, (uint32_t)g * 32u, (uint32_t)T.tile0 * (uint32_t)kTile, lane, 0, 0,
                   a.ctr->leaf_base};
   TLBox own = empty_box();
-  if (r0 + lane < Q.n) {
-    const float4 p = a.qpos[(int64_t)g * 32 + lane], d = a.qdir[(int64_t)g * 32 + lane];
+  if (r0 + lane < qn) {
+    const float4 *r = a.q + 2 * ((int64_t)g * 32 + lane);
+    const float4 p = r[0], d = r[1];
     own = swept_box(p, d, a.frames[inst], a.Llo, a.Lhi, a.half);
     ws.qpos[lane] = p;
     ws.qdir[lane] = d;
   }
-  put_box(ws.qbox + 2 * lane, own);
   const TLBox all = warp_union(own);
-  unsigned long long node_tests = 0, narrow = 0, leaves = 0;
-  const int top = T.top;
+  unsigned long long node_tests = 0, narrow = 0;
+  unsigned leaves = 0;
+  const int top = tl_top_level(tn);
   int lev = top, base = 0;
-  unsigned mask = 0u, lanes = 0u;  // children to descend into; lane c: the lanes that overlap c
-  bool fresh = true;               // the children of (lev, base) are still to be tested
+  unsigned mask = 0u;      // children of (lev, base) to descend into
+  unsigned near = 0u;      // level 1: leaves that overlap the union,
+  uint32_t hits = 0u;      // and which of them overlap this lane's box
+  bool fresh = true;       // the children of (lev, base) are still to be tested
   while (true) {
     if (fresh) {
-      const int cnt = min(32, T.cnt[lev] - base), c = base + lane;
+      const int cnt = min(32, tl_level_count(tn, lev) - base), c = base + lane;
       const int sh = 5 * (lev - 1);
-      bool ok = lane < cnt && ((long long)c << sh) < c1 && ((long long)(c + 1) << sh) > c0;
+      const bool ok = lane < cnt && ((long long)c << sh) < c1 && ((long long)(c + 1) << sh) > c0;
       const TLBox b = ok ? get_box(a.box + 2 * ((size_t)T.lev[lev] + c)) : empty_box();
-      ok = tl_overlap(b, all);
-      unsigned m = __ballot_sync(0xffffffffu, ok);
-      node_tests += (unsigned)(cnt + 32 * __popc(m));
+      near = __ballot_sync(0xffffffffu, tl_overlap(b, all));
+      node_tests += (unsigned)(cnt + 32 * __popc(near));
       mask = 0u;
-      if (m) {
-        __syncwarp();
-        put_box(ws.cbox + 2 * lane, b);
-        __syncwarp();
-        do {
-          const int k = __ffs(m) - 1;
-          m &= m - 1u;
-          const unsigned w = __ballot_sync(0xffffffffu, tl_overlap(get_box(ws.cbox + 2 * k), own));
-          if (lane == k) lanes = w;
-          if (w) mask |= 1u << k;
-        } while (m);
+      if (near) {
+        hits = test_boxes(ws, b, near, own, lane);
+        const uint32_t any = __reduce_or_sync(0xffffffffu, hits);
+        mask = __ballot_sync(0xffffffffu, (near >> lane & 1u) &&
+                                              (any >> __popc(near & ((1u << lane) - 1u)) & 1u));
       }
       fresh = false;
     }
@@ -549,34 +831,18 @@ __global__ void __launch_bounds__(32 * kColWarps) k_collide(ColArgs a) {
         const int k = __ffs(mask) - 1;
         mask &= mask - 1u;
         const int j0 = (base + k) * 32;
-        const bool ok = j0 + lane < T.n;
+        const bool ok = j0 + lane < tn;
         const TLBox b = ok ? get_box(a.box + 2 * ((size_t)T.lev[0] + j0 + lane)) : empty_box();
-        unsigned mb = __ballot_sync(0xffffffffu, tl_overlap(b, all));
-        unsigned mq = __shfl_sync(0xffffffffu, lanes, k);
+        const unsigned mb = __ballot_sync(0xffffffffu, tl_overlap(b, all));
+        const unsigned mq =
+            __ballot_sync(0xffffffffu, hits >> __popc(near & ((1u << k) - 1u)) & 1u);
         ++leaves;
         const int nb = __popc(mb), nq = __popc(mq);
         narrow += (unsigned)(nb * nq);
-        if (nb <= nq) {
-          if (!mb) continue;
-          __syncwarp();
-          put_box(ws.cbox + 2 * lane, b);
-          __syncwarp();
-          do {
-            const int j = __ffs(mb) - 1;
-            mb &= mb - 1u;
-            const bool hit = tl_overlap(get_box(ws.cbox + 2 * j), own);
-            const unsigned m = __ballot_sync(0xffffffffu, hit);
-            if (m) out.add(hit, m, (uint32_t)lane << 27 | (uint32_t)(j0 + j));
-          } while (mb);
-        } else {
-          do {
-            const int q = __ffs(mq) - 1;
-            mq &= mq - 1u;
-            const bool hit = tl_overlap(get_box(ws.qbox + 2 * q), b);
-            const unsigned m = __ballot_sync(0xffffffffu, hit);
-            if (m) out.add(hit, m, (uint32_t)q << 27 | (uint32_t)(j0 + lane));
-          } while (mq);
-        }
+        if (nb == 0) continue;
+        const bool by_tree = nb <= nq;
+        out.add(by_tree ? test_boxes(ws, b, mb, own, lane) : test_boxes(ws, own, mq, b, lane),
+                by_tree, (uint32_t)j0);
       }
     while (!mask && lev < top) {  // up to the next level with children left
       ++lev;
@@ -600,7 +866,7 @@ __global__ void __launch_bounds__(32 * kColWarps) k_collide(ColArgs a) {
   if (lane == 0) {
     if (node_tests) atomicAdd(&a.ctr->node_tests, node_tests);
     if (narrow) atomicAdd(&a.ctr->narrow_tests, narrow);
-    if (leaves) atomicAdd(&a.ctr->leaf_pairs, leaves);
+    if (leaves) atomicAdd(&a.ctr->leaf_pairs, (unsigned long long)leaves);
   }
 }
 
@@ -649,9 +915,10 @@ __global__ void __launch_bounds__(256) k_decide(TravArgs a) {
     }
     bool open = false;
     if (ok)
-      open = !tl_exact_sure_miss(a.mA, __float_as_uint(__ldg(a.A.dir + pr.x).w), a.mB,
-                                 __float_as_uint(__ldg(a.B.dir + pr.y).w), a.ct, a.dt,
-                                 (double)a.nk.r2max);
+      open = !tl_exact_sure_miss(
+          a.mA, __float_as_uint(__ldg(a.A.dir + (size_t)pr.x * a.A.stride).w), a.mB,
+          __float_as_uint(__ldg(a.B.dir + (size_t)pr.y * a.B.stride).w), a.ct, a.dt,
+          (double)a.nk.r2max);
     const unsigned m = __ballot_sync(0xffffffffu, open);
     if (open) pend[warp][np + __popc(m & ((1u << lane) - 1u))] = pr;
     np += __popc(m);

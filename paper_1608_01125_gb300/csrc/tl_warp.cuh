@@ -31,13 +31,14 @@ __device__ __forceinline__ void decide_pairs(const TravArgs &a, const uint2 pr, 
   int outcome = TL_MISS;
   uint32_t oi = 0u, oj = 0u;
   if (ok) {
-    const float4 da = __ldg(a.A.dir + pr.x), db = __ldg(a.B.dir + pr.y);
+    const size_t ia = (size_t)pr.x * a.A.stride, jb = (size_t)pr.y * a.B.stride;
+    const float4 da = __ldg(a.A.dir + ia), db = __ldg(a.B.dir + jb);
     oi = __float_as_uint(da.w);
     oj = __float_as_uint(db.w);
     if (FP64) {
       outcome = tl_exact_hit(a.mA, oi, a.mB, oj, a.ct, a.dt, a.kappa) ? TL_HIT : TL_MISS;
     } else {
-      const float4 pa = __ldg(a.A.pos + pr.x), pb = __ldg(a.B.pos + pr.y);
+      const float4 pa = __ldg(a.A.pos + ia), pb = __ldg(a.B.pos + jb);
       outcome = tl_narrow32(pa, da, pb, db, a.nk, sbin);
     }
   }
