@@ -38,7 +38,8 @@
 // first.
 //
 // Once few hits are left open (kTail), block 0 runs the remaining rounds
-// alone, its phases separated by __syncthreads instead of grid barriers.
+// alone, the hits in its registers, its phases separated by __syncthreads instead of
+// grid barriers.
 //
 // Layout: a photon's slots of both round parities share one 32-byte record
 // (one sector), and the photons' FP64 positions and directions are packed once
@@ -54,7 +55,13 @@ namespace {
 constexpr unsigned long long kNoKey = ~0ull;
 constexpr unsigned kNoIdx = ~0u;
 constexpr int kThreads = 1024;
-constexpr long long kTail = 2 * kThreads;  // open hits below which block 0 goes on alone
+// open hits below which block 0 goes on alone, kTailHits per thread in registers: a round
+// is then a chain of L2 round trips instead of two grid barriers and the lists.  One SM's
+// share of the L2 sets the line: with 8 hits per thread in this tail a step of 2 x 2048
+// photons (17,000 hits) takes 363 us, with 4 305, 2 277, 1 272, and with a quarter of
+// that 284.
+constexpr int kTailHits = 1;
+constexpr long long kTail = kTailHits * kThreads;
 
 enum : uint8_t { kOpen = 0, kDone = 1 };
 enum : int { kFlagBadInput = 1, kFlagRounds = 2, kFlagBarrier = 4 };
@@ -62,8 +69,8 @@ enum : int { kFlagBadInput = 1, kFlagRounds = 2, kFlagBarrier = 4 };
 // Device control block of a call, zeroed before the launch.
 struct DepCtl {
   unsigned cnt[2];  // entries of list[0], list[1]
-  unsigned arrive;  // grid barrier: blocks arrived
-  unsigned gen;     // grid barrier: generation
+  unsigned arrive;  // grid barrier: blocks arrived, over all barriers of the call
+  unsigned pad0;
   int flag;         // kFlag* bits
   int tie[2];       // by round parity: some hit met its own time key at a photon in R1
   int pad;
@@ -160,37 +167,33 @@ __device__ __forceinline__ void block_sum(double &s, unsigned long long &c, doub
 
 // Grid-wide barrier of the cooperative launch.  Every thread makes its writes
 // visible at device scope (a fence) before the block arrives; thread 0 then
-// arrives on a counter, the last one to arrive resets it and advances the
-// generation the others wait on, and every waiter fences again after it sees
-// the new generation.  The wait is bounded: on a timeout (or when another
+// arrives on a counter that only grows and waits until every block has arrived as often
+// as this one (`done`, its barriers so far); each fences again.  One atomic and one poll
+// on the critical path (a counter reset and a generation word took three more round
+// trips).  The wait is bounded: on a timeout (or when another
 // block already gave up) the block sets kFlagBarrier, marks the slots dirty
 // and the call returns false, after which the block leaves the kernel; the
 // others then give up at their next barrier.
-__device__ bool grid_sync(const DepArgs &g) {
+__device__ bool grid_sync(const DepArgs &g, unsigned &done) {
   __shared__ int ok_s;
   __threadfence();
   __syncthreads();
+  ++done;
   if (threadIdx.x == 0) {
     int ok = 1;
     DepCtl *ctl = g.ctl;
-    volatile unsigned *gen = &ctl->gen;
-    const unsigned g0 = *gen;
-    __threadfence();
-    if (atomicAdd(&ctl->arrive, 1u) == gridDim.x - 1) {
-      atomicExch(&ctl->arrive, 0u);
-      __threadfence();
-      atomicAdd(&ctl->gen, 1u);
-    } else {
-      long long it = 0;
-      while (*gen == g0) {
-        if ((*(volatile int *)&ctl->flag & kFlagBarrier) || ++it > g.spin) {
-          atomicOr(&ctl->flag, kFlagBarrier);
-          atomicExch(g.dirty, 1);
-          ok = 0;
-          break;
-        }
-        __nanosleep(64);
+    const unsigned want = done * gridDim.x;
+    unsigned have = atomicAdd(&ctl->arrive, 1u) + 1u;
+    long long it = 0;
+    while (have < want) {
+      if ((*(volatile int *)&ctl->flag & kFlagBarrier) || ++it > g.spin) {
+        atomicOr(&ctl->flag, kFlagBarrier);
+        atomicExch(g.dirty, 1);
+        ok = 0;
+        break;
       }
+      __nanosleep(32);
+      have = *(volatile unsigned *)&ctl->arrive;
     }
     __threadfence();
     ok_s = ok;
@@ -224,29 +227,16 @@ __global__ void k_dep_pack(TLBeam A, TLBeam B, DepPhoton *pa, DepPhoton *pb) {
   }
 }
 
-// Phase separation: grid-wide between the rounds every block shares, the
-// block's own barrier once block 0 runs the tail alone.
-template <bool kBlock>
-__device__ __forceinline__ bool phase_sync(const DepArgs &g) {
-  if (kBlock) {  // reads go through L2 (__ldcg): the block's writes first reach it
-    __threadfence();
-    __syncthreads();
-    return true;
-  }
-  return grid_sync(g);
-}
-
 // Rounds from round r (R1 skipped for round 0: it ran with the t* keys) over
 // the nr open hits of `cur` (nullptr: every hit), work items tid0, tid0 +
-// stride, ...  Returns 0 when no hit is left open, 1 (grid mode only) when at
+// stride, ...  Returns 0 when no hit is left open, 1 when at
 // most kTail are, -1 on a failed barrier, -2 when the rounds ran out.
-template <bool kBlock>
 __device__ int run_rounds(const DepArgs &g, long long &nr, const unsigned *&cur, long long &r,
-                          long long tid0, long long stride) {
+                          long long tid0, long long stride, unsigned &done) {
   const int lane = threadIdx.x & 31;
   DepCtl *ctl = g.ctl;
   for (;; ++r) {
-    if (!kBlock && nr <= kTail) return 1;
+    if (nr <= kTail) return 1;
     if (r > g.n) return -2;  // unreachable: every round resolves the earliest open hit
     const int b = (int)(r & 1), nb = b ^ 1;
     unsigned *cntn = b ? &ctl->cnt[0] : &ctl->cnt[1];
@@ -275,7 +265,7 @@ __device__ int run_rounds(const DepArgs &g, long long &nr, const unsigned *&cur,
         if ((atomicMin(&g.sA[h.x].t[b], k) == k) | (atomicMin(&g.sB[h.y].t[b], k) == k))
           atomicOr(tie, 1);
       }
-      if (!phase_sync<kBlock>(g)) return -1;
+      if (!grid_sync(g, done)) return -1;
     }
     const bool ties = __ldcg(tie) != 0;
     // R2
@@ -287,7 +277,7 @@ __device__ int run_rounds(const DepArgs &g, long long &nr, const unsigned *&cur,
       if (__ldcg(&g.sA[h.x].t[b]) == k) atomicMin(&g.sA[h.x].p[b], h.y);
       if (__ldcg(&g.sB[h.y].t[b]) == k) atomicMin(&g.sB[h.y].p[b], h.x);
     }
-    if (ties && !phase_sync<kBlock>(g)) return -1;
+    if (ties && !grid_sync(g, done)) return -1;
     // R3 (warp-uniform trip count, for the ballot of the compaction)
     for (long long i0 = tid0 - lane; i0 < nr; i0 += stride) {
       const long long i = i0 + lane;
@@ -325,25 +315,124 @@ __device__ int run_rounds(const DepArgs &g, long long &nr, const unsigned *&cur,
         if (keep) listn[base + __popc(m & ((1u << lane) - 1u))] = e;
       }
     }
-    if (!phase_sync<kBlock>(g)) return -1;
+    if (!grid_sync(g, done)) return -1;
     nr = (long long)__ldcg(cntn);
     cur = listn;
     if (nr == 0) return 0;
   }
 }
 
+// The rounds of the last nr <= kTail open hits by block 0 alone, from round r: each
+// thread keeps up to kTailHits of them in registers to the end.  Round 0 (the list is every
+// hit) has had its R1 with the t* keys.  Photons' slots and remaining weights are read
+// and written through L2; a fence and the block's barrier separate the phases.  Returns 0,
+// or -2 when the rounds ran out.
+__device__ int tail_rounds(const DepArgs &g, long long nr, const unsigned *cur, long long &r) {
+  __shared__ int tie_s[2];
+  unsigned hx[kTailHits], hy[kTailHits], id[kTailHits];
+  unsigned long long key[kTailHits];
+  unsigned open = 0u;
+#pragma unroll
+  for (int q = 0; q < kTailHits; ++q) {
+    const long long i = threadIdx.x + (long long)q * kThreads;
+    hx[q] = hy[q] = id[q] = 0u;
+    key[q] = 0ull;
+    if (i < nr) {
+      id[q] = cur ? __ldcg(cur + i) : (unsigned)i;
+      if (cur || __ldcg(g.state + id[q]) == kOpen) {
+        const uint2 h = __ldcg(g.hits + id[q]);
+        hx[q] = h.x;
+        hy[q] = h.y;
+        key[q] = __ldcg(g.key + id[q]);
+        open |= 1u << q;
+      }
+    }
+  }
+  if (threadIdx.x < 2) tie_s[threadIdx.x] = r == 0 ? __ldcg(&g.ctl->tie[threadIdx.x]) : 0;
+  __syncthreads();
+  for (;; ++r) {
+    if (r > g.n) return -2;  // unreachable: every round resolves the earliest open hit
+    const int b = (int)(r & 1), nb = b ^ 1;
+    if (r > 0) {
+      // R1
+      unsigned used = 0u;  // a photon used up: delta stays 0
+#pragma unroll
+      for (int q = 0; q < kTailHits; ++q)
+        if (open >> q & 1u)
+          used |= (unsigned)(!(__ldcg(g.rem_a + hx[q]) > 0.0) | !(__ldcg(g.rem_b + hy[q]) > 0.0))
+                  << q;
+      open &= ~used;
+      bool tie = false;
+#pragma unroll
+      for (int q = 0; q < kTailHits; ++q)
+        if (open >> q & 1u)
+          tie |= (atomicMin(&g.sA[hx[q]].t[b], key[q]) == key[q]) |
+                 (atomicMin(&g.sB[hy[q]].t[b], key[q]) == key[q]);
+      if (tie) tie_s[b] = 1;
+      __threadfence();
+      __syncthreads();
+    }
+    const bool ties = tie_s[b] != 0;
+    // R2
+    if (ties) {
+#pragma unroll
+      for (int q = 0; q < kTailHits; ++q)
+        if (open >> q & 1u) {
+          if (__ldcg(&g.sA[hx[q]].t[b]) == key[q]) atomicMin(&g.sA[hx[q]].p[b], hy[q]);
+          if (__ldcg(&g.sB[hy[q]].t[b]) == key[q]) atomicMin(&g.sB[hy[q]].p[b], hx[q]);
+        }
+      __threadfence();
+      __syncthreads();
+    }
+    // R3
+    unsigned ready = 0u;
+#pragma unroll
+    for (int q = 0; q < kTailHits; ++q)
+      if (open >> q & 1u) {
+        const DepSlot *qa = g.sA + hx[q], *qb = g.sB + hy[q];
+        if (__ldcg(&qa->t[b]) == key[q] && __ldcg(&qb->t[b]) == key[q] &&
+            (!ties || (__ldcg(&qa->p[b]) == hy[q] && __ldcg(&qb->p[b]) == hx[q])))
+          ready |= 1u << q;
+      }
+#pragma unroll
+    for (int q = 0; q < kTailHits; ++q)
+      if (open >> q & 1u) {
+        DepSlot *qa = g.sA + hx[q], *qb = g.sB + hy[q];
+        qa->t[nb] = kNoKey;  // the next round's slots of both photons start empty
+        qa->p[nb] = kNoIdx;
+        qb->t[nb] = kNoKey;
+        qb->p[nb] = kNoIdx;
+        if (ready >> q & 1u) {
+          const double ra = __ldcg(g.rem_a + hx[q]), rb = __ldcg(g.rem_b + hy[q]);
+          const double d = ra < rb ? ra : rb;
+          g.rem_a[hx[q]] = __dsub_rn(ra, d);
+          g.rem_b[hy[q]] = __dsub_rn(rb, d);
+          g.delta[id[q]] = d;
+        }
+      }
+    open &= ~ready;
+    if (threadIdx.x == 0) tie_s[nb] = 0;  // (nb's flag was last read before the R1 barrier)
+    __threadfence();
+    if (!__syncthreads_or(open != 0u)) return 0;
+  }
+}
+
 // One depletion call.  Values that other threads wrote in an earlier phase
 // are read with __ldcg (from L2), so no stale L1 line is seen.
 __global__ void __launch_bounds__(kThreads, 1) k_deplete(DepArgs g) {
-  const long long gtid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  // warps dealt to the blocks in turn, so that a short list spreads over all of them (the
+  // t* phase is bound by the SMs' FP64 pipes)
+  const long long gtid =
+      ((threadIdx.x >> 5) * (long long)gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31);
   const long long gstride = (long long)gridDim.x * blockDim.x;
   DepCtl *ctl = g.ctl;
+  unsigned done = 0u;  // grid barriers passed
 
   // slots left dirty by a call that failed: every photon's slots back to empty
   if (__ldcg(g.dirty)) {
     for (long long q = gtid; q < g.na; q += gstride) clear_slot(g.sA + q);
     for (long long q = gtid; q < g.nb; q += gstride) clear_slot(g.sB + q);
-    if (!grid_sync(g)) return record_failure(g, TRILENS_ERR_TIMEOUT);
+    if (!grid_sync(g, done)) return record_failure(g, TRILENS_ERR_TIMEOUT);
     if (gtid == 0) atomicExch(g.dirty, 0);  // every block has read it
   }
 
@@ -369,7 +458,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_deplete(DepArgs g) {
         atomicOr(&ctl->tie[0], 1);
     }
   }
-  if (!grid_sync(g)) return record_failure(g, TRILENS_ERR_TIMEOUT);
+  if (!grid_sync(g, done)) return record_failure(g, TRILENS_ERR_TIMEOUT);
   if (__ldcg(&ctl->flag) & kFlagBadInput) {  // nothing changed but delta
     if (gtid == 0) atomicExch(g.dirty, 1);
     return record_failure(g, TRILENS_ERR_INVALID);
@@ -378,14 +467,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_deplete(DepArgs g) {
   long long nr = g.n;            // hits open at the start of round r
   const unsigned *cur = nullptr;  // their list (round 0: every hit, in order)
   long long r = 0;
-  int st = run_rounds<false>(g, nr, cur, r, gtid, gstride);
+  int st = run_rounds(g, nr, cur, r, gtid, gstride, done);
   if (st == 1) {
     // the tail: block 0 alone; the others wait for it at the next barrier
     if (blockIdx.x == 0) {
-      st = run_rounds<true>(g, nr, cur, r, threadIdx.x, blockDim.x);
+      st = tail_rounds(g, nr, cur, r);
       if (st == -2 && threadIdx.x == 0) atomicOr(&ctl->flag, kFlagRounds);
     }
-    if (!grid_sync(g)) return record_failure(g, TRILENS_ERR_TIMEOUT);
+    if (!grid_sync(g, done)) return record_failure(g, TRILENS_ERR_TIMEOUT);
     st = (__ldcg(&ctl->flag) & kFlagRounds) ? -2 : 0;
   }
   if (st == -1) return record_failure(g, TRILENS_ERR_TIMEOUT);
@@ -416,7 +505,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_deplete(DepArgs g) {
       g.pcnt[blockIdx.x] = c;
     }
   }
-  if (!grid_sync(g)) return record_failure(g, TRILENS_ERR_TIMEOUT);
+  if (!grid_sync(g, done)) return record_failure(g, TRILENS_ERR_TIMEOUT);
   if (blockIdx.x == 0) {
     __syncthreads();  // ss, sc reused
     double s = 0.0;
@@ -562,7 +651,9 @@ static int dep_launch(trilens_ctx *c, int64_t step, const uint32_t *hits, int64_
   g.dirty = d.dirty;
   g.out = out;
   g.spin = c->p.spin_limit;  // iterations of 64 ns sleeps per barrier wait
-  const long long nblk = (n_hits + kThreads - 1) / kThreads;
+  // a block per 512 hits (see k_deplete's order of warps): more spread the t* phase further,
+  // and lengthen the barriers (50,000 photons' step: 209 us at 1024, 194 at 512, 204 at 256)
+  const long long nblk = (n_hits + 511) / 512;
   const int blocks = (int)std::min<long long>(nblk, d.max_blocks);
   CK(cudaMemsetAsync(d.ctl, 0, sizeof(DepCtl), s));
   void *args[] = {&g};
