@@ -219,32 +219,12 @@ TLNarrowConst tl_narrow_const(double dt_fs, double kappa) {
 
 static void free_beam(tl::BuildBufs &w) {
   cudaFree(w.stat);
-  cudaFree(w.pos_u);
-  cudaFree(w.dir_u);
   cudaFree(w.rec);
   cudaFree(w.cell);
   cudaFree(w.count);
   cudaFree(w.start);
   cudaFree(w.scan_st);
-  cudaFree(w.val[0]);
-  cudaFree(w.val[1]);
-  cudaFree(w.key[0]);
-  cudaFree(w.key[1]);
-  cudaFree(w.nodes);
-  cudaFree(w.parent_leaf);
-  cudaFree(w.parent_node);
-  cudaFree(w.rpre);
-  cudaFree(w.rsuf);
-  cudaFree(w.rtile);
-  cudaFree(w.rsuper);
-  cudaFree(w.nfirst);
-  cudaFree(w.nlast);
-  cudaFree(w.nlev);
-  cudaFree(w.sort_status);
-  cudaFree(w.sort_ep);
-  cudaFree(w.sort_raw);
-  cudaFree(w.sort_hist);
-  cudaFree(w.sort_tile);
+  cudaFree(w.full);
   memset(&w, 0, sizeof(w));
 }
 
@@ -285,6 +265,38 @@ static int beam_moments(trilens_ctx *c, const TLFrame &f, double mom[2][15], dou
   return TRILENS_OK;
 }
 
+// The statistical regime's arrays of m photons, in order in one buffer (256-byte aligned
+// each); the bytes they take.
+static size_t carve_full(tl::BuildBufs &w, char *base, size_t m) {
+  size_t at = 0;
+  auto take = [&](auto *&p, size_t count) {
+    p = reinterpret_cast<std::remove_reference_t<decltype(p)>>(base + at);
+    at = (at + sizeof(*p) * count + 255) & ~(size_t)255;
+  };
+  take(w.pos_u, m);
+  take(w.dir_u, m);
+  for (int q = 0; q < 2; ++q) {
+    take(w.key[q], m);
+    take(w.val[q], m);
+  }
+  take(w.sort_status, (size_t)w.sort_tiles * 256);
+  take(w.sort_ep, 9);
+  take(w.sort_raw, 8 * 256);
+  take(w.sort_hist, 8 * 256);
+  take(w.sort_tile, 8);
+  take(w.nodes, m);
+  take(w.parent_leaf, m);
+  take(w.parent_node, m);
+  take(w.rpre, 6 * m);
+  take(w.rsuf, 6 * m);
+  take(w.rtile, 6 * (size_t)tl::refit_tiles((int64_t)m));
+  take(w.rsuper, tl::refit_super_floats((int64_t)m));
+  take(w.nfirst, m);
+  take(w.nlast, m);
+  take(w.nlev, m);
+  return at;
+}
+
 // the statistical regime's hierarchies and the seeded traversal's queues, on first use
 int ensure_full(trilens_ctx *c) {
   if (c->full_ready) return TRILENS_OK;
@@ -297,32 +309,19 @@ int ensure_full(trilens_ctx *c) {
   for (int k = 0; k < 2; ++k) {
     tl::BuildBufs &w = c->w[k];
     const size_t m = (size_t)std::max<int64_t>(c->beam[k].n, 1);
-    CK(dalloc(&w.pos_u, m));
-    CK(dalloc(&w.dir_u, m));
-    CK(tl::launch_static_soa(c->beam[k], w, c->stream));
-    for (int q = 0; q < 2; ++q) {
-      CK(dalloc(&w.key[q], m));
-      CK(dalloc(&w.val[q], m));
-    }
     w.sort_tiles = (int64_t)((m + TL_SORT_TILE - 1) / TL_SORT_TILE);
     w.sort_epoch = 0;
-    CK(dalloc(&w.sort_status, (size_t)w.sort_tiles * 256));
-    CK(dalloc(&w.sort_ep, 9));
-    CK(dalloc(&w.sort_raw, 8 * 256));
+    // one allocation per beam (one by one, the arrays took a fifth of the first call)
+    if (!w.full) CK(dalloc(&w.full, carve_full(w, nullptr, m)));
+    carve_full(w, w.full, m);
+    CK(tl::launch_static_soa(c->beam[k], w, c->stream));
     CK(cudaMemsetAsync(w.sort_raw, 0, sizeof(uint32_t) * 8 * 256, c->stream));
-    CK(dalloc(&w.sort_hist, 8 * 256));
-    CK(dalloc(&w.sort_tile, 8));
-    CK(dalloc(&w.nodes, m));
-    CK(dalloc(&w.parent_leaf, m));
-    CK(dalloc(&w.parent_node, m));
-    CK(dalloc(&w.rpre, 6 * m));
-    CK(dalloc(&w.rsuf, 6 * m));
-    CK(dalloc(&w.rtile, 6 * (size_t)tl::refit_tiles((int64_t)m)));
-    CK(dalloc(&w.rsuper, tl::refit_super_floats((int64_t)m)));
-    CK(dalloc(&w.nfirst, m));
-    CK(dalloc(&w.nlast, m));
-    CK(dalloc(&w.nlev, m));
   }
+  int lo = 0, hi = 0;
+  CK(cudaDeviceGetStreamPriorityRange(&lo, &hi));
+  if (!c->cut_stream)
+    CK(cudaStreamCreateWithPriority(&c->cut_stream, cudaStreamNonBlocking, hi));
+  if (!c->sum_stream) CK(cudaStreamCreateWithFlags(&c->sum_stream, cudaStreamNonBlocking));
   const unsigned long long warps = (unsigned long long)c->trav_blocks * c->trav_warps;
   int rc = alloc_queue(c, std::max<unsigned long long>(
                               1 << 20, 2ull * warps * (unsigned long long)c->p.stack_depth));
@@ -467,6 +466,8 @@ void trilens_destroy(trilens_ctx *c) {
   if (c->gexec) cudaGraphExecDestroy(c->gexec);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   if (c->side_stream) cudaStreamDestroy(c->side_stream);
+  if (c->sum_stream) cudaStreamDestroy(c->sum_stream);
+  if (c->cut_stream) cudaStreamDestroy(c->cut_stream);
   if (c->fork_ev) cudaEventDestroy(c->fork_ev);
   if (c->join_ev) cudaEventDestroy(c->join_ev);
   for (int ph = 0; ph < PH_COUNT; ++ph)

@@ -174,7 +174,9 @@ struct BuildBufs {
   uint2 *cell;
   uint32_t *count, *start, *scan_st;
   int64_t cells;
-  // from here to sort_ep: the statistical regime's, allocated with it
+  // from here to sort_ep (nfirst to nlev too): the statistical regime's, one buffer `full`
+  // allocated with it
+  char *full;
   float4 *pos_u, *dir_u;      // unsorted SoA32
   unsigned long long *key[2];
   uint32_t *val[2];

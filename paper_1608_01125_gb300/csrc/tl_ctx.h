@@ -86,6 +86,9 @@ struct trilens_ctx {
   // context's stream (the two builds are independent)
   cudaStream_t side_stream = nullptr;
   cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
+  // statistical regime: the cut's chain of small kernels (high priority), and the moments'
+  // sums inside the blocks, both beside the other moments' kernels
+  cudaStream_t cut_stream = nullptr, sum_stream = nullptr;
   cudaGraphExec_t gexec = nullptr;
   int64_t g_first = -1, g_steps = 0;
   double *g_yields = nullptr;

@@ -4,6 +4,26 @@
 
 namespace tl {
 
+// running sums of six moments over a beam's sorted photons: up to the front of a 32-photon
+// chunk, and within the chunk up to the ends of the cut nodes
+struct PreSums {
+  double *bsum;  // [6][block of 1024]
+  double *tot;   // [6][chunk in block][block]: the chunks' sums, then the running sums
+  double *end;   // [n + 1][6], at the ends alone
+  int64_t blocks;
+};
+size_t pre_doubles(int64_t n);  // workspace of one beam
+PreSums pre_sums(double *buf, int64_t n);
+
+struct PreBeam {
+  const float4 *pos, *dir;  // sorted SoA (dir.w = input index)
+  const unsigned long long *key;  // sorted keys
+  const double *w;          // weights of the input, null: 1
+  int64_t n;
+  int key_bits;
+  PreSums sums;
+};
+
 // one hierarchy as the level-L cut and the feature gather see it
 struct CutTree {
   const TLNode *nodes;
@@ -11,7 +31,7 @@ struct CutTree {
   const uint32_t *nfirst;       // first photon of every inner node's range
   const uint8_t *nlev;          // level of every inner node
   const float4 *dir;            // sorted SoA (w = input index)
-  const double *pre;            // 6 prefix sums of n + 1 doubles each
+  PreSums pre;                  // running moments of the sorted photons
   int64_t n;
   uint32_t super;
   int bucket;  // leaf bucket size: inner nodes of at most this many photons are buckets
@@ -31,12 +51,14 @@ struct CutArgs {
   unsigned *status;
 };
 
-cudaError_t launch_prefix_moments(const TLBeam &B, const float4 *pos, const float4 *dir, int64_t n,
-                                  double *bsum, double *pre, cudaStream_t s);
+cudaError_t launch_prefix_moments(const PreBeam &a, const PreBeam &b, int L, cudaStream_t s,
+                                  cudaStream_t side, cudaEvent_t blocks_ev, cudaEvent_t tile_ev);
+cudaError_t prefix_prepare();
 cudaError_t launch_cut_level(const CutArgs &a, int blocks, cudaStream_t s);
 cudaError_t launch_features(const CutTree &A, const CutTree &B, const uint4 *cut,
                             const unsigned *cut_count, unsigned cap, float *feat, float *st,
-                            double dt, double kappa, int blocks, cudaStream_t s);
+                            double dt, double kappa, const unsigned *build_status, int blocks,
+                            cudaStream_t s);
 cudaError_t launch_labels_prep(const CutTree &T, int L, uint32_t *cid_node, uint32_t *cid_slot,
                                uint2 *flist, unsigned *fcount, unsigned fcap, uint32_t *cut_of,
                                uint32_t *inv, cudaStream_t s);
@@ -54,7 +76,7 @@ cudaError_t launch_attribute(const uint2 *hits, const unsigned long long *nhits,
 cudaError_t launch_estimate(const float *out, const float *st, float st_scale, const uint4 *cut,
                             const unsigned *cut_count, unsigned cap, float tau, double *pred,
                             uint2 *fb, unsigned *fb_count, unsigned fb_cap, int blocks,
-                            cudaStream_t s, uint8_t *flag = nullptr);
+                            cudaStream_t s, uint8_t *flag = nullptr, double *sums = nullptr);
 // small helpers: op 0 copies cut refs (uint4 -> uint2), op 1 writes log1p of
 // doubles as floats, op 2 / op 3 add n doubles / floats into *c (a double)
 cudaError_t launch_sur_misc(int op, const void *a, const void *b, void *c, int64_t n,

@@ -15,6 +15,7 @@
 
 constexpr int kBatch = 8192;
 constexpr int kTauBins = 64;
+constexpr int kCutRec = 4 + 256;
 // edges of the fallback-threshold bins of the calibration table: 2^(g/2 - 10)
 static inline double tau_edge(int g) { return std::ldexp(1.0, -10) * std::pow(2.0, 0.5 * g); }
 
@@ -32,10 +33,13 @@ struct SurrogateState {
   double cal_tau[64];
   int adam_step = 0;
   // per-step buffers
-  double *pre[2]{}, *bsum[2]{};
+  double *pre[2]{};  // tl::PreSums
   uint2 *lvl[2]{};
   unsigned lvl_cap = 0;
-  unsigned *lcount = nullptr;  // device, per level
+  // device record of the cut, set and read back as one: [0] pairs, [1] status, [2..3] the
+  // root pair, [4..] pairs per level
+  unsigned *rec = nullptr;
+  unsigned *lcount = nullptr;
   uint4 *cut = nullptr;
   unsigned cut_cap = 0;
   unsigned *cut_count = nullptr;
@@ -44,6 +48,7 @@ struct SurrogateState {
   double *pred = nullptr, *scal = nullptr;
   uint2 *fb = nullptr, *seeds = nullptr;
   unsigned *fb_count = nullptr;
+  cudaEvent_t ev[4]{};
   // labels
   uint32_t *cid_node[2]{}, *cid_slot[2]{}, *cut_of[2]{}, *inv[2]{};
   uint2 *flist[2]{};
@@ -73,7 +78,6 @@ static void sfree(SurrogateState *s) {
   cudaFree(s->err);
   for (int k = 0; k < 2; ++k) {
     cudaFree(s->pre[k]);
-    cudaFree(s->bsum[k]);
     cudaFree(s->lvl[k]);
     cudaFree(s->cid_node[k]);
     cudaFree(s->cid_slot[k]);
@@ -81,10 +85,10 @@ static void sfree(SurrogateState *s) {
     cudaFree(s->inv[k]);
     cudaFree(s->flist[k]);
   }
-  cudaFree(s->lcount);
+  cudaFree(s->rec);
+  for (int k = 0; k < 4; ++k)
+    if (s->ev[k]) cudaEventDestroy(s->ev[k]);
   cudaFree(s->cut);
-  cudaFree(s->cut_count);
-  cudaFree(s->status);
   cudaFree(s->feat);
   cudaFree(s->st);
   cudaFree(s->out);
@@ -164,8 +168,7 @@ static int ensure_state(trilens_ctx *c) {
   CK(cudaMemsetAsync(s->err, 0, sizeof(int), c->stream));
   for (int k = 0; k < 2; ++k) {
     const int64_t n = std::max<int64_t>(c->beam[k].n, 1);
-    CK(dalloc(&s->pre[k], (size_t)6 * (n + 1)));
-    CK(dalloc(&s->bsum[k], (size_t)6 * ((n + 1023) / 1024 + 1)));
+    CK(dalloc(&s->pre[k], tl::pre_doubles(n)));
     CK(dalloc(&s->cid_node[k], (size_t)n));
     CK(dalloc(&s->cid_slot[k], (size_t)2 * n));
     CK(dalloc(&s->cut_of[k], (size_t)n));
@@ -173,9 +176,12 @@ static int ensure_state(trilens_ctx *c) {
   }
   s->fcap = (unsigned)std::min<int64_t>(std::max(c->beam[0].n, c->beam[1].n) + 16, 1ll << 30);
   for (int k = 0; k < 2; ++k) CK(dalloc(&s->flist[k], s->fcap));
-  CK(dalloc(&s->lcount, 256));
-  CK(dalloc(&s->cut_count, 1));
-  CK(dalloc(&s->status, 1));
+  CK(tl::prefix_prepare());
+  for (int k = 0; k < 4; ++k) CK(cudaEventCreateWithFlags(&s->ev[k], cudaEventDisableTiming));
+  CK(dalloc(&s->rec, kCutRec));
+  s->cut_count = s->rec;
+  s->status = s->rec + 1;
+  s->lcount = s->rec + 4;
   CK(dalloc(&s->fb_count, 1));
   CK(dalloc(&s->fcount, 2));
   CK(dalloc(&s->scal, 4));
@@ -189,7 +195,7 @@ static tl::CutTree cut_tree(trilens_ctx *c, int k) {
   t.nfirst = c->w[k].nfirst;
   t.nlev = c->w[k].nlev;
   t.dir = c->w[k].dir;
-  t.pre = c->sur->pre[k];
+  t.pre = tl::pre_sums(c->sur->pre[k], c->beam[k].n);
   t.n = c->beam[k].n;
   t.super = (uint32_t)(t.n > 1 ? t.n - 1 : 0);
   t.bucket = c->p.leaf_bucket;
@@ -199,18 +205,25 @@ static tl::CutTree cut_tree(trilens_ctx *c, int k) {
 // moments, level-L cut pairs and their features for the built step
 static int sur_cut(trilens_ctx *c, int L, unsigned *ncut) {
   SurrogateState *s = c->sur;
+  // The cut's chain of small kernels runs beside the moments' (all on one stream where the
+  // phases are timed), with high priority: a kernel behind another's queue of blocks waits
+  // for the whole queue (2 x 1e6 photons: 755 us a step, 705 us this way).
+  const cudaStream_t cs = c->timing ? c->stream : c->cut_stream;
+  CK(cudaEventRecord(s->ev[0], c->stream));
+  CK(cudaStreamWaitEvent(cs, s->ev[0], 0));
+  tl::PreBeam pb[2];
+  for (int k = 0; k < 2; ++k)
+    pb[k] = {c->w[k].pos, c->w[k].dir, c->w[k].key[c->sel[k]], c->beam[k].w, c->beam[k].n,
+             c->key_bits[k], tl::pre_sums(s->pre[k], c->beam[k].n)};
+  CK(tl::launch_prefix_moments(pb[0], pb[1], L, c->stream, c->timing ? c->stream : c->sum_stream,
+                               s->ev[1], s->ev[2]));
   for (int attempt = 0; attempt < 6; ++attempt) {
-    for (int k = 0; k < 2; ++k)
-      CK(tl::launch_prefix_moments(c->beam[k], c->w[k].pos, c->w[k].dir, c->beam[k].n, s->bsum[k],
-                                   s->pre[k], c->stream));
-    CK(cudaMemsetAsync(s->lcount, 0, sizeof(unsigned) * 256, c->stream));
-    CK(cudaMemsetAsync(s->cut_count, 0, sizeof(unsigned), c->stream));
-    CK(cudaMemsetAsync(s->status, 0, sizeof(unsigned), c->stream));
-    const uint2 root = make_uint2((uint32_t)(c->beam[0].n > 1 ? c->beam[0].n - 1 : 0),
-                                  (uint32_t)(c->beam[1].n > 1 ? c->beam[1].n - 1 : 0));
     const unsigned one = (c->beam[0].n > 0 && c->beam[1].n > 0) ? 1u : 0u;
-    CK(cudaMemcpyAsync(s->lvl[0], &root, sizeof(uint2), cudaMemcpyHostToDevice, c->stream));
-    CK(cudaMemcpyAsync(s->lcount, &one, sizeof(unsigned), cudaMemcpyHostToDevice, c->stream));
+    unsigned rec[kCutRec] = {};
+    rec[2] = (unsigned)(c->beam[0].n > 1 ? c->beam[0].n - 1 : 0);
+    rec[3] = (unsigned)(c->beam[1].n > 1 ? c->beam[1].n - 1 : 0);
+    rec[4] = one;
+    CK(cudaMemcpyAsync(s->rec, rec, sizeof(rec), cudaMemcpyHostToDevice, cs));
     tl::CutArgs a;
     a.A = cut_tree(c, 0);
     a.B = cut_tree(c, 1);
@@ -223,23 +236,37 @@ static int sur_cut(trilens_ctx *c, int L, unsigned *ncut) {
     int level = 0;
     unsigned left = one;
     while (left > 0 && level < 250) {
-      for (int q = 0; q < 8 && level < 250; ++q, ++level) {
-        a.in = s->lvl[level & 1];
+      // a level of the cut is at least one bit deeper in both trees, below the super
+      // roots: L + 2 levels end it, and up to a depth of 30 the host does not ask before
+      const int batch = level == 0 ? std::min(L + 2, 32) : 8;
+      if (level > 0) {  // not before the features have read the list so far
+        CK(cudaEventRecord(s->ev[0], c->stream));
+        CK(cudaStreamWaitEvent(cs, s->ev[0], 0));
+      }
+      for (int q = 0; q < batch && level < 250; ++q, ++level) {
+        a.in = level ? s->lvl[level & 1] : reinterpret_cast<const uint2 *>(s->rec + 2);
         a.out = s->lvl[(level + 1) & 1];
         a.counts = s->lcount + level;
-        CK(tl::launch_cut_level(a, 4 * c->n_sm, c->stream));
+        CK(tl::launch_cut_level(a, 4 * c->n_sm, cs));
       }
-      CK(cudaMemcpyAsync(&left, s->lcount + level, sizeof(unsigned), cudaMemcpyDeviceToHost,
-                         c->stream));
+      // the features of what is complete when the cut ends here, without the host's word
+      CK(cudaEventRecord(s->ev[3], cs));
+      CK(cudaStreamWaitEvent(c->stream, s->ev[3], 0));
+      CK(tl::launch_features(a.A, a.B, s->cut, s->cut_count, s->cut_cap, s->feat, s->st,
+                             c->p.dt_fs, c->p.kappa, c->build_status, 16 * c->n_sm, c->stream));
+      CK(cudaMemcpyAsync(c->build_status_host, c->build_status, sizeof(unsigned),
+                         cudaMemcpyDeviceToHost, cs));
+      CK(cudaMemcpyAsync(rec, s->rec, sizeof(rec), cudaMemcpyDeviceToHost, cs));
+      CK(cudaStreamSynchronize(cs));
+      left = rec[4 + level];
+    }
+    if (!one) {  // an empty beam
+      CK(cudaMemcpyAsync(c->build_status_host, c->build_status, sizeof(unsigned),
+                         cudaMemcpyDeviceToHost, c->stream));
       CK(cudaStreamSynchronize(c->stream));
     }
-    unsigned st = 0;
-    CK(cudaMemcpyAsync(ncut, s->cut_count, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaMemcpyAsync(&st, s->status, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaMemcpyAsync(c->build_status_host, c->build_status, sizeof(unsigned),
-                       cudaMemcpyDeviceToHost, c->stream));
-    CK(cudaStreamSynchronize(c->stream));
-    const unsigned bst = *c->build_status_host;
+    *ncut = rec[0];
+    const unsigned st = rec[1], bst = *c->build_status_host;
     if (bst & (TL_ST_TIMEOUT | TL_ST_BADTREE)) {  // the hierarchy of this step is invalid
       c->w[0].sort_epoch = c->w[1].sort_epoch = 0;
       CK(cudaMemsetAsync(c->build_status, 0, sizeof(unsigned), c->stream));
@@ -249,11 +276,8 @@ static int sur_cut(trilens_ctx *c, int L, unsigned *ncut) {
       return fail(c, TRILENS_ERR_CUDA, "the refit met a node reference out of range (internal error)");
     }
     if (left > 0) return fail(c, TRILENS_ERR_STACK, "cut traversal did not finish");
-    if (!(st & TL_ST_FRONT_OVF)) {
-      CK(tl::launch_features(a.A, a.B, s->cut, s->cut_count, s->cut_cap, s->feat, s->st,
-                             c->p.dt_fs, c->p.kappa, 4 * c->n_sm, c->stream));
-      return TRILENS_OK;
-    }
+    if (!(st & TL_ST_FRONT_OVF)) return TRILENS_OK;
+    CK(cudaStreamSynchronize(c->stream));  // the features of the list that overflowed
     int rc = cut_buffers(c, std::max(2 * s->cut_cap, *ncut + (*ncut >> 2) + 1024));
     if (rc) return rc;
   }
@@ -589,14 +613,19 @@ int trilens_surrogate_step(trilens_ctx *c, int64_t step, int32_t level_L, float 
   CK(cudaEventRecord(e1, c->stream));
   CK(tl::mlp_forward(s->prm, s->norm, s->feat, ncut, s->out, c->n_sm, s->err, c->p.spin_limit,
                      c->stream));
-  CK(cudaMemsetAsync(s->fb_count, 0, sizeof(unsigned), c->stream));
+  // sums of the predictions and of the ST rates, then the number of fallback pairs
+  unsigned *const fbc = reinterpret_cast<unsigned *>(s->scal + 2);
+  CK(cudaMemsetAsync(s->scal, 0, 3 * sizeof(double), c->stream));
   CK(tl::launch_estimate(s->out, s->st, (float)s->st_calib, s->cut, s->cut_count, s->cut_cap, tau,
-                         s->pred, s->fb, s->fb_count, s->cut_cap, 4 * c->n_sm, c->stream));
+                         s->pred, s->fb, fbc, s->cut_cap, 4 * c->n_sm, c->stream, nullptr,
+                         s->scal));
   CK(cudaEventRecord(e2, c->stream));
+  double sums[3];
+  CK(cudaMemcpyAsync(sums, s->scal, sizeof(sums), cudaMemcpyDeviceToHost, c->stream));
+  CK(cudaStreamSynchronize(c->stream));
+  const double est = sums[0], st = sums[1];
   unsigned nfb = 0;
-  CK(cudaMemcpyAsync(&nfb, s->fb_count, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
-  double est = 0, st = 0;
-  if ((rc = dsum(c, 2, s->pred, ncut, &est)) || (rc = dsum(c, 3, s->st, ncut, &st))) return rc;
+  memcpy(&nfb, sums + 2, sizeof(nfb));
   double fb_exact = 0;
   if (nfb > 0) {
     const double keep_c = c->tot_count, keep_w = c->tot_weighted;
