@@ -27,7 +27,7 @@ size_t partial_bytes();
 cudaError_t launch_yield_inst(const TravArgs &a, const uint32_t *inst_of_a, double *yields,
                               int blocks, cudaStream_t s);
 cudaError_t launch_pair_products(const TLBeam &a, const TLBeam &b, const uint32_t *hits,
-                                 int64_t n_hits, unsigned long long seed, double *out, int n_sm,
+                                 int64_t n_hits, unsigned long long seed, double *out,
                                  cudaStream_t s);
 cudaError_t launch_step_finish(const TLCounters *ctr, unsigned *run_status, TLRunAcc *acc,
                                cudaStream_t s);
@@ -1459,10 +1459,6 @@ int trilens_pair_products(const trilens_beam *a, const trilens_beam *b, const ui
   if (!beam_ok(a) || !beam_ok(b) || n_hits < 0 || n_hits >= (1ll << 40)) return TRILENS_ERR_INVALID;
   if (n_hits == 0) return TRILENS_OK;
   if (!hits || !out || a->n == 0 || b->n == 0) return TRILENS_ERR_INVALID;
-  int dev = 0, n_sm = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return TRILENS_ERR_CUDA;
   TLBeam ta, tb;
   const trilens_beam *bs[2] = {a, b};
   TLBeam *ts[2] = {&ta, &tb};
@@ -1473,7 +1469,7 @@ int trilens_pair_products(const trilens_beam *a, const trilens_beam *b, const ui
     t.dx = bs[k]->dx; t.dy = bs[k]->dy; t.dz = bs[k]->dz;
     t.E = bs[k]->E; t.w = bs[k]->w;
   }
-  if (tl::launch_pair_products(ta, tb, hits, n_hits, (unsigned long long)seed, out, n_sm,
+  if (tl::launch_pair_products(ta, tb, hits, n_hits, (unsigned long long)seed, out,
                                (cudaStream_t)stream) != cudaSuccess)
     return TRILENS_ERR_CUDA;
   return TRILENS_OK;
