@@ -174,6 +174,26 @@ static double host_sigma_max() { return host_sigma(host_sigma_peak_s()); }
 // an upper bound of Eq. BWcross over s (for conservative tests elsewhere)
 double tl_sigma_max_bound() { return host_sigma_max() * (1.0 + 1e-6); }
 
+// the pads' A(q): r(s) s^q at its largest, over r_max (see tl_set_pads); in steps of 3 %
+// of s - 1 up to s = 1e12 (r s^q is smooth, so 1e-3 covers the steps, and falls beyond)
+static TLPadTable make_pad_table() {
+  double a[kPadQ] = {};
+  const double smax = host_sigma_max();
+  for (double x = 1e-3; x < 1e12; x *= 1.03) {
+    double v = sqrt(host_sigma(1.0 + x) / smax);
+    const double p = pow(1.0 + x, 0.04);
+    for (int k = 0; k < kPadQ; ++k, v *= p) a[k] = std::max(a[k], v);
+  }
+  TLPadTable t;
+  for (int k = 0; k < kPadQ; ++k) t.a[k] = (float)(a[k] * (1.0 + 1e-3));
+  return t;
+}
+
+static const TLPadTable &pad_table() {
+  static const TLPadTable t = make_pad_table();
+  return t;
+}
+
 static float round_up(double x) {
   float f = (float)x;
   if ((double)f < x) f = nextafterf(f, INFINITY);
@@ -358,11 +378,13 @@ static int layout(trilens_ctx *c, const std::vector<int64_t> sizes[2]) {
   for (int k = 0; k < 2; ++k) {
     std::vector<TLInst> in(ni);
     std::vector<uint32_t> tile_inst;
-    int64_t tile = 0, cells = 0;
+    int64_t tile = 0, cells = 0, first = 0;
     for (size_t q = 0; q < ni; ++q) {
       TLInst &I = in[q];
       memset(&I, 0, sizeof(I));
       I.n = (int)sizes[k][q];
+      I.first = (int)first;
+      first += sizes[k][q];
       I.tile0 = (int)tile;
       I.bits = order_bits_for(sizes[k][q]);
       I.cell0 = (uint32_t)cells;
@@ -546,6 +568,7 @@ static int ctx_create(trilens_ctx **out, const trilens_beam *a, const trilens_be
     // one-time: the beams' mean directions (the frame), then their moments and extremes in
     // the frame, for the grids and boxes of every step
     c->frame0 = tl_ident_frame();
+    double mean[2][5] = {}, le[2][2] = {};
     if (c->beam[0].n > 0 && c->beam[1].n > 0) {
       const int nd = tl::mean_doubles();
       std::vector<double> h(2 * (size_t)nd);
@@ -560,17 +583,20 @@ static int ctx_create(trilens_ctx **out, const trilens_beam *a, const trilens_be
       if (!me) me = cudaStreamSynchronize(c->stream);
       cudaFree(part);
       CK(me);
-      double mean[2][3] = {};
-      for (int k = 0; k < 2; ++k)
+      for (int k = 0; k < 2; ++k) {
         for (int q = 0; q < nd; ++q)
-          mean[k][q % 3] += h[(size_t)k * nd + q] / (double)tl::mean_count(c->beam[k].n);
+          mean[k][q % 5] += h[(size_t)k * nd + q] / (double)tl::mean_count(c->beam[k].n);
+        le[k][0] = mean[k][3];
+        le[k][1] = sqrt(std::max(mean[k][4] - mean[k][3] * mean[k][3], 0.0));
+      }
       c->frame0 = tl_make_frame(mean[0], mean[1]);
     }
-    CK(cudaMemcpyAsync(c->frames, &c->frame0, sizeof(TLFrame), cudaMemcpyHostToDevice, c->stream));
     if ((rc = beam_moments(c, c->frame0, c->fmoments, c->ext))) {
       trilens_destroy(c);
       return rc;
     }
+    tl_set_pads(c->frame0, pad_table(), c->ext[0], c->ext[1], le[0], le[1], c->half);
+    CK(cudaMemcpyAsync(c->frames, &c->frame0, sizeof(TLFrame), cudaMemcpyHostToDevice, c->stream));
   }
   CK(tl::sort_prepare());
   CK(tl::refit_prepare());
@@ -647,7 +673,7 @@ static void step_grids(trilens_ctx *c, double T, TLGrid g[2]) {
     const TLFrame &f = c->frame0;
     ru[k] = (double)f.r[3 * k] * f.u[0] + (double)f.r[3 * k + 1] * f.u[1] +
             (double)f.r[3 * k + 2] * f.u[2];
-    s[k] = 2.0 * c->half;
+    s[k] = 2.0 * f.typ;
     for (int h = 0; h < 2; ++h) {
       const double *m = c->fmoments[h], n = (double)std::max<int64_t>(c->beam[h].n, 1);
       const double mean = m[3 + k] / n;
@@ -746,6 +772,7 @@ static int build_exact(trilens_ctx *c, int64_t step) {
     b.Llo = c->L_lo;
     b.Lhi = c->L_hi;
     b.half = c->half;
+    b.beam = k;
     b.box = c->box;
     b.build_status = c->build_status;
     CK(tl::launch_boxes(b, c->n_tiles[k], c->n_inst, c->max_top, st));
@@ -1093,7 +1120,17 @@ int trilens_batch_create(trilens_ctx **out, const trilens_beam *a, const trilens
       CK(tl::launch_inst_bounds(c->beam[k], c->inst_of[k], nullptr, n_inst, c->inst_tmp,
                                 c->inst_bounds[k], c->stream));
     }
-    CK(tl::launch_inst_frames(c->inst_bounds[0], c->inst_bounds[1], n_inst, c->frames, c->stream));
+    double *le = nullptr;  // ln E of the instances, beam after beam
+    CK(dalloc(&le, (size_t)4 * n_inst));
+    cudaError_t fe = cudaSuccess;
+    for (int k = 0; k < 2 && !fe; ++k)
+      fe = tl::launch_inst_energy(c->beam[k], c->insts[k], n_inst, le + 2 * (size_t)k * n_inst,
+                                  c->stream);
+    if (!fe)
+      fe = tl::launch_inst_frames(c->inst_bounds[0], c->inst_bounds[1], le, le + 2 * (size_t)n_inst,
+                                  pad_table(), c->half, n_inst, c->frames, c->stream);
+    cudaFree(le);  // (waits for the kernels)
+    CK(fe);
     for (int k = 0; k < 2; ++k)  // the bounds in every instance's frame
       CK(tl::launch_inst_bounds(c->beam[k], c->inst_of[k], c->frames, n_inst, c->inst_tmp,
                                 c->inst_bounds[k], c->stream));

@@ -19,6 +19,9 @@ struct TLFrame {
   float r[9];
   float u[3];
   int ident;
+  // half-width across its path of a photon's box of beam k: amp[k] E^xp (tl_photon_pad);
+  // typ: that of a typical photon
+  float amp[2], xp, typ;
   int pad[3];
 };
 
@@ -37,7 +40,8 @@ struct TLGrid {
 // photons that can meet the other beam in a step are sorted; how many, the running sum
 // of the cells tells (tl_live).
 struct TLInst {
-  int n;            // photons
+  int n;            // photons,
+  int first;        // from this one of the input on
   int tile0;        // first tile
   int bits;         // its photons are ordered by 2^bits cells,
   uint32_t cell0;   // from this one on
@@ -58,7 +62,7 @@ __host__ __device__ inline int tl_top_level(int n) {
 constexpr int kTile = 1024;  // sorted photons per tile (a level-2 node)
 
 __host__ __device__ inline TLFrame tl_ident_frame() {
-  TLFrame f{};
+  TLFrame f{};  // (no pads: set by tl_set_pads)
   f.r[0] = f.r[4] = f.r[8] = 1.0f;
   f.ident = 1;
   return f;
@@ -114,6 +118,53 @@ __host__ __device__ inline TLFrame tl_make_frame(const double a[3], const double
     f.r[6 + k] = (float)w[k];
   }
   return f;
+}
+
+// Pads by energy.  A pair collides within r(s), s = E_i E_j (1 - cos) / (2 m^2 c^4), and r
+// falls with s beyond its peak at s ~ 2 (r^2 ~ ln s / s): most pairs meet far inside r_max.
+// With r(s) <= A r_max s^-q for every s (A = max of r s^q / r_max) and s >= s_i s_j,
+// s_k = lambda_k E_k sqrt(cmin / 2) / m c^2 (cmin: least 1 - cos of the beams;
+// lambda_a lambda_b = 1), r <= A r_max s_i^-q s_j^-q <= A r_max (s_i^-2q + s_j^-2q) / 2:
+// a pad of its own for each photon, whose sums cover every pair.  A photon's pad
+// is at most r_max, which covers its pairs alone.  q is the one with the least pads near
+// the beams' mean ln E, 0 (r_max / 2 for all) where none is below that.  64 steps of
+// 2 x 1M photons of 5 MeV 12.3 ms with r_max / 2, 10.1 ms now; a step of 2 x 4M with a
+// broad spectrum 7.16 ms, 6.60 ms.
+constexpr int kPadQ = 12;  // q = 0.04 k
+struct TLPadTable {
+  float a[kPadQ];
+};
+
+// e: 12 values each, the beams' extremes as in tl_beam_box, whose directions bound cos
+// (2e-5 covers their FP32 rounding and that of the frame); mean and standard deviation of
+// ln E of each beam.
+__host__ __device__ inline void tl_set_pads(TLFrame &f, const TLPadTable &t, const double *ea,
+                                            const double *eb, const double la[2],
+                                            const double lb[2], double half) {
+  double cmin = 1.0 - 2e-5;
+  for (int k = 0; k < 3; ++k) {
+    const double a0 = ea[3 + k], a1 = ea[9 + k], b0 = eb[3 + k], b1 = eb[9 + k];
+    cmin -= fmax(fmax(a0 * b0, a0 * b1), fmax(a1 * b0, a1 * b1));
+  }
+  const double m2 = TL_MEC2 * TL_MEC2, st = 0.5 * cmin * exp(la[0] + lb[0]) / m2;
+  const double sd = fmax(la[1], lb[1]);
+  int best = 0;
+  double least = 0.95;
+  for (int k = 1; k < kPadQ && cmin > 1e-3 && st > 0.0; ++k) {
+    const double c = (double)t.a[k] * exp(0.04 * k * (2.0 * sd - log(st)));
+    if (c < least) {
+      least = c;
+      best = k;
+    }
+  }
+  f.xp = -0.08f * (float)best;
+  for (int k = 0; k < 2; ++k) {
+    const double lam = exp(0.5 * (k ? la[0] - lb[0] : lb[0] - la[0]));
+    f.amp[k] = best ? (float)(half * (double)t.a[best] * (1.0 + 1e-5) *
+                              exp((double)f.xp * log(lam * sqrt(0.5 * cmin / m2))))
+                    : (float)half;
+  }
+  f.typ = (float)(best ? half * (double)t.a[best] * exp(-0.04 * best * log(st)) : half);
 }
 
 // The grid of `bits` bits in all over [lo, lo + range]: each bit halves the cells of
@@ -191,6 +242,12 @@ __device__ __forceinline__ void seg_axis(float p, float dc, float Llo, float Lhi
                                          float &lo, float &hi) {
   swept_axis(p, __fmaf_ru(fabsf(p), 1.1920928955078125e-7f, 1e-30f), dc,
              __fmaf_ru(fabsf(dc), 1.1920928955078125e-7f, 1e-30f), Llo, Lhi, half, lo, hi);
+}
+
+// A photon's pad (E in FP32): the margin in amp covers the rounding of the power.
+__device__ __forceinline__ float tl_photon_pad(const TLFrame &f, int beam, float E, float half) {
+  if (f.xp == 0.0f) return half;
+  return fminf(2.0f * half, fmaf(f.amp[beam], exp2f(f.xp * log2f(E)), 1e-9f));
 }
 
 // A photon's swept box in the frame.  Each coordinate of R P from the rounded inputs

@@ -20,33 +20,41 @@ namespace tl {
 
 // ---------------------------------------------------------------- frames and grids
 
-// Sums of d over up to kSample photons of a beam, evenly spaced (3 FP64 values per block,
-// added by the host): the beam's mean direction, for the choice of the frame.
+// Sums of d, ln E and ln^2 E over up to kSample photons of a beam, evenly spaced (5 FP64
+// values per block, added by the host): the beam's mean direction, for the choice of the
+// frame, and its typical energy, for the pads.
 constexpr int kSampleBlocks = 64, kSample = 65536;
 
+__device__ __forceinline__ float ln_energy(double E) {
+  return logf(fminf(fmaxf((float)E, 1e-18f), 1e18f));
+}
+
 __global__ void __launch_bounds__(256) k_mean_dir(TLBeam b, double *part) {
-  __shared__ double sm[8][3];
+  __shared__ double sm[8][5];
   const int64_t n = b.n < kSample ? b.n : kSample;
-  double m[3] = {0.0, 0.0, 0.0};
+  double m[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
   for (int64_t t = blockIdx.x * 256 + threadIdx.x; t < n; t += kSampleBlocks * 256) {
     const int64_t i = t * b.n / n;
     m[0] += b.dx[i];
     m[1] += b.dy[i];
     m[2] += b.dz[i];
+    const double le = (double)ln_energy(b.E[i]);
+    m[3] += le;
+    m[4] += le * le;
   }
-  for (int q = 0; q < 3; ++q)
+  for (int q = 0; q < 5; ++q)
     for (int off = 16; off; off >>= 1) m[q] += __shfl_xor_sync(0xffffffffu, m[q], off);
   if ((threadIdx.x & 31) == 0)
-    for (int q = 0; q < 3; ++q) sm[threadIdx.x >> 5][q] = m[q];
+    for (int q = 0; q < 5; ++q) sm[threadIdx.x >> 5][q] = m[q];
   __syncthreads();
-  if (threadIdx.x < 3) {
+  if (threadIdx.x < 5) {
     double t = 0.0;
     for (int w = 0; w < 8; ++w) t += sm[w][threadIdx.x];
-    part[blockIdx.x * 3 + threadIdx.x] = t;
+    part[blockIdx.x * 5 + threadIdx.x] = t;
   }
 }
 
-int mean_doubles() { return 3 * kSampleBlocks; }
+int mean_doubles() { return 5 * kSampleBlocks; }
 int64_t mean_count(int64_t n) { return n < kSample ? n : kSample; }
 
 cudaError_t launch_mean_dir(const TLBeam &b, double *part, cudaStream_t s) {
@@ -216,8 +224,44 @@ cudaError_t launch_inst_bounds(const TLBeam &b, const uint32_t *inst_of, const T
   return cudaGetLastError();
 }
 
-// Frames of a batch's instances, from the middle of each beam's range of directions.
-__global__ void k_inst_frames(const double *ba, const double *bb, int n_inst, TLFrame *out) {
+// Mean and standard deviation of ln E over up to 1024 photons, evenly spaced, of every
+// instance of a beam: a block each.
+__global__ void __launch_bounds__(256) k_inst_energy(const double *E, const TLInst *inst,
+                                                     double *out) {
+  __shared__ double sm[8][2];
+  const TLInst &I = inst[blockIdx.x];
+  const int n = min(I.n, 1024);
+  double m[2] = {0.0, 0.0};
+  for (int t = threadIdx.x; t < n; t += 256) {
+    const double le = (double)ln_energy(E[I.first + (int64_t)t * I.n / n]);
+    m[0] += le;
+    m[1] += le * le;
+  }
+  for (int q = 0; q < 2; ++q) {
+    for (int off = 16; off; off >>= 1) m[q] += __shfl_xor_sync(0xffffffffu, m[q], off);
+    if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5][q] = m[q];
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w)
+      for (int q = 0; q < 2; ++q) sm[0][q] += sm[w][q];
+    const double mean = sm[0][0] / max(n, 1);
+    out[2 * blockIdx.x] = mean;
+    out[2 * blockIdx.x + 1] = sqrt(fmax(sm[0][1] / max(n, 1) - mean * mean, 0.0));
+  }
+}
+
+cudaError_t launch_inst_energy(const TLBeam &b, const TLInst *inst, int n_inst, double *out,
+                               cudaStream_t s) {
+  k_inst_energy<<<n_inst, 256, 0, s>>>(b.E, inst, out);
+  return cudaGetLastError();
+}
+
+// Frames of a batch's instances, from the middle of each beam's range of directions, and
+// their pads; le: mean and standard deviation of ln E of either beam.
+__global__ void k_inst_frames(const double *ba, const double *bb, const double *lea,
+                              const double *leb, TLPadTable pads, double half, int n_inst,
+                              TLFrame *out) {
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= n_inst) return;
   double a[3], b[3];
@@ -225,12 +269,15 @@ __global__ void k_inst_frames(const double *ba, const double *bb, int n_inst, TL
     a[k] = 0.5 * (ba[12 * q + 3 + k] + ba[12 * q + 9 + k]);
     b[k] = 0.5 * (bb[12 * q + 3 + k] + bb[12 * q + 9 + k]);
   }
-  out[q] = tl_make_frame(a, b);  // an empty beam's bounds are NaN or infinite: the lab frame
+  TLFrame f = tl_make_frame(a, b);  // an empty beam's bounds are NaN or infinite: the lab frame
+  tl_set_pads(f, pads, ba + 12 * q, bb + 12 * q, lea + 2 * q, leb + 2 * q, half);
+  out[q] = f;
 }
 
-cudaError_t launch_inst_frames(const double *ba, const double *bb, int n_inst, TLFrame *out,
-                               cudaStream_t s) {
-  k_inst_frames<<<(n_inst + 127) / 128, 128, 0, s>>>(ba, bb, n_inst, out);
+cudaError_t launch_inst_frames(const double *ba, const double *bb, const double *lea,
+                               const double *leb, const TLPadTable &pads, double half, int n_inst,
+                               TLFrame *out, cudaStream_t s) {
+  k_inst_frames<<<(n_inst + 127) / 128, 128, 0, s>>>(ba, bb, lea, leb, pads, half, n_inst, out);
   return cudaGetLastError();
 }
 
@@ -248,7 +295,7 @@ __global__ void k_inst_grid(const double *ba, const double *bb, const TLFrame *f
   for (int k = 0; k < 3; ++k) {
     ru[k] = (double)f.r[3 * k] * f.u[0] + (double)f.r[3 * k + 1] * f.u[1] +
             (double)f.r[3 * k + 2] * f.u[2];
-    s[k] = 2.0 * half;
+    s[k] = 2.0 * f.typ;
     for (int h = 0; h < 2; ++h) {
       const double mean = 0.5 * (bd[h][3 + k] + bd[h][9 + k]) - ru[k];
       const double sd = 0.125 * (bd[h][9 + k] - bd[h][3 + k]);
@@ -589,7 +636,9 @@ __global__ void __launch_bounds__(kTile) k_boxes(BoxArgs a) {
   TLBox b = empty_box();
   if (r < n) {
     const int64_t p = (int64_t)tile * kTile + t;
-    b = swept_box(a.rec[2 * p], a.rec[2 * p + 1], a.frames[q], a.Llo, a.Lhi, a.half);
+    const float4 pe = a.rec[2 * p];
+    b = swept_box(pe, a.rec[2 * p + 1], a.frames[q], a.Llo, a.Lhi,
+                  tl_photon_pad(a.frames[q], a.beam, pe.w, a.half));
     put_box(a.box + 2 * ((size_t)I.lev[0] + r), b);
   }
   b = warp_union(b);
@@ -796,7 +845,8 @@ __global__ void __launch_bounds__(32 * kColWarps, 8) k_collide(ColArgs a) {
   if (r0 + lane < qn) {
     const float4 *r = a.q + 2 * ((int64_t)g * 32 + lane);
     const float4 p = r[0], d = r[1];
-    own = swept_box(p, d, a.frames[inst], a.Llo, a.Lhi, a.half);
+    own = swept_box(p, d, a.frames[inst], a.Llo, a.Lhi,
+                    tl_photon_pad(a.frames[inst], a.swap, p.w, a.half));
     ws.qpos[lane] = p;
     ws.qdir[lane] = d;
   }

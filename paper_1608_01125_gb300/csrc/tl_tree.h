@@ -43,6 +43,7 @@ struct BoxArgs {
   const uint32_t *tile_inst;  // instance of each tile (batches, else NULL)
   const TLFrame *frames;
   float Llo, Lhi, half;
+  int beam;
   float4 *box;
   const unsigned *build_status;
 };
@@ -73,8 +74,11 @@ size_t moment_doubles();
 cudaError_t launch_beam_moments(const TLBeam &b, const TLFrame &f, double *out, cudaStream_t s);
 cudaError_t launch_inst_bounds(const TLBeam &b, const uint32_t *inst_of, const TLFrame *frames,
                                int n_inst, long long *tmp, double *out, cudaStream_t s);
-cudaError_t launch_inst_frames(const double *ba, const double *bb, int n_inst, TLFrame *out,
+cudaError_t launch_inst_energy(const TLBeam &b, const TLInst *inst, int n_inst, double *out,
                                cudaStream_t s);
+cudaError_t launch_inst_frames(const double *ba, const double *bb, const double *lea,
+                               const double *leb, const TLPadTable &pads, double half, int n_inst,
+                               TLFrame *out, cudaStream_t s);
 cudaError_t launch_inst_grid(const double *ba, const double *bb, const TLFrame *frames,
                              const TLInst *ia, const TLInst *ib, int n_inst, double T, double L,
                              double half, TLGrid *ga, TLGrid *gb, cudaStream_t s);
