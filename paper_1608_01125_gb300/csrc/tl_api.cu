@@ -104,6 +104,7 @@ static tl::ColArgs col_args(trilens_ctx *c, int p) {
   a.items = c->n_tiles[t] > 0 ? (g1 - g0) * a.slices : 0;
   a.fp64 = c->p.precision == TRILENS_FP64;
   a.swap = t == 0;
+  a.needles = c->needles;
   return a;
 }
 
@@ -596,6 +597,7 @@ static int ctx_create(trilens_ctx **out, const trilens_beam *a, const trilens_be
       return rc;
     }
     tl_set_pads(c->frame0, pad_table(), c->ext[0], c->ext[1], le[0], le[1], c->half);
+    tl_set_needles(c->frame0, c->ext[0], c->ext[1], c->L64, c->half);
     CK(cudaMemcpyAsync(c->frames, &c->frame0, sizeof(TLFrame), cudaMemcpyHostToDevice, c->stream));
   }
   CK(tl::sort_prepare());
@@ -662,13 +664,20 @@ static int join_builds(trilens_ctx *c, bool fork) {
   return TRILENS_OK;
 }
 
+// Photon pairs are told by their needles (tl_set_needles) in steps where more than this
+// many photons of the tree's beam have swept boxes that meet a photon's, at the beam's
+// density: 614 in the step of 2 x 4M photons that they take from 6.60 to 4.62 ms, 11 in the
+// run of 2 x 1M (10.1 and 10.4 ms), 0.8 in the step of 2 x 16M (3.70 and 3.99 ms).  Batches
+// keep the boxes (2 x 64 instances of up to 131072 photons 6.9 and 7.2 ms).
+constexpr double kNeedlePairs = 64.0;
+
 // The ordering grids of a single problem's beams for the step with travel T to the
 // swept boxes' centres: per axis of the frame the mean of the centres +- 5 standard
 // deviations, in closed form from the moments (centres outside are clamped to the edge
 // cells; the grid only shapes the tree), and cells in the proportions of the boxes'
 // extents: pad plus the travel of a typical photon of either beam.
 static void step_grids(trilens_ctx *c, double T, TLGrid g[2]) {
-  double ru[3], s[3];
+  double ru[3], s[3], near = 0.0;
   for (int k = 0; k < 3; ++k) {
     const TLFrame &f = c->frame0;
     ru[k] = (double)f.r[3 * k] * f.u[0] + (double)f.r[3 * k + 1] * f.u[1] +
@@ -683,6 +692,7 @@ static void step_grids(trilens_ctx *c, double T, TLGrid g[2]) {
   }
   for (int h = 0; h < 2; ++h) {
     double lo[3], range[3];
+    double vol = 15.75;  // (2 pi)^1.5: of a Gaussian beam's peak density
     for (int k = 0; k < 3; ++k) {
       const double *m = c->fmoments[h], n = (double)std::max<int64_t>(c->beam[h].n, 1);
       const double mean = (m[k] + T * m[3 + k]) / n;
@@ -690,10 +700,13 @@ static void step_grids(trilens_ctx *c, double T, TLGrid g[2]) {
       const double sd5 = 5.0 * sqrt(std::max(msq - mean * mean, 0.0));
       lo[k] = mean - 0.5 * c->L64 * ru[k] - sd5;
       range[k] = 2.0 * sd5;
+      vol *= 0.2 * sd5 / s[k];
     }
+    if (h == c->tree) near = (double)c->beam[h].n / vol;
     g[h] = tl_make_grid(lo, range, s, c->order_bits[h]);
     tl_beam_box(c->ext[1 - h], c->ext[1 - h][12], c->ext[1 - h][13], c->frame0, T - 0.5 * c->L64, c->L64, c->half, g[h].clo, g[h].chi);
   }
+  c->needles = c->frame0.axis >= 0 && near > kNeedlePairs;
 }
 
 // The exact path's order of both beams and the tree of the smaller one.
@@ -773,6 +786,7 @@ static int build_exact(trilens_ctx *c, int64_t step) {
     b.Lhi = c->L_hi;
     b.half = c->half;
     b.beam = k;
+    b.needles = c->needles;
     b.box = c->box;
     b.build_status = c->build_status;
     CK(tl::launch_boxes(b, c->n_tiles[k], c->n_inst, c->max_top, st));

@@ -39,6 +39,7 @@ struct trilens_ctx {
   // exact path: one frame per instance; the photons of both beams in tiles; a tree over
   // the smaller beam
   TLFrame frame0{};
+  bool needles = false;  // the built step's photon pairs are told by their needles
   TLFrame *frames = nullptr;
   int tree = 1;                  // the beam with the tree
   TLInst *insts[2]{};            // device, per instance

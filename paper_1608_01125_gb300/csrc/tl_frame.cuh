@@ -22,7 +22,11 @@ struct TLFrame {
   // half-width across its path of a photon's box of beam k: amp[k] E^xp (tl_photon_pad);
   // typ: that of a typical photon
   float amp[2], xp, typ;
-  int pad[3];
+  // photon pairs compared at the time they pass each other (tl_set_needles): closing axis
+  // (-1: none), 1 / closing velocity, half the step, window, and the pads' terms
+  int axis;
+  float inv, hl, lt, gain, add, ep, ec;
+  int fill[3];
 };
 
 // Ordering grid of one instance and step: cell = (x' - lo) scale, nb bits per axis,
@@ -158,6 +162,7 @@ __host__ __device__ inline void tl_set_pads(TLFrame &f, const TLPadTable &t, con
     }
   }
   f.xp = -0.08f * (float)best;
+  f.axis = -1;
   for (int k = 0; k < 2; ++k) {
     const double lam = exp(0.5 * (k ? la[0] - lb[0] : lb[0] - la[0]));
     f.amp[k] = best ? (float)(half * (double)t.a[best] * (1.0 + 1e-5) *
@@ -165,6 +170,64 @@ __host__ __device__ inline void tl_set_pads(TLFrame &f, const TLPadTable &t, con
                     : (float)half;
   }
   f.typ = (float)(best ? half * (double)t.a[best] * exp(-0.04 * best * log(st)) : half);
+}
+
+// Needles.  Where the beams close along one axis of the frame with nearly one velocity vc,
+// a pair that collides does so close to the time lambda0 = -dZ0 / vc (in units of length, 0
+// to L in the step) at which it would pass with exactly that velocity: the closest approach
+// within hs, the sum of the pads, has |dZ| <= hs, so with vlo the least closing velocity and
+// delta the largest |dV / vc - 1| it lies within Terr = (hs / vlo) (1 + delta) + L delta of
+// lambda0, and across the axis |dX(lambda0)| <= hs + DV Terr, DV the largest difference of
+// velocities there.  So a pair can be told by u = lambda0 - L / 2 in the window
+// |u| <= L / 2 + Terr, and |dXm + dVx u| <= hs (1 + DV (1 + delta) / vlo) + DV L delta,
+// Xm the middle of the photon's path: a square of the pads' size, where swept boxes also
+// hold all of both photons' travel (1 % of the pairs that they leave is left of a step of
+// 2 x 4M photons).  u is the sum of -Z / vc - L / 2 of beam A's photon and Z / vc of beam
+// B's.  FP32: a coordinate is off by 6u of the sum of the lengths turned (u = 2^-24), in u
+// by that over vc; ep and ec take 16u and more of each (tl_needle).
+// Beams without such an axis (delta > 0.1) keep the boxes, and so do those whose photons
+// travel less than kNeedleTravel pads across it in a step (the spread of directions taken as
+// an eighth of their range): there the two tests leave the same pairs.
+constexpr double kNeedleTravel = 3.0;
+
+inline void tl_set_needles(TLFrame &f, const double *ea, const double *eb,
+                                               double L, double half) {
+  f.axis = -1;
+  double best = 0.0;
+  int m = -1;
+  for (int k = 0; k < 3; ++k) {
+    const double c = fabs(ea[3 + k] + ea[9 + k] - eb[3 + k] - eb[9 + k]);
+    if (c > best) {
+      best = c;
+      m = k;
+    }
+  }
+  if (m < 0) return;
+  // closing velocities of a pair, 1e-6 for the rounding of the extremes and of the frame
+  const double v0 = ea[3 + m] - eb[9 + m] - 2e-6, v1 = ea[9 + m] - eb[3 + m] + 2e-6;
+  const double vc = 0.5 * (v0 + v1), vlo = fmin(fabs(v0), fabs(v1));
+  if (!(v0 * v1 > 0.0) || !(vlo > 0.05)) return;
+  const double delta = 0.5 * (v1 - v0) / fabs(vc) + 1e-6;
+  if (!(delta < 0.1)) return;
+  double DV = 0.0, sd = 0.0;
+  for (int k = 0; k < 3; ++k)
+    if (k != m) {
+      const double ra = 0.125 * (ea[9 + k] - ea[3 + k]), rb = 0.125 * (eb[9 + k] - eb[3 + k]);
+      DV = fmax(DV, fmax(fabs(ea[9 + k] - eb[3 + k]), fabs(ea[3 + k] - eb[9 + k])));
+      sd = fmax(sd, ra * ra + rb * rb);
+    }
+  if (!(L * sqrt(sd) > kNeedleTravel * 2.0 * (double)f.typ)) return;
+  DV += 2e-6;
+  if (!(DV < 4.0)) return;
+  const double up = 1.0 + 1e-5;
+  f.axis = m;
+  f.inv = (float)(1.0 / vc);
+  f.hl = (float)(0.5 * L);
+  f.lt = (float)((0.5 * L + 4.0 * half / vlo * (1.0 + delta) + L * delta) * up);
+  f.gain = (float)((1.0 + DV * (1.0 + delta) / vlo) * up);
+  f.add = (float)(0.5 * DV * L * delta * up);
+  f.ep = (float)(0x1p-20 * (1.0 + fabs(1.0 / vc)) * (1.0 + DV) * up);
+  f.ec = (float)(0x1p-18 * (L + (double)f.lt) * (1.0 + DV) * up);
 }
 
 // The grid of `bits` bits in all over [lo, lo + range]: each bit halves the cells of
@@ -248,6 +311,36 @@ __device__ __forceinline__ void seg_axis(float p, float dc, float Llo, float Lhi
 __device__ __forceinline__ float tl_photon_pad(const TLFrame &f, int beam, float E, float half) {
   if (f.xp == 0.0f) return half;
   return fminf(2.0f * half, fmaf(f.amp[beam], exp2f(f.xp * log2f(E)), 1e-9f));
+}
+
+// A photon as a needle: middle of its path across the closing axis, time, velocities across,
+// pad, and the rounding of its time.
+struct TLNeedle {
+  float x, y, w, vx, vy, h, e;
+};
+
+__device__ __forceinline__ TLNeedle tl_needle(const TLFrame &f, int beam, const float4 p,
+                                              const float4 d, float pad) {
+  float X[3] = {p.x, p.y, p.z}, V[3] = {d.x, d.y, d.z};
+  if (!f.ident) {
+    const float vx = d.x - f.u[0], vy = d.y - f.u[1], vz = d.z - f.u[2];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      X[k] = fmaf(f.r[3 * k], p.x, fmaf(f.r[3 * k + 1], p.y, f.r[3 * k + 2] * p.z));
+      V[k] = fmaf(f.r[3 * k], vx, fmaf(f.r[3 * k + 1], vy, f.r[3 * k + 2] * vz));
+    }
+  }
+  const int m = f.axis;
+  const float z = m == 0 ? X[0] : (m == 1 ? X[1] : X[2]);
+  TLNeedle n;
+  n.vx = m == 0 ? V[1] : V[0];
+  n.vy = m == 2 ? V[1] : V[2];
+  n.x = fmaf(n.vx, f.hl, m == 0 ? X[1] : X[0]);
+  n.y = fmaf(n.vy, f.hl, m == 2 ? X[1] : X[2]);
+  n.w = beam ? z * f.inv : fmaf(-z, f.inv, -f.hl);
+  n.e = fmaf(f.ep, fabsf(p.x) + fabsf(p.y) + fabsf(p.z), f.ec);
+  n.h = (fmaf(f.gain, pad, f.add) + n.e) * (1.0f + 0x1p-20f);
+  return n;
 }
 
 // A photon's swept box in the frame.  Each coordinate of R P from the rounded inputs

@@ -621,9 +621,25 @@ __device__ __forceinline__ TLBox get_box(const float4 *src) {
   return TLBox{a.x, a.y, a.z, a.w, c.x, c.y};
 }
 
-// One block per tile: every photon's swept box, the boxes of the tile's 32 runs of 32
+// a needle, likewise
+__device__ __forceinline__ void put_needle(float4 *dst, const TLNeedle &n) {
+  dst[0] = make_float4(n.x, n.y, n.w, n.vx);
+  dst[1] = make_float4(n.vy, n.h, n.e, 0.0f);
+}
+__device__ __forceinline__ TLNeedle get_needle(const float4 *src) {
+  const float4 a = src[0], b = src[1];
+  return TLNeedle{a.x, a.y, a.z, a.w, b.x, b.y, b.z};
+}
+// never met: no time is within its window
+__device__ __forceinline__ TLNeedle no_needle() {
+  return TLNeedle{0.0f, 0.0f, __int_as_float(0x7f800000), 0.0f, 0.0f, 0.0f, 0.0f};
+}
+
+// One block per tile: every photon's swept box (its needle where the frame has a closing
+// axis: the box then only goes into the unions), the boxes of the tile's 32 runs of 32
 // photons (level 1) and the tile's own (level 2).  One pass over the sorted photons;
 // unions by shuffles, no links and no second pass.
+template <bool NEEDLES>
 __global__ void __launch_bounds__(kTile) k_boxes(BoxArgs a) {
   __shared__ TLBox wb[32];
   if (*a.build_status & TL_ST_TIMEOUT) return;  // keys unsorted: the build is abandoned
@@ -637,9 +653,13 @@ __global__ void __launch_bounds__(kTile) k_boxes(BoxArgs a) {
   if (r < n) {
     const int64_t p = (int64_t)tile * kTile + t;
     const float4 pe = a.rec[2 * p];
-    b = swept_box(pe, a.rec[2 * p + 1], a.frames[q], a.Llo, a.Lhi,
-                  tl_photon_pad(a.frames[q], a.beam, pe.w, a.half));
-    put_box(a.box + 2 * ((size_t)I.lev[0] + r), b);
+    const float4 de = a.rec[2 * p + 1];
+    const TLFrame &f = a.frames[q];
+    const float pad = tl_photon_pad(f, a.beam, pe.w, a.half);
+    b = swept_box(pe, de, f, a.Llo, a.Lhi, pad);
+    float4 *dst = a.box + 2 * ((size_t)I.lev[0] + r);
+    if (!NEEDLES) put_box(dst, b);
+    else put_needle(dst, tl_needle(f, a.beam, pe, de, pad));
   }
   b = warp_union(b);
   if (lane == 0) {
@@ -673,7 +693,8 @@ __global__ void __launch_bounds__(1024) k_upper(const TLInst *inst, const uint32
 
 cudaError_t launch_boxes(const BoxArgs &a, int tiles, int n_inst, int max_top, cudaStream_t s) {
   if (tiles <= 0) return cudaSuccess;
-  k_boxes<<<tiles, kTile, 0, s>>>(a);
+  if (a.needles) k_boxes<true><<<tiles, kTile, 0, s>>>(a);
+  else k_boxes<false><<<tiles, kTile, 0, s>>>(a);
   if (max_top >= 3) k_upper<<<n_inst, 1024, 0, s>>>(a.inst, a.start, a.box);
   return cudaGetLastError();
 }
@@ -742,6 +763,7 @@ struct Pairs {
   // every lane's pairs: bit r of bits stands for box r of the cnt last tested, this lane
   // for its photon (by_tree) or for photon j0 + lane of the tree
   __device__ __forceinline__ void add(uint32_t bits, bool by_tree, uint32_t j0) {
+    if (!__any_sync(0xffffffffu, bits != 0u)) return;
     int inc = __popc(bits);
     const int own = inc;
 #pragma unroll
@@ -750,7 +772,6 @@ struct Pairs {
       if (lane >= off) inc += t;
     }
     const int total = __shfl_sync(0xffffffffu, inc, 31);
-    if (total == 0) return;
     // what does not fit the list at once (dense leaves) goes in rounds of one per lane
     if (np + total <= kPend) {
       int at = np + inc - own;
@@ -803,6 +824,29 @@ __device__ __forceinline__ uint32_t test_boxes(ColSmem &ws, const TLBox &src, un
   return bits;
 }
 
+// The same for needles, with the window lt: ~14 instructions for 32 pairs.
+__device__ __forceinline__ uint32_t test_needles(ColSmem &ws, const TLNeedle &src, unsigned sel,
+                                                 const TLNeedle &cmp, float lt, int lane) {
+  __syncwarp();
+  if (sel >> lane & 1u) {
+    const int r = __popc(sel & ((1u << lane) - 1u));
+    put_needle(ws.cbox + 2 * r, src);
+    ws.id[r] = (uint8_t)lane;
+  }
+  __syncwarp();
+  const int cnt = __popc(sel);
+  uint32_t bits = 0u;
+#pragma unroll 4
+  for (int r = 0; r < cnt; ++r) {
+    const float4 c = ws.cbox[2 * r];
+    const float2 g = *reinterpret_cast<const float2 *>(ws.cbox + 2 * r + 1);
+    const float u = c.z + cmp.w;
+    const float x = fmaf(c.w - cmp.vx, u, c.x - cmp.x), y = fmaf(g.x - cmp.vy, u, c.y - cmp.y);
+    if (fabsf(u) <= lt && fmaxf(fabsf(x), fabsf(y)) <= g.y + cmp.h) bits |= 1u << r;
+  }
+  return bits;
+}
+
 // One warp: 32 consecutive photons of the query beam, one per lane, against the tree.
 // A node's 32 children are tested by 32 lanes at once against the union of the warp's
 // boxes; those that overlap it are tested by every lane against its own box, and
@@ -814,9 +858,10 @@ __device__ __forceinline__ uint32_t test_boxes(ColSmem &ws, const TLBox &src, un
 // and lane-private 64-byte records).  Few groups (small beams): the tree is cut into
 // `slices` contiguous parts of its sorted photons, one warp each per group.
 // Measured (with the first look, which was k_narrow's): 2 x 4M statistical step 15.0 ms
-// for the dual descent and its narrow phase, 6.1 ms now; 2 x 16M at 90 degrees
+// for the dual descent and its narrow phase, 6.1 ms by boxes (half of it the first look at
+// pairs whose boxes meet at different times), 3.8 ms by needles; 2 x 16M at 90 degrees
 // 7.3 ms, 1.1 ms now (there the turned frame is most of it).
-template <bool FP64>
+template <bool FP64, bool NEEDLES>
 __global__ void __launch_bounds__(32 * kColWarps, 8) k_collide(ColArgs a) {
   __shared__ ColSmem wsm[kColWarps];
   __shared__ float suf[TL_SBINS];
@@ -841,16 +886,30 @@ __global__ void __launch_bounds__(32 * kColWarps, 8) k_collide(ColArgs a) {
   ColSmem &ws = wsm[warp];
   Pairs<FP64> out{a, ws, suf, (uint32_t)g * 32u, (uint32_t)T.tile0 * (uint32_t)kTile, lane, 0, 0,
                   a.ctr->leaf_base};
+  const TLFrame &f = a.frames[inst];
   TLBox own = empty_box();
+  TLNeedle ndl = no_needle();
   if (r0 + lane < qn) {
     const float4 *r = a.q + 2 * ((int64_t)g * 32 + lane);
     const float4 p = r[0], d = r[1];
-    own = swept_box(p, d, a.frames[inst], a.Llo, a.Lhi,
-                    tl_photon_pad(a.frames[inst], a.swap, p.w, a.half));
+    const float pad = tl_photon_pad(f, a.swap, p.w, a.half);
+    own = swept_box(p, d, f, a.Llo, a.Lhi, pad);
+    if (NEEDLES) ndl = tl_needle(f, a.swap, p, d, pad);
     ws.qpos[lane] = p;
     ws.qdir[lane] = d;
   }
   const TLBox all = warp_union(own);
+  // where and when the warp's needles are: x, y and w of the whole window
+  float lt = 0.0f;
+  TLBox span = empty_box();
+  if (NEEDLES) {
+    lt = f.lt + __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(ndl.e)));
+    if (r0 + lane < qn) {
+      const float ax = fmaf(fabsf(ndl.vx), lt, ndl.h), ay = fmaf(fabsf(ndl.vy), lt, ndl.h);
+      span = TLBox{ndl.x - ax, ndl.y - ay, ndl.w, ndl.x + ax, ndl.y + ay, ndl.w};
+    }
+    span = warp_union(span);
+  }
   unsigned long long node_tests = 0, narrow = 0;
   unsigned leaves = 0;
   const int top = tl_top_level(tn);
@@ -882,10 +941,29 @@ __global__ void __launch_bounds__(32 * kColWarps, 8) k_collide(ColArgs a) {
         mask &= mask - 1u;
         const int j0 = (base + k) * 32;
         const bool ok = j0 + lane < tn;
-        const TLBox b = ok ? get_box(a.box + 2 * ((size_t)T.lev[0] + j0 + lane)) : empty_box();
-        const unsigned mb = __ballot_sync(0xffffffffu, tl_overlap(b, all));
+        const float4 *src = a.box + 2 * ((size_t)T.lev[0] + j0 + lane);
         const unsigned mq =
             __ballot_sync(0xffffffffu, hits >> __popc(near & ((1u << k) - 1u)) & 1u);
+        if (NEEDLES) {
+          const TLNeedle b = ok ? get_needle(src) : no_needle();
+          const float l = lt + __uint_as_float(
+                                   __reduce_max_sync(0xffffffffu, __float_as_uint(b.e)));
+          const float ax = fmaf(fabsf(b.vx), l, b.h), ay = fmaf(fabsf(b.vy), l, b.h);
+          const unsigned mb = __ballot_sync(
+              0xffffffffu, b.x + ax >= span.lx && b.x - ax <= span.hx && b.y + ay >= span.ly &&
+                               b.y - ay <= span.hy && b.w + span.hz >= -l && b.w + span.lz <= l);
+          ++leaves;
+          const int nb = __popc(mb), nq = __popc(mq);
+          narrow += (unsigned)(nb * nq);
+          if (nb == 0) continue;
+          const bool by_tree = nb <= nq;
+          out.add(by_tree ? test_needles(ws, b, mb, ndl, l, lane)
+                          : test_needles(ws, ndl, mq, b, l, lane),
+                  by_tree, (uint32_t)j0);
+          continue;
+        }
+        const TLBox b = ok ? get_box(src) : empty_box();
+        const unsigned mb = __ballot_sync(0xffffffffu, tl_overlap(b, all));
         ++leaves;
         const int nb = __popc(mb), nq = __popc(mq);
         narrow += (unsigned)(nb * nq);
@@ -923,8 +1001,9 @@ __global__ void __launch_bounds__(32 * kColWarps, 8) k_collide(ColArgs a) {
 cudaError_t launch_collide(const ColArgs &a, cudaStream_t s) {
   if (a.items <= 0) return cudaSuccess;
   const unsigned blocks = (unsigned)((a.items + kColWarps - 1) / kColWarps);
-  if (a.fp64) k_collide<true><<<blocks, 32 * kColWarps, 0, s>>>(a);
-  else k_collide<false><<<blocks, 32 * kColWarps, 0, s>>>(a);
+  auto *const k = a.needles ? (a.fp64 ? k_collide<true, true> : k_collide<false, true>)
+                            : (a.fp64 ? k_collide<true, false> : k_collide<false, false>);
+  k<<<blocks, 32 * kColWarps, 0, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -43,7 +43,7 @@ struct BoxArgs {
   const uint32_t *tile_inst;  // instance of each tile (batches, else NULL)
   const TLFrame *frames;
   float Llo, Lhi, half;
-  int beam;
+  int beam, needles;
   float4 *box;
   const unsigned *build_status;
 };
@@ -65,6 +65,7 @@ struct ColArgs {
   int group0;       // first group of this part
   int slices;       // parts of the tree per group
   int fp64, swap;   // swap: the tree is beam A's
+  int needles;      // the tree's level 0 holds needles
 };
 
 int mean_doubles();  // per-block sums of launch_mean_dir
