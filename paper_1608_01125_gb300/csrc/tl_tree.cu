@@ -550,10 +550,9 @@ cudaError_t launch_cell_scan(uint32_t *count, uint32_t *start, int64_t cells, ui
 // one full 32-byte sector written per photon; beside that it keeps GB300's FP64 pipe
 // busy (six operations and three conversions per photon at 2 per clock and SM).
 __global__ void __launch_bounds__(256) k_place(PlaceArgs a) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.b.n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const uint2 c = a.cell[i];
-    if (c.x == TL_NONE) continue;
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const uint2 c = i < a.b.n ? a.cell[i] : make_uint2(TL_NONE, 0u);
+  if (c.x != TL_NONE) {
     int64_t to = (int64_t)__ldg(a.start + c.x) + c.y;
     const float4 s0 = a.stat[2 * i], d = a.stat[2 * i + 1];
     const double dx = a.b.dx[i], dy = a.b.dy[i], dz = a.b.dz[i];
@@ -575,7 +574,9 @@ __global__ void __launch_bounds__(256) k_place(PlaceArgs a) {
 cudaError_t launch_place(const PlaceArgs &a, cudaStream_t s) {
   if (a.b.n <= 0) return cudaSuccess;
   const int64_t nb = (a.b.n + 255) / 256;
-  k_place<<<(int)(nb < 8 * 152 ? nb : 8 * 152), 256, 0, s>>>(a);
+  // a block per 256 photons: a fixed grid of 8 per SM leaves SMs idle at its end (both
+  // beams of 16M photons at 90 degrees: 3.69 ms a step with it, 3.45 without)
+  k_place<<<(unsigned)nb, 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 
