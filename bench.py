@@ -1,13 +1,14 @@
 """Benchmark: exact Breit-Wheeler collision detection, 2 x 1,048,576 photons.
 
 One benchmark step = one full run of the head-on workload: 64 time steps of
-5 fs, each a hierarchy build of both beams plus the collision step (dual
-traversal, FP32 narrow phase, FP64 band re-test, yield), inputs resident in
-HBM.  The metric is the narrow-phase photon-pair tests per second: photon
-pairs that reach the exact closest-approach test (the work the method
-does after the hierarchy has pruned).  Collided pairs/s and the all-pairs
-equivalent N_A * N_B * time steps per second are reported beside it as
-context.
+5 fs, each the order of both beams and the tree of one plus the collision step
+(descent by groups of 32 photons, pair tests, FP64 band re-test, yield), inputs
+resident in HBM.  The metric is the narrow-phase photon-pair tests per second:
+photon pairs that the tree leaves to be told pair by pair, by the pair's own swept
+boxes or passing point first and by the closest-approach test where that leaves
+them (the work the method does after the hierarchy has pruned).  Collided pairs/s
+and the all-pairs equivalent N_A * N_B * time steps per second are reported beside
+it as context, and the time of a run, which fewer tests shorten.
 
   python bench.py [--gpus N --steps K --warmup W] [--impl reference]
 
@@ -44,34 +45,21 @@ SINGLE_THREAD_STEPS = (4, 36)
 FALLBACK_HBM_GBS = 6800.0
 PHASES = ("propagate", "sort", "gather", "emit", "refit", "expand", "traverse", "narrow", "band",
           "yield")
-# FP32 operations of the narrow test's prefix (threshold and quick miss), which
-# decides most photon pairs: the invariant s and its bound (13), the relative
-# position and direction and their products (15), the reciprocal and the
-# closest approach (8), the position sum and the quick-miss comparisons (11)
-NARROW_OPS_PER_TEST = 47
+# operations of the pair test that every counted pair gets: six comparisons of two
+# boxes, their conjunction and the bit kept (a needle's test takes 14); the tests of
+# groups and nodes, the lists and the closest-approach test of what is left come on top
+PAIR_OPS_PER_TEST = 10
 # GB300 FP32 lanes: 152 SMs x 128 per SM at the 2070 MHz maximum SM clock
 FP32_OPS_PEAK = 152 * 128 * 2.07e9
 
 
-def algorithmic_bytes(phase: str, na: int, nb: int, key_bits: tuple, hits: float, band: float):
-    """Bytes one launch of a phase must move at least (per beam launches use
-    that beam's size; traversal and later phases cover both beams)."""
-    n = na + nb
-    if phase == "propagate":   # p0, d (6 doubles) and the FP32 direction in; x, y, z + key + index out
-        return 48 + 16 + 12 + 12, "photon"
-    if phase == "sort":        # per pass: key + index read and written
-        return 24, "photon-pass"
-    if phase == "gather":      # index, random float4 x2 read, float4 x2 written
-        return 4 + 32 + 32, "photon"
-    if phase == "emit":        # keys read, child refs + counts + parent written
-        return 8 + 16 + 4, "photon"
-    if phase == "refit":       # sorted SoA, parent links and ranges read; two child boxes per node
-        return 32 + 8 + 4 + 4 + 48, "photon"
-    if phase == "traverse":    # node records of both trees once + the leaf pairs written
-        return 64, "photon"
-    if phase == "narrow":      # sorted photon records once + the leaf pairs read + output pairs
-        return 32, "photon"
-    return 8, "pair"
+def algorithmic_bytes(phase: str) -> int:
+    """Bytes per photon that a phase of one beam must move at least."""
+    if phase == "propagate":   # order: FP32 record in, cell and rank out, one count
+        return 32 + 8 + 4
+    if phase == "sort":        # two cells a photon scanned (count in and cleared, sum out);
+        return 24 + 8 + 4 + 32 + 48 + 32  # cell, sum, record, p0 and d in, sorted record out
+    return 32 + 32             # refit (boxes): sorted record in, box out
 
 
 def read_peaks():
@@ -204,11 +192,11 @@ def cpu_baseline(wl, a, b, first=0, nsteps=None):
                                         f"{tests1} narrow-phase tests"}}
 
 
-# FP64 operations per hit of the pair products, counted from the kernel: 26
-# for the photons' sums, the invariant mass and the CoM momentum, ~16 for the
-# direction (1.27 Marsaglia tries of 2 draws), 4 divisions, 2 x 16 for the two
-# boosts; 3 square roots; divisions and square roots counted as one each
-PAIR_FP64_OPS = 26 + 16 + 4 + 32 + 3
+# FP64 operations per hit of the pair products, counted from the kernel: 19 for the
+# photons' sums, the invariant mass and the CoM momentum, 12 for the direction (its
+# rejections are told in FP32), 3 for q, 21 for both boosts; 5 divisions and 3 square
+# roots counted as one each
+PAIR_FP64_OPS = 19 + 12 + 3 + 21 + 8
 FP64_NOMINAL_TFLOPS = 1.25  # GB300 dense FP64, nominal (no measured figure here)
 
 
@@ -455,20 +443,16 @@ def crossing_timing(dev, stream, peak, peak_src, steps=(120, 129, 141, 160)):
                      "leaf_pairs": st["leaf_pairs"]})
     col.timing(False)
     col.close()
-    n_ab = wl.a.n + wl.b.n
     tt = sum(r["traverse"] for r in rows)
-    tbytes = sum(64.0 * n_ab + 8.0 * r["leaf_pairs"] for r in rows)
-    ach = tbytes / (tt / 1e3) / 1e9
+    ach = PAIR_OPS_PER_TEST * sum(r["narrow_tests"] for r in rows) / (tt / 1e3)
     tot = sum(sum(r[p] for p in PHASES) for r in rows)
     return {"workload": wl.name, "photons_per_beam": wl.a.n, "time_steps_timed": list(steps),
             "tuning": tuned, "ms_per_step": tot / len(rows), "per_step": rows,
             "narrow_tests_per_s": sum(r["narrow_tests"] for r in rows) / (tot / 1e3),
             "collided_pairs_per_s": sum(r["hits"] for r in rows) / (tot / 1e3),
-            "traverse_roofline": {"bound": "hbm", "achieved": ach, "peak": peak,
-                                  "peak_source": peak_src, "unit": "GB/s", "frac": ach / peak,
-                                  "algorithmic_bytes": tbytes, "ms": tt,
-                                  "unit_of_work": "node records of both trees once, leaf pairs "
-                                                  "written, per step"}}
+            "traverse_roofline": {"bound": "alu", "achieved": ach, "peak": FP32_OPS_PEAK,
+                                  "unit": "op/s", "frac": ach / FP32_OPS_PEAK, "ms": tt,
+                                  "ops_per_test": PAIR_OPS_PER_TEST}}
 
 
 def run_reference(args, wl):
@@ -681,75 +665,51 @@ def run_ours(args, wl):
             dist.destroy_process_group()
         return
     peak, peak_src = read_peaks()
-    # rooflines of the traversal (HBM: its algorithmic bytes per step), the
-    # narrow phase (FP32 ALU: the test prefix's operations) and the dominant
-    # build phase, each from the per-phase device times of the step-by-step
-    # runs; the dominant one by time is the line's roofline
-    n_ab = wl.a.n + wl.b.n
-    leaves = sum(r["leaves"] for r in per_step)  # one run
-    steps_total = K * nsteps
-    builds = 2 * steps_total  # one build per beam and step
+    # rooflines from the per-phase device times of the step-by-step runs: the descent
+    # with its pair tests (issue of the pair tests' operations) and the build's phases
+    # (HBM); the dominant one by time is the line's roofline
+    n_half = (wl.a.n + wl.b.n) / 2
+    trav_steps = max(launches["propagate"] // 2, 1)  # steps whose beams can meet, all runs
 
-    def hbm(phase, algo, launch_ms, note):
-        ach = algo / (launch_ms / 1e3) / 1e9
+    def hbm(phase, per_photon, ms_per_beam, note):
+        algo = per_photon * n_half
+        ach = algo / (ms_per_beam / 1e3) / 1e9
         return {"kernel": phase, "bound": "hbm", "achieved": ach, "peak": peak,
                 "peak_source": peak_src, "unit": "GB/s", "frac": ach / peak, "traffic": None,
-                "algorithmic_bytes_per_launch": algo, "launch_ms": launch_ms, "unit_of_work": note}
+                "algorithmic_bytes_per_launch": algo, "launch_ms": ms_per_beam,
+                "unit_of_work": note}
 
-    roofs = {}
-    roofs["traverse"] = hbm("traverse", 64.0 * n_ab + 8.0 * leaves / nsteps,
-                            phase_ms["traverse"] / steps_total,
-                            "one step: node records of both trees once, leaf pairs written")
-    ops = NARROW_OPS_PER_TEST * tests / K / nsteps
-    nms = phase_ms["narrow"] / steps_total
-    roofs["narrow"] = {"kernel": "narrow", "bound": "alu", "unit": "FP32 op/s",
-                       "achieved": ops / (nms / 1e3), "peak": FP32_OPS_PEAK,
-                       "peak_source": "derived: 152 SMs x 128 FP32 lanes x 2.07 GHz",
-                       "frac": ops / (nms / 1e3) / FP32_OPS_PEAK, "launch_ms": nms,
-                       "ops_per_test": NARROW_OPS_PER_TEST, "traffic": None}
-    for ph in ("sort", "refit", "emit", "propagate"):
-        per_unit, _ = algorithmic_bytes(ph, wl.a.n, wl.b.n, None, 0, 0)
-        if ph == "sort":  # the unit is one digit pass over one beam
-            passes = max(launches[ph] - builds, 1)  # minus one scan per build
-            roofs[ph] = hbm(ph, per_unit * n_ab / 2, phase_ms[ph] / passes, "one pass, one beam")
-        else:
-            roofs[ph] = hbm(ph, per_unit * n_ab / 2, phase_ms[ph] / builds, "one beam's build")
+    def alu(n_tests, t_ms):
+        ach = PAIR_OPS_PER_TEST * n_tests / (t_ms / 1e3)
+        return {"achieved": ach, "frac": ach / FP32_OPS_PEAK}
+
+    roofs = {"traverse": {"kernel": "traverse", "bound": "alu", "unit": "op/s",
+                          "peak": FP32_OPS_PEAK,
+                          "peak_source": "derived: 152 SMs x 128 lanes x 2.07 GHz",
+                          "launch_ms": phase_ms["traverse"] / trav_steps,
+                          "ops_per_test": PAIR_OPS_PER_TEST, "traffic": None,
+                          **alu(tests, phase_ms["traverse"])}}
+    for ph, beams, note in (("propagate", 2, "order of one beam: cells and ranks"),
+                            ("sort", 2, "one beam: running sum of the cells, photons placed"),
+                            ("refit", 1, "boxes of the tree's beam")):
+        roofs[ph] = hbm(ph, algorithmic_bytes(ph), phase_ms[ph] / (beams * trav_steps), note)
     dom = max(roofs, key=lambda p: phase_ms[p])
     # busy steps: those with at least 5% of the peak step's narrow-phase tests
     peak_tests = max(r["tests"] for r in per_step) if per_step else 0
     busy = [r for r in per_step if peak_tests and r["tests"] >= 0.05 * peak_tests]
     tb = sum(r["traverse"] for r in busy)
-    tn = sum(r["narrow"] for r in busy)
-    busy_bytes = sum(64.0 * n_ab + 8.0 * r["leaves"] for r in busy)
-    busy_ops = NARROW_OPS_PER_TEST * sum(r["tests"] for r in busy)
-    roofs["traverse"]["busy_steps"] = {
-        "steps": [r["step"] for r in busy], "ms": tb, "algorithmic_bytes": busy_bytes,
-        "achieved": busy_bytes / (tb / 1e3) / 1e9 if tb > 0 else None,
-        "frac": busy_bytes / (tb / 1e3) / 1e9 / peak if tb > 0 else None,
-        "per_step_ms": [round(r["traverse"], 4) for r in busy]}
-    roofs["narrow"]["busy_steps"] = {
-        "steps": [r["step"] for r in busy], "ms": tn,
-        "achieved": busy_ops / (tn / 1e3) if tn > 0 else None,
-        "frac": busy_ops / (tn / 1e3) / FP32_OPS_PEAK if tn > 0 else None,
-        "per_step_ms": [round(r["narrow"], 4) for r in busy],
-        "narrow_tests": [r["tests"] for r in busy]}
-    # DRAM traffic from profiles/traffic.txt: the traversal's on busy steps (with
-    # the capture's own algorithmic bytes: the leaf-pair count depends on the
-    # knobs), the build kernels' per launch like their rooflines
-    tr = read_traffic("traverse")
-    if tr is not None:
-        dram, algo = float(tr["bytes_per_launch"]), float(tr["algorithmic_bytes_per_launch"])
-        roofs["traverse"]["busy_steps"]["traffic"] = {
-            "steps": tr["steps"], "knobs": tr["knobs"], "dram_bytes_per_launch": dram,
-            "algorithmic_bytes_per_launch": algo, "dram_over_algorithmic": dram / algo}
+    if tb > 0:
+        roofs["traverse"]["busy_steps"] = {
+            "steps": [r["step"] for r in busy], "ms": tb,
+            **alu(sum(r["tests"] for r in busy), tb),
+            "per_step_ms": [round(r["traverse"], 4) for r in busy],
+            "narrow_tests": [r["tests"] for r in busy]}
     roofline = dict(roofs[dom])
-    td = read_traffic(dom) if dom != "traverse" else None
+    td = read_traffic(dom)
     roofline["traffic"] = float(td["bytes_per_launch"]) if td is not None else None
     roofline["traffic_note"] = (
-        "DRAM bytes were captured on busy steps only (rooflines.traverse.busy_steps.traffic)"
-        if dom == "traverse" else
-        ("dram__bytes_read.sum + dram__bytes_write.sum per launch, profiles/traffic.txt"
-         if td is not None else "not captured for this kernel"))
+        "dram__bytes_read.sum + dram__bytes_write.sum per launch, profiles/traffic.txt"
+        if td is not None else "not captured for this kernel")
     cpu = (cpu_baseline(wl, a_np, b_np, first, nsteps)
            if (world == 1 and not args.no_cpu_baseline) else None)
     line = {
@@ -770,9 +730,11 @@ def run_ours(args, wl):
         "stepwise_ms_per_run": statistics.mean(sw_ms),
         "roofline": roofline,
         "rooflines": roofs,
-        "roofline_note": "per-launch averages over every launch of the run (most time steps "
-                         "are almost empty: the bunches cross in the first ~10); busy_steps "
-                         "gives the steps where they cross",
+        "roofline_note": "per-launch averages over every launch of the run (the bunches cross "
+                         "in the first ~10 steps, and steps whose beams are apart launch "
+                         "nothing); busy_steps gives the steps where they cross",
+        "narrow_tests_note": "pairs the tree leaves to be told pair by pair: by their own swept "
+                             "boxes first, by the closest-approach test where those meet",
         "pair_products": pairs,
         "depletion": depl,
         "ip_regime": ipr,
@@ -781,8 +743,10 @@ def run_ours(args, wl):
         "cpu_baseline": cpu,
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d,
                 "d2h_bytes_per_step": 16},
-        # the graph holds the step-by-step path's kernels plus one status kernel per step
-        "gpu_launches": int(sum(launches.values())) + K * nsteps,
+        # the graph holds the build's kernels and six more (start, descent, decision, band,
+        # yield, totals) per step whose beams can meet
+        "gpu_launches": int(sum(launches[p] for p in ("propagate", "sort", "refit")))
+                        + 6 * trav_steps,
         "tuning": tuned,
         "clocks": clk.summary(),
     }
