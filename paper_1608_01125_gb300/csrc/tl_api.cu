@@ -363,15 +363,16 @@ int ensure_full(trilens_ctx *c) {
   return TRILENS_OK;
 }
 
-// bits of the cells that order n photons: 2 to 4 cells per photon spread evenly, so up
-// to a leaf's worth of photons per cell where a Gaussian bunch is densest (ten times the
-// cells per photon cost more to scan than the finer order saves), and at most 2^23, whose
-// counts (32 MB a beam) stay in L2 for the atomics: both beams of 16M photons at 90 degrees
-// 3.45 ms a step with 2^25, 3.21 with 2^23, 3.29 with 2^22
+// Bits of the cells that order n photons: 2 to 4 cells per photon spread evenly, so up to a
+// leaf's worth of photons per cell where a Gaussian bunch is densest (ten times the cells per
+// photon cost more to scan than the finer order saves).  Large beams take 2^23, whose counts
+// (32 MB) stay in L2 for the atomics, or half a cell per photon: both beams of 16M photons
+// at 90 degrees 3.45 ms a step with 2^25, 3.21 with 2^23, 3.29 with 2^22; of 5e7 photons
+// 11.8 ms with 2^27, 10.9 with 2^25, 11.5 with 2^23.
 static int order_bits_for(int64_t n) {
   int lg = 0;
   while ((1ll << lg) < n) ++lg;
-  return std::max(4, std::min(lg + 1, 23));
+  return std::max(4, std::min(lg + 1, std::max(23, lg - 1)));
 }
 
 // The exact path's layout of both beams (sizes[k]: photons of every instance).

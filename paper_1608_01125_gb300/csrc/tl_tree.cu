@@ -5,7 +5,8 @@
 // The smaller beam (the tree's) gets a packed tree over its sorted photons with 32
 // children per node (as in Kamel and Faloutsos, "Hilbert R-tree", VLDB 1994: leaves
 // are runs of the curve, so there are no links to build): k_boxes writes every
-// photon's swept box and the boxes of levels 1 and 2, k_upper those above.  The other
+// photon's swept box (in dense steps its needle, tl_frame.cuh) and the boxes of levels 1
+// and 2, k_upper those above.  The other
 // beam needs no tree: k_collide descends the tree with 32 of its consecutive photons
 // at a time, one per lane, and gives the photon pairs whose boxes overlap the first
 // look of the narrow phase; k_decide decides what that leaves.
