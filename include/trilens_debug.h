@@ -105,6 +105,11 @@ int trilens_debug_band_stress(uint64_t seed, int64_t n_pairs, double dt_fs, doub
                               unsigned long long *counts, double *sample, int64_t n_sample,
                               trilens_stream_t stream);
 
+/* *n: how often the context has captured a run (trilens_run, trilens_batch_run) so
+ * far.  A run is captured again when its steps change or when a buffer or shape that
+ * the captured one holds was replaced.  INVALID for a NULL context or n. */
+int trilens_debug_captures(trilens_ctx *c, int64_t *n);
+
 /* The FP32 narrow phase's sure-miss radii per bin of the invariant s (host
  * only, no GPU): bin 0 holds s < 1; bin 1 + 8 e + k holds s in
  * [2^e (1 + k/8), 2^e (1 + (k+1)/8)) for e = 0..23, the last bin also every

@@ -118,6 +118,8 @@ def lib() -> ctypes.CDLL:
         L.trilens_debug_stall_sort.restype = ctypes.c_int
         L.trilens_debug_set_spin_limit.argtypes = [vp, i64]
         L.trilens_debug_set_spin_limit.restype = ctypes.c_int
+        L.trilens_debug_captures.argtypes = [vp, ctypes.POINTER(i64)]
+        L.trilens_debug_captures.restype = ctypes.c_int
         L.trilens_debug_set_cut_cap.argtypes = [vp, ctypes.c_int32]
         L.trilens_debug_set_cut_cap.restype = ctypes.c_int
         L.trilens_debug_shrink_buffers.argtypes = [vp, i64]
@@ -477,6 +479,11 @@ class Collider:
 
     def debug_set_parts(self, parts: int):
         _check(lib().trilens_debug_set_parts(self.ctx, int(parts)), self.ctx)
+
+    def debug_captures(self) -> int:
+        n = ctypes.c_int64(0)
+        _check(lib().trilens_debug_captures(self.ctx, ctypes.byref(n)), self.ctx)
+        return int(n.value)
 
     def debug_set_spin_limit(self, limit: int):
         _check(lib().trilens_debug_set_spin_limit(self.ctx, int(limit)), self.ctx)

@@ -48,6 +48,7 @@ constexpr unsigned long long kLeafListMax = 1ull << 30;
 // pairs): a larger list, or more parts
 static int leaves_for(trilens_ctx *c, unsigned long long need) {
   if (need + need / 4 + 1024 <= kLeafListMax) return grow(c, &c->leaves, &c->leaf_cap, need);
+  drop_run(c);
   if (c->leaf_cap < kLeafListMax) {
     cudaFree(c->leaves);
     c->leaves = nullptr;
@@ -353,6 +354,7 @@ int ensure_full(trilens_ctx *c) {
   const unsigned long long cap = std::min<unsigned long long>(
       std::max<unsigned long long>(1 << 20, 16ull * (c->beam[0].n + c->beam[1].n)), 1ull << 29);
   if (c->leaf_cap < cap) {
+    drop_run(c);
     cudaFree(c->leaves);
     c->leaves = nullptr;
     c->leaf_cap = 0;
@@ -489,7 +491,7 @@ void trilens_destroy(trilens_ctx *c) {
   cudaFree(c->inst_tmp);
   cudaFree(c->run_status);
   cudaFreeHost(c->run_status_host);
-  if (c->gexec) cudaGraphExecDestroy(c->gexec);
+  drop_run(c);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   if (c->side_stream) cudaStreamDestroy(c->side_stream);
   if (c->sum_stream) cudaStreamDestroy(c->sum_stream);
@@ -1178,10 +1180,7 @@ static int graph_collide(trilens_ctx *c, int64_t step, double *yields) {
 }
 
 static int capture_run(trilens_ctx *c, int64_t first, int64_t steps, double *yields) {
-  if (c->gexec) {
-    cudaGraphExecDestroy(c->gexec);
-    c->gexec = nullptr;
-  }
+  drop_run(c);
   const int timing = c->timing;
   c->timing = 0;
   cudaStream_t saved = c->stream;
@@ -1210,6 +1209,7 @@ static int capture_run(trilens_ctx *c, int64_t first, int64_t steps, double *yie
   e = cudaGraphInstantiate(&c->gexec, g, 0);
   cudaGraphDestroy(g);
   if (e != cudaSuccess) return fail(c, TRILENS_ERR_CUDA, "instantiate: %s", cudaGetErrorString(e));
+  ++c->g_captures;
   c->g_first = first;
   c->g_steps = steps;
   c->g_yields = yields;
@@ -1246,10 +1246,6 @@ static int replay_run(trilens_ctx *c, int64_t first_step, int64_t steps, double 
       return rc;
     if (st & TL_ST_BAND_OVF && (rc = grow(c, &c->band, &c->band_cap, m.max_band))) return rc;
     if (st & TL_ST_LEAFQ && (rc = leaves_for(c, m.max_leaves))) return rc;
-    if (c->gexec) {
-      cudaGraphExecDestroy(c->gexec);
-      c->gexec = nullptr;
-    }
   }
   return fail(c, TRILENS_ERR_STACK, "captured run kept overflowing");
 }
@@ -1338,10 +1334,7 @@ static int apply_tuning(trilens_ctx *c, int bucket, int depth, int warps, int bu
       if (rcq) return rcq;
     }
   }
-  if (c->gexec) {  // a captured run holds the old shapes
-    cudaGraphExecDestroy(c->gexec);
-    c->gexec = nullptr;
-  }
+  drop_run(c);  // a captured run holds the old shapes
   c->built_step = c->exact_step = c->full_step = -1;  // the leaf bucket changes the hierarchy
   return TRILENS_OK;
 }
@@ -1592,10 +1585,13 @@ int trilens_debug_phase_ms(trilens_ctx *c, double *out, int64_t *launches, int r
 int trilens_debug_set_parts(trilens_ctx *c, int32_t parts) {
   if (!c || parts < 1 || parts > 4096) return TRILENS_ERR_INVALID;
   c->parts = parts;
-  if (c->gexec) {  // a captured run holds the old part count
-    cudaGraphExecDestroy(c->gexec);
-    c->gexec = nullptr;
-  }
+  drop_run(c);  // a captured run holds the old part count
+  return TRILENS_OK;
+}
+
+int trilens_debug_captures(trilens_ctx *c, int64_t *n) {
+  if (!c || !n) return TRILENS_ERR_INVALID;
+  *n = c->g_captures;
   return TRILENS_OK;
 }
 
@@ -1609,10 +1605,7 @@ int trilens_debug_shrink_buffers(trilens_ctx *c, int64_t cap) {
   if (!c || cap < 1) return TRILENS_ERR_INVALID;
   CK(cudaSetDevice(c->device));
   CK(cudaStreamSynchronize(c->stream));
-  if (c->gexec) {  // a captured run holds the old buffers
-    cudaGraphExecDestroy(c->gexec);
-    c->gexec = nullptr;
-  }
+  drop_run(c);  // a captured run holds the old buffers
   const unsigned long long n = (unsigned long long)cap;
   cudaFree(c->hits);
   cudaFree(c->band);
@@ -1642,10 +1635,7 @@ int trilens_debug_set_key_bits(trilens_ctx *c, int32_t bits) {
   }
   for (int k = 0; k < 2; ++k)  // at most what the cells are allocated for
     c->order_bits[k] = std::min(order_bits_for(c->beam[k].n), 3 * bits);
-  if (c->gexec) {  // a captured run holds the old pass count
-    cudaGraphExecDestroy(c->gexec);
-    c->gexec = nullptr;
-  }
+  drop_run(c);  // a captured run holds the old pass count
   c->built_step = c->exact_step = c->full_step = -1;
   return TRILENS_OK;
 }

@@ -92,6 +92,7 @@ struct trilens_ctx {
   cudaStream_t cut_stream = nullptr, sum_stream = nullptr;
   cudaGraphExec_t gexec = nullptr;
   int64_t g_first = -1, g_steps = 0;
+  int64_t g_captures = 0;  // runs captured so far
   double *g_yields = nullptr;
   TLRunAcc *run_acc = nullptr;       // device totals of a captured single-context run
   unsigned *run_status = nullptr;
@@ -167,8 +168,17 @@ static inline int alloc_spill(trilens_ctx *c, unsigned per_warp, unsigned long l
   return TRILENS_OK;
 }
 
+// A captured run holds the hit, band and candidate buffers, the part count and the shapes
+// of its launches by value: whatever replaces one of them drops the run, and the next
+// trilens_run or trilens_batch_run captures it again.
+static inline void drop_run(trilens_ctx *c) {
+  if (c->gexec) cudaGraphExecDestroy(c->gexec);
+  c->gexec = nullptr;
+}
+
 static inline int grow(trilens_ctx *c, uint2 **buf, unsigned long long *cap, unsigned long long need) {
   unsigned long long nc = std::max<unsigned long long>(need + need / 4 + 1024, *cap * 2);
+  drop_run(c);
   cudaFree(*buf);
   *buf = nullptr;
   *cap = 0;
