@@ -1554,6 +1554,7 @@ int trilens_reset_yield(trilens_ctx *c) {
 // TRILENS_ERR_TIMEOUT instead of a hang.
 int trilens_debug_stall_sort(trilens_ctx *c, int on) {
   if (!c) return TRILENS_ERR_INVALID;
+  drop_run(c);  // a captured run holds the old setting
   c->debug_stall_sort = on;
   return TRILENS_OK;
 }
@@ -1597,6 +1598,7 @@ int trilens_debug_captures(trilens_ctx *c, int64_t *n) {
 
 int trilens_debug_set_spin_limit(trilens_ctx *c, int64_t limit) {
   if (!c || limit < 1) return TRILENS_ERR_INVALID;
+  drop_run(c);  // a captured run holds the old limit
   c->p.spin_limit = limit;
   return TRILENS_OK;
 }

@@ -281,9 +281,11 @@ __host__ __device__ inline void tl_beam_box(const double *e, double p1, double d
 
 #ifdef __CUDACC__
 
-// photons of an instance that are sorted this step
+// photons of an instance that are sorted this step (never more than it has, also where the
+// running sum is not valid: a wait of its scan ran out)
 __device__ __forceinline__ int tl_live(const TLInst &I, const uint32_t *start) {
-  return (int)(__ldg(start + I.cell0 + (1u << I.bits)) - __ldg(start + I.cell0));
+  const int n = (int)(__ldg(start + I.cell0 + (1u << I.bits)) - __ldg(start + I.cell0));
+  return max(0, min(n, I.n));
 }
 
 // Swept interval of one axis in FP32 interval arithmetic with directed rounding: the

@@ -677,7 +677,8 @@ __global__ void __launch_bounds__(kTile) k_boxes(BoxArgs a) {
 
 // Levels 3 and up of one instance's tree per block, a warp per node.
 __global__ void __launch_bounds__(1024) k_upper(const TLInst *inst, const uint32_t *start,
-                                                float4 *box) {
+                                                float4 *box, const unsigned *build_status) {
+  if (*build_status & TL_ST_TIMEOUT) return;  // (k_boxes has written nothing)
   const TLInst &I = inst[blockIdx.x];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int n = tl_live(I, start), top = tl_top_level(n);
@@ -697,7 +698,7 @@ cudaError_t launch_boxes(const BoxArgs &a, int tiles, int n_inst, int max_top, c
   if (tiles <= 0) return cudaSuccess;
   if (a.needles) k_boxes<true><<<tiles, kTile, 0, s>>>(a);
   else k_boxes<false><<<tiles, kTile, 0, s>>>(a);
-  if (max_top >= 3) k_upper<<<n_inst, 1024, 0, s>>>(a.inst, a.start, a.box);
+  if (max_top >= 3) k_upper<<<n_inst, 1024, 0, s>>>(a.inst, a.start, a.box, a.build_status);
   return cudaGetLastError();
 }
 
