@@ -49,6 +49,7 @@ struct CutArgs {
   unsigned *cut_count;
   unsigned cut_cap;
   unsigned *status;
+  const unsigned *build_status;
 };
 
 cudaError_t launch_prefix_moments(const PreBeam &a, const PreBeam &b, int L, cudaStream_t s,

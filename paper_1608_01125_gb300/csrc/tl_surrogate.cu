@@ -338,6 +338,7 @@ __device__ __forceinline__ void append(bool pred, uint2 v, uint2 *buf, unsigned 
 // otherwise the non-cut sides are split and the overlapping child pairs go
 // to the next level.
 __global__ void __launch_bounds__(256) k_cut_level(CutArgs a) {
+  if (*a.build_status & (TL_ST_TIMEOUT | TL_ST_BADTREE)) return;  // no valid links to follow
   const unsigned nin = min(a.counts[0], a.cap);
   const int lane = threadIdx.x & 31;
   const unsigned nround = (nin + 31u) & ~31u;

@@ -238,6 +238,7 @@ static int sur_cut(trilens_ctx *c, int L, unsigned *ncut) {
     a.cut_count = s->cut_count;
     a.cut_cap = s->cut_cap;
     a.status = s->status;
+    a.build_status = c->build_status;
     int level = 0;
     unsigned left = one;
     while (left > 0 && level < 250) {
