@@ -274,6 +274,7 @@ static int sur_cut(trilens_ctx *c, int L, unsigned *ncut) {
     *ncut = rec[0];
     const unsigned st = rec[1], bst = *c->build_status_host;
     if (bst & (TL_ST_TIMEOUT | TL_ST_BADTREE)) {  // the hierarchy of this step is invalid
+      c->exact_step = c->full_step = -1;
       c->w[0].sort_epoch = c->w[1].sort_epoch = 0;
       CK(cudaMemsetAsync(c->build_status, 0, sizeof(unsigned), c->stream));
       CK(cudaStreamSynchronize(c->stream));
