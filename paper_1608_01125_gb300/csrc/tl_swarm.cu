@@ -150,7 +150,9 @@ __global__ void __launch_bounds__(kThreads) k_swarm_mark(MarkArgs g) {
   const int w0 = (tid >> 5) % groups;  // warps start apart: one's finds spare the others' tests
   for (int gi = 0; gi < groups; ++gi) {
     const int gr = gi + w0 < groups ? gi + w0 : gi + w0 - groups;
-    unsigned bm = *(volatile unsigned *)&sm[gr];
+    // one lane reads the word, which other warps add to: bm, todo and all are the warp's
+    unsigned bm = lane == 0 ? *(volatile unsigned *)&sm[gr] : 0u;
+    bm = __shfl_sync(0xffffffffu, bm, 0);
     const unsigned bm0 = bm;
     const int cnt = min(kMarkGroup, m - gr * kMarkGroup);
     unsigned todo = cnt == 32 ? 0xffffffffu : (1u << cnt) - 1u;
@@ -187,6 +189,7 @@ __global__ void __launch_bounds__(kThreads) k_swarm_mark(MarkArgs g) {
       }
     }
     if (lane == 0 && bm != bm0) atomicOr(&sm[gr], bm);
+    __syncwarp();
   }
   if (known && !known0) g.mark_a[i] = 1;
   __syncthreads();
