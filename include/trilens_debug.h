@@ -110,6 +110,10 @@ int trilens_debug_band_stress(uint64_t seed, int64_t n_pairs, double dt_fs, doub
  * the captured one holds was replaced.  INVALID for a NULL context or n. */
 int trilens_debug_captures(trilens_ctx *c, int64_t *n);
 
+/* Host only: 1 if a grid barrier that waits for its counter of arrivals to come to
+ * `want` lets go at `have`, else 0.  Both count modulo 2^32. */
+int trilens_debug_arrived(uint32_t have, uint32_t want);
+
 /* The FP32 narrow phase's sure-miss radii per bin of the invariant s (host
  * only, no GPU): bin 0 holds s < 1; bin 1 + 8 e + k holds s in
  * [2^e (1 + k/8), 2^e (1 + (k+1)/8)) for e = 0..23, the last bin also every

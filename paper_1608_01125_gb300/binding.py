@@ -118,6 +118,8 @@ def lib() -> ctypes.CDLL:
         L.trilens_debug_stall_sort.restype = ctypes.c_int
         L.trilens_debug_set_spin_limit.argtypes = [vp, i64]
         L.trilens_debug_set_spin_limit.restype = ctypes.c_int
+        L.trilens_debug_arrived.argtypes = [ctypes.c_uint32, ctypes.c_uint32]
+        L.trilens_debug_arrived.restype = ctypes.c_int
         L.trilens_debug_captures.argtypes = [vp, ctypes.POINTER(i64)]
         L.trilens_debug_captures.restype = ctypes.c_int
         L.trilens_debug_set_cut_cap.argtypes = [vp, ctypes.c_int32]

@@ -72,6 +72,12 @@ enum {
   TL_ST_BADTREE = 128   // the refit met a node reference out of range (an internal error)
 };
 
+// Whether a counter that only grows, modulo 2^32, has come to `want` (it is never 2^31 or
+// more away).
+__host__ __device__ inline bool tl_arrived(unsigned have, unsigned want) {
+  return (int)(have - want) >= 0;
+}
+
 // Per-step device counters; zeroed by the step's init kernel.
 struct TLCounters {
   unsigned long long hits;         // colliding pairs found (may exceed capacity)

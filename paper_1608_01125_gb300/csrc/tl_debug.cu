@@ -21,3 +21,7 @@ extern "C" int trilens_debug_eval64(const double *x, double *out, int64_t n, int
   k_sigma64<<<(unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream>>>(x, out, n, which);
   return cudaGetLastError() == cudaSuccess ? TRILENS_OK : TRILENS_ERR_CUDA;
 }
+
+extern "C" int trilens_debug_arrived(uint32_t have, uint32_t want) {
+  return tl_arrived(have, want) ? 1 : 0;
+}

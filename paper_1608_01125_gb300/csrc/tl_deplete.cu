@@ -185,7 +185,7 @@ __device__ bool grid_sync(const DepArgs &g, unsigned &done) {
     const unsigned want = done * gridDim.x;
     unsigned have = atomicAdd(&ctl->arrive, 1u) + 1u;
     long long it = 0;
-    while (have < want) {
+    while (!tl_arrived(have, want)) {  // (a long chain of rounds wraps the counter)
       if ((*(volatile int *)&ctl->flag & kFlagBarrier) || ++it > g.spin) {
         atomicOr(&ctl->flag, kFlagBarrier);
         atomicExch(g.dirty, 1);
