@@ -329,13 +329,17 @@ int trilens_collide_batch(const trilens_beam *a, const trilens_beam *b, const tr
                           int32_t n_inst, int64_t steps, double *yields, trilens_stream_t stream);
 
 /* ---- tuning -----------------------------------------------------------------
- * The hit set never depends on these knobs; only the time does.
- *   leaf_bucket  photons per hierarchy leaf (1..32)
+ * Knobs of the statistical regime's hierarchies and of the seeded traversal that serves
+ * its labels and its exact fallback.  The hit set never depends on them, and the exact path
+ * (trilens_build, trilens_collide_step, trilens_run, batches) uses none.
+ *   leaf_bucket  photons per hierarchy leaf (1..32); a leaf that holds more than a level-L
+ *                node is a cloud of the level-L cut, so a model stands for the bucket it was
+ *                trained with
  *   stack_depth  traversal stack entries per warp in shared memory (64..4096; the
  *                rest of a warp's stack is its private spill area in global memory)
  *   block_shape  traversal warps per block (1..8)
  *   budget       traversal iterations a warp spends on one work item before it
- *                hands the rest on, as chunks of 8 node pairs, to the step's
+ *                hands the rest on, as chunks of 32 node pairs, to the step's
  *                device work queue, where idle warps take them (0 = never;
  *                default 16) */
 
@@ -347,11 +351,14 @@ int trilens_set_tuning(trilens_ctx *c, int32_t leaf_bucket, int32_t stack_depth,
 /* Current knobs into out[4] (leaf_bucket, stack_depth, block_shape, budget). */
 int trilens_get_tuning(trilens_ctx *c, int32_t out[4]);
 
-/* Autotuner.  If cache_path (a JSON file; NULL = no cache) holds an entry for
- * this context's configuration class (beam sizes rounded to powers of two,
- * instance count, precision, SM count), apply it.  Otherwise time build +
- * collide of the n_steps sample steps while sweeping each knob in turn (the
- * others held at the best so far), apply the fastest, and record it in the
+/* Autotuner of stack_depth, block_shape and budget; leaf_bucket stays as it is.  If
+ * cache_path (a JSON file; NULL = no cache) holds an entry for this context's configuration
+ * class (beam sizes rounded to powers of two, instance count, precision, SM count; level and
+ * leaf bucket where the context has samples or a model of the statistical regime), apply it.
+ * Otherwise, in a context with samples or a model, time the seeded traversal of the n_steps
+ * sample steps' cut pairs while sweeping each knob in turn (the others held at the best so
+ * far), and apply the fastest; in any other context no knob acts on anything, the sample
+ * steps are built and collided and the current knobs kept.  The choice is recorded in the
  * cache.  Tuning runs are not added to the yield.  chosen (host, 4 ints) may
  * be NULL.  Synchronises the stream. */
 int trilens_autotune(trilens_ctx *c, const int64_t *steps, int32_t n_steps,

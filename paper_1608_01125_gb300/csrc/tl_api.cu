@@ -1355,14 +1355,16 @@ int trilens_get_tuning(trilens_ctx *c, int32_t out[4]) {
   return TRILENS_OK;
 }
 
-// key of a configuration class: sizes rounded to powers of two, precision,
-// SM count
+// key of a configuration class: sizes rounded to powers of two, precision, SM count, and
+// the level and leaf bucket of a context that uses the statistical regime
 static void tuning_key(trilens_ctx *c, char *key, size_t len) {
   int la = 0, lb = 0;
   while ((1ll << la) < std::max<int64_t>(c->beam[0].n, 1)) ++la;
   while ((1ll << lb) < std::max<int64_t>(c->beam[1].n, 1)) ++lb;
-  snprintf(key, len, "nA2^%d_nB2^%d_inst%d_prec%d_sm%d", la, lb, c->n_inst, c->p.precision,
-           c->n_sm);
+  const int at = snprintf(key, len, "nA2^%d_nB2^%d_inst%d_prec%d_sm%d", la, lb, c->n_inst,
+                          c->p.precision, c->n_sm);
+  if (surrogate_level(c) >= 0)
+    snprintf(key + at, len - at, "_L%d_b%d", surrogate_level(c), c->p.leaf_bucket);
 }
 
 static bool cache_lookup(const char *path, const char *key, int v[4]) {
@@ -1418,31 +1420,35 @@ static void cache_store(const char *path, const char *key, const int v[4], doubl
   rename(tmp.c_str(), path);
 }
 
-// time build + collide over the sample steps with the current tuning
-// the faster of two timed passes over the sample steps (one pass is noisy
-// enough to flip close choices)
+// The time of the sample steps with the current knobs: of what they act on, the seeded
+// traversal of the steps' cut pairs, where the context uses the statistical regime, else of
+// build + collide.  The faster of two passes (one is noisy enough to flip close choices).
 static int time_steps(trilens_ctx *c, const int64_t *steps, int n, double *ms) {
+  const bool seeded = surrogate_level(c) >= 0;
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
   const double keep_count = c->tot_count, keep_w = c->tot_weighted;
   double best = 1e30;
   for (int rep = 0; rep < 2; ++rep) {
+    double sum = 0.0;
     CK(cudaEventRecord(e0, c->stream));
     for (int i = 0; i < n; ++i) {
-      int rc = trilens_build(c, steps[i]);
-      if (!rc) rc = trilens_collide_step(c, steps[i], nullptr, 0, nullptr);
+      float f = 0.f;
+      int rc = seeded ? surrogate_time_step(c, steps[i], &f) : trilens_build(c, steps[i]);
+      if (!rc && !seeded) rc = trilens_collide_step(c, steps[i], nullptr, 0, nullptr);
       if (rc) {
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
         return rc;
       }
+      sum += (double)f;
     }
     CK(cudaEventRecord(e1, c->stream));
     CK(cudaEventSynchronize(e1));
     float f = 0.f;
     CK(cudaEventElapsedTime(&f, e0, e1));
-    best = std::min(best, (double)f);
+    best = std::min(best, seeded ? sum : (double)f);
   }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
@@ -1456,32 +1462,31 @@ int trilens_autotune(trilens_ctx *c, const int64_t *steps, int32_t n_steps,
                      const char *cache_path, int32_t chosen[4]) {
   if (!c || !steps || n_steps < 1) return TRILENS_ERR_INVALID;
   CK(cudaSetDevice(c->device));
-  char key[128];
+  char key[160];
   tuning_key(c, key, sizeof(key));
+  const int bucket = c->p.leaf_bucket;  // kept: it says what a cloud is (and is not a matter of time)
   int v[4];
   if (cache_lookup(cache_path, key, v)) {
+    v[0] = bucket;
     int rc = apply_tuning(c, v[0], v[1], v[2], v[3]);
     if (rc) return rc;
     if (chosen)
       for (int i = 0; i < 4; ++i) chosen[i] = v[i];
     return TRILENS_OK;
   }
-  // coordinate descent over the four knobs, each swept with the others
+  // coordinate descent over the seeded traversal's knobs, each swept with the others
   // fixed at the best so far (stack depth first: a shallow stack moves work
   // to the spill areas, which would bias the other sweeps); results never
-  // depend on the knobs, only time does
-  int best[4] = {c->p.leaf_bucket, c->p.stack_depth, c->p.block_shape, c->budget};
-  static const int cand[4][5] = {{1, 2, 4, 8, 16}, {256, 512, 1024, 0, 0}, {2, 4, 8, 0, 0},
-                                 {8, 16, 32, 64, 0}};
-  static const int order[4] = {1, 0, 2, 3};
+  // depend on them, only time does.  Where nothing they act on is used, the current ones stay.
+  int best[4] = {bucket, c->p.stack_depth, c->p.block_shape, c->budget};
+  static const int cand[4][4] = {{0, 0, 0, 0}, {256, 512, 1024, 0}, {2, 4, 8, 0}, {8, 16, 32, 64}};
   double best_ms = 1e30;
   int rc = apply_tuning(c, best[0], best[1], best[2], best[3]);
   if (rc) return rc;
   if ((rc = time_steps(c, steps, n_steps, &best_ms))) return rc;  // warm-up
   if ((rc = time_steps(c, steps, n_steps, &best_ms))) return rc;
-  for (int oi = 0; oi < 4; ++oi) {
-    const int knob = order[oi];
-    for (int j = 0; j < 5 && cand[knob][j]; ++j) {
+  for (int knob = 1; knob < 4 && surrogate_level(c) >= 0; ++knob) {
+    for (int j = 0; j < 4 && cand[knob][j]; ++j) {
       int t[4] = {best[0], best[1], best[2], best[3]};
       t[knob] = cand[knob][j];
       if (t[knob] == best[knob]) continue;

@@ -200,4 +200,8 @@ void surrogate_free(trilens_ctx *c);
 void deplete_free(trilens_ctx *c);
 double tl_sigma_max_bound();
 TLNarrowConst tl_narrow_const(double dt_fs, double kappa);
+// the level of the statistical regime's samples or model, -1 if there is none
+int surrogate_level(const trilens_ctx *c);
+// device time of the seeded traversal of all of step's cut pairs at that level
+int surrogate_time_step(trilens_ctx *c, int64_t step, float *ms);
 extern "C" int surrogate_total(trilens_ctx *c, int level, double *out);

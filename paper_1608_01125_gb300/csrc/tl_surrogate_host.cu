@@ -334,6 +334,31 @@ static int sur_labels(trilens_ctx *c, int L, double ct, unsigned ncut, double *t
   return TRILENS_OK;
 }
 
+int surrogate_level(const trilens_ctx *c) { return c->sur ? c->sur->level : -1; }
+
+int surrogate_time_step(trilens_ctx *c, int64_t step, float *ms) {
+  SurrogateState *s = c->sur;
+  *ms = 0.0f;
+  int rc = trilens_build(c, step);
+  if (rc) return rc;
+  unsigned ncut = 0;
+  if ((rc = sur_cut(c, s->level, &ncut)) || ncut == 0) return rc;
+  CK(tl::launch_sur_misc(0, s->cut, nullptr, s->seeds, ncut, c->stream));
+  cudaEvent_t e0, e1;
+  CK(cudaEventCreate(&e0));
+  CK(cudaEventCreate(&e1));
+  cudaError_t e = cudaEventRecord(e0, c->stream);
+  if (!e) rc = run_exact(c, TL_C * ((double)step * c->p.dt_fs), s->seeds, ncut, nullptr);
+  if (!e) e = cudaEventRecord(e1, c->stream);
+  if (!e) e = cudaEventSynchronize(e1);
+  if (!e) e = cudaEventElapsedTime(ms, e0, e1);
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+  if (rc) return rc;
+  CK(e);
+  return TRILENS_OK;
+}
+
 static int append_samples(trilens_ctx *c, unsigned ncut) {
   SurrogateState *s = c->sur;
   if (s->tn + ncut > s->tcap) {
