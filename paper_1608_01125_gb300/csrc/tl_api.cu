@@ -86,7 +86,7 @@ static tl::ColArgs col_args(trilens_ctx *c, int p) {
   a.tinst = c->insts[t];
   a.qstart = c->w[q].start;
   a.tstart = c->w[t].start;
-  a.tile_inst = c->tile_inst[q];
+  a.group_inst = c->group_inst[q];
   a.frames = c->frames;
   a.Llo = c->L_lo;
   a.Lhi = c->L_hi;
@@ -95,14 +95,14 @@ static tl::ColArgs col_args(trilens_ctx *c, int p) {
   a.ctr = c->ctr;
   a.cand = c->leaves;
   a.cand_cap = c->leaf_cap;
-  const long long groups = 32ll * c->n_tiles[q];
+  const long long groups = c->n_groups[q];
   const long long g0 = groups * p / c->parts, g1 = groups * (p + 1) / c->parts;
   a.group0 = (int)g0;
   a.slices = 1;
   if (g1 > g0)
     a.slices = (int)std::min<long long>(
         64, std::max<long long>(1, (long long)kColWarpsPerSm * c->n_sm / (g1 - g0)));
-  a.items = c->n_tiles[t] > 0 ? (g1 - g0) * a.slices : 0;
+  a.items = c->n_groups[t] > 0 ? (g1 - g0) * a.slices : 0;
   a.fp64 = c->p.precision == TRILENS_FP64;
   a.swap = t == 0;
   a.needles = c->needles;
@@ -383,29 +383,34 @@ static int layout(trilens_ctx *c, const std::vector<int64_t> sizes[2]) {
   const size_t ni = sizes[0].size();
   for (int k = 0; k < 2; ++k) {
     std::vector<TLInst> in(ni);
-    std::vector<uint32_t> tile_inst;
-    int64_t tile = 0, cells = 0, first = 0;
+    std::vector<uint32_t> group_inst;
+    int64_t group = 0, cells = 0, first = 0;
     for (size_t q = 0; q < ni; ++q) {
       TLInst &I = in[q];
       memset(&I, 0, sizeof(I));
       I.n = (int)sizes[k][q];
       I.first = (int)first;
       first += sizes[k][q];
-      I.tile0 = (int)tile;
       I.bits = order_bits_for(sizes[k][q]);
       I.cell0 = (uint32_t)cells;
       cells += 1ll << in[q].bits;
-      const int64_t t = (sizes[k][q] + kTile - 1) / kTile;
-      if (ni > 1) tile_inst.insert(tile_inst.end(), (size_t)t, (uint32_t)q);
-      tile += t;
+      // (a tile's groups behind a small instance count as that instance's, without photons)
+      if (sizes[k][q] > kTile) group = (group + 31) & ~31ll;
+      if (ni > 1 && q > 0) group_inst.resize((size_t)group, (uint32_t)q - 1u);
+      I.group0 = (int)group;
+      group += (sizes[k][q] + 31) / 32;
+      if (sizes[k][q] > kTile) group = (group + 31) & ~31ll;
+      if (ni > 1) group_inst.resize((size_t)group, (uint32_t)q);
     }
-    c->n_tiles[k] = (int)tile;
+    const int64_t tile = (group + 31) / 32;
+    if (ni > 1) group_inst.resize((size_t)tile * 32, (uint32_t)ni - 1u);
+    c->n_groups[k] = (int)tile * 32;
     if (k == c->tree) {  // levels 0..2 tile by tile, then what is above
       uint64_t up = (uint64_t)tile * (kTile + 32 + 1);
       for (size_t q = 0; q < ni; ++q) {
-        in[q].lev[0] = (uint32_t)((uint64_t)in[q].tile0 * kTile);
-        in[q].lev[1] = (uint32_t)((uint64_t)tile * kTile + (uint64_t)in[q].tile0 * 32);
-        in[q].lev[2] = (uint32_t)((uint64_t)tile * (kTile + 32) + (uint64_t)in[q].tile0);
+        in[q].lev[0] = (uint32_t)((uint64_t)in[q].group0 * 32);
+        in[q].lev[1] = (uint32_t)((uint64_t)tile * kTile + (uint64_t)in[q].group0);
+        in[q].lev[2] = (uint32_t)((uint64_t)tile * (kTile + 32) + (uint64_t)(in[q].group0 / 32));
         const int top = tl_top_level(in[q].n);
         for (int l = 3; l <= top; ++l) {
           in[q].lev[l] = (uint32_t)up;
@@ -419,8 +424,8 @@ static int layout(trilens_ctx *c, const std::vector<int64_t> sizes[2]) {
     CK(cudaMemcpyAsync(c->insts[k], in.data(), sizeof(TLInst) * ni, cudaMemcpyHostToDevice,
                        c->stream));
     if (ni > 1) {
-      CK(dalloc(&c->tile_inst[k], tile_inst.size()));
-      CK(cudaMemcpyAsync(c->tile_inst[k], tile_inst.data(), sizeof(uint32_t) * tile_inst.size(),
+      CK(dalloc(&c->group_inst[k], group_inst.size()));
+      CK(cudaMemcpyAsync(c->group_inst[k], group_inst.data(), sizeof(uint32_t) * group_inst.size(),
                          cudaMemcpyHostToDevice, c->stream));
     }
     const int rc = alloc_beam(c, c->w[k], c->beam[k].n, tile * kTile, cells);
@@ -482,7 +487,7 @@ void trilens_destroy(trilens_ctx *c) {
     cudaFree(c->inst_of[k]);
     cudaFree(c->inst_bounds[k]);
     cudaFree(c->insts[k]);
-    cudaFree(c->tile_inst[k]);
+    cudaFree(c->group_inst[k]);
     cudaFree(c->grids[k]);
     for (int a = 0; a < 8; ++a) cudaFree(c->owned[k][a]);
   }
@@ -767,7 +772,7 @@ static int build_exact(trilens_ctx *c, int64_t step) {
     memset(&pl, 0, sizeof(pl));
     pl.b = c->beam[k];
     pl.ct = ct;
-    pl.n_pad = (int64_t)c->n_tiles[k] * kTile;
+    pl.n_pad = (int64_t)c->n_groups[k] * 32;
     pl.stat = w.stat;
     pl.cell = w.cell;
     pl.start = w.start;
@@ -785,7 +790,7 @@ static int build_exact(trilens_ctx *c, int64_t step) {
     b.rec = w.rec;
     b.inst = c->insts[k];
     b.start = w.start;
-    b.tile_inst = c->tile_inst[k];
+    b.group_inst = c->group_inst[k];
     b.frames = c->frames;
     b.Llo = c->L_lo;
     b.Lhi = c->L_hi;
@@ -794,7 +799,7 @@ static int build_exact(trilens_ctx *c, int64_t step) {
     b.needles = c->needles;
     b.box = c->box;
     b.build_status = c->build_status;
-    CK(tl::launch_boxes(b, c->n_tiles[k], c->n_inst, c->max_top, st));
+    CK(tl::launch_boxes(b, c->n_groups[k] / 32, c->n_inst, c->max_top, st));
     tmark(c, PH_REFIT, k, 1);
     c->phase_launches[PH_REFIT] += c->max_top >= 3 ? 2 : 1;
   }

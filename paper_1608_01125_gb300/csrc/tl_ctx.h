@@ -43,9 +43,9 @@ struct trilens_ctx {
   TLFrame *frames = nullptr;
   int tree = 1;                  // the beam with the tree
   TLInst *insts[2]{};            // device, per instance
-  uint32_t *tile_inst[2]{};      // device, instance of every tile (batches)
+  uint32_t *group_inst[2]{};     // device, instance of every group of 32 photons (batches)
   TLGrid *grids[2]{};            // device, per instance (batches)
-  int n_tiles[2]{};
+  int n_groups[2]{};             // a multiple of 32
   int max_top = 1;               // over the trees of all instances
   double ext[2][14]{};           // extremes of R p0 and R d (tl_beam_box; not batches)
   bool apart = false;            // the beams' boxes do not meet at exact_step

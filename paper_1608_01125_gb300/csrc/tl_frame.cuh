@@ -38,15 +38,17 @@ struct TLGrid {
   float clo[3], chi[3];
 };
 
-// One instance's photons of one beam in the exact path's layout: tiles of 1024
-// sorted photons from tile0 on, and its tree, an implicit one with 32 children per
-// node over the sorted photons: level 0 the photons, level l nodes of 32^l.  Only the
+// One instance's photons of one beam in the exact path's layout: groups of 32 sorted photons
+// from group0 on, and its tree, an implicit one with 32 children per
+// node over the sorted photons: level 0 the photons, level l nodes of 32^l.  An instance of
+// more than 1024 photons starts on a tile of 32 groups and takes whole tiles (its level 2);
+// smaller ones, whose trees end at level 1, share tiles.  Only the
 // photons that can meet the other beam in a step are sorted; how many, the running sum
 // of the cells tells (tl_live).
 struct TLInst {
   int n;            // photons,
   int first;        // from this one of the input on
-  int tile0;        // first tile
+  int group0;       // first group
   int bits;         // its photons are ordered by 2^bits cells,
   uint32_t cell0;   // from this one on
   uint32_t lev[6];  // first box of each level
@@ -63,7 +65,7 @@ __host__ __device__ inline int tl_top_level(int n) {
   return l;
 }
 
-constexpr int kTile = 1024;  // sorted photons per tile (a level-2 node)
+constexpr int kTile = 1024;  // sorted photons per tile (a level-2 node of a larger instance)
 
 __host__ __device__ inline TLFrame tl_ident_frame() {
   TLFrame f{};  // (no pads: set by tl_set_pads)

@@ -563,7 +563,7 @@ __global__ void __launch_bounds__(256) k_place(PlaceArgs a) {
                     __double2float_rn(__dadd_rn(a.b.pz[i], __dmul_rn(a.ct, dz))), s0.w);
     if (a.inst_of) {
       const TLInst &I = a.inst[a.inst_of[i]];
-      to += (int64_t)I.tile0 * kTile - (int64_t)__ldg(a.start + I.cell0);
+      to += (int64_t)I.group0 * 32 - (int64_t)__ldg(a.start + I.cell0);
     }
     if ((uint64_t)to < (uint64_t)a.n_pad) {  // always, unless the scan's wait expired
       a.rec[2 * to] = p;
@@ -638,22 +638,25 @@ __device__ __forceinline__ TLNeedle no_needle() {
 }
 
 // One block per tile: every photon's swept box (its needle where the frame has a closing
-// axis: the box then only goes into the unions), the boxes of the tile's 32 runs of 32
-// photons (level 1) and the tile's own (level 2).  One pass over the sorted photons;
-// unions by shuffles, no links and no second pass.
+// axis: the box then only goes into the unions), the boxes of the tile's 32 groups of 32
+// photons (level 1) and, in an instance of more than one tile, the tile's own (level 2).  One
+// pass over the sorted photons; unions by shuffles, no links and no second pass.  A warp finds
+// its own instance: 65536 instances of 8 photons with a tile of 1024 each took 24.7 ms and
+// 6.4 GB for 16 steps, with a group of 32 each 5.2 ms and 0.4 GB.
 template <bool NEEDLES>
 __global__ void __launch_bounds__(kTile) k_boxes(BoxArgs a) {
   __shared__ TLBox wb[32];
   if (*a.build_status & TL_ST_TIMEOUT) return;  // keys unsorted: the build is abandoned
-  const int tile = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const uint32_t q = a.tile_inst ? a.tile_inst[tile] : 0u;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5, g = blockIdx.x * 32 + warp;
+  const uint32_t q = a.group_inst ? a.group_inst[g] : 0u;
   const TLInst &I = a.inst[q];
   const int n = tl_live(I, a.start);
-  const int k = tile - I.tile0, r = k * kTile + t;
-  if (k * kTile >= n) return;
+  const int k = g - I.group0, r = k * 32 + lane;
+  const bool whole = I.n > kTile;  // the tile is one instance's (the same for all its warps)
+  if (whole && (k & ~31) * 32 >= n) return;
   TLBox b = empty_box();
   if (r < n) {
-    const int64_t p = (int64_t)tile * kTile + t;
+    const int64_t p = (int64_t)g * 32 + lane;
     const float4 pe = a.rec[2 * p];
     const float4 de = a.rec[2 * p + 1];
     const TLFrame &f = a.frames[q];
@@ -666,12 +669,13 @@ __global__ void __launch_bounds__(kTile) k_boxes(BoxArgs a) {
   b = warp_union(b);
   if (lane == 0) {
     wb[warp] = b;
-    if (r < n) put_box(a.box + 2 * ((size_t)I.lev[1] + k * 32 + warp), b);
+    if (r < n) put_box(a.box + 2 * ((size_t)I.lev[1] + k), b);
   }
+  if (!whole) return;
   __syncthreads();
   if (warp == 0) {
     b = warp_union(wb[lane]);
-    if (lane == 0) put_box(a.box + 2 * ((size_t)I.lev[2] + k), b);
+    if (lane == 0) put_box(a.box + 2 * ((size_t)I.lev[2] + (k >> 5)), b);
   }
 }
 
@@ -877,17 +881,16 @@ __global__ void __launch_bounds__(32 * kColWarps, 8) k_collide(ColArgs a) {
   const long long item = blockIdx.x * (long long)kColWarps + warp;
   if (item >= a.items) return;
   const int g = a.group0 + (int)(item / a.slices), slice = (int)(item % a.slices);
-  const int tile = g >> 5;
-  const uint32_t inst = a.tile_inst ? a.tile_inst[tile] : 0u;
+  const uint32_t inst = a.group_inst ? a.group_inst[g] : 0u;
   const TLInst &Q = a.qinst[inst], &T = a.tinst[inst];
-  const int r0 = (g - Q.tile0 * 32) * 32, qn = tl_live(Q, a.qstart);
+  const int r0 = (g - Q.group0) * 32, qn = tl_live(Q, a.qstart);
   if (r0 >= qn) return;
   const int tn = tl_live(T, a.tstart), leaves_n = tl_level_count(tn, 1);
   const int c0 = (int)((long long)leaves_n * slice / a.slices);
   const int c1 = (int)((long long)leaves_n * (slice + 1) / a.slices);
   if (c0 == c1) return;
   ColSmem &ws = wsm[warp];
-  Pairs<FP64> out{a, ws, suf, (uint32_t)g * 32u, (uint32_t)T.tile0 * (uint32_t)kTile, lane, 0, 0,
+  Pairs<FP64> out{a, ws, suf, (uint32_t)g * 32u, (uint32_t)T.group0 * 32u, lane, 0, 0,
                   a.ctr->leaf_base};
   const TLFrame &f = a.frames[inst];
   TLBox own = empty_box();

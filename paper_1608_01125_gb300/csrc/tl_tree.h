@@ -40,7 +40,7 @@ struct BoxArgs {
   const float4 *rec;
   const TLInst *inst;
   const uint32_t *start;
-  const uint32_t *tile_inst;  // instance of each tile (batches, else NULL)
+  const uint32_t *group_inst;  // instance of each group (batches, else NULL)
   const TLFrame *frames;
   float Llo, Lhi, half;
   int beam, needles;
@@ -54,7 +54,7 @@ struct ColArgs {
   const float4 *box;                        // the tree
   const TLInst *qinst, *tinst;
   const uint32_t *qstart, *tstart;  // running sums of their cells
-  const uint32_t *tile_inst;  // instance of each query tile (batches, else NULL)
+  const uint32_t *group_inst;  // instance of each query group (batches, else NULL)
   const TLFrame *frames;
   float Llo, Lhi, half;
   TLNarrowConst nk;
