@@ -989,8 +989,10 @@ int run_exact(trilens_ctx *c, double ct, const uint2 *seeds, unsigned n_seeds, i
       again = true;
     }
     if (st & TL_ST_SPILL_OVF) {  // the queue: larger, and every slot the sentinel again
+      // (a pass stops soon after the queue is full, so what it asked for says little: four
+      // times as large, up to the largest)
       const unsigned long long need = kQueueChunk * (h.q_tail + h.q_tail / 4 + 1024);
-      if ((rc = alloc_queue(c, std::max(need, 2 * c->queue_cap)))) return rc;
+      if ((rc = alloc_queue(c, std::max(need, std::min(4 * c->queue_cap, 1ull << 30))))) return rc;
       again = true;
     }
     if (st & TL_ST_PRIV_OVF) {  // a warp's spill area: twice as large
@@ -1002,7 +1004,11 @@ int run_exact(trilens_ctx *c, double ct, const uint2 *seeds, unsigned n_seeds, i
       again = true;
     }
     if (!again) break;
-    if (++retries > 8) return fail(c, TRILENS_ERR_STACK, "buffers kept overflowing");
+    if (++retries > 16)  // each makes room for at least twice as much of something
+      return fail(c, TRILENS_ERR_STACK,
+                  "buffers kept overflowing (status 0x%x; queue of %llu node pairs, %llu chunks "
+                  "asked for; spill areas of %u)",
+                  st, c->queue_cap, (unsigned long long)h.q_tail, c->spill_per_warp);
   }
   if (retries_out) *retries_out = retries;
   return TRILENS_OK;
