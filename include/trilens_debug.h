@@ -110,6 +110,11 @@ int trilens_debug_band_stress(uint64_t seed, int64_t n_pairs, double dt_fs, doub
  * the captured one holds was replaced.  INVALID for a NULL context or n. */
 int trilens_debug_captures(trilens_ctx *c, int64_t *n);
 
+/* *on: 1 if the built step's photon pairs are told at the time they pass each other
+ * (dense steps of beams whose photons travel far across the closing axis), 0 if by their
+ * swept boxes.  INVALID for a NULL context or on, or where the exact path has built no step. */
+int trilens_debug_needles(trilens_ctx *c, int32_t *on);
+
 /* Host only: 1 if a grid barrier that waits for its counter of arrivals to come to
  * `want` lets go at `have`, else 0.  Both count modulo 2^32. */
 int trilens_debug_arrived(uint32_t have, uint32_t want);

@@ -120,6 +120,8 @@ def lib() -> ctypes.CDLL:
         L.trilens_debug_set_spin_limit.restype = ctypes.c_int
         L.trilens_debug_arrived.argtypes = [ctypes.c_uint32, ctypes.c_uint32]
         L.trilens_debug_arrived.restype = ctypes.c_int
+        L.trilens_debug_needles.argtypes = [vp, ctypes.POINTER(i32)]
+        L.trilens_debug_needles.restype = ctypes.c_int
         L.trilens_debug_captures.argtypes = [vp, ctypes.POINTER(i64)]
         L.trilens_debug_captures.restype = ctypes.c_int
         L.trilens_debug_set_cut_cap.argtypes = [vp, ctypes.c_int32]
@@ -481,6 +483,11 @@ class Collider:
 
     def debug_set_parts(self, parts: int):
         _check(lib().trilens_debug_set_parts(self.ctx, int(parts)), self.ctx)
+
+    def debug_needles(self) -> bool:
+        on = ctypes.c_int32(0)
+        _check(lib().trilens_debug_needles(self.ctx, ctypes.byref(on)), self.ctx)
+        return bool(on.value)
 
     def debug_captures(self) -> int:
         n = ctypes.c_int64(0)

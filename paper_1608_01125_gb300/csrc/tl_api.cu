@@ -1612,6 +1612,12 @@ int trilens_debug_captures(trilens_ctx *c, int64_t *n) {
   return TRILENS_OK;
 }
 
+int trilens_debug_needles(trilens_ctx *c, int32_t *on) {
+  if (!c || !on || c->exact_step < 0) return TRILENS_ERR_INVALID;
+  *on = c->needles ? 1 : 0;
+  return TRILENS_OK;
+}
+
 int trilens_debug_set_spin_limit(trilens_ctx *c, int64_t limit) {
   if (!c || limit < 1) return TRILENS_ERR_INVALID;
   drop_run(c);  // a captured run holds the old limit
