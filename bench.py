@@ -3,10 +3,12 @@
 One benchmark step = one full run of the head-on workload: 64 time steps of
 5 fs, each the order of both beams and the tree of one plus the collision step
 (descent by groups of 32 photons, pair tests, FP64 band re-test, yield), inputs
-resident in HBM.  The metric is the narrow-phase photon-pair tests per second:
-photon pairs that the tree leaves to be told pair by pair, by the pair's own swept
-boxes or passing point first and by the closest-approach test where that leaves
-them (the work the method does after the hierarchy has pruned).  Collided pairs/s
+resident in HBM.  The metric is photon-pair tests per second: photon pairs that the
+hierarchy leaves to be told one by one.  Here a pair's first test is that of its own
+swept boxes or passing point, and the closest-approach test follows where that leaves
+it; the oracle of the reference arm has the closest-approach test only, so a ratio of
+the two arms compares pairs told, not operations, and the times of a run say what the
+hierarchies' pruning is worth.  Collided pairs/s
 and the all-pairs equivalent N_A * N_B * time steps per second are reported beside
 it as context, and the time of a run, which fewer tests shorten.
 
@@ -35,7 +37,7 @@ sys.path.insert(0, ROOT)
 
 from paper_1608_01125_gb300 import synth  # noqa: E402
 
-METRIC = "narrow-phase photon-pair tests/s at 2x1M (photon pairs given the exact test per second)"
+METRIC = "photon-pair tests/s at 2x1M (photon pairs the hierarchy leaves to be told one by one)"
 UNIT = "pair-tests/s"
 # the oracle's CPU samples: every 4th time step (a systematic sample of the
 # run's busy and empty steps), all host cores; single-threaded (as the paper
@@ -408,12 +410,11 @@ def ip_regime_timing(dev, stream, reps=3, cpu=True):
             "cpu_baseline": cpu_line}
 
 
-def crossing_timing(dev, stream, peak, peak_src, steps=(120, 129, 141, 160)):
+def crossing_timing(dev, stream, steps=(120, 129, 141, 160)):
     """The large exact workload (2 x 5e7 photons crossing at 90 degrees, Gamma
     energies, 2 fs steps): a few of its busy time steps built and collided one
-    at a time with per-phase device times (CUDA events).  Here the two
-    hierarchies (2 x 5e7 x 64 B of node records) are far larger than the L2,
-    so the traversal's HBM fraction is measured where it can matter.  The
+    at a time with per-phase device times (CUDA events).  The sorted photons (32 B
+    each) and the tree over one beam (33 B per photon) are far larger than the L2.  The
     hit counts of steps 129, 141 and 160 are the oracle's (the GPU tests
     compare their checksums)."""
     import torch
@@ -424,8 +425,6 @@ def crossing_timing(dev, stream, peak, peak_src, steps=(120, 129, 141, 160)):
     A, B = binding.to_device(a_np, dev), binding.to_device(b_np, dev)
     del a_np, b_np
     col = binding.Collider(A, B, wl.dt, wl.kappa, precision=binding.FP32_BAND, stream=stream)
-    tuned = col.autotune([steps[1]], os.path.join(ROOT, "paper_1608_01125_gb300",
-                                                  "_tuning_cache.json"))
     col.timing(True)
     rows = []
     for k in steps:
@@ -447,7 +446,7 @@ def crossing_timing(dev, stream, peak, peak_src, steps=(120, 129, 141, 160)):
     ach = PAIR_OPS_PER_TEST * sum(r["narrow_tests"] for r in rows) / (tt / 1e3)
     tot = sum(sum(r[p] for p in PHASES) for r in rows)
     return {"workload": wl.name, "photons_per_beam": wl.a.n, "time_steps_timed": list(steps),
-            "tuning": tuned, "ms_per_step": tot / len(rows), "per_step": rows,
+            "ms_per_step": tot / len(rows), "per_step": rows,
             "narrow_tests_per_s": sum(r["narrow_tests"] for r in rows) / (tot / 1e3),
             "collided_pairs_per_s": sum(r["hits"] for r in rows) / (tot / 1e3),
             "traverse_roofline": {"bound": "alu", "achieved": ach, "peak": FP32_OPS_PEAK,
@@ -630,7 +629,7 @@ def run_ours(args, wl):
             if rank == 0 and not args.no_depletion else None)
     ipr = (ip_regime_timing(dev, stream, cpu=not args.no_cpu_baseline)
            if rank == 0 and not args.no_ip else None)
-    crossing = (crossing_timing(dev, stream, *read_peaks())
+    crossing = (crossing_timing(dev, stream)
                 if rank == 0 and not args.no_crossing else None)
     # the learned statistical regime on a 2 x 1e6 sample of the statistical
     # workload's shape (config 3's full size runs with --workload statistical)
@@ -800,11 +799,11 @@ def surrogate_eval(n, kappa, L, train_seeds, test_seed, taus=(1e30,), epochs=30,
     (weights U[1,10], Gamma(2, 5 MeV) energies, head-on Gaussian beams,
     32 steps of 20 fs) with n macro-photons per beam: a network trained on
     the draws train_seeds (all steps, level L) estimates the draw test_seed.
-    The exact GPU traversal of the same steps, with autotuned knobs, is the
+    The exact GPU path of the same steps is the
     reference for the yield error and the time; beside the network: the
     paper's ST rate of the same node pairs (no network, no fitted scale) and
     that rate times the one scale fitted on the training pairs.  Device times
-    with CUDA events: exact = frontier + traversal + narrow phase + band +
+    with CUDA events: exact = descent + narrow phase + band +
     yield after each step's build; surrogate = cut traversal, features,
     network, estimate and the exact fallback."""
     import torch
@@ -834,10 +833,8 @@ def surrogate_eval(n, kappa, L, train_seeds, test_seed, taus=(1e30,), epochs=30,
     exact = ms_exact = ms_build = 0.0
     acc = {t: dict(sur=0.0, st=0.0, ms=0.0, pairs=0, fb=0) for t in taus}
     with binding.Collider(a0, b0, wl0.dt, kappa) as col:
-        trained_knobs = col.tuning()  # the hierarchy the network was trained on
-        tuned = col.autotune([wl0.steps // 2 - 1, wl0.steps // 2, wl0.steps // 2 + 1])
         col.timing(True)
-        for k in range(wl0.steps):  # the exact traversal with the fastest knobs
+        for k in range(wl0.steps):  # the exact path
             col.phase_ms(reset=True)
             col.build(k)
             col.collide(k)
@@ -845,8 +842,6 @@ def surrogate_eval(n, kappa, L, train_seeds, test_seed, taus=(1e30,), epochs=30,
             ms_exact += sum(ph[p] for p in ("expand", "traverse", "narrow", "band", "yield"))
             ms_build += sum(ph[p] for p in ("propagate", "sort", "gather", "emit", "refit"))
             exact += col.stats()["weighted"]
-        col.set_tuning(*[trained_knobs[k] for k in ("leaf_bucket", "stack_depth", "block_shape",
-                                                    "budget")])
         col.surrogate_load(model)
         for k in range(wl0.steps):  # the surrogate on the level-L cut it was trained on
             for t in taus:
@@ -870,8 +865,7 @@ def surrogate_eval(n, kappa, L, train_seeds, test_seed, taus=(1e30,), epochs=30,
                     "fallback_pairs": q["fb"]})
     return {"photons_per_beam": n, "kappa": kappa, "level_L": L, "time_steps": wl0.steps,
             "train": f"seeds {list(train_seeds)}, all steps", "test": f"seed {test_seed}, all steps",
-            "train_samples": info["samples"], "train_s": t_train, "exact_tuning": tuned,
-            "results": out}
+            "train_samples": info["samples"], "train_s": t_train, "results": out}
 
 
 def run_statistical(args):
@@ -893,8 +887,7 @@ def run_statistical(args):
                            "time_steps": wl.steps, "level_L": args.level, "tau": q["tau"],
                            "train": r["train"], "test": r["test"]},
                 **{k: v for k, v in q.items() if k != "tau"},
-                "train_samples": r["train_samples"], "train_s": r["train_s"],
-                "exact_tuning": r["exact_tuning"]}
+                "train_samples": r["train_samples"], "train_s": r["train_s"]}
         print(json.dumps(line), flush=True)
 
 
