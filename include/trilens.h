@@ -7,8 +7,8 @@
  * during the step (Sec. 2.1: a BV grows by the distance its particles travel in
  * one step, so collisions are found before they happen), descends it with groups
  * of the other beam's photons by the axis-aligned overlap test (Eq. CollDet;
- * depth first, Sec. 2.2), and tests the surviving photon pairs.  A pair (i in A, j in B) collides in step
- * k when
+ * depth first, Sec. 2.2), and tests the surviving photon pairs.  A pair (i in A, j
+ * in B) collides in step k when
  *     s = E_i E_j (1 - cos Phi) / (2 m_e^2 c^4) > 1           (Eq. eq.Cond)
  *     t* = time of the pair's closest approach, 0 <= t* - t_k < dt
  *     d(t*)^2 < r^2 = kappa sigma(s) / pi,  sigma from Eq. BWcross
@@ -102,7 +102,8 @@ typedef struct {
 } trilens_step_stats;
 
 /* Create a context for beams a and b (both kept by pointer; arrays must stay
- * valid).  Allocates the workspace for both beams.  Returns INVALID for
+ * valid and unchanged: FP32 copies and the extremes of positions, directions and
+ * energies are taken here, and decide what every step leaves out).  Allocates the workspace for both beams.  Returns INVALID for
  * n < 0, n >= 2^27, missing arrays, dt <= 0, kappa <= 0 or tuning fields out
  * of range; NOMEM if the workspace does not fit. */
 int trilens_create(trilens_ctx **out, const trilens_beam *a, const trilens_beam *b,
@@ -142,7 +143,8 @@ int trilens_yield(trilens_ctx *c, int32_t mode, int32_t level_L, double *count,
 /* Run time steps first_step .. first_step+steps-1 of a single (non-batch)
  * context -- trilens_build + trilens_collide_step for each, in step order --
  * as one captured CUDA graph on the context's stream, with no host round
- * trip between steps.  The graph is captured on the first call and replayed while (first_step, steps) stay the same.  Adds the
+ * trip between steps.  The graph is captured on the first call and replayed while (first_step,
+ * steps) stay the same and no call in between replaced a buffer that it holds.  Adds the
  * run's yield to the cumulative yield; out (host, may be NULL) receives the
  * run's totals: step = steps, count, weighted, the checksums (hsum summed,
  * hxor xored over the steps) and the work counters.  Hit lists are not

@@ -36,8 +36,8 @@ int trilens_debug_set_parts(trilens_ctx *c, int32_t parts);
 int trilens_debug_set_spin_limit(trilens_ctx *c, int64_t limit);
 
 /* Resolution of a single context's keys: bits per axis of the statistical regime's
- * Morton keys (4..21), and three times as many (at most 30) for the exact path's
- * Hilbert keys.  The hit set never depends on it (the hierarchy only prunes); tests
+ * Morton keys (4..21), and three times as many in all, at most the default, for the exact
+ * path's cells.  The hit set never depends on it (the hierarchy only prunes); tests
  * use it to check that, and to time the sort against tree quality.  The next
  * collisions need a fresh build.  INVALID for a NULL or batch context or bits
  * outside 4..21. */

@@ -676,9 +676,11 @@ static int join_builds(trilens_ctx *c, bool fork) {
 
 // Photon pairs are told by their needles (tl_set_needles) in steps where more than this
 // many photons of the tree's beam have swept boxes that meet a photon's, at the beam's
-// density: 614 in the step of 2 x 4M photons that they take from 6.60 to 4.62 ms, 11 in the
-// run of 2 x 1M (10.1 and 10.4 ms), 0.8 in the step of 2 x 16M (3.70 and 3.99 ms).  Batches
-// keep the boxes (2 x 64 instances of up to 131072 photons 6.9 and 7.2 ms).
+// density.  Time of a step with boxes over that with needles, 75 steps of 60,000 to 4M photons
+// of four shapes, head-on, at 0.6 and at 1.57 rad: 0.91 to 1.03 where 5 to 45 boxes meet a
+// photon's, 0.87 to 1.09 at 45 to 65, 0.97 to 1.14 at 65 to 120, 0.99 to 1.31 at 120 to 270, 1.25
+// to 1.8 at 360 to 1340 (2 x 4M photons 6.60 to 4.62 ms); below 1 beyond 65 only at 1.57 rad, by 3 %.
+// Batches keep the boxes (2 x 64 instances of up to 131072 photons 6.9 and 7.2 ms).
 constexpr double kNeedlePairs = 64.0;
 
 // The ordering grids of a single problem's beams for the step with travel T to the
@@ -714,7 +716,8 @@ static void step_grids(trilens_ctx *c, double T, TLGrid g[2]) {
     }
     if (h == c->tree) near = (double)c->beam[h].n / vol;
     g[h] = tl_make_grid(lo, range, s, c->order_bits[h]);
-    tl_beam_box(c->ext[1 - h], c->ext[1 - h][12], c->ext[1 - h][13], c->frame0, T - 0.5 * c->L64, c->L64, c->half, g[h].clo, g[h].chi);
+    const double *e = c->ext[1 - h];
+    tl_beam_box(e, e[12], e[13], c->frame0, T - 0.5 * c->L64, c->L64, c->half, g[h].clo, g[h].chi);
   }
   c->needles = c->frame0.axis >= 0 && near > kNeedlePairs;
 }
@@ -901,7 +904,7 @@ static int status_failure(trilens_ctx *c, unsigned trav_st, unsigned build_st) {
   CK(cudaStreamSynchronize(c->stream));
   if (build_st & TL_ST_TIMEOUT)
     return fail(c, TRILENS_ERR_TIMEOUT,
-                "a device wait reached spin_limit=%lld (the radix sort's look-back)",
+                "a device wait reached spin_limit=%lld (the look-back of a build's scan or sort)",
                 (long long)c->p.spin_limit);
   if (trav_st & TL_ST_TIMEOUT)
     return fail(c, TRILENS_ERR_TIMEOUT,

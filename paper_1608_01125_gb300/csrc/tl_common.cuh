@@ -109,7 +109,7 @@ struct TLRunAcc {
   double weighted;
   unsigned long long hsum, hxor;
   unsigned long long narrow_tests, node_tests, leaf_pairs, band;
-  unsigned long long max_hits, max_band, max_handed;  // largest per-step list and queue sizes
+  unsigned long long max_hits, max_band;  // largest per-step list sizes
   unsigned long long max_leaves;
 };
 

@@ -59,7 +59,9 @@ constexpr int kThreads = 1024;
 // is then a chain of L2 round trips instead of two grid barriers and the lists.  One SM's
 // share of the L2 sets the line: with 8 hits per thread in this tail a step of 2 x 2048
 // photons (17,000 hits) takes 363 us, with 4 305, 2 277, 1 272, and with a quarter of
-// that 284.
+// that 284.  Depletions of 300 to 1M hits among 4096 to 1M photons, unit and mixed weights (26
+// cases): 1 hit per thread is the fastest or within 4 % of it everywhere, 2 take up to 14 %
+// longer and 4 up to 57 %.
 constexpr int kTailHits = 1;
 constexpr long long kTail = kTailHits * kThreads;
 
@@ -650,7 +652,7 @@ static int dep_launch(trilens_ctx *c, int64_t step, const uint32_t *hits, int64_
   g.ctl = d.ctl;
   g.dirty = d.dirty;
   g.out = out;
-  g.spin = c->p.spin_limit;  // iterations of 64 ns sleeps per barrier wait
+  g.spin = c->p.spin_limit;  // polls of a barrier's counter per wait, 32 ns of sleep between them
   // a block per 512 hits (see k_deplete's order of warps): more spread the t* phase further,
   // and lengthen the barriers (50,000 photons' step: 209 us at 1024, 194 at 512, 204 at 256)
   const long long nblk = (n_hits + 511) / 512;

@@ -155,8 +155,8 @@ __device__ __forceinline__ bool group_mma(FwdSmem &S, int g, uint32_t d, const v
 // GELU on the CUDA cores (384 erff per row against 72 kFLOP of products); one group of
 // 128 threads per SM left its schedulers idle between dependent instructions and during
 // its own products, so a block runs four groups, each with its own rows, accumulator
-// columns and barrier, around one copy of the weights.  200,003 rows: 197 us with one
-// group, TL_FWD_US now.
+// columns and barrier, around one copy of the weights.  A call for 200,003 rows: 423 us with
+// one group and allocations on every call (197 us of it the kernel), 137 us now.
 __global__ void __launch_bounds__(kThreads, 1)
     k_mlp_forward(const float *__restrict__ prm, const float *__restrict__ norm,
                   const float *__restrict__ x, int64_t M, float *out, int *err, long long spin) {

@@ -626,7 +626,6 @@ __global__ void k_step_finish(const TLCounters *ctr, unsigned *run_status, TLRun
     acc->band += ctr->band;
     if (ctr->hits > acc->max_hits) acc->max_hits = ctr->hits;
     if (ctr->band > acc->max_band) acc->max_band = ctr->band;
-    if (ctr->q_tail > acc->max_handed) acc->max_handed = ctr->q_tail;
     if (ctr->max_part_leaves > acc->max_leaves) acc->max_leaves = ctr->max_part_leaves;
   }
 }

@@ -371,9 +371,9 @@ cudaError_t launch_static(const TLBeam &b, float4 *stat, cudaStream_t s) {
 
 // Every photon's cell, from its swept box's centre in the frame (FP32), counted there:
 // the count it finds is its rank in the cell.  With the cells' running sum that is its
-// place, so a beam is ordered by one counting sort with 2 to 4 cells per photon (three
-// or four radix passes took 29 us each for 1M photons; the scan takes 13 us, the move
-// 30).
+// place, so a beam is ordered by one counting sort with 2 to 4 cells per photon, half a cell
+// for beams beyond 16M photons (three or four radix passes took 29 us each for 1M photons;
+// the scan takes 13 us, the move 30).
 // The order inside a cell is that of the atomics and changes from run to run; it shapes
 // the tree and nothing else.  A photon whose swept box misses the box of the whole other
 // beam is left out of the step here: its 32 bytes are all that is read of it.  The test
@@ -446,7 +446,7 @@ cudaError_t launch_order(const OrderArgs &a, cudaStream_t s) {
 // over the preceding tiles' words 32 at a time (Merrill and Garland 2016, "Single-pass
 // parallel prefix scan with decoupled look-back").  Tiles are numbered in the order blocks
 // start, so a tile only waits on running ones; every wait is bounded by spin (then
-// TL_ST_TIMEOUT is recorded and the sums are not used).  Words: 2 flag bits and a 27-bit
+// TL_ST_TIMEOUT is recorded and the sums are not used).  Words: 2 flag bits and a 28-bit
 // sum (beams hold fewer than 2^27 photons), cleared by k_order.
 constexpr int kScanThreads = 1024, kScanCells = 16, kScanTile = kScanThreads * kScanCells;
 constexpr uint32_t kScanSum = 1u << 30, kScanPre = 2u << 30, kScanVal = (1u << 28) - 1u;
