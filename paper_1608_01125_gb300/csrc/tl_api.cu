@@ -734,15 +734,17 @@ static int build_exact(trilens_ctx *c, int64_t step) {
                             c->stream));
   else
     step_grids(c, T, grid);
-  c->exact_step = step;
-  c->full_step = -1;  // the two builds share the sorted photons
+  c->exact_step = c->full_step = -1;  // the two builds share the sorted photons
   // The root of the descent, tested on the host: where the boxes of all swept boxes of
   // the two beams do not meet (Eq. CollDet), no photon of one meets one of the other,
   // and the step has nothing to order or to test.
   c->apart = c->beam[0].n <= 0 || c->beam[1].n <= 0;
   for (int k = 0; k < 3 && !batch; ++k)
     c->apart = c->apart || grid[0].clo[k] > grid[1].chi[k] || grid[1].clo[k] > grid[0].chi[k];
-  if (c->apart) return TRILENS_OK;
+  if (c->apart) {
+    c->exact_step = step;
+    return TRILENS_OK;
+  }
   bool fork;
   if (int rc = fork_builds(c, &fork)) return rc;
   for (int k = 0; k < 2; ++k) {
@@ -806,12 +808,15 @@ static int build_exact(trilens_ctx *c, int64_t step) {
     tmark(c, PH_REFIT, k, 1);
     c->phase_launches[PH_REFIT] += c->max_top >= 3 ? 2 : 1;
   }
-  return join_builds(c, fork);
+  if (int rc = join_builds(c, fork)) return rc;
+  c->exact_step = step;
+  return TRILENS_OK;
 }
 
 // The statistical regime's binary hierarchies of both beams, in Morton order.
 static int build_full(trilens_ctx *c, int64_t step) {
   if (int rc = ensure_full(c)) return rc;
+  c->exact_step = c->full_step = -1;
   const double ct = TL_C * ((double)step * c->p.dt_fs);
   const double T = ct + 0.5 * c->L64;
   bool fork;
@@ -865,7 +870,6 @@ static int build_full(trilens_ctx *c, int64_t step) {
   }
   if (int rc = join_builds(c, fork)) return rc;
   c->full_step = step;
-  c->exact_step = -1;
   return TRILENS_OK;
 }
 
@@ -1211,6 +1215,7 @@ static int capture_run(trilens_ctx *c, int64_t first, int64_t steps, double *yie
     rc = build_exact(c, k);
     if (rc == TRILENS_OK && !c->apart) rc = graph_collide(c, k, yields);
   }
+  c->exact_step = -1;  // (captured, not built)
   cudaGraph_t g = nullptr;
   e = cudaStreamEndCapture(c->cap_stream, &g);
   c->stream = saved;
